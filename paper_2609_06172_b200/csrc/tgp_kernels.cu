@@ -1204,11 +1204,11 @@ static void launch_gemv(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, 
     tgpk_last_gemm_kernel = "tgp_wstream_kernel";
 }
 
-// Same product for blocks with two to eight 16-row groups per SM: one CTA owns ROWS rows of W and its NW warps split K
+// Same product for blocks of a short K with two to eight 16-row groups per SM: one CTA owns ROWS rows of W and its NW warps split K
 // (interleaved chunks of 32*U), so n/ROWS CTAs of NW warps fill the machine where n/16 warps would not.  The partial
 // tiles meet in shared memory and are summed in warp order: deterministic.  RPC <= ROWS: rows a CTA owns (the tile's
 // remaining rows re-read its last row and are not stored; a row's sum does not depend on its place in the tile).
-// (Blocks of fewer rows take tgp_wstream_mma_group_kernel.)
+// (Blocks of fewer rows or a longer K take tgp_wstream_mma_group_kernel.)
 template <int NB, int U, int NW, int ROWS, int RPC = ROWS>
 __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const bf16 *A, const bf16 *__restrict__ W, float *__restrict__ C,
                                                               uint32_t Mrows, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int accumulate) {
@@ -1267,7 +1267,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const b
     }
 }
 
-// The product for blocks of fewer than two 16-row groups per SM, one block or a list of blocks that read the same
+// The product for 3 - 32 activation rows on blocks of few rows or of a long K (pick_skinny), one block or a list of blocks that read the same
 // activations (the pieces of one matrix; the q, k and v projections): one persistent CTA per SM walks the row groups
 // as one list, RG consecutive groups at a time, whose MMAs share each activation fragment - every CTA reads its K
 // slices of all activation rows from L2, so at 16 rows per CTA that traffic equals the weights'; RG row groups divide
@@ -1457,6 +1457,10 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
 // ROWS rows.  The choice depends on the block alone, so a block computes the same bits alone or as part of a group.
 struct SkinnyPick { int nb, u, nw, rows; bool split, persistent; };
 
+// 17 - 32 activation rows on a block of at least this many weight rows: the tiled GEMM with the weights as its 128-row operand is
+// ahead of the weight-streaming kernels (n=8192, K=8192, M=32: 33 us against 41 us)
+constexpr uint32_t TILES_WIN_ROWS = 8065;
+
 static int device_sms() {
     static int sms = 0;
     if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
@@ -1468,13 +1472,22 @@ static SkinnyPick pick_skinny(uint32_t M, uint32_t n, uint32_t K) {
     SkinnyPick k;
     k.nb = M <= 8 ? 1 : M <= 16 ? 2 : 4;
     k.split = n < 16u * 8u * sms;                         // too few 16-row groups to give every SM eight warps
-    // fewer than two 16-row groups per SM: one persistent CTA per SM walks the row groups of the block, or of a list of such
-    // blocks (tgp_wstream_mma_group_kernel).  One choice per class of M for all of them, so that the pieces of a matrix share
-    // a launch whatever the rows of its last piece:
+    // One persistent CTA per SM walks the row groups of the block, or of a list of such blocks (tgp_wstream_mma_group_kernel).
+    // It is bound by HBM: its loads never drain between row groups (n=14336, K=4096: 18.5 us = 6.36 TB/s at M=8, 23.2 us at
+    // M=16; one CTA per row group took 22.7 and 31.6 us.  n=32000, K=4096, M=8: 40.1 us against 55.3 us of one warp per 16
+    // rows).  Its warps share K in chunks of 4096 columns, so a short K leaves most of them without work: with two or more
+    // row groups per SM it is taken from K=3072 on at M <= 8 (K=2048: ahead from five row groups per SM on - n=32000: 23.1 us
+    // against 29.5 us, n=6144: 6.3 us against 5.6 us) and from K=4096 on at M <= 32 (K=2048, M=16, n=12288: 15.1 us against 11.5 us).
+    // Up to 16 rows that holds for any n; 17 - 32 rows on 8192 or more weight rows take the tiled GEMM (tgpk_gemm).
+    // One choice per class of M for all of them, so that the pieces of a matrix share a launch whatever the rows of its
+    // last piece:
     //   M <= 8   16 warps, 8 load steps per warp and chunk
     //   M <= 16  8 warps of twice the registers, 16 load steps: room for the activation fragments of a register set
     //   M <= 32  the same with 8 load steps (four groups of activation rows take the registers)
-    k.persistent = k.split && groups16 < 2u * sms;
+    const bool few = k.split && groups16 < 2u * sms;
+    const bool deep = k.nb == 1 ? K >= 3072 || (K >= 2048 && groups16 >= 5u * sms) : K >= 4096 && (M <= 16 || n < TILES_WIN_ROWS);
+    k.persistent = few || deep;
+    if (k.persistent) k.split = true;
     if (k.persistent) {
         k.nw = k.nb == 1 ? 16 : 8;
         k.u = k.nb == 1 ? 8 : k.nb == 2 ? 16 : 8;
@@ -1701,9 +1714,7 @@ int tgpk_gemm(const void *A, const void *W, float *C, uint32_t M, uint32_t n, ui
     if (!M || !n) return TGP_OK;
     if (K % 8 || !K) return TGP_E_INVAL;
     const bf16 *a = (const bf16 *)A, *w = (const bf16 *)W;
-    // 17 - 32 activation rows on a block of 64 or more 128-row tiles: the tiled GEMM with the weights as its 128-row operand
-    // is ahead of the weight-streaming kernel (n=8192, K=8192, M=32: 33 us against 41 us)
-    const bool tiles_win = M > 16 && (n + 127) / 128 >= 64 && g_gemm_impl == 0;
+    const bool tiles_win = M > 16 && n >= TILES_WIN_ROWS && g_gemm_impl == 0;
     if (M >= 3 && M <= 32 && K % 32 == 0 && g_skinny_impl == 0 && !tiles_win) {
         GemvParts p;
         memset(&p, 0, sizeof(p));

@@ -706,3 +706,25 @@ def test_skinny_tensor_core_gemv_matches_oracle_and_cuda_core_path(M, n, K, accu
     assert np.abs(outs[0] - outs[1]).max() < 2e-5 * scale + 1e-7
     for out in outs:
         assert np.array_equal(out[:, :4], c0[:, :4]) and np.array_equal(out[:, 4 + n:], c0[:, 4 + n:])
+
+
+# blocks on either side of the lines that send a product of 3 - 32 rows to the persistent list kernel: K below / at 2048 and 3072
+# (M <= 8) and 4096 (M <= 32), row counts around five 16-row groups per SM, a ragged last group, a K that ends inside a warp's chunk
+@pytest.mark.parametrize("M,ns,K", [(3, (4737,), 3072), (8, (4800, 4737), 3104), (8, (11840, 12000), 2048), (5, (11800,), 2080), (9, (4737, 5000), 4096),
+                                    (16, (9001,), 4128), (17, (4737, 8064), 4096), (32, (8065,), 4096)])
+def test_blocks_of_many_rows_take_the_list_kernel_with_the_same_bits_alone_and_in_a_list(M, ns, K):
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(M * K + len(ns))
+    A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
+    Ws = [(torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16() for n in ns]
+    c0 = [torch.randn((M, n), device=DEV, generator=gen) for n in ns]
+    alone, listed = [c.clone() for c in c0], [c.clone() for c in c0]
+    for W, C, n in zip(Ws, alone, ns):
+        tb.k_gemm(A, W, C, M, n, K, n, 0, True)
+    tb.k_gemm_group(A, Ws, listed, M, list(ns), K, list(ns), True)
+    torch.cuda.synchronize()
+    for W, a, b, c in zip(Ws, alone, listed, c0):
+        assert torch.equal(a, b)
+        want = A.double() @ W.double().T + c.double()
+        # fp32 sums of K products of N(0, 1) x N(0, 0.02): errors of a few 2^-24 of the partial sums' size, bounded as in the tests above
+        assert float((a.double() - want).abs().max()) < 2e-5 * float(want.abs().max())
