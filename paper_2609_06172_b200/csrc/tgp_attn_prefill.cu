@@ -2,7 +2,10 @@
 // (64 queries, query head, sequence).  Flash-style: K/V blocks of 64 keys are gathered through the KV tile
 // pointer table with cp.async (double-buffered), S = Q K^T and O += P V run on mma.sync m16n8k16 (bf16 in,
 // fp32 accumulate), the softmax is online (running max / sum per row) in registers.  P is rounded to bf16
-// for the second product; that is the one rounding of this path the CPU oracle does not mirror.
+// for the second product; that is the one rounding of this path the CPU oracle does not mirror.  Where no row has more
+// than 64 keys (SPLIT_P, one key block) what that rounding leaves over is multiplied with V too, so P counts with 16 bits: with
+// few keys nothing averages the rounding out (one layer of the Mixtral widths, 16 keys: largest logit error 0.033 -> 0.020),
+// and one block costs 0.2 us more (3.1 -> 3.3 us); with 1600 keys it would be 67 -> 80 us and gain nothing.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cstdint>
@@ -49,7 +52,7 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
 // the 8 rows an ldmatrix phase reads fall into different banks
 template <int DH> __device__ __forceinline__ uint32_t tile_off(uint32_t r, uint32_t c) { return r * (DH * 2) + ((c ^ (r & 7u)) << 4); }
 
-template <int DH>
+template <int DH, bool SPLIT_P>
 __global__ void __launch_bounds__(128) tgp_attn_prefill_mma_kernel(PArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     constexpr int CH = DH / 8;                              // 16-byte chunks per row
@@ -151,12 +154,22 @@ __global__ void __launch_bounds__(128) tgp_attn_prefill_mma_kernel(PArgs a) {
         for (int kk = 0; kk < BN / 16; ++kk) {
             uint32_t pf[4] = {pack2(s[2 * kk][0], s[2 * kk][1]), pack2(s[2 * kk][2], s[2 * kk][3]),
                               pack2(s[2 * kk + 1][0], s[2 * kk + 1][1]), pack2(s[2 * kk + 1][2], s[2 * kk + 1][3])};
+            uint32_t pl[4];
+            if constexpr (SPLIT_P) {                        // what the rounding of P left over
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 h = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162 *>(&pf[i]));
+                    const float *sv = &s[2 * kk + (i >> 1)][(i & 1) * 2];
+                    pl[i] = pack2(sv[0] - h.x, sv[1] - h.y);
+                }
+            }
 #pragma unroll
             for (int nt = 0; nt < DH / 8; nt += 2) {
                 uint32_t b0, b1, b2, b3;
                 ldsm4t(smem_u32(Vst + tile_off<DH>(kk * 16 + (lane & 7) + 8 * ((lane >> 3) & 1), nt + (lane >> 4))), b0, b1, b2, b3);
                 mma16816(o[nt], pf, b0, b1);
                 mma16816(o[nt + 1], pf, b2, b3);
+                if constexpr (SPLIT_P) { mma16816(o[nt], pl, b0, b1); mma16816(o[nt + 1], pl, b2, b3); }
             }
         }
         __syncthreads();                                    // everyone is done with this stage before it is refilled
@@ -183,22 +196,20 @@ __global__ void __launch_bounds__(128) tgp_attn_prefill_mma_kernel(PArgs a) {
 
 extern thread_local uint64_t tgpk_launches;
 
-int tgpk_attn_prefill_tc(const void *qb, const TgpTilePtrs &tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0, cudaStream_t st) {
-    PArgs a{(const bf16 *)qb, (bf16 *)ob, c->Hq, c->Hkv, c->TK, q_len, pos0, 1.4426950408889634f / sqrtf((float)c->Dh), tiles};
-    dim3 grid((q_len + BM - 1) / BM, c->Hq, B);
-    static bool attr64 = false, attr128 = false;
-    if (c->Dh == 64) {
-        constexpr int SM = (BM + 4 * BN) * 64 * 2;
-        if (!attr64) { if (cudaFuncSetAttribute(tgp_attn_prefill_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM) != cudaSuccess) return TGP_E_CUDA; attr64 = true; }
-        tgp_attn_prefill_mma_kernel<64><<<grid, 128, SM, st>>>(a);
-    } else if (c->Dh == 128) {
-        constexpr int SM = (BM + 4 * BN) * 128 * 2;
-        if (!attr128) { if (cudaFuncSetAttribute(tgp_attn_prefill_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM) != cudaSuccess) return TGP_E_CUDA; attr128 = true; }
-        tgp_attn_prefill_mma_kernel<128><<<grid, 128, SM, st>>>(a);
-    } else {
-        return TGP_E_INVAL;
-    }
+template <int DH, bool SPLIT_P>
+static int launch(const PArgs &a, uint32_t B, cudaStream_t st) {
+    constexpr int SM = (BM + 4 * BN) * DH * 2;
+    static bool attr_set = false;
+    if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_prefill_mma_kernel<DH, SPLIT_P>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM) != cudaSuccess) return TGP_E_CUDA; attr_set = true; }
+    tgp_attn_prefill_mma_kernel<DH, SPLIT_P><<<dim3((a.q_len + BM - 1) / BM, a.Hq, B), 128, SM, st>>>(a);
     if (cudaGetLastError() != cudaSuccess) return TGP_E_CUDA;
     tgpk_launches += 1;
     return TGP_OK;
+}
+
+int tgpk_attn_prefill_tc(const void *qb, const TgpTilePtrs &tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0, cudaStream_t st) {
+    PArgs a{(const bf16 *)qb, (bf16 *)ob, c->Hq, c->Hkv, c->TK, q_len, pos0, 1.4426950408889634f / sqrtf((float)c->Dh), tiles};
+    if (c->Dh == 64) return pos0 + q_len <= BN ? launch<64, true>(a, B, st) : launch<64, false>(a, B, st);
+    if (c->Dh == 128) return pos0 + q_len <= BN ? launch<128, true>(a, B, st) : launch<128, false>(a, B, st);
+    return TGP_E_INVAL;
 }
