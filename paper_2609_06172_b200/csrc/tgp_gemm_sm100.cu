@@ -14,7 +14,9 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
+#include <algorithm>
 #include <cstdint>
+#include <cstring>
 #include "tgp.h"
 #include "tgp_kernels.h"
 #include "tgp_sm100.cuh"
@@ -337,158 +339,380 @@ __global__ void __launch_bounds__(192, 1) tgp_matmul_tc_persistent_kernel(const 
     }
 }
 
-// ---- paired variant: one 256 x 256 tile per CTA pair (cta_group::2) -------------------------------------------------
+// ---- paired variant: tiles of 256 weight rows x up to 256 activation rows per CTA pair (cta_group::2) ----------------
 // What limits the kernel above is not the tensor pipe but what an SM can pull from L2: 48 KB per 64-wide K block is
-// 54 B per clock, and the MMA thread waits for data a third of the time.  Here the two CTAs of a cluster sit on the two
-// SMs of a TPC and share one MMA of M = 256: each loads its own 128 rows of A and HALF of the 256 rows of W (B), 32 KB
-// per K block for the same arithmetic per SM; a stage holds two K blocks (128 wide: half the barrier hand-overs of 64-wide
-// stages, 4 % faster), three stages deep.  Only the even CTA (the leader) issues MMAs; the TMA loads
-// of both CTAs count on the leader's `full` barrier; an MMA commit arrives on the `empty` / `acc_full` barriers of both
-// CTAs; both CTAs drain their own 128 rows of the accumulator from their own TMEM and arrive (the odd one remotely) on
-// the leader's `acc_empty`.  No multicast load anywhere.  Same bounded waits and error word; a cluster barrier before
-// TMEM is freed keeps either CTA from leaving while its partner still works on its memory.
-constexpr int Q_HALVES = 2, Q_STAGES = 6 / Q_HALVES;   // a stage holds Q_HALVES 64-wide K blocks
+// 54 B per clock, and the MMA thread waits for data a third of the time.  Here the two CTAs of a pair sit on the two
+// SMs of a TPC and share one MMA: its 256 rows are WEIGHT rows (128 per CTA), its N columns activation rows, of which each
+// CTA loads half - 32 KB per K block at N = 256 for the same arithmetic per SM.  Weights as rows means that a warp's 32
+// TMEM lanes are 32 consecutive columns of C: every store, residual add and gate load of the epilogue is one full line of
+// one output row (with activations as rows each lane walked a row of its own: the SwiGLU epilogue of 32768 x 4096 x 4096
+// took 1280 us against 970 us of the plain one), and N follows the batch: ceil(M / tiles) rounded up to 32, so that M = 603
+// costs 3 x 224 rows and not 3 x 256.
+//   Parts.  Up to TGP_GEMM_GROUP_MAX weight blocks that read the same activations are walked as one list of tiles.
+//   Pairs are persistent, with two accumulators in TMEM: the epilogue of a tile overlaps the MMAs of the next.
+//   A stage holds two 64-wide K blocks (half the barrier hand-overs of one, 4 % faster), p.stages of them.  Only the
+// even CTA of a pair (its leader) issues MMAs; the TMA loads of both CTAs count on the leader's `full` barrier; an MMA
+// commit arrives on the `empty` / `acc_full` barriers of both; the epilogue warps of both arrive on the leader's `acc_empty`.
+// No multicast load anywhere.  Same bounded waits and error word; a cluster barrier before TMEM is freed keeps a CTA from
+// leaving while its partner may still touch its memory.
+//   The launch is a programmatic dependent one: barriers, TMEM and tensor maps are set up while the previous kernel drains.
+constexpr int Q_WARPS = 10, Q_EPI = Q_WARPS - 2;       // TMA, MMA, eight epilogue warps (two per TMEM lane quarter)
+constexpr int KH = 2;                                  // 64-wide K blocks per stage
 
-__global__ void __launch_bounds__(192, 1) tgp_matmul_tc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                                                              float *__restrict__ C, uint32_t M, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int accumulate, const Epi ep) {
+struct ListArgs {
+    CUtensorMap x, w[TGP_GEMM_GROUP_MAX];
+    float *C[TGP_GEMM_GROUP_MAX];
+    uint32_t n[TGP_GEMM_GROUP_MAX], ldc[TGP_GEMM_GROUP_MAX], tiles[TGP_GEMM_GROUP_MAX];      // tiles: of weight rows, per part
+    uint32_t count, tiles_n, M, N, tiles_m, K, stages, slices;                              // N: activation rows per tile
+    int accumulate;
+    Epi ep;                                                                                 // with one part only
+};
+
+// 32 activation rows of one column of C, from element offset `at` on, `cnt` of them inside the matrix.  A warp's lanes are neighbouring
+// columns: every access is one full line of one row.  The gates are all requested before the first is used; a product
+// added to C goes out as one add per element by one thread - the rounded sum of load, add and store, but not waited for.
+__device__ __forceinline__ void store32(const ListArgs &p, uint32_t part, size_t at, uint32_t ldc, const float (&v)[32], uint32_t cnt) {
+    if (p.ep.aout) {
+        const float *g = p.ep.gate + at;
+        __nv_bfloat16 *a = p.ep.aout + at;
+        float gv[32];
+#pragma unroll
+        for (uint32_t j = 0; j < 32; ++j) gv[j] = j < cnt ? g[(size_t)j * ldc] : 0.f;
+#pragma unroll
+        for (uint32_t j = 0; j < 32; ++j)
+            if (j < cnt) a[(size_t)j * ldc] = __float2bfloat16_rn(gv[j] / (1.0f + expf(-gv[j])) * v[j]);
+        return;
+    }
+    float *C = p.C[part] + at;
+    if (p.accumulate) {
+#pragma unroll
+        for (uint32_t j = 0; j < 32; ++j) if (j < cnt) atomicAdd(C + (size_t)j * ldc, v[j]);
+    } else {
+#pragma unroll
+        for (uint32_t j = 0; j < 32; ++j) if (j < cnt) C[(size_t)j * ldc] = v[j];
+    }
+}
+
+__global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(const __grid_constant__ ListArgs p) {
     extern __shared__ uint8_t smem_raw[];
-    constexpr int A_BYTES = BM * BK * 2, B_BYTES = (P_BN / 2) * BK * 2, STAGE_BYTES = Q_HALVES * (A_BYTES + B_BYTES);
-    constexpr int QK = Q_HALVES * BK;
+    constexpr uint32_t W_BYTES = BM * BK * 2;                     // one K block of this CTA's 128 weight rows
+    const uint32_t N = p.N, ST = p.stages;
+    const uint32_t X_BYTES = N / 2 * BK * 2, HALF = W_BYTES + X_BYTES, STAGE = KH * HALF;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + Q_STAGES * STAGE_BYTES);      // used in the leader only
-    uint64_t *empty = full + Q_STAGES;
-    uint64_t *acc_full = empty + Q_STAGES;           // [2]
-    uint64_t *acc_empty = acc_full + 2;              // [2], used in the leader only: 4 warps of each CTA
+    // barriers ahead of the ring (the first 1024 bytes): full[8], empty[8], acc_full[2], acc_empty[2], TMEM slot, flag
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem);          // used in the leader only
+    uint64_t *empty = full + 8;
+    uint64_t *acc_full = empty + 8;                               // [2]
+    uint64_t *acc_empty = acc_full + 2;                           // [2], used in the leader only: the epilogue warps of both CTAs
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
     volatile uint32_t *failed = tmem_slot + 1;
+    uint8_t *ring = smem + 1024;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank(), pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
-    const uint32_t num_k = (K + QK - 1) / QK;
-    const uint32_t tiles_m = (M + 2 * BM - 1) / (2 * BM), tiles_n = (n + P_BN - 1) / P_BN, tiles = tiles_m * tiles_n;
+    const uint32_t num_k = (p.K + KH * BK - 1) / (KH * BK);                         // stages per tile; a block past K reads zeros
+    const uint32_t tiles = p.tiles_m * p.tiles_n;
+    const uint32_t buf_cols = N <= 64 ? 64u : N <= 128 ? 128u : 256u;               // TMEM columns of one accumulator
 
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (threadIdx.x == 0) {
-        for (int s = 0; s < Q_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 8); }
+        for (uint32_t s = 0; s < 8; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * Q_EPI); }
         *failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 2) {                                  // the same warp in both CTAs of the pair
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2 * buf_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    cluster_sync_all();                               // barriers of both CTAs initialised, TMEM allocated
+    cluster_sync_all();                               // barriers of all CTAs initialised, TMEM allocated
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
 
-    auto tile_origin = [&](uint32_t tile, uint32_t &m0, uint32_t &n0) {       // of the pair's 256 x 256 tile
-        const uint32_t group = tile / (GROUP_M * tiles_n), first_m = group * GROUP_M;
-        const uint32_t rows_in_group = min((uint32_t)GROUP_M, tiles_m - first_m);
-        const uint32_t in_group = tile - group * GROUP_M * tiles_n;
-        m0 = (first_m + in_group % rows_in_group) * (2 * BM);
-        n0 = (in_group / rows_in_group) * P_BN;
+    // Tile order: groups of GROUP_M activation tiles are swept across all weight tiles before the next group starts (see the
+    // per-tile kernel above).  part: the weight block, w0: first weight row of the tile in it, m0: first activation row
+    auto tile_origin = [&](uint32_t tile, uint32_t &part, uint32_t &w0, uint32_t &m0) {
+        const uint32_t group = tile / (GROUP_M * p.tiles_n), first_m = group * GROUP_M;
+        const uint32_t rows_in_group = min((uint32_t)GROUP_M, p.tiles_m - first_m);
+        const uint32_t in_group = tile - group * GROUP_M * p.tiles_n;
+        m0 = (first_m + in_group % rows_in_group) * N;
+        uint32_t wt = in_group / rows_in_group;
+        part = 0;
+        while (part + 1 < p.count && wt >= p.tiles[part]) wt -= p.tiles[part++];
+        w0 = wt * (2 * BM);
     };
 
     if (warp == 0) {
-        if (lane == 0) {                              // TMA thread of this CTA: its rows of A, its half of B
-            uint32_t it = 0, armed = 0;
+        if (lane == 0) {                              // TMA thread of this CTA: its 128 weight rows, its half of the activation rows
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            uint32_t it = 0, s = 0, ph = 0;
             const uint32_t withhold = pair == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;     // test hook: both CTAs of the first pair never load this stage
-            for (uint32_t tile = pair; tile < tiles; tile += pairs) {
-                uint32_t m0, n0;
-                tile_origin(tile, m0, n0);
-                bool ok = true;
+            bool ok = true;
+            for (uint32_t tile = pair; tile < tiles && ok; tile += pairs) {
+                uint32_t part, w0, m0;
+                tile_origin(tile, part, w0, m0);
+                const CUtensorMap *mw = &p.w[part];
                 for (uint32_t kb = 0; kb < num_k; ++kb, ++it) {
-                    const uint32_t s = it % Q_STAGES, ph = (it / Q_STAGES) & 1;
                     if (it == withhold) { ok = false; break; }
                     if (*failed || !mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } ok = false; break; }
-                    if (rank == 0) mbar_expect_tx(&full[s], 2 * STAGE_BYTES);
+                    if (rank == 0) mbar_expect_tx(&full[s], 2 * STAGE);
 #pragma unroll
-                    for (int h = 0; h < Q_HALVES; ++h) {
-                        tma_load_2d_pair(smem + s * STAGE_BYTES + h * (A_BYTES + B_BYTES), &tmA, (int)(kb * QK + h * BK), (int)(m0 + rank * BM), &full[s]);
-                        tma_load_2d_pair(smem + s * STAGE_BYTES + h * (A_BYTES + B_BYTES) + A_BYTES, &tmB, (int)(kb * QK + h * BK), (int)(n0 + rank * (P_BN / 2)), &full[s]);
+                    for (int h = 0; h < KH; ++h) {
+                        const int k = (int)((kb * KH + h) * BK);
+                        tma_load_2d_pair(ring + s * STAGE + h * HALF, mw, k, (int)(w0 + rank * BM), &full[s]);
+                        tma_load_2d_pair(ring + s * STAGE + h * HALF + W_BYTES, &p.x, k, (int)(m0 + rank * (N / 2)), &full[s]);
                     }
-                    armed = it + 1;
+                    if (++s == ST) { s = 0; ph ^= 1; }
                 }
-                if (!ok) break;
             }
             if (*failed && rank == 0) {               // loads of both CTAs still in flight land on these barriers (bounded wait)
                 volatile uint32_t never = 0;
-                for (uint32_t q = armed > Q_STAGES ? armed - Q_STAGES : 0; q < armed; ++q) mbar_wait(&full[q % Q_STAGES], (q / Q_STAGES) & 1, &never);
+                for (uint32_t q = it > ST ? it - ST : 0; q < it; ++q) mbar_wait(&full[q % ST], (q / ST) & 1, &never);
             }
         }
+        __syncwarp();
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {                 // MMA thread of the pair
-            constexpr uint32_t idesc = umma_idesc_pair(P_BN);
-            uint32_t it = 0, lt = 0;
+            const uint32_t idesc = umma_idesc_pair(N);
+            uint32_t s = 0, ph = 0, lt = 0;
             bool ok = true;
             for (uint32_t tile = pair; tile < tiles && ok; tile += pairs, ++lt) {
                 const uint32_t buf = lt & 1, use = lt >> 1;
                 if (*failed || !mbar_wait(&acc_empty[buf], (use & 1) ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | 0x80 | (int)buf); } break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t tacc = tmem_base + buf * P_BN;
-                for (uint32_t kb = 0; kb < num_k; ++kb, ++it) {
-                    const uint32_t s = it % Q_STAGES, ph = (it / Q_STAGES) & 1;
+                const uint32_t tacc = tmem_base + buf * buf_cols;
+                for (uint32_t kb = 0; kb < num_k; ++kb) {
                     if (*failed || !mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-                    for (uint32_t h = 0; h < Q_HALVES; ++h) {
-                        const uint64_t da = umma_desc(smem_u32(smem + s * STAGE_BYTES + h * (A_BYTES + B_BYTES)));
-                        const uint64_t db = umma_desc(smem_u32(smem + s * STAGE_BYTES + h * (A_BYTES + B_BYTES) + A_BYTES));
+                    for (uint32_t h = 0; h < KH; ++h) {
+                        const uint64_t dw = umma_desc(smem_u32(ring + s * STAGE + h * HALF));
+                        const uint64_t dx = umma_desc(smem_u32(ring + s * STAGE + h * HALF + W_BYTES));
 #pragma unroll
-                        for (uint32_t k = 0; k < BK / 16; ++k) umma_pair(tacc, da + 2 * k, db + 2 * k, idesc, (kb | h | k) != 0);
+                        for (uint32_t k = 0; k < BK / 16; ++k) umma_pair(tacc, dw + 2 * k, dx + 2 * k, idesc, (kb | h | k) != 0);
                     }
                     umma_commit_pair(&empty[s]);
+                    if (++s == ST) { s = 0; ph ^= 1; }
                 }
                 if (ok) umma_commit_pair(&acc_full[buf]);
             }
         }
+        __syncwarp();
     } else {
-        const uint32_t quarter = warp & 3;
-        const bool vec = ((ldc | col0) & 3u) == 0 && (reinterpret_cast<uintptr_t>(C) & 15u) == 0;
+        asm volatile("griddepcontrol.wait;" ::: "memory");        // what C, the gate and a hold is the previous kernel's work
+        const uint32_t quarter = warp & 3, half = (warp - 2) >> 2, wrow = rank * BM + quarter * 32 + lane;
         uint32_t lt = 0;
         for (uint32_t tile = pair; tile < tiles; tile += pairs, ++lt) {
             const uint32_t buf = lt & 1, use = lt >> 1;
+            uint32_t part, w0, m0;
+            tile_origin(tile, part, w0, m0);
             bool ready = !*failed && mbar_wait(&acc_full[buf], use & 1, failed);
             if (!ready && !*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, 3 << 8); }
             ready = __all_sync(0xffffffffu, ready && !*failed);
             if (!ready) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            uint32_t m0, n0;
-            tile_origin(tile, m0, n0);
-            const uint32_t row = m0 + rank * BM + quarter * 32 + lane;
+            const uint32_t row = w0 + wrow, ldc = p.ldc[part], rows = min(N, p.M - m0);      // this lane's column of C; activation rows of the tile
+            const bool mine = row < p.n[part];
 #pragma unroll 1
-            for (uint32_t c = 0; c < P_BN / 32; ++c) {
+            for (uint32_t c = half * 32; c < N; c += 64) {        // 32 activation rows at a time
                 float v[32];
-                tmem_ld32(tmem_base + ((quarter * 32) << 16) + buf * P_BN + c * 32, v);
-                const uint32_t col = n0 + c * 32;
-                if (row < M && col < n) {
-                    float *dst = C + (size_t)row * ldc + col0 + col;
-                    if (ep.aout) swiglu_store32(ep, (size_t)row * ldc + col0 + col, v, min(32u, n - col));
-                    else if (vec && col + 32 <= n) {
-#pragma unroll
-                        for (int j = 0; j < 32; j += 4) {
-                            float4 o = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                            if (accumulate) { const float4 old = *reinterpret_cast<const float4 *>(dst + j); o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
-                            *reinterpret_cast<float4 *>(dst + j) = o;
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (col + j < n) dst[j] = accumulate ? dst[j] + v[j] : v[j];
-                    }
-                }
+                tmem_ld32(tmem_base + ((quarter * 32) << 16) + buf * buf_cols + c, v);
+                store32(p, part, (size_t)(m0 + c) * ldc + row, ldc, v, mine && c < rows ? rows - c : 0);
             }
-            // this warp has read its quarter of this CTA's half of the buffer: tell the pair's MMA thread
+            // this warp has read its share of this CTA's half of the buffer: tell the pair's MMA thread
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive_remote(&acc_empty[buf], 0);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncwarp();
     cluster_sync_all();                               // neither CTA frees TMEM or leaves while its partner may still touch it
     if (warp == 2) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * buf_cols) : "memory");
+    }
+}
+
+// ---- up to 128 activation rows, and products of few tiles: one tile of 128 weight rows per CTA ----------------------
+// A product of up to 128 activation rows is bound by HBM, one of more rows and few tiles by the length of K.  Every CTA takes 128
+// weight rows (the rows of the MMA; N <= 128 activation rows, a multiple of 16, are its columns) and a slice of K.  One CTA
+// per MMA and not a pair: an MMA costs 75 cycles for N <= 128, a pair's 128 for any N <= 256 (112 SMs of pairs would take
+// their weights in no faster than HBM delivers them), and there are four times as many tiles to share out.
+//   K slices: a block of few tiles is split along K over the SL CTAs of a cluster; their partial tiles meet in shared memory
+// and are summed pairwise.  The split depends on M, n and K alone: a block computes the same bits alone or in a list.
+//   Ring: 200 KB where the launch gives an SM one CTA (M=61, n=14336, K=4096: 24.9 us; 28.4 us with 100 KB), else 100 KB, so that
+// an SM holds two (28672 rows: 43.0 us; 50.3 us with 200 KB).
+constexpr uint32_t S_RING = 100 * 1024, S_RING_LONE = 200 * 1024, S_STAGES = 12;
+
+// Sum of the SL partial tiles of a cluster ([activation row][128 weight rows] fp32 at `addr` in every CTA), neighbours first: J activation
+// rows `stride` bytes apart, four weight rows each.  All loads are under way before the first sum (a load
+// from another CTA of the cluster takes about 0.3 us).
+template <int SL, int J>
+__device__ __forceinline__ void sum_slices(uint32_t addr, uint32_t stride, float4 (&sum)[J]) {
+    float4 v[SL][J];
+#pragma unroll
+    for (uint32_t q = 0; q < SL; ++q)
+#pragma unroll
+        for (uint32_t j = 0; j < J; ++j) v[q][j] = ld_remote_f32x4(addr + j * stride, q);
+#pragma unroll
+    for (uint32_t w = 1; w < SL; w *= 2)
+#pragma unroll
+        for (uint32_t q = 0; q < SL; q += 2 * w)
+#pragma unroll
+            for (uint32_t j = 0; j < J; ++j) {
+                v[q][j].x += v[q + w][j].x; v[q][j].y += v[q + w][j].y; v[q][j].z += v[q + w][j].z; v[q][j].w += v[q + w][j].w;
+            }
+#pragma unroll
+    for (uint32_t j = 0; j < J; ++j) sum[j] = v[0][j];
+}
+
+// four consecutive columns of one row of C (element offset `at` in its geometry, `cnt` of them inside the matrix)
+__device__ __forceinline__ void store4(float *C, size_t at, const float4 &v, uint32_t cnt, int accumulate, const Epi &ep, bool vec) {
+    const float f[4] = {v.x, v.y, v.z, v.w};
+    if (ep.aout) {
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i)
+            if (i < cnt) { const float g = ep.gate[at + i]; ep.aout[at + i] = __float2bfloat16_rn(g / (1.0f + expf(-g)) * f[i]); }
+    } else if (accumulate) {
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) if (i < cnt) atomicAdd(C + at + i, f[i]);
+    } else if (vec && cnt == 4) {
+        *reinterpret_cast<float4 *>(C + at) = v;
+    } else {
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) if (i < cnt) C[at + i] = f[i];
+    }
+}
+
+__global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_constant__ ListArgs p) {
+    extern __shared__ uint8_t smem_raw[];
+    constexpr uint32_t W_BYTES = BM * BK * 2;
+    const uint32_t N = p.N, ST = p.stages, SL = p.slices, STAGE = W_BYTES + N * BK * 2;
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    // barriers ahead of the ring (the first 1024 bytes): full[S_STAGES], empty[S_STAGES], acc_full, TMEM slot, flag
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem), *empty = full + S_STAGES, *acc_full = empty + S_STAGES;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_full + 1);
+    volatile uint32_t *failed = tmem_slot + 1;
+    uint8_t *ring = smem + 1024;
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t slice = SL > 1 ? cluster_ctarank() : 0, tile = blockIdx.x / SL;
+    const uint32_t kblocks = (p.K + BK - 1) / BK, kb_lo = kblocks * slice / SL, num_k = kblocks * (slice + 1) / SL - kb_lo;
+    const uint32_t cols = N <= 32 ? 32u : N <= 64 ? 64u : 128u;                     // TMEM columns
+    const uint32_t m0 = tile % p.tiles_m * N, rows = min(N, p.M - m0);              // this tile's activation rows
+    uint32_t part = 0, wt = tile / p.tiles_m;
+    while (part + 1 < p.count && wt >= p.tiles[part]) wt -= p.tiles[part++];
+    const uint32_t w0 = wt * BM;
+    const CUtensorMap *mw = &p.w[part];
+
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (threadIdx.x == 0) {
+        for (uint32_t s = 0; s < S_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        mbar_init(acc_full, 1);
+        *failed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&p.x) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(mw) : "memory");
+    }
+    if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            uint32_t s = 0, ph = 0, armed = 0;
+            const uint32_t withhold = blockIdx.x == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;     // test hook: this stage is never loaded
+            for (uint32_t kb = 0; kb < num_k; ++kb) {
+                if (kb == withhold) break;
+                if (*failed || !mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } break; }
+                mbar_expect_tx(&full[s], STAGE);
+                tma_load_2d(ring + s * STAGE, mw, (int)((kb_lo + kb) * BK), (int)w0, &full[s]);
+                tma_load_2d(ring + s * STAGE + W_BYTES, &p.x, (int)((kb_lo + kb) * BK), (int)m0, &full[s]);
+                armed = kb + 1;
+                if (++s == ST) { s = 0; ph ^= 1; }
+            }
+            if (*failed) {
+                volatile uint32_t never = 0;
+                for (uint32_t q = armed > ST ? armed - ST : 0; q < armed; ++q) mbar_wait(&full[q % ST], (q / ST) & 1, &never);
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = umma_idesc((int)N);
+            uint32_t s = 0, ph = 0;
+            bool ok = true;
+            for (uint32_t kb = 0; kb < num_k; ++kb) {
+                if (*failed || !mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t dw = umma_desc(smem_u32(ring + s * STAGE)), dx = umma_desc(smem_u32(ring + s * STAGE + W_BYTES));
+#pragma unroll
+                for (uint32_t k = 0; k < BK / 16; ++k) umma(tmem_base, dw + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
+                umma_commit(&empty[s]);
+                if (++s == ST) { s = 0; ph ^= 1; }
+            }
+            if (ok) umma_commit(acc_full);
+        }
+        __syncwarp();
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");        // what C holds is the previous kernel's work
+        bool ready = !*failed && mbar_wait(acc_full, 0, failed);
+        if (!ready && !*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, 3 << 8); }
+        ready = __all_sync(0xffffffffu, ready && !*failed);
+        if (ready) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t quarter = warp & 3, wrow = quarter * 32 + lane, row = w0 + wrow, ldc = p.ldc[part];
+            const bool mine = row < p.n[part];
+#pragma unroll 1
+            for (uint32_t c = 0; c < N; c += 32) {
+                float v[32];
+                tmem_ld32(tmem_base + ((quarter * 32) << 16) + c, v);          // (N = 16, 48, ...: the columns past N are not used)
+                if (SL > 1) {                                      // this slice's partial over the idle ring
+                    float *part_s = reinterpret_cast<float *>(ring) + wrow;
+#pragma unroll
+                    for (uint32_t j = 0; j < 32; ++j) if (c + j < N) part_s[(c + j) * BM] = v[j];
+                    continue;
+                }
+                const size_t at = (size_t)(m0 + c) * ldc + row;
+                store32(p, part, at, ldc, v, mine && c < rows ? rows - c : 0);
+            }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    }
+    if (SL > 1) {
+        cluster_sync_all();                           // every slice's partial tile is in its CTA's shared memory
+        if (warp >= 2) {
+            uint32_t bad = 0;
+            for (uint32_t q = 0; q < SL; ++q) bad |= ld_remote_u32(smem_u32((const void *)failed), q);
+            const uint32_t row = w0 + 4 * lane, n = p.n[part], ldc = p.ldc[part], ew = warp - 2, j_hi = N * (slice + 1) / SL;
+            const uint32_t cnt = bad || row >= n ? 0u : min(4u, n - row), base = smem_u32(ring) + lane * 16;
+            const bool vec = (ldc & 3u) == 0 && (reinterpret_cast<uintptr_t>(p.C[part]) & 15u) == 0;
+            for (uint32_t j0 = N * slice / SL + ew; j0 < j_hi; j0 += 8) {
+                float4 sum[2];                                     // rows j0 and j0 + 4 (past this slice's share: read, not stored)
+                const uint32_t at = base + j0 * (BM * 4);
+                if (SL == 2) sum_slices<2, 2>(at, 4 * BM * 4, sum);
+                else sum_slices<4, 2>(at, 4 * BM * 4, sum);
+#pragma unroll
+                for (uint32_t j = 0; j < 2; ++j) {
+                    const uint32_t m = j0 + 4 * j;
+                    if (m < rows && m < j_hi) store4(p.C[part], (size_t)(m0 + m) * ldc + row, sum[j], cnt, p.accumulate, p.ep, vec);
+                }
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();                           // no CTA leaves while another may still read its partial tile
+    } else {
+        __syncthreads();
+    }
+    if (warp == 2) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(cols) : "memory");
     }
 }
 
@@ -514,8 +738,138 @@ static bool launch_tile(const CUtensorMap &ma, const CUtensorMap &mb, float *C, 
     return true;
 }
 
-static int g_tc_variant = 0;     // 0 auto, 1 force the 128x128 per-tile kernel, 2 the persistent 128x256 kernel, 3 the paired 256x256 kernel,
+static int g_tc_variant = 0;     // 0 and 3 the paired kernel, 1 force the 128x128 per-tile kernel, 2 the persistent 128x256 kernel,
                                  // 4 the per-tile kernel with the weights as the 128-row operand (M <= 128 only; else as 0)
+
+bool tgpk_gemm_tc_forced() { return g_tc_variant != 0; }
+
+static uint32_t tc_sms() {
+    static int sms = 0;
+    if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
+    return (uint32_t)sms;
+}
+
+// K slices of a block in the one-tile-per-CTA kernel, 0: the paired kernel serves it.  The choice depends on M, n and K of the block
+// alone.  Measured (us; M=61 unless stated):
+//   n=4096, K=4096        22.4 unsplit, 15.3 in two slices, 11.9 in four, 12.4 in eight
+//   n=2048, K=8192        41.6, 24.7, 15.4, 21.1 (few clusters of eight fit the GPU at a time: no eight anywhere)
+//   n=8192, K=8192        42.4, 28.1, 26.4 (256 CTAs, two per SM)
+//   n=8192 twice, K=2048  14.4, 16.5, 22.2; n=32000, K=4096: 46.2, 51.3, 62.3
+//   M=509, n=2048, K=8192 22.7 in four slices, 33.9 in pairs; M=200, n=4096, K=14336: 35.2, 55.5; M=603, n=4096+1024+1024, K=4096:
+//                         26.5 in pairs, 35 with k and v in slices of their own; M=256, n=4096+1024+1024 and 4096, K=4096: 39.6 in pairs, 45.8
+static uint32_t cta_slices(uint32_t M, uint32_t n, uint32_t K) {
+    const uint32_t tiles = (n + BM - 1) / BM * ((M + BM - 1) / BM), sms = tc_sms();
+    if (tiles * 4 <= 2 * sms && K >= 8192) return 4;
+    if (M > BM) return 0;
+    if (tiles * 4 <= sms && K >= 1024) return 4;
+    return tiles * 2 <= sms && K >= 1024 ? 2 : 1;
+}
+
+// Estimated cycles of the paired kernel for `wt` tiles of 256 weight rows at M activation rows in tiles of N: a K block of a
+// pair takes 512 cycles of the tensor pipe at any N <= 256, and (16384 + 64 N) bytes per SM from L2 at 40 bytes a clock.
+static uint64_t pair_cost(uint32_t M, uint32_t wt, uint32_t K, uint32_t N, uint32_t pairs) {
+    const uint64_t kblocks = (K + BK - 1) / BK, tiles = (uint64_t)((M + N - 1) / N) * wt;
+    return (tiles + pairs - 1) / pairs * (kblocks * std::max<uint64_t>(512, (16384 + 64 * N) / 40) + 600);
+}
+
+// Activation rows per tile: the fewest tiles that hold M rows, or up to two more where smaller tiles fill the pairs better.
+static uint32_t pair_rows(uint32_t M, uint32_t wt, uint32_t K, uint32_t pairs) {
+    const uint32_t t0 = (M + 255) / 256;
+    uint32_t best = 0;
+    uint64_t cost = 0;
+    for (uint32_t t = t0; t <= (g_tc_variant == 3 ? t0 : t0 + 2); ++t) {                 // (forced: the largest tiles)
+        const uint32_t N = ((M + t - 1) / t + 31) / 32 * 32;
+        const uint64_t c = pair_cost(M, wt, K, N, pairs);
+        if (!best || c < cost) { best = N; cost = c; }
+    }
+    return best;
+}
+
+static int launch_pair(ListArgs &p, cudaStream_t st) {
+    constexpr uint32_t RING = 227u * 1024u - 2048u;
+    static bool attr_set = false;
+    if (!attr_set) {
+        if (cudaFuncSetAttribute(tgp_matmul_tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, RING + 2048) != cudaSuccess) return TGP_E_CUDA;
+        attr_set = true;
+    }
+    const uint32_t stage = KH * (BM * BK * 2 + p.N / 2 * BK * 2);
+    p.stages = std::min(8u, RING / stage);
+    const uint32_t tiles = p.tiles_m * p.tiles_n, pairs_max = tc_sms() / 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * std::min(tiles, pairs_max));
+    cfg.blockDim = dim3(Q_WARPS * 32);
+    cfg.dynamicSmemBytes = 2048 + p.stages * stage;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, tgp_matmul_tc_pair_kernel, p) == cudaSuccess ? TGP_OK : TGP_E_CUDA;
+}
+
+static int launch_stream(ListArgs &p, cudaStream_t st) {
+    static bool attr_set = false;
+    if (!attr_set) {
+        if (cudaFuncSetAttribute(tgp_wstream_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, S_RING_LONE + 2048) != cudaSuccess) return TGP_E_CUDA;
+        attr_set = true;
+    }
+    const uint32_t stage = BM * BK * 2 + p.N * BK * 2, ctas = p.tiles_m * p.tiles_n * p.slices;
+    p.stages = std::min(S_STAGES, (ctas <= tc_sms() ? S_RING_LONE : S_RING) / stage);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(192);
+    cfg.dynamicSmemBytes = 2048 + std::max(p.stages * stage, p.slices > 1 ? p.N * (uint32_t)BM * 4u : 0u);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = p.slices; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = p.slices > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, tgp_wstream_tc_kernel, p) == cudaSuccess ? TGP_OK : TGP_E_CUDA;
+}
+
+uint32_t tgpk_gemm_tc_class(uint32_t M, uint32_t n, uint32_t K) { return cta_slices(M, n, K) + 1; }
+
+// Blocks of equal tgpk_gemm_tc_class() over the same activations, in one launch.
+int tgpk_gemm_tc_list(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t M, uint32_t K,
+                      int accumulate, cudaStream_t st, const float *gate, void *aout) {
+    if (!count || count > TGP_GEMM_GROUP_MAX || !M || !K || K % 8) return TGP_E_INVAL;
+    ListArgs p;
+    memset(&p, 0, sizeof(p));
+    p.ep = Epi{aout ? gate : nullptr, gate ? (__nv_bfloat16 *)aout : nullptr};
+    if (p.ep.aout && (accumulate || count != 1)) return TGP_E_INVAL;
+    const bool stream = g_tc_variant != 3 && cta_slices(M, n[0], K) != 0;
+    const uint32_t rows_w = stream ? BM : 2 * BM;
+    uintptr_t bits = reinterpret_cast<uintptr_t>(A);
+    for (uint32_t s = 0; s < count; ++s) {
+        bits |= reinterpret_cast<uintptr_t>(W[s]);
+        p.C[s] = C[s]; p.n[s] = n[s]; p.ldc[s] = ldc[s]; p.tiles[s] = (n[s] + rows_w - 1) / rows_w;
+        p.tiles_n += p.tiles[s];
+    }
+    if (bits & 15u) return TGP_E_INVAL;                                                                  // TMA needs 16-byte aligned bases
+    p.count = count; p.M = M; p.K = K; p.accumulate = accumulate;
+    if (stream) {
+        p.slices = cta_slices(M, n[0], K);
+        const uint32_t t = (M + BM - 1) / BM;
+        p.N = ((M + t - 1) / t + 15) / 16 * 16;
+    } else {
+        p.slices = 1;
+        p.N = pair_rows(M, p.tiles_n, K, tc_sms() / 2);
+    }
+    p.tiles_m = (M + p.N - 1) / p.N;
+    if (!make_map(&p.x, A, M, K, stream ? p.N : p.N / 2)) return TGP_E_CUDA;
+    for (uint32_t s = 0; s < count; ++s) if (!make_map(&p.w[s], W[s], n[s], K, BM)) return TGP_E_CUDA;
+    const int rc = stream ? launch_stream(p, st) : launch_pair(p, st);
+    if (rc) return rc;
+    tgpk_launches += 1;
+    tgpk_last_gemm_kernel = stream ? "tgp_wstream_tc_kernel" : "tgp_matmul_tc_pair_kernel";
+    return TGP_OK;
+}
 
 int tgpk_gemm_tc(const void *A, const void *W, float *C, uint32_t M, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int accumulate, cudaStream_t st,
                  const float *gate, void *aout) {
@@ -524,15 +878,13 @@ int tgpk_gemm_tc(const void *A, const void *W, float *C, uint32_t M, uint32_t n,
     if (ep.aout && accumulate) return TGP_E_INVAL;
     if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W)) & 15u) return TGP_E_INVAL;     // TMA needs 16-byte aligned bases
     if (K % 8) return TGP_E_INVAL;                                                                       // and 16-byte row strides
-    static int sms = 0;
-    if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
-    // Up to 64 activation rows on a block with 128-row tiles for a good part of the SMs: the weights become the 128-row
-    // operand (see tgp_matmul_tc_kernel), the activations the narrow one.  A CTA takes in about 100 GB/s through its TMA ring
-    // whatever the tile, so the form pays from 64 weight tiles on (n=8192, K=8192, M=64: 34 us against 47 us), for more
-    // than 32 rows from 32 tiles on (n=4096, K=14336, M=64: 48 us against 70 us); with fewer tiles the weight-streaming
-    // kernels and the narrow tiles below have more CTAs at work
-    const uint32_t w_tiles = (n + BM - 1) / BM;
-    if (!ep.aout && M <= 128 && (g_tc_variant == 4 || (g_tc_variant == 0 && M <= 64 && (w_tiles >= 64 || (M > 32 && w_tiles >= 32))))) {
+    if (g_tc_variant == 0 || g_tc_variant == 3 || (g_tc_variant == 4 && (ep.aout || M > 128))) {
+        float *Cb = C + col0;
+        return tgpk_gemm_tc_list(A, 1, &W, &Cb, &n, &ldc, M, K, accumulate, st, gate ? gate + col0 : nullptr, aout ? (__nv_bfloat16 *)aout + col0 : nullptr);
+    }
+    // the kernels of one CTA per tile, by request only (they cross-check the paired one)
+    const uint32_t sms = tc_sms();
+    if (g_tc_variant == 4) {                                     // the weights as the 128-row operand, M <= 128
         CUtensorMap mw, mx;
         const uint32_t bx = M <= 32 ? 32 : M <= 64 ? 64 : 128;
         if (!make_map(&mw, W, n, K, BM) || !make_map(&mx, A, M, K, bx)) return TGP_E_CUDA;
@@ -544,61 +896,27 @@ int tgpk_gemm_tc(const void *A, const void *W, float *C, uint32_t M, uint32_t n,
         tgpk_last_gemm_kernel = "tgp_matmul_tc_kernel (weights as the 128-row operand)";
         return TGP_OK;
     }
-    const uint32_t tiles_p = ((M + BM - 1) / BM) * ((n + P_BN - 1) / P_BN);
-    const uint32_t tiles_q = ((M + 2 * BM - 1) / (2 * BM)) * ((n + P_BN - 1) / P_BN);
-    // measured on 8192 x {640 .. 4096} x {4096, 14336}, {1024 .. 4096} x 4096 x 4096 and {512, 1024} x 8192 x 2048: the paired
-    // kernel is ahead as soon as every pair of SMs has a 256 x 256 tile, the persistent one from about 64 tiles of 128 x 256
-    const bool paired = g_tc_variant == 3 || (g_tc_variant == 0 && 2 * tiles_q >= (uint32_t)sms);
-    const bool persistent = !paired && (g_tc_variant == 2 || (g_tc_variant == 0 && tiles_p >= 64u));
-    // small problems, one tile per CTA: an MMA into one accumulator costs the same 75 cycles for N = 32 as for N = 128, so
-    // a CTA's time is set by its K loop, and narrower tiles simply put more CTAs to work: the widest tile that still
-    // gives every SM one
-    const uint32_t tm = (M + BM - 1) / BM;
-    uint32_t bn = BN;
-    // ... as long as the A panel is not re-read by more than 32 column tiles (L2 bandwidth then takes over)
-    if (g_tc_variant == 0) while (bn > 32 && tm * ((n + bn - 1) / bn) < (uint32_t)sms && (n + bn / 2 - 1) / (bn / 2) <= 32) bn /= 2;
+    const bool persistent = g_tc_variant == 2;
     CUtensorMap ma, mb;
-    if (!make_map(&ma, A, M, K, BM) || !make_map(&mb, W, n, K, paired ? P_BN / 2 : persistent ? P_BN : bn)) return TGP_E_CUDA;
-    if (paired) {
-        constexpr int SMEM = Q_STAGES * Q_HALVES * (BM * BK * 2 + (P_BN / 2) * BK * 2) + 160 + 1024;
-        static bool attr_q = false;
-        if (!attr_q) {
-            if (cudaFuncSetAttribute(tgp_matmul_tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess) return TGP_E_CUDA;
-            attr_q = true;
-        }
-        const uint32_t pairs_max = (uint32_t)sms / 2, npairs = tiles_q < pairs_max ? tiles_q : pairs_max;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2 * npairs);
-        cfg.blockDim = dim3(192);
-        cfg.dynamicSmemBytes = SMEM;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, tgp_matmul_tc_pair_kernel, ma, mb, C, M, n, K, ldc, col0, accumulate, ep) != cudaSuccess) return TGP_E_CUDA;
-    } else if (persistent) {
+    if (!make_map(&ma, A, M, K, BM) || !make_map(&mb, W, n, K, persistent ? P_BN : BN)) return TGP_E_CUDA;
+    if (persistent) {
+        const uint32_t tiles_p = ((M + BM - 1) / BM) * ((n + P_BN - 1) / P_BN);
         constexpr int SMEM = P_STAGES * (BM * BK * 2 + P_BN * BK * 2) + 128 + 1024;
         static bool attr_p = false;
         if (!attr_p) {
             if (cudaFuncSetAttribute(tgp_matmul_tc_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess) return TGP_E_CUDA;
             attr_p = true;
         }
-        tgp_matmul_tc_persistent_kernel<<<tiles_p < (uint32_t)sms ? tiles_p : (uint32_t)sms, 192, SMEM, st>>>(ma, mb, C, M, n, K, ldc, col0, accumulate, ep);
-    } else if (bn == 128) {
+        tgp_matmul_tc_persistent_kernel<<<tiles_p < sms ? tiles_p : sms, 192, SMEM, st>>>(ma, mb, C, M, n, K, ldc, col0, accumulate, ep);
+    } else {
         // fewer tiles than SMs: one CTA per SM, so the ring may take all of shared memory (a 3-stage ring leaves a lone
         // CTA waiting on L2 latency); otherwise two CTAs per SM with three stages each
-        const bool lone = tm * ((n + 127) / 128) <= (uint32_t)sms;
+        const bool lone = ((M + BM - 1) / BM) * ((n + 127) / 128) <= sms;
         if (!(lone ? launch_tile<128, 2, 3>(ma, mb, C, M, n, K, ldc, col0, accumulate, st, ep) : launch_tile<128, 3, 1>(ma, mb, C, M, n, K, ldc, col0, accumulate, st, ep))) return TGP_E_CUDA;
-    } else if (bn == 64) {
-        if (!launch_tile<64, 3, 3>(ma, mb, C, M, n, K, ldc, col0, accumulate, st, ep)) return TGP_E_CUDA;
-    } else {
-        if (!launch_tile<32, 3, 3>(ma, mb, C, M, n, K, ldc, col0, accumulate, st, ep)) return TGP_E_CUDA;
     }
     if (cudaGetLastError() != cudaSuccess) return TGP_E_CUDA;
     tgpk_launches += 1;
-    tgpk_last_gemm_kernel = paired ? "tgp_matmul_tc_pair_kernel" : persistent ? "tgp_matmul_tc_persistent_kernel" : "tgp_matmul_tc_kernel";
+    tgpk_last_gemm_kernel = persistent ? "tgp_matmul_tc_persistent_kernel" : "tgp_matmul_tc_kernel";
     return TGP_OK;
 }
 

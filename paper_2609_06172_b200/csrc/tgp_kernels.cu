@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(256) tgp_wstream_splitk_kernel(const bf16 *A, 
     }
 }
 
-// ---- skinny GEMM for 3 <= M <= 32 activation rows: weight streaming through mma.sync ---------------------------
+// ---- skinny GEMM for 3 <= M <= 16 activation rows: weight streaming through mma.sync ---------------------------
 // out^T[16 rows of W, 8 activation rows] += W[16 x 16] * x^T[16 x 8] per instruction.  Each lane loads 16 contiguous
 // bytes (8 values of K) of W rows g and g+8 and of activation row g straight from global memory; the 8 values feed two
 // instructions.  Which physical k lands in which logical k-slot of the instruction does not matter for a dot product
@@ -1173,12 +1173,13 @@ int tgpk_rmsnorm(const float *x, uint32_t ldx, const void *g, void *h, uint32_t 
     return TGP_OK;
 }
 
-static int g_skinny_impl = 0;    // 0: tensor-core skinny kernel for 3 <= M <= 32; 1: CUDA-core GEMV (an on-device cross-check)
+static int g_skinny_impl = 0;    // 0: tensor-core skinny kernels for 3 <= M <= 16; 1: CUDA-core GEMV (an on-device cross-check)
 static int g_gemm_impl = 0;      // 0: tensor cores for M > 16; 1: CUDA-core tiles (kept as an on-device cross-check)
 static int g_gemv_splitk = 1;    // small-n blocks at M <= 2: CTA per RB rows with K split over its warps (0: one warp per row)
 static int g_gemm_group = 1;     // products over the same activations: one launch where the parts allow it (0: always one launch each)
 static int g_gemv_balance = 1;   // grouped skinny launches: rows per group chosen so that every persistent CTA gets the same number of groups
 static int g_gemv_pdl = 1;       // consecutive weight-streaming launches may overlap (programmatic dependent launch)
+bool tgpk_launch_overlap() { return g_gemv_pdl != 0; }
 
 template <int MT, int R, int U>
 static void launch_gemv(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int acc, cudaStream_t st) {
@@ -1267,7 +1268,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const b
     }
 }
 
-// The product for 3 - 32 activation rows on blocks of few rows or of a long K (pick_skinny), one block or a list of blocks that read the same
+// The product for 3 - 16 activation rows on blocks of few rows or of a long K (pick_skinny), one block or a list of blocks that read the same
 // activations (the pieces of one matrix; the q, k and v projections): one persistent CTA per SM walks the row groups
 // as one list, RG consecutive groups at a time, whose MMAs share each activation fragment - every CTA reads its K
 // slices of all activation rows from L2, so at 16 rows per CTA that traffic equals the weights'; RG row groups divide
@@ -1280,11 +1281,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
     constexpr int UL = ROWS == 8 ? 2 * U : U;             // half a tile per load step: twice the steps in flight
     constexpr int G = RG, SK = UL / (2 * G);              // a register set holds SK load steps of G groups: two sets are as many loads as UL steps of one group
     static_assert(UL % (2 * G) == 0 && SK >= 1, "row groups per CTA must divide half the load steps");
-    // the warps' partial tiles: static where they fit the 48 KB a kernel may declare, else the launch's dynamic shared memory
-    constexpr bool PART_DYNAMIC = (size_t)NW * G * NB * 4 * 32 * 4 > 48 * 1024;
-    __shared__ float part_static[PART_DYNAMIC ? 1 : NW * G * NB * 4 * 32];
-    extern __shared__ float part_dynamic[];
-    float (*part)[G * NB * 4][32] = reinterpret_cast<float (*)[G * NB * 4][32]>(PART_DYNAMIC ? part_dynamic : part_static);
+    __shared__ float part[NW][G * NB * 4][32];            // the warps' partial tiles
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, c = lane & 3;
     uint32_t grp0 = blockIdx.x * G;
     if (grp0 >= groups_total) return;
@@ -1452,14 +1449,22 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
     }
 }
 
-// Which skinny kernel serves a block of n rows at M activation rows: NB groups of 8 activation rows, U load steps in
+// Which skinny kernel serves a block of n rows at M activation rows: NB groups of 8 activation rows (M <= 16), U load steps in
 // flight, and for blocks too small to give every SM eight 16-row warps the split-K kernel with NW warps per CTA over
 // ROWS rows.  The choice depends on the block alone, so a block computes the same bits alone or as part of a group.
 struct SkinnyPick { int nb, u, nw, rows; bool split, persistent; };
 
-// 17 - 32 activation rows on a block of at least this many weight rows: the tiled GEMM with the weights as its 128-row operand is
-// ahead of the weight-streaming kernels (n=8192, K=8192, M=32: 33 us against 41 us)
+// 9 - 16 activation rows on a block of at least this many weight rows (64 tiles of 128): the tcgen05 kernel is ahead of the
+// mma.sync ones (M=16: n=28672, K=8192 76 us against 85 us; two blocks of 8192 rows, K=2048 15 us against 22 us; n=32000, K=4096
+// 46 us either way; below, n=4096, K=4096: 11.3 us against 8.4 us).  From 17 rows on it is ahead on blocks of any size (M=32:
+// n=6144 in three blocks, K=4096 14.7 us against 18.4 us; n=4096, K=14336 24 us against 35 us).
 constexpr uint32_t TILES_WIN_ROWS = 8065;
+
+// a product that the tcgen05 kernels serve (tgpk_gemm_tc)
+static bool takes_tiles(uint32_t M, uint32_t n, uint32_t K) {
+    if (g_gemm_impl || K % 8) return false;
+    return M > 16 || (M >= 9 && n >= TILES_WIN_ROWS && g_skinny_impl == 0 && !tgpk_gemm_tc_forced());
+}
 
 static int device_sms() {
     static int sms = 0;
@@ -1470,31 +1475,29 @@ static int device_sms() {
 static SkinnyPick pick_skinny(uint32_t M, uint32_t n, uint32_t K) {
     const uint32_t sms = (uint32_t)device_sms(), groups16 = (n + 15) / 16;
     SkinnyPick k;
-    k.nb = M <= 8 ? 1 : M <= 16 ? 2 : 4;
+    k.nb = M <= 8 ? 1 : 2;
     k.split = n < 16u * 8u * sms;                         // too few 16-row groups to give every SM eight warps
     // One persistent CTA per SM walks the row groups of the block, or of a list of such blocks (tgp_wstream_mma_group_kernel).
     // It is bound by HBM: its loads never drain between row groups (n=14336, K=4096: 18.5 us = 6.36 TB/s at M=8, 23.2 us at
     // M=16; one CTA per row group took 22.7 and 31.6 us.  n=32000, K=4096, M=8: 40.1 us against 55.3 us of one warp per 16
     // rows).  Its warps share K in chunks of 4096 columns, so a short K leaves most of them without work: with two or more
     // row groups per SM it is taken from K=3072 on at M <= 8 (K=2048: ahead from five row groups per SM on - n=32000: 23.1 us
-    // against 29.5 us, n=6144: 6.3 us against 5.6 us) and from K=4096 on at M <= 32 (K=2048, M=16, n=12288: 15.1 us against 11.5 us).
-    // Up to 16 rows that holds for any n; 17 - 32 rows on 8192 or more weight rows take the tiled GEMM (tgpk_gemm).
+    // against 29.5 us, n=6144: 6.3 us against 5.6 us) and from K=4096 on at M <= 16 (K=2048, M=16, n=12288: 15.1 us against 11.5 us).
     // One choice per class of M for all of them, so that the pieces of a matrix share a launch whatever the rows of its
     // last piece:
     //   M <= 8   16 warps, 8 load steps per warp and chunk
     //   M <= 16  8 warps of twice the registers, 16 load steps: room for the activation fragments of a register set
-    //   M <= 32  the same with 8 load steps (four groups of activation rows take the registers)
     const bool few = k.split && groups16 < 2u * sms;
-    const bool deep = k.nb == 1 ? K >= 3072 || (K >= 2048 && groups16 >= 5u * sms) : K >= 4096 && (M <= 16 || n < TILES_WIN_ROWS);
+    const bool deep = k.nb == 1 ? K >= 3072 || (K >= 2048 && groups16 >= 5u * sms) : K >= 4096;
     k.persistent = few || deep;
     if (k.persistent) k.split = true;
     if (k.persistent) {
         k.nw = k.nb == 1 ? 16 : 8;
-        k.u = k.nb == 1 ? 8 : k.nb == 2 ? 16 : 8;
+        k.u = k.nb == 1 ? 8 : 16;
         k.rows = 16;
     } else {
         k.nw = 8;
-        k.u = M <= 16 ? 4 : 2;
+        k.u = 4;
         k.rows = 16;
     }
     return k;
@@ -1565,16 +1568,6 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
             if (per_cta == 4) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 8, 16, 4>, A, p, Mrows, total, K, acc, rpc, early);
             else if (per_cta == 2) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 8, 16, 2>, A, p, Mrows, total, K, acc, rpc, early);
             else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 8, 16, 1>, A, p, Mrows, total, K, acc, rpc, early);
-        } else if constexpr (NB == 4 && U == 8) {
-            if (per_cta == 4) {
-                // four groups of 32 activation rows: the warps' partial tiles take 64 KB of dynamic shared memory
-                constexpr size_t smem = (size_t)8 * 4 * NB * 4 * 32 * 4;
-                static bool attr_set = false;
-                if (!attr_set) { cudaFuncSetAttribute(tgp_wstream_mma_group_kernel<NB, U, 8, 16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); attr_set = true; }
-                cfg.dynamicSmemBytes = smem;
-                cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 8, 16, 4>, A, p, Mrows, total, K, acc, rpc, early);
-            } else if (per_cta == 2) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 8, 16, 2>, A, p, Mrows, total, K, acc, rpc, early);
-            else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 8, 16, 1>, A, p, Mrows, total, K, acc, rpc, early);
         }
     } else if constexpr (STREAMS) {
         if (!k.split) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_kernel<NB, U>, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);
@@ -1584,8 +1577,7 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
 
 static void launch_skinny_pick(const bf16 *A, const GemvParts &p, const SkinnyPick &k, uint32_t Mrows, uint32_t K, int acc, cudaStream_t st) {
     if (k.nb == 1) { if (k.u == 8) launch_skinny<1, 8>(A, p, k, Mrows, K, acc, st); else launch_skinny<1, 4>(A, p, k, Mrows, K, acc, st); }
-    else if (k.nb == 2) { if (k.u == 16) launch_skinny<2, 16>(A, p, k, Mrows, K, acc, st); else launch_skinny<2, 4>(A, p, k, Mrows, K, acc, st); }
-    else { if (k.u == 8) launch_skinny<4, 8>(A, p, k, Mrows, K, acc, st); else launch_skinny<4, 2>(A, p, k, Mrows, K, acc, st); }
+    else { if (k.u == 16) launch_skinny<2, 16>(A, p, k, Mrows, K, acc, st); else launch_skinny<2, 4>(A, p, k, Mrows, K, acc, st); }
 }
 
 template <int MT, int RB, int U>
@@ -1653,29 +1645,36 @@ static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows,
 }
 
 // Which products may share a launch: those with the same non-zero key.  A key names the kernel a block takes on its own
-// (M <= 2: tgp_wstream_kernel<MT, 1, 8>; 3 <= M <= 32: one instance of the split-K skinny kernel); blocks of so many rows that
-// they fill the machine alone, and the shapes served by other kernels, have key 0 and are launched alone.
+// (M <= 2: tgp_wstream_kernel<MT, 1, 8>; 3 <= M <= 32: one instance of the persistent list kernel, or the tcgen05 kernel and
+// split of K); blocks of so many rows that they fill the machine alone, and the shapes served by other kernels, have key 0 and
+// are launched alone.
 uint32_t tgpk_gemm_group_key(uint32_t M, uint32_t n, uint32_t K) {
     if (!g_gemm_group || !M || !n || !K || K % 8) return 0;
-    if (M >= 3 && M <= 32 && K % 32 == 0 && g_skinny_impl == 0) {
-        const SkinnyPick k = pick_skinny(M, n, K);
-        // the blocks served by the persistent 16-warp kernel, which walks the row groups of any number of blocks
-        return k.persistent ? (0x1000000u | (uint32_t)k.nb | (uint32_t)k.u << 4 | (uint32_t)k.nw << 8 | (uint32_t)k.rows << 16) : 0;
-    }
     if (M <= 2) return (n < 2 * 148 * 16 && !(g_gemv_splitk && K >= 8192)) ? M : 0;
-    return 0;
+    if (M > 32) return 0;
+    if (takes_tiles(M, n, K)) return tgpk_gemm_tc_forced() ? 0 : 0x2000000u | tgpk_gemm_tc_class(M, n, K);
+    if (M > 16 || K % 32 || g_skinny_impl) return 0;
+    const SkinnyPick k = pick_skinny(M, n, K);
+    return k.persistent ? (0x1000000u | (uint32_t)k.nb | (uint32_t)k.u << 4 | (uint32_t)k.nw << 8 | (uint32_t)k.rows << 16) : 0;
 }
 
 int tgpk_gemm_group(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t M, uint32_t K,
                     int accumulate, cudaStream_t st) {
     if (!count || !M) return TGP_OK;
     const uint32_t key = tgpk_gemm_group_key(M, n[0], K);
-    bool same = key != 0 && count >= 2 && count <= TGP_GEMM_GROUP_MAX;
+    bool same = key != 0 && key < 0x2000000u && count >= 2 && count <= TGP_GEMM_GROUP_MAX;
     for (uint32_t s = 1; s < count && same; ++s) same = tgpk_gemm_group_key(M, n[s], K) == key;
     if (!same) {
-        for (uint32_t s = 0; s < count; ++s) {
-            const int rc = tgpk_gemm(A, W[s], C[s], M, n[s], K, ldc[s], 0, accumulate, st);
+        // neighbours that one tcgen05 kernel serves with one split of K share a launch, at any M; other parts are launched alone
+        auto tc_class = [&](uint32_t s) { return g_gemm_group && n[s] && takes_tiles(M, n[s], K) && !tgpk_gemm_tc_forced() ? tgpk_gemm_tc_class(M, n[s], K) : 0u; };
+        for (uint32_t s = 0; s < count;) {
+            const uint32_t cls = tc_class(s);
+            uint32_t e = s + 1;
+            while (cls && e < count && e - s < TGP_GEMM_GROUP_MAX && tc_class(e) == cls) ++e;
+            const int rc = e - s > 1 ? tgpk_gemm_tc_list(A, e - s, W + s, C + s, n + s, ldc + s, M, K, accumulate, st)
+                                     : tgpk_gemm(A, W[s], C[s], M, n[s], K, ldc[s], 0, accumulate, st);
             if (rc) return rc;
+            s = e;
         }
         return TGP_OK;
     }
@@ -1714,26 +1713,12 @@ int tgpk_gemm(const void *A, const void *W, float *C, uint32_t M, uint32_t n, ui
     if (!M || !n) return TGP_OK;
     if (K % 8 || !K) return TGP_E_INVAL;
     const bf16 *a = (const bf16 *)A, *w = (const bf16 *)W;
-    const bool tiles_win = M > 16 && n >= TILES_WIN_ROWS && g_gemm_impl == 0;
-    if (M >= 3 && M <= 32 && K % 32 == 0 && g_skinny_impl == 0 && !tiles_win) {
+    if (takes_tiles(M, n, K)) return tgpk_gemm_tc(A, W, C, M, n, K, ldc, col0, accumulate, st);
+    if (M >= 3 && M <= 16 && K % 32 == 0 && g_skinny_impl == 0) {
         GemvParts p;
         memset(&p, 0, sizeof(p));
         p.W[0] = w; p.C[0] = C + col0; p.n[0] = n; p.ldc[0] = ldc; p.count = 1;
         launch_skinny_pick(a, p, pick_skinny(M, n, K), M, K, accumulate, st);
-    } else if (M > 32 && M <= 64 && K % 32 == 0 && g_skinny_impl == 0 && g_gemm_impl == 0 && n < 4096) {
-        // 33 - 64 activation rows on a block of few rows: the tiled GEMM would run a handful of CTAs with a serial K loop
-        // (n=1024, K=4096: 15.8 us); two weight-streaming launches of half the rows each read the block twice, the
-        // second time from L2, and are faster (9.9 us); from 32 tiles of 128 rows on the tiled GEMM takes the weights as its
-        // 128-row operand instead
-        const uint32_t m1 = (M + 1) / 2;
-        for (uint32_t m0 = 0; m0 < M; m0 += m1) {
-            const uint32_t mr = M - m0 < m1 ? M - m0 : m1;
-            GemvParts p;
-            memset(&p, 0, sizeof(p));
-            p.W[0] = w; p.C[0] = C + (size_t)m0 * ldc + col0; p.n[0] = n; p.ldc[0] = ldc; p.count = 1;
-            launch_skinny_pick(a + (size_t)m0 * K, p, pick_skinny(mr, n, K), mr, K, accumulate, st);
-            if (m0) tgpk_launches += 1;
-        }
     } else if (M <= 16) {
         for (uint32_t m0 = 0; m0 < M; m0 += 8) {
             uint32_t mr = M - m0 < 8 ? M - m0 : 8;
@@ -1745,8 +1730,6 @@ int tgpk_gemm(const void *A, const void *W, float *C, uint32_t M, uint32_t n, ui
             else launch_gemv_rows<8>(am, w, cm, mr, n, K, ldc, col0, accumulate, st);
             if (m0) tgpk_launches += 1;
         }
-    } else if (g_gemm_impl == 0) {
-        return tgpk_gemm_tc(A, W, C, M, n, K, ldc, col0, accumulate, st);
     } else {
         dim3 grid((n + 63) / 64, (M + 63) / 64);
         tgp_matmul_simt_kernel<<<grid, 256, 0, st>>>(a, w, C, M, n, K, ldc, col0, accumulate);

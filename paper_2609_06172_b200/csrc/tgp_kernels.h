@@ -23,6 +23,15 @@ int tgpk_gemm_group(const void *A, uint32_t count, const void *const *W, float *
 // stores aout[m, col0 + j] = bf16(silu(gate[m, col0 + j]) * acc) (gate fp32 and aout bf16 in C's geometry); not with accumulate
 int tgpk_gemm_tc(const void *A, const void *W, float *C, uint32_t M, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int accumulate, cudaStream_t st,
                  const float *gate = nullptr, void *aout = nullptr);
+// blocks over the same activations in one launch of a tcgen05 kernel (gate / aout with one block only); all of them must
+// have the same tgpk_gemm_tc_class() (kernel and split of K, never 0), then each computes the bits it computes alone
+uint32_t tgpk_gemm_tc_class(uint32_t M, uint32_t n, uint32_t K);
+int tgpk_gemm_tc_list(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t M, uint32_t K,
+                      int accumulate, cudaStream_t st, const float *gate = nullptr, void *aout = nullptr);
+// a kernel other than the automatic choice is selected (tgp_k_gemm_tc_variant)
+bool tgpk_gemm_tc_forced();
+// programmatic dependent launches are switched on (tgp_k_gemv_overlap)
+bool tgpk_launch_overlap();
 // true if a product of M activation rows takes the tensor-core GEMM, whose epilogue can apply SwiGLU (M > 128, tensor cores selected)
 bool tgpk_swiglu_fusable(uint32_t M);
 int tgpk_rope_kv(const float *q32, const float *k32, const float *v32, void *qb, const TgpTilePtrs &tiles, const float *cos_t, const float *sin_t,

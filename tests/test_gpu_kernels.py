@@ -728,3 +728,56 @@ def test_blocks_of_many_rows_take_the_list_kernel_with_the_same_bits_alone_and_i
         want = A.double() @ W.double().T + c.double()
         # fp32 sums of K products of N(0, 1) x N(0, 0.02): errors of a few 2^-24 of the partial sums' size, bounded as in the tests above
         assert float((a.double() - want).abs().max()) < 2e-5 * float(want.abs().max())
+
+
+# the tcgen05 kernels on either side of their dispatch lines: one tile per CTA unsplit / in 2 / in 4 slices of K (ragged row tiles, K that
+# ends inside a 64-wide block or leaves slices of unequal length), the line at 8192 columns above 128 activation rows, the paired
+# kernel's activation tiles (one of 160 rows, three of 224, the last one ragged), lists of ragged parts
+@pytest.mark.parametrize("M,ns,K", [(17, (4736, 129), 1024), (33, (130, 1), 1032), (61, (9400, 4737), 1024), (64, (9473,), 2048), (128, (4737,), 8192),
+                                    (16, (8065, 8193), 512), (129, (257, 255), 8184), (129, (257, 255), 8192), (300, (2300,), 8200), (603, (300, 513), 1096),
+                                    (100, (33,) * 8, 1024)])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_tcgen05_products_alone_and_in_a_list(M, ns, K, accumulate):
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(M * K + len(ns))
+    A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
+    Ws = [(torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16() for n in ns]
+    lds = [n + 4 * (s % 3) for s, n in enumerate(ns)]
+    c0 = [torch.randn((M, ld), device=DEV, generator=gen) for ld in lds]
+    alone, listed = [c.clone() for c in c0], [c.clone() for c in c0]
+    for W, C, n, ld in zip(Ws, alone, ns, lds):
+        tb.k_gemm(A, W, C, M, n, K, ld, 0, accumulate)
+    tb.k_gemm_group(A, Ws, listed, M, list(ns), K, lds, accumulate)
+    torch.cuda.synchronize()
+    assert tb.k_gemm_status() == 0
+    for W, a, b, c, n in zip(Ws, alone, listed, c0, ns):
+        assert torch.equal(a, b) and torch.equal(a[:, n:], c[:, n:])
+        want = A.double() @ W.double().T + (c[:, :n].double() if accumulate else 0)
+        assert float((a[:, :n].double() - want).abs().max()) < 2e-5 * float(want.abs().max())
+
+
+def test_tcgen05_product_in_slices_gives_up_on_a_wait_that_runs_out_and_recovers():
+    """The one-tile-per-CTA kernel with K in four slices: the grid's first CTA never loads its second block, so the waits for its
+    tile run out; no CTA of its cluster stores anything, every other tile is right, and the next launch is correct."""
+    M, n, K = 61, 300, 2048
+    A, W = bf16_dev(rnd_bits(53, M * K).reshape(M, K)), bf16_dev(rnd_bits(54, n * K).reshape(n, K))
+    want = (A.double() @ W.double().T).cpu().numpy()
+    SENT = 12345.0
+    tb.k_status_clear()
+    try:
+        tb.k_wait_test(2_000_000, 1)
+        Cd = torch.full((M, n), SENT, dtype=torch.float32, device=DEV)
+        tb.k_gemm(A, W, Cd, M, n, K, n, 0, 0)
+        torch.cuda.synchronize()
+        assert tb.k_gemm_status() != 0
+        got = Cd.cpu().numpy()
+        assert (got[:, :128] == SENT).all()
+        assert np.abs(got[:, 128:] - want[:, 128:]).max() < 2e-5 * np.abs(want).max()
+    finally:
+        tb.k_wait_test(0, -1)
+        tb.k_status_clear()
+    Cd = torch.zeros((M, n), dtype=torch.float32, device=DEV)
+    tb.k_gemm(A, W, Cd, M, n, K, n, 0, 0)
+    torch.cuda.synchronize()
+    assert tb.k_gemm_status() == 0
+    assert np.abs(Cd.cpu().numpy() - want).max() < 2e-5 * np.abs(want).max()

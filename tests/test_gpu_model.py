@@ -233,6 +233,27 @@ def test_prefill_swiglu_in_the_up_projection_epilogue_gives_the_same_bits():
     check_logits([runs[(0, 1)][0][0]], [ref])
 
 
+def test_prefill_swiglu_epilogue_of_a_product_split_along_k_gives_the_same_bits():
+    """A long K and few tiles above 128 activation rows: the up projection runs in four K slices per tile, and the CTA that sums a
+    tile's partials applies SwiGLU."""
+    cfg = replace(si.CONFIGS[1], L=1, d=8192, F=704, Hq=2, Hkv=1, Dh=64, V=512, B=1, S=200, T=0, TK=64, budget_rule="half_w")
+    lay, pool, s, blobs, T = setup(cfg, n_dec=0)
+    r = Runner(s, cfg.B * cfg.S)
+    prompt = si.prompt_tokens(cfg)
+    runs = []
+    for enable in (1, 0):
+        tb.k_swiglu_epilogue(enable)
+        r.reset()
+        st = r.step(tb.PREFILL, prompt, cfg.S, want_stats=True)
+        runs.append((r.logits.cpu().numpy().copy(), st.n_launches))
+    tb.k_swiglu_epilogue(1)
+    s.close()
+    assert tb.k_gemm_status() == 0
+    assert np.array_equal(runs[0][0], runs[1][0]) and runs[1][1] - runs[0][1] == cfg.L
+    ref = forward.OracleModel(cfg, si.weights_as_bits(lay), dtype=np.float32).step(prompt, 0)
+    check_logits([runs[0][0]], [ref])
+
+
 @pytest.mark.parametrize("bits", [tb.BIT_ZC, 15])
 def test_adjacent_small_copies_are_coalesced_without_changing_a_bit(bits):
     """Consecutive loads whose pool ranges and arena slots continue one another travel in one copy: with nothing pinned
