@@ -55,6 +55,8 @@ template <int DH> __device__ __forceinline__ uint32_t tile_off(uint32_t r, uint3
 template <int DH, bool SPLIT_P>
 __global__ void __launch_bounds__(128) tgp_attn_prefill_mma_kernel(PArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");       // a programmatic dependent launch: the next one's latency overlaps this kernel,
+    asm volatile("griddepcontrol.wait;" ::: "memory");                    // which reads nothing before the previous one has finished
     constexpr int CH = DH / 8;                              // 16-byte chunks per row
     constexpr int TILE = BN * DH * 2;
     uint8_t *Qs = smem, *Ks = smem + BM * DH * 2, *Vs = Ks + 2 * TILE;
@@ -201,8 +203,14 @@ static int launch(const PArgs &a, uint32_t B, cudaStream_t st) {
     constexpr int SM = (BM + 4 * BN) * DH * 2;
     static bool attr_set = false;
     if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_prefill_mma_kernel<DH, SPLIT_P>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM) != cudaSuccess) return TGP_E_CUDA; attr_set = true; }
-    tgp_attn_prefill_mma_kernel<DH, SPLIT_P><<<dim3((a.q_len + BM - 1) / BM, a.Hq, B), 128, SM, st>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return TGP_E_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((a.q_len + BM - 1) / BM, a.Hq, B); cfg.blockDim = dim3(128); cfg.dynamicSmemBytes = SM; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, tgp_attn_prefill_mma_kernel<DH, SPLIT_P>, a) != cudaSuccess) return TGP_E_CUDA;
     tgpk_launches += 1;
     return TGP_OK;
 }

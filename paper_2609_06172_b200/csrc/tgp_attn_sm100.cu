@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
     volatile uint32_t *failed = tmem_slot + 1;
 
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (smem_u32(smem) & 1023u) {                            // the swizzle assumes 1024-byte aligned tiles
         if (tid == 0) atomicCAS(&g_attn_tc_error, 0, 5);
         return;
@@ -125,6 +126,8 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmQ) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tmKV) : "memory");
+        // a programmatic dependent launch: the set-up above and the TMEM allocation overlap the previous kernel, which wrote Q, K and V
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         next_k(Q_BYTES);                                     // K_0 and, on the same barrier, Q
 #pragma unroll
         for (uint32_t kb = 0; kb < KB; ++kb) tma_load_2d(Qs + kb * (BQ * 128), &tmQ, hq * DH + kb * 64, b * a.q_len + q0, bar_k);
@@ -136,7 +139,8 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    __syncthreads();                                         // (after the TMA thread's wait for the previous kernel: nothing below runs before it)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t tmem_S = tmem_base, tmem_O = tmem_base + 64, tmem_P = tmem_base + 192;     // P: two buffers of 32 columns (bf16 pairs)
@@ -354,6 +358,26 @@ template <int DH> constexpr int smem_bytes() { return (DH / 64) * (BQ + 4 * BKV)
 
 extern thread_local uint64_t tgpk_launches;
 
+template <int DH>
+static int launch(const CUtensorMap &mq, const CUtensorMap &mkv, const CUtensorMap &mo, const TArgs &a, uint32_t B, cudaStream_t st) {
+    static bool attr_set = false;
+    if (!attr_set) {
+        if (cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<DH>()) != cudaSuccess) return TGP_E_CUDA;
+        cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<DH>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        attr_set = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((a.q_len + BQ - 1) / BQ, a.Hq, B); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = smem_bytes<DH>(); cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, tgp_attn_prefill_tc_kernel<DH>, mq, mkv, mo, a) != cudaSuccess) return TGP_E_CUDA;
+    tgpk_launches += 1;
+    return TGP_OK;
+}
+
 int tgpk_attn_prefill_tc5(const void *qb, const TgpTilePtrs &tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0, cudaStream_t st) {
     if (c->Dh != 64 && c->Dh != 128) return TGP_E_INVAL;
     const uint32_t n_tiles = (pos0 + q_len + c->TK - 1) / c->TK;
@@ -381,26 +405,7 @@ int tgpk_attn_prefill_tc5(const void *qb, const TgpTilePtrs &tiles, void *ob, co
         !tensor_map_bf16_2d(&mkv, (const void *)lo, (hi - lo) / row_bytes + tile_rows, c->Dh, row_bytes, BKV) ||
         !tensor_map_bf16_2d(&mo, ob, (uint64_t)B * q_len, (uint64_t)c->Hq * c->Dh, (uint64_t)c->Hq * c->Dh * 2, BQ))
         return TGP_E_CUDA;
-    dim3 grid((q_len + BQ - 1) / BQ, c->Hq, B);
-    static bool attr64 = false, attr128 = false;
-    if (c->Dh == 64) {
-        if (!attr64) {
-            if (cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<64>()) != cudaSuccess) return TGP_E_CUDA;
-            cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<64>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-            attr64 = true;
-        }
-        tgp_attn_prefill_tc_kernel<64><<<grid, THREADS, smem_bytes<64>(), st>>>(mq, mkv, mo, a);
-    } else {
-        if (!attr128) {
-            if (cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<128>()) != cudaSuccess) return TGP_E_CUDA;
-            cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<128>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-            attr128 = true;
-        }
-        tgp_attn_prefill_tc_kernel<128><<<grid, THREADS, smem_bytes<128>(), st>>>(mq, mkv, mo, a);
-    }
-    if (cudaGetLastError() != cudaSuccess) return TGP_E_CUDA;
-    tgpk_launches += 1;
-    return TGP_OK;
+    return c->Dh == 64 ? launch<64>(mq, mkv, mo, a, B, st) : launch<128>(mq, mkv, mo, a, B, st);
 }
 
 int tgpk_attn_wait_test(unsigned long long limit_ns, int withhold_step) {

@@ -473,6 +473,7 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
         __syncwarp();
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {                 // MMA thread of the pair
+            asm volatile("griddepcontrol.wait;" ::: "memory");    // the limit of its waits counts from here
             const uint32_t idesc = umma_idesc_pair(N);
             uint32_t s = 0, ph = 0, lt = 0;
             bool ok = true;
@@ -645,6 +646,7 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
         __syncwarp();
     } else if (warp == 1) {
         if (lane == 0) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");    // the limit of its waits counts from here
             const uint32_t idesc = umma_idesc((int)N);
             uint32_t s = 0, ph = 0;
             bool ok = true;
