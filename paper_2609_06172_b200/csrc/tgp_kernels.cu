@@ -52,6 +52,12 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+static int device_sms() {
+    static int sms = 0;
+    if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
+    return sms;
+}
+
 static int g_small_pdl = 1;      // small kernels are launched as programmatic dependents of their predecessor (0: plain launches)
 
 template <typename... KArgs, typename... Args>
@@ -97,29 +103,54 @@ __device__ __forceinline__ float sumsq4(float ss, const float4 &v) {
     return __fadd_rn(ss, __fmaf_rn(v.w, v.w, __fmaf_rn(v.z, v.z, __fmaf_rn(v.y, v.y, __fmul_rn(v.x, v.x)))));
 }
 
-__global__ void tgp_rmsnorm_kernel(const float *x, uint32_t ldx, const bf16 *__restrict__ g, bf16 *h, uint32_t d, float eps) {
+// One CTA of 256 threads per row.  NV > 0: the row has at most NV x 1024 elements, which stay in registers between the two passes, and
+// every load, the gains' too, is under way before the first is used: a decode step's norms are two latencies long (8 rows of
+// 4096: 5.4 -> 3.5 us from the end of the kernel before).  NV == 0: longer rows, read twice, and gains or
+// outputs that are not 8-byte aligned.  The sum of squares is the same
+// for every NV: thread t adds elements 4 t, 4 (t + 256), ... in that order.
+template <int NV>
+__global__ void __launch_bounds__(256) tgp_rmsnorm_kernel(const float *x, uint32_t ldx, const bf16 *__restrict__ g, bf16 *h, uint32_t d, float eps) {
     pdl_enter();
-    __shared__ float red[32];
+    __shared__ float red[8];
     const float4 *row = reinterpret_cast<const float4 *>(x + (size_t)blockIdx.x * ldx);
+    const uint2 *gg = reinterpret_cast<const uint2 *>(g);
+    uint2 *out = reinterpret_cast<uint2 *>(h + (size_t)blockIdx.x * d);
+    const uint32_t n4 = d / 4;
+    float4 v[NV ? NV : 1];
+    uint2 gv[NV ? NV : 1];
     float ss = 0.f;
-    for (uint32_t i = threadIdx.x; i < d / 4; i += blockDim.x) ss = sumsq4(ss, row[i]);
+    if constexpr (NV > 0) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) { const uint32_t k = threadIdx.x + 256 * i; if (k < n4) v[i] = row[k]; }
+#pragma unroll
+        for (int i = 0; i < NV; ++i) { const uint32_t k = threadIdx.x + 256 * i; if (k < n4) gv[i] = gg[k]; }
+#pragma unroll
+        for (int i = 0; i < NV; ++i) if (threadIdx.x + 256 * i < n4) ss = sumsq4(ss, v[i]);
+    } else {
+        for (uint32_t i = threadIdx.x; i < n4; i += 256) ss = sumsq4(ss, row[i]);
+    }
     ss = warp_sum(ss);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        float t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-        t = warp_sum(t);
-        if (threadIdx.x == 0) red[0] = 1.0f / sqrtf(t / (float)d + eps);
-    }
-    __syncthreads();
-    const float r = red[0];
-    __nv_bfloat162 *out = reinterpret_cast<__nv_bfloat162 *>(h + (size_t)blockIdx.x * d);
-    const __nv_bfloat162 *gg = reinterpret_cast<const __nv_bfloat162 *>(g);
-    for (uint32_t i = threadIdx.x; i < d / 4; i += blockDim.x) {
-        float4 v = row[i];
-        float2 g0 = __bfloat1622float2(gg[2 * i]), g1 = __bfloat1622float2(gg[2 * i + 1]);
-        out[2 * i] = __floats2bfloat162_rn(v.x * r * g0.x, v.y * r * g0.y);
-        out[2 * i + 1] = __floats2bfloat162_rn(v.z * r * g1.x, v.w * r * g1.y);
+    // every warp adds the eight partial sums itself, in the one order
+    const float t = warp_sum((threadIdx.x & 31) < 8 ? red[threadIdx.x & 31] : 0.f);
+    const float r = 1.0f / sqrtf(t / (float)d + eps);
+    auto scaled = [&](const float4 &w, const uint2 &gw) {
+        const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gw.x)), g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gw.y));
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(w.x * r * g0.x, w.y * r * g0.y), hi = __floats2bfloat162_rn(w.z * r * g1.x, w.w * r * g1.y);
+        return make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+    };
+    if constexpr (NV > 0) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) { const uint32_t k = threadIdx.x + 256 * i; if (k < n4) out[k] = scaled(v[i], gv[i]); }
+    } else {
+        const __nv_bfloat162 *g2 = reinterpret_cast<const __nv_bfloat162 *>(g);
+        __nv_bfloat162 *o2 = reinterpret_cast<__nv_bfloat162 *>(h + (size_t)blockIdx.x * d);
+        for (uint32_t i = threadIdx.x; i < n4; i += 256) {
+            const uint2 w = scaled(row[i], make_uint2(*reinterpret_cast<const uint32_t *>(&g2[2 * i]), *reinterpret_cast<const uint32_t *>(&g2[2 * i + 1])));
+            o2[2 * i] = *reinterpret_cast<const __nv_bfloat162 *>(&w.x);
+            o2[2 * i + 1] = *reinterpret_cast<const __nv_bfloat162 *>(&w.y);
+        }
     }
 }
 
@@ -508,6 +539,37 @@ __global__ void tgp_rope_kv_kernel(RopeArgs a) {
     }
 }
 
+// The same for heads of 64 or 128 dimensions and 16-byte aligned buffers: a thread takes four neighbouring dimensions and their
+// partners half a head away - two 16-byte loads, two 8-byte stores - and a position's heads are spread over gridDim.y CTAs,
+// so that a decode step of a few sequences is one item per thread (8 positions of 48 heads x 128: 11 us with one CTA of twelve
+// dependent rounds per position, 2.5 us now; 32768 positions of them: 381 us, 5.8 TB/s at 208 us now).
+template <int DH>
+__global__ void __launch_bounds__(256) tgp_rope_kv_vec_kernel(RopeArgs a) {
+    pdl_enter();
+    constexpr uint32_t HALF = DH / 2, V = HALF / 4;              // items per head
+    const uint32_t m = blockIdx.x, b = m / a.q_len, pos = a.pos0 + m - b * a.q_len;
+    const uint32_t qd = a.Hq * DH, kd = a.Hkv * DH, j = pos / a.TK, slot = pos - j * a.TK;
+    for (uint32_t idx = blockIdx.y * blockDim.x + threadIdx.x; idx < (a.Hq + 2 * a.Hkv) * V; idx += gridDim.y * blockDim.x) {
+        const uint32_t h = idx / V, i = idx % V * 4;
+        const bool rot = h < a.Hq + a.Hkv;
+        const uint32_t hk = h < a.Hq ? h : rot ? h - a.Hq : h - a.Hq - a.Hkv;
+        const float *s = h < a.Hq ? a.q32 + (size_t)m * qd : (rot ? a.k32 : a.v32) + (size_t)m * kd;
+        s += hk * DH + i;
+        float4 x0 = *reinterpret_cast<const float4 *>(s), x1 = *reinterpret_cast<const float4 *>(s + HALF);
+        if (rot) {
+            const float4 c = *reinterpret_cast<const float4 *>(a.cos_t + (size_t)pos * HALF + i), sv = *reinterpret_cast<const float4 *>(a.sin_t + (size_t)pos * HALF + i);
+            const float4 y0 = x0, y1 = x1;
+            x0 = make_float4(y0.x * c.x - y1.x * sv.x, y0.y * c.y - y1.y * sv.y, y0.z * c.z - y1.z * sv.z, y0.w * c.w - y1.w * sv.w);
+            x1 = make_float4(y1.x * c.x + y0.x * sv.x, y1.y * c.y + y0.y * sv.y, y1.z * c.z + y0.z * sv.z, y1.w * c.w + y0.w * sv.w);
+        }
+        bf16 *o = h < a.Hq ? a.qb + (size_t)m * qd + hk * DH
+                           : reinterpret_cast<bf16 *>(rot ? a.tiles.k[j] : a.tiles.v[j]) + ((size_t)(b * a.Hkv + hk) * a.TK + slot) * DH;
+        const __nv_bfloat162 p[4] = {__floats2bfloat162_rn(x0.x, x0.y), __floats2bfloat162_rn(x0.z, x0.w), __floats2bfloat162_rn(x1.x, x1.y), __floats2bfloat162_rn(x1.z, x1.w)};
+        *reinterpret_cast<uint2 *>(o + i) = make_uint2(*reinterpret_cast<const uint32_t *>(&p[0]), *reinterpret_cast<const uint32_t *>(&p[1]));
+        *reinterpret_cast<uint2 *>(o + i + HALF) = make_uint2(*reinterpret_cast<const uint32_t *>(&p[2]), *reinterpret_cast<const uint32_t *>(&p[3]));
+    }
+}
+
 // ---- attention -------------------------------------------------------------------------------------
 struct AttnArgs {
     const bf16 *qb; bf16 *ob; float *scratch;
@@ -801,19 +863,36 @@ __global__ void __launch_bounds__(256, 2) tgp_attn_decode_group_kernel(AttnArgs 
     }
 }
 
+// One warp holds 32 partials' maxima and sums in its lanes at a time, so the loads of a round are independent of one another, and the
+// outputs of four partials are under way at once: two latencies for up to 32 partials instead of two per partial.
 template <int DH>
-__global__ void tgp_attn_decode_merge_kernel(AttnArgs a) {
+__global__ void __launch_bounds__(DH) tgp_attn_decode_merge_kernel(AttnArgs a) {
     pdl_enter();
-    const uint32_t hq = blockIdx.x, b = blockIdx.y, i = threadIdx.x;
+    const uint32_t hq = blockIdx.x, b = blockIdx.y, i = threadIdx.x, lane = threadIdx.x & 31;
     const uint32_t nt = a.n_parts ? a.n_parts : (a.pos0 + 1 + a.TK - 1) / a.TK;
     const float *part = a.scratch + (size_t)(b * a.Hq + hq) * a.n_tiles * (DH + 2);
-    float mx = -INFINITY;
-    for (uint32_t t = 0; t < nt; ++t) mx = fmaxf(mx, part[t * (DH + 2)]);
-    float l = 0.f, o = 0.f;
-    for (uint32_t t = 0; t < nt; ++t) {
-        const float w = expf(part[t * (DH + 2)] - mx);
-        l += w * part[t * (DH + 2) + 1];
-        o += w * part[t * (DH + 2) + 2 + i];
+    float m0 = lane < nt ? part[lane * (DH + 2)] : -INFINITY, mx = m0;
+    const float l0 = lane < nt ? part[lane * (DH + 2) + 1] : 0.f;
+    for (uint32_t t = lane + 32; t < nt; t += 32) mx = fmaxf(mx, part[t * (DH + 2)]);
+    mx = warp_max(mx);
+    float l = 0.f, o = 0.f, w = 0.f, lw = 0.f;
+    for (uint32_t t0 = 0; t0 < nt; t0 += 4) {
+        float v[4];
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q) v[q] = t0 + q < nt ? part[(t0 + q) * (DH + 2) + 2 + i] : 0.f;
+        if ((t0 & 31) == 0) {                                  // the weights of the next 32 partials, one per lane
+            const uint32_t t = t0 + lane;
+            const float mt = t0 == 0 ? m0 : t < nt ? part[t * (DH + 2)] : -INFINITY;
+            lw = t0 == 0 ? l0 : t < nt ? part[t * (DH + 2) + 1] : 0.f;
+            w = t < nt ? expf(mt - mx) : 0.f;
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q)
+            if (t0 + q < nt) {
+                const float wt = __shfl_sync(0xffffffffu, w, (t0 + q) & 31), lt = __shfl_sync(0xffffffffu, lw, (t0 + q) & 31);
+                l += wt * lt;
+                o += wt * v[q];
+            }
     }
     a.ob[(size_t)b * a.Hq * DH + hq * DH + i] = __float2bfloat16_rn(o / l);
 }
@@ -1009,25 +1088,69 @@ __global__ void tgp_swiglu_kernel(const float4 *g, const float4 *u, __nv_bfloat1
 }
 
 // ---- argmax, lowest index on ties -----------------------------------------------------------------
-__global__ void __launch_bounds__(1024) tgp_argmax_kernel(const float *logits, int32_t *out, uint32_t V) {
+// A row is shared by the CTAs of a cluster (8 for long rows): each scans a contiguous part with four independent 16-byte loads per
+// thread under way, and the parts' winners meet in the first CTA's shared memory (8 rows of 32000: 9.5 us with one CTA of 1024
+// threads and one dependent element per thread and round, 3.4 us now, from the end of the kernel before).
+__global__ void __launch_bounds__(256) tgp_argmax_kernel(const float *logits, int32_t *out, uint32_t V, int vec) {
     pdl_enter();
-    __shared__ float bv[32];
-    __shared__ uint32_t bi[32];
-    const float *row = logits + (size_t)blockIdx.x * V;
+    __shared__ float bv[8], cv[8];
+    __shared__ uint32_t bi[8], ci[8];
+    uint32_t rank, parts;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(parts));
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float *row = logits + (size_t)(blockIdx.x / parts) * V;
+    const uint32_t per = ((V + parts - 1) / parts + 3) / 4 * 4, lo = min(V, rank * per), hi = min(V, lo + per);
     // the index starts at 0, not at a sentinel: a row of NaNs (no comparison holds) must still give a legal token id
     float best = -INFINITY; uint32_t idx = 0u;
-    for (uint32_t j = threadIdx.x; j < V; j += blockDim.x) { float v = row[j]; if (v > best || (v == best && j < idx)) { best = v; idx = j; } }
     auto merge = [](float &v, uint32_t &i, float ov, uint32_t oi) { if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; } };
+    if (vec) {
+        for (uint32_t j0 = lo + threadIdx.x * 4; j0 < hi; j0 += 4096) {
+            float4 v[4];
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) v[q] = j0 + 1024 * q < hi ? *reinterpret_cast<const float4 *>(row + j0 + 1024 * q) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                const uint32_t j = j0 + 1024 * q;
+                if (v[q].x > best) { best = v[q].x; idx = j; }          // a thread's indices ascend: the first of equals stays
+                if (v[q].y > best) { best = v[q].y; idx = j + 1; }
+                if (v[q].z > best) { best = v[q].z; idx = j + 2; }
+                if (v[q].w > best) { best = v[q].w; idx = j + 3; }
+            }
+        }
+    } else {
+        for (uint32_t j = lo + threadIdx.x; j < hi; j += 256) { const float v = row[j]; if (v > best) { best = v; idx = j; } }
+    }
 #pragma unroll
     for (int o = 16; o; o >>= 1) merge(best, idx, __shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, idx, o));
-    if ((threadIdx.x & 31) == 0) { bv[threadIdx.x >> 5] = best; bi[threadIdx.x >> 5] = idx; }
+    if (lane == 0) { bv[warp] = best; bi[warp] = idx; }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        best = threadIdx.x < (blockDim.x >> 5) ? bv[threadIdx.x] : -INFINITY;
-        idx = threadIdx.x < (blockDim.x >> 5) ? bi[threadIdx.x] : 0u;
+    if (warp == 0) {
+        best = lane < 8 ? bv[lane] : -INFINITY;
+        idx = lane < 8 ? bi[lane] : 0u;
 #pragma unroll
-        for (int o = 16; o; o >>= 1) merge(best, idx, __shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, idx, o));
+        for (int o = 4; o; o >>= 1) merge(best, idx, __shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, idx, o));
+    }
+    if (parts == 1) {
         if (threadIdx.x == 0) out[blockIdx.x] = (int32_t)idx;
+        return;
+    }
+    if (threadIdx.x == 0) {                                    // to slot `rank` of the cluster's first CTA
+        uint32_t rv, ri;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(rv) : "r"((uint32_t)__cvta_generic_to_shared(&cv[rank])));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(ri) : "r"((uint32_t)__cvta_generic_to_shared(&ci[rank])));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(rv), "f"(best) : "memory");
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ri), "r"(idx) : "memory");
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank == 0 && warp == 0) {
+        best = lane < parts ? cv[lane] : -INFINITY;
+        idx = lane < parts ? ci[lane] : 0u;
+#pragma unroll
+        for (int o = 4; o; o >>= 1) merge(best, idx, __shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, idx, o));
+        if (lane == 0) out[blockIdx.x / parts] = (int32_t)idx;
     }
 }
 
@@ -1168,7 +1291,11 @@ int tgpk_embed(const void *table, const int32_t *tok, float *x, uint32_t M, uint
 int tgpk_rmsnorm(const float *x, uint32_t ldx, const void *g, void *h, uint32_t M, uint32_t d, float eps, cudaStream_t st) {
     if (!M) return TGP_OK;
     if (d % 4 || ldx % 4) return TGP_E_INVAL;
-    launch_pdl(tgp_rmsnorm_kernel, dim3(M), dim3(256), 0, st, x, ldx, (const bf16 *)g, (bf16 *)h, d, eps);
+#define TGP_RMSNORM(NV_) launch_pdl(tgp_rmsnorm_kernel<NV_>, dim3(M), dim3(256), 0, st, x, ldx, (const bf16 *)g, (bf16 *)h, d, eps)
+    // (many long rows: read twice by more CTAs per SM - 8192 rows of 8192: 63.0 us, 65.5 us from registers)
+    if (((reinterpret_cast<uintptr_t>(g) | reinterpret_cast<uintptr_t>(h)) & 7u) || (d > 4096 && M > 1024)) TGP_RMSNORM(0);
+    else if (d <= 1024) TGP_RMSNORM(1); else if (d <= 2048) TGP_RMSNORM(2); else if (d <= 4096) TGP_RMSNORM(4); else if (d <= 8192) TGP_RMSNORM(8); else TGP_RMSNORM(0);
+#undef TGP_RMSNORM
     LAUNCH_CHECK(1);
     return TGP_OK;
 }
@@ -1466,12 +1593,6 @@ static bool takes_tiles(uint32_t M, uint32_t n, uint32_t K) {
     return M > 16 || (M >= 9 && n >= TILES_WIN_ROWS && g_skinny_impl == 0 && !tgpk_gemm_tc_forced());
 }
 
-static int device_sms() {
-    static int sms = 0;
-    if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
-    return sms;
-}
-
 static SkinnyPick pick_skinny(uint32_t M, uint32_t n, uint32_t K) {
     const uint32_t sms = (uint32_t)device_sms(), groups16 = (n + 15) / 16;
     SkinnyPick k;
@@ -1745,7 +1866,15 @@ int tgpk_rope_kv(const float *q32, const float *k32, const float *v32, void *qb,
                  const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0, cudaStream_t st) {
     if (!B || !q_len) return TGP_OK;
     RopeArgs a{q32, k32, v32, (bf16 *)qb, cos_t, sin_t, c->Hq, c->Hkv, c->Dh, c->TK, q_len, pos0, tiles};
-    launch_pdl(tgp_rope_kv_kernel, dim3(B * q_len), dim3(256), 0, st, a);
+    uintptr_t bits = reinterpret_cast<uintptr_t>(q32) | reinterpret_cast<uintptr_t>(k32) | reinterpret_cast<uintptr_t>(v32) | reinterpret_cast<uintptr_t>(cos_t) |
+                     reinterpret_cast<uintptr_t>(sin_t) | reinterpret_cast<uintptr_t>(qb);
+    for (uint32_t j = pos0 / c->TK; j <= (pos0 + q_len - 1) / c->TK && j < TGP_MAX_TILES; ++j) bits |= reinterpret_cast<uintptr_t>(tiles.k[j]) | reinterpret_cast<uintptr_t>(tiles.v[j]);
+    const uint32_t items = (c->Hq + 2 * c->Hkv) * (c->Dh / 8);
+    // CTAs per position: one item per thread while the positions alone do not fill the GPU (four CTAs of 256 threads per SM)
+    const uint32_t split = std::max(1u, std::min((items + 255) / 256, 4u * (uint32_t)device_sms() / (B * q_len)));
+    if (c->Dh == 64 && (bits & 15u) == 0) launch_pdl(tgp_rope_kv_vec_kernel<64>, dim3(B * q_len, split), dim3(256), 0, st, a);
+    else if (c->Dh == 128 && (bits & 15u) == 0) launch_pdl(tgp_rope_kv_vec_kernel<128>, dim3(B * q_len, split), dim3(256), 0, st, a);
+    else launch_pdl(tgp_rope_kv_kernel, dim3(B * q_len), dim3(256), 0, st, a);
     LAUNCH_CHECK(1);
     return TGP_OK;
 }
@@ -1840,7 +1969,19 @@ int tgpk_swiglu(const float *g, const float *u, void *ab, uint64_t n, cudaStream
 
 int tgpk_argmax(const float *logits, int32_t *out, uint32_t B, uint32_t V, cudaStream_t st) {
     if (!B) return TGP_OK;
-    launch_pdl(tgp_argmax_kernel, dim3(B), dim3(1024), 0, st, logits, out, V);
+    // rows of up to 4096 logits are one round of one CTA
+    const uint32_t parts = V > 4096 ? 8 : 1;
+    const int vec = V % 4 == 0 && (reinterpret_cast<uintptr_t>(logits) & 15u) == 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(B * parts); cfg.blockDim = dim3(256); cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = parts; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    cudaLaunchKernelEx(&cfg, tgp_argmax_kernel, logits, out, V, vec);
     LAUNCH_CHECK(1);
     return TGP_OK;
 }

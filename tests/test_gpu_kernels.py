@@ -781,3 +781,79 @@ def test_tcgen05_product_in_slices_gives_up_on_a_wait_that_runs_out_and_recovers
     torch.cuda.synchronize()
     assert tb.k_gemm_status() == 0
     assert np.abs(Cd.cpu().numpy() - want).max() < 2e-5 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("d", [1024, 1028, 2048, 2052, 4096, 4100, 8192, 8196])
+@pytest.mark.parametrize("M,shift", [(3, 0), (2, 2), (2049, 0)])
+def test_rmsnorm_row_lengths_around_its_register_variants(d, M, shift):
+    """Row lengths at and just past what the variants hold in registers, a row stride longer than the row, gains and outputs
+    that are 4-byte but not 8-byte aligned (shift), many long rows."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(d + M)
+    x = torch.randn((M, d + 4), device=DEV, generator=gen) * 3
+    g = (1 + 0.1 * torch.randn(d + shift, device=DEV, generator=gen)).bfloat16()[shift:]
+    h = torch.zeros(M * d + shift, dtype=torch.bfloat16, device=DEV)
+    tb.k_rmsnorm(x, d + 4, g, h[shift:], M, d, 1e-5)
+    torch.cuda.synchronize()
+    xd = x[:, :d].double()
+    want = xd / torch.sqrt((xd * xd).mean(dim=1, keepdim=True) + 1e-5) * g.double()
+    bf16_close(h[shift:].view(M, d).float().cpu().numpy(), want.float().bfloat16().float().cpu().numpy())
+
+
+@pytest.mark.parametrize("Dh,shift", [(64, 0), (128, 0), (128, 2), (32, 0)])
+@pytest.mark.parametrize("B,S,pos0", [(1, 1, 0), (3, 1, 70), (2, 37, 50), (1, 700, 3)])
+def test_rope_and_kv_append_vector_and_general_forms(Dh, shift, B, S, pos0):
+    """The four-dimensions-a-thread form and the general one (a head size it does not serve, a query buffer that is not 16-byte
+    aligned) against double precision: positions across tile edges, one CTA and several per position."""
+    Hq, Hkv, TK = 6, 2, 16
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=S, T=0, B=B, d=Hq * Dh)
+    cfg = replace(cfg, S=S + pos0)
+    mc = model_cfg(cfg)
+    nt = (pos0 + S + TK - 1) // TK
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(Dh + S)
+    q, k, v = (torch.randn((B * S, h * Dh), device=DEV, generator=gen) for h in (Hq, Hkv, Hkv))
+    kt, vt = ([torch.full((B * Hkv * TK, Dh), 5.0, dtype=torch.bfloat16, device=DEV) for _ in range(nt)] for _ in range(2))
+    cos, sin = (torch.randn((pos0 + S, Dh // 2), device=DEV, generator=gen) for _ in range(2))
+    qb = torch.zeros(B * S * Hq * Dh + shift, dtype=torch.bfloat16, device=DEV)
+    tb.k_rope_kv(q, k, v, qb[shift:], kt, vt, cos, sin, mc, B, S, pos0)
+    torch.cuda.synchronize()
+
+    def rot(x, h):
+        x = x.double().view(B, S, h, Dh)
+        c, s_ = cos[pos0:].double().view(1, S, 1, -1), sin[pos0:].double().view(1, S, 1, -1)
+        a, b = x[..., :Dh // 2], x[..., Dh // 2:]
+        return torch.cat([a * c - b * s_, b * c + a * s_], dim=-1)
+
+    # half a bf16 step of the result, plus the fp32 rounding of two products of factors below 6 (3 x 36 x 2^-24), which is what is
+    # left where they cancel
+    close = lambda got, want: bool(((got.double() - want).abs() <= 2.0 ** -8 * want.abs() + 1e-5).all())
+    assert close(qb[shift:].view(B, S, Hq, Dh), rot(q, Hq))
+    for tiles, want in ((kt, rot(k, Hkv)), (vt, v.double().view(B, S, Hkv, Dh))):
+        cache = torch.stack([t.view(B, Hkv, TK, Dh) for t in tiles], dim=2).reshape(B, Hkv, nt * TK, Dh)
+        assert close(cache[:, :, pos0:pos0 + S].transpose(1, 2), want)
+        assert (cache[:, :, :pos0] == 5.0).all() and (cache[:, :, pos0 + S:] == 5.0).all()      # nothing else is touched
+
+
+@pytest.mark.parametrize("V", [1, 5, 4096, 4097, 4100, 32000, 50001, 131072])
+def test_argmax_parts_ties_and_special_values(V):
+    """One CTA and a cluster of eight per row, vector and scalar loads, parts that are empty or end inside a vector: the lowest
+    index of equal maxima wherever they lie, infinities, rows of NaN."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(V)
+    rows = [torch.randn(V, device=DEV, generator=gen) for _ in range(9)]
+    for i, r in enumerate(rows[:4]):
+        at = torch.randint(0, V, (3,), device=DEV, generator=gen)
+        r[at] = 7.5 if i < 3 else float("inf")
+    rows[4][:] = 1.25
+    rows[5][:] = float("-inf")
+    rows[6][:] = float("nan")
+    rows[7][V // 2:] = float("nan")
+    rows[8][V - 1] = 9.0
+    lg = torch.stack(rows)
+    out = torch.full((9,), -7, dtype=torch.int32, device=DEV)
+    tb.k_argmax(lg, out, 9, V)
+    torch.cuda.synchronize()
+    a = lg.cpu().numpy()
+    want = [0 if not np.any(r > -np.inf) else int(np.flatnonzero(r == np.nanmax(r))[0]) for r in a]
+    assert out.cpu().tolist() == want
