@@ -42,6 +42,13 @@ struct TgpEngine {
     float *topk_gate = nullptr, *egate = nullptr, *y32 = nullptr, *bias_dev = nullptr;
     char *hg = nullptr, *spill = nullptr;
     int32_t *ecount_host = nullptr;                      // pinned mirror of the per-expert counts
+    int32_t *epos = nullptr;                             // place of a token in the lists of its experts
+    // counts of the steps whose experts ran without the host looking at them, written by the router kernel: [steps, L, E] of the
+    // plan in mapped host memory (sized by tgp_run_reset()); the slots to fold into run_counts when someone asks
+    int32_t *count_log = nullptr;
+    size_t count_log_words = 0;
+    std::vector<size_t> count_slots;
+    uint32_t step_tokens = 0;                            // tokens of the step being executed
     std::vector<uint32_t> cnt;                           // counts of the layer being executed
     int32_t cur_expert = -1;
     uint32_t max_tokens = 0;
@@ -88,7 +95,7 @@ struct TgpEngine {
 
 static inline uint64_t up256(uint64_t x) { return (x + 255) / 256 * 256; }
 
-struct WsLayout { uint64_t tok, amax, x, h, q32, k32, v32, qb, ob, g32, u32, ab, hf, cos_t, sin_t, scratch, topk_idx, topk_gate, erow, egate, ecount, hg, y32, bias, spill, total; };
+struct WsLayout { uint64_t tok, amax, x, h, q32, k32, v32, qb, ob, g32, u32, ab, hf, cos_t, sin_t, scratch, topk_idx, topk_gate, erow, egate, ecount, epos, hg, y32, bias, spill, total; };
 
 static WsLayout ws_layout(const tgp_model_cfg &c, uint64_t Mx) {
     WsLayout w{};
@@ -107,6 +114,7 @@ static WsLayout ws_layout(const tgp_model_cfg &c, uint64_t Mx) {
     if (c.E) {
         w.topk_idx = take(Mx * 2 * 4); w.topk_gate = take(Mx * 2 * 4);
         w.erow = take((uint64_t)c.E * Mx * 4); w.egate = take((uint64_t)c.E * Mx * 4); w.ecount = take((uint64_t)c.E * 4);
+        w.epos = take(Mx * 2 * 4);
         w.hg = take(Mx * c.d * 2); w.y32 = take(Mx * c.d * 4); w.bias = take((uint64_t)c.L * c.E * 4);
         w.spill = take(std::max<uint64_t>((uint64_t)c.F * c.d * 2, 512));        // one whole expert matrix: the largest block a fallback fetches
     }
@@ -147,6 +155,7 @@ void tgp_engine_free(tgp_ctx *ctx) {
     for (cudaStream_t xs : e->xcopy) if (xs) cudaStreamDestroy(xs);
     if (e->wb_stream) cudaStreamDestroy(e->wb_stream);
     if (e->ecount_host) cudaFreeHost(e->ecount_host);
+    if (e->count_log) cudaFreeHost(e->count_log);
     delete e;
     ctx->eng = nullptr;
 }
@@ -214,7 +223,7 @@ int tgp_model_bind(tgp_ctx *ctx, const tgp_model_cfg *cfg, const tgp_role_entry 
     e->max_tokens = max_tokens;
     if (c.E) {
         e->topk_idx = (int32_t *)(b + w.topk_idx); e->topk_gate = (float *)(b + w.topk_gate); e->erow = (int32_t *)(b + w.erow);
-        e->egate = (float *)(b + w.egate); e->ecount = (int32_t *)(b + w.ecount); e->hg = b + w.hg; e->y32 = (float *)(b + w.y32);
+        e->egate = (float *)(b + w.egate); e->ecount = (int32_t *)(b + w.ecount); e->epos = (int32_t *)(b + w.epos); e->hg = b + w.hg; e->y32 = (float *)(b + w.y32);
         e->bias_dev = (float *)(b + w.bias); e->spill = b + w.spill;
         CU(ctx, cudaMemcpy(e->bias_dev, ctx->router_bias.data(), (size_t)c.L * c.E * 4, cudaMemcpyHostToDevice));
         CU(ctx, cudaHostAlloc((void **)&e->ecount_host, (size_t)c.E * 4, cudaHostAllocDefault));
@@ -260,6 +269,15 @@ int tgp_run_reset(tgp_ctx *ctx) {
     e->advised = false;                                  // the plan may have changed since the last run
     for (uint64_t &r : e->recent_objects) r = ~0ull;
     ctx->run_counts.clear();
+    e->count_slots.clear();
+    const size_t words = ctx->steps.size() * ctx->cfg.L * ctx->cfg.E;
+    if (words > e->count_log_words) {
+        if (e->count_log) CU(ctx, cudaFreeHost(e->count_log));
+        e->count_log = nullptr;
+        e->count_log_words = 0;
+        CU(ctx, cudaHostAlloc((void **)&e->count_log, words * 4, cudaHostAllocMapped));
+        e->count_log_words = words;
+    }
     return TGP_OK;
 }
 
@@ -478,14 +496,19 @@ static int run_expert_block(tgp_ctx *ctx, const TgpRole &r, const void *W, uint3
     const int32_t *rows = e->erow + (size_t)r.expert * e->max_tokens;
     const float *gates = e->egate + (size_t)r.expert * e->max_tokens;
     int rc = TGP_OK;
+    auto product = [&](const void *A, float *C, uint32_t ldc) {
+        C += r.row0;
+        if (tgpk_expert_rows(e->step_tokens, K)) return tgpk_gemm_rows(A, 1, &W, &C, &r.rows, &ldc, me, e->step_tokens, K, cs);
+        return tgpk_gemm(A, W, C, me, r.rows, K, ldc, 0, 0, cs);
+    };
     switch (r.kind) {
     case TGP_K_WG:
         if (r.row0 == 0 && (rc = tgpk_gather_rows(e->h, rows, e->hg, me, c.d, cs))) return rc;
-        return tgpk_gemm(e->hg, W, e->g32, me, r.rows, K, c.F, r.row0, 0, cs);
+        return product(e->hg, e->g32, c.F);
     case TGP_K_WU:
-        return tgpk_gemm(e->hg, W, e->u32, me, r.rows, K, c.F, r.row0, 0, cs);
+        return product(e->hg, e->u32, c.F);
     case TGP_K_WD:
-        if ((rc = tgpk_gemm(e->ab, W, e->y32, me, r.rows, K, c.d, r.row0, 0, cs))) return rc;
+        if ((rc = product(e->ab, e->y32, c.d))) return rc;
         if (r.row0 + r.rows == c.d) rc = tgpk_scatter_add(e->x, e->y32, rows, gates, me, c.d, cs);
         return rc;
     default:
@@ -555,6 +578,42 @@ static bool gemm_target(const TgpEngine *e, const tgp_model_cfg &c, const TgpRol
     }
 }
 
+// The expert ops of a layer, [first, first + result), as one launch of tgpk_experts(): every expert is traced (so none can be routed to
+// that is not here), the blocks fit its tables and are on the device or on their way, and no copy waits for one of them.
+// 0: they run one by one.
+static uint32_t expert_span(const tgp_ctx *ctx, uint32_t first, uint32_t end, int32_t layer, uint32_t M, TgpExperts *x) {
+    const TgpEngine *e = ctx->eng;
+    const tgp_model_cfg &c = ctx->cfg;
+    if (!tgpk_gemm_grouping() || !tgpk_expert_rows(M, c.d) || c.F % 32 || c.E > TGP_MOE_EXPERTS || (uint64_t)M * c.topk > e->max_tokens) return 0;
+    memset(x, 0, sizeof(*x));
+    uint32_t seen[3][TGP_MOE_EXPERTS] = {}, per[2] = {0, 0}, n = 0;        // rows of each matrix listed so far; rows per block of (gate, up) and down
+    for (; first + n < end; ++n) {
+        const TgpOp &o = ctx->ops[first + n];
+        if (o.layer != layer || (o.kind != TGP_OP_GEMM && o.kind != TGP_OP_SWIGLU)) break;
+        if (ctx->plan.op_is_wait_target[first + n]) return 0;
+        if (ctx->plan.op_last_place[first + n] >= 0 && (size_t)ctx->plan.op_last_place[first + n] >= e->next_cmd) return 0;
+        if (o.kind == TGP_OP_SWIGLU) continue;
+        const TgpRole *r = role_of(ctx, o, 0);
+        if (!r || r->expert < 0 || (uint32_t)r->expert >= c.E || !r->rows) return 0;
+        const uint32_t kind = r->kind == TGP_K_WG ? 0u : r->kind == TGP_K_WU ? 1u : r->kind == TGP_K_WD ? 2u : 3u;
+        if (kind == 3) return 0;
+        const uint32_t rows = kind == 2 ? c.d : c.F, K = kind == 2 ? c.F : c.d, cls = kind == 2;
+        if (ctx->tensors[ctx->acc[o.acc0].tensor].size != 2ull * r->rows * K) return 0;
+        if (!per[cls]) per[cls] = r->rows;
+        const uint32_t b = r->row0 / per[cls];
+        if (r->row0 != seen[kind][r->expert] || r->row0 % per[cls] || b >= TGP_MOE_BLOCKS || (r->rows != per[cls] && r->row0 + r->rows != rows)) return 0;
+        const char *W = where(ctx, o, 0);
+        if ((uintptr_t)W & 15u) return 0;
+        x->w[kind][r->expert][b] = W;
+        seen[kind][r->expert] += r->rows;
+    }
+    for (uint32_t k = 0; k < c.E; ++k) if (seen[0][k] != c.F || seen[1][k] != c.F || seen[2][k] != c.d) return 0;
+    x->h = e->h; x->a = e->ab; x->y = e->y32; x->x = e->x;
+    x->rows = e->erow; x->counts = e->ecount; x->idx = e->topk_idx; x->pos = e->epos; x->gate = e->topk_gate;
+    x->E = c.E; x->topk = c.topk; x->M = M; x->d = c.d; x->F = c.F; x->per_f = per[0]; x->per_d = per[1]; x->stride = e->max_tokens;
+    return n;
+}
+
 extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_host, uint32_t B, uint32_t q_len,
                         float *logits_dev, int32_t *argmax_dev, void *compute_stream, void *copy_stream, tgp_step_stats *stats) {
     if (!ctx || !logits_dev) return TGP_E_INVAL;
@@ -587,6 +646,9 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
     struct ChainScope { bool was; ChainScope() : was(tgpk_chain_ok) { tgpk_chain_ok = true; } ~ChainScope() { tgpk_chain_ok = was; } } chain_scope;
     uint32_t n_cmds = 0, n_mismatch = 0;
     e->cur_expert = -1;
+    e->step_tokens = M;
+    TgpExperts moe;
+    uint32_t moe_first = 0, moe_span = 0;                    // the expert ops of the layer at hand that run as one launch
     if (stats) CU(ctx, cudaEventRecord(e->t0, cs));
     const int32_t *tok = e->amax;
     if (tokens_host) { CU(ctx, cudaMemcpyAsync(e->tok, tokens_host, (size_t)M * 4, cudaMemcpyHostToDevice, cs)); tok = e->tok; }
@@ -623,7 +685,7 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
                 GemmTarget t;
                 if (!r.rows || !gemm_target(e, c, r, M, B, logits_dev, &t) || !t.Mrows || t.Mrows > 32) break;
                 const uint32_t Kj = (uint32_t)(ctx->tensors[ctx->acc[f.acc0].tensor].size / (2ull * r.rows));
-                const uint32_t key = tgpk_gemm_group_key(t.Mrows, r.rows, Kj);
+                const uint32_t key = r.expert >= 0 && tgpk_expert_rows(M, Kj) ? (tgpk_gemm_grouping() ? 0x3000000u : 0u) : tgpk_gemm_group_key(t.Mrows, r.rows, Kj);
                 if (!key) break;
                 if (j == 0) { g0 = t; gK = Kj; key0 = key; g_expert = r.expert; }
                 else if (t.A != g0.A || t.acc != g0.acc || t.Mrows != g0.Mrows || Kj != gK || key != key0 || r.expert != g_expert) break;
@@ -634,7 +696,9 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
             if (key_out) *key_out = key0;
             return cnt;
         };
-        if (ring && o.kind == TGP_OP_GEMM && !e->tap) {
+        if (moe_span && i == moe_first) {
+            span = moe_span;
+        } else if (ring && o.kind == TGP_OP_GEMM && !e->tap) {
             uint32_t cnt = form_group(i, nullptr);
             // A grouped launch keeps the ring slots of its first blocks until its last block has arrived and the launch has
             // run, and the copies that wait for those slots start that much later: the link idles.  So a block whose slot a
@@ -710,6 +774,7 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
             break;
         }
         case TGP_OP_GEMM: {
+            if (moe_span && i == moe_first) { rc = tgpk_experts(moe, cs); break; }
             const TgpRole *rp = role_of(ctx, o, 0);
             if (!rp || !rp->rows) return tgp_fail(ctx, TGP_E_MISMATCH, "GEMM op on a tensor with no model role");
             const tgp_access &a = ctx->acc[o.acc0];
@@ -723,7 +788,8 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
                     e->cur_expert = g_expert;
                     const int32_t *rows = e->erow + (size_t)g_expert * e->max_tokens;
                     if (g_gather && (rc = tgpk_gather_rows(e->h, rows, e->hg, g0.Mrows, c.d, cs))) break;
-                    if ((rc = tgpk_gemm_group(g0.A, span, gW, gC, gn, gld, g0.Mrows, gK, 0, cs))) break;
+                    rc = tgpk_expert_rows(M, gK) ? tgpk_gemm_rows(g0.A, span, gW, gC, gn, gld, g0.Mrows, M, gK, cs) : tgpk_gemm_group(g0.A, span, gW, gC, gn, gld, g0.Mrows, gK, 0, cs);
+                    if (rc) break;
                     if (g_scatter) rc = tgpk_scatter_add(e->x, e->y32, rows, e->egate + (size_t)g_expert * e->max_tokens, g0.Mrows, c.d, cs);
                     break;
                 }
@@ -750,9 +816,14 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
         }
         case TGP_OP_ROUTER: {
             if (!c.E || !o.nacc) return tgp_fail(ctx, TGP_E_MISMATCH, "router op in a dense model or without its weight");
-            rc = tgpk_router(e->h, where(ctx, o, 0), e->bias_dev + (size_t)o.layer * c.E, e->topk_idx, e->topk_gate, e->erow, e->egate, e->ecount,
-                             M, e->max_tokens, c.d, c.E, c.topk, cs);
+            const size_t slot = ((size_t)e->next_step * c.L + o.layer) * c.E;
+            if (ctx->run_counts.size() < slot + c.E) ctx->run_counts.resize(slot + c.E, 0);
+            moe_span = ring && !e->tap && !e->op_timing && slot + c.E <= e->count_log_words ? expert_span(ctx, i + 1, st.op0 + st.nops, o.layer, M, &moe) : 0;
+            moe_first = i + 1;
+            rc = tgpk_router(e->h, where(ctx, o, 0), e->bias_dev + (size_t)o.layer * c.E, e->topk_idx, e->topk_gate, e->erow, e->egate, e->ecount, e->epos,
+                             moe_span ? e->count_log + slot : nullptr, M, e->max_tokens, c.d, c.E, c.topk, cs);
             if (rc) break;
+            if (moe_span) { e->count_slots.push_back(slot); break; }       // the expert kernels read the counts on the device
             // the host needs the counts to size the expert launches (and to detect experts the trace does not list)
             CU(ctx, cudaMemcpyAsync(e->ecount_host, e->ecount, (size_t)c.E * 4, cudaMemcpyDeviceToHost, cs));
             CU(ctx, cudaStreamSynchronize(cs));
@@ -763,8 +834,6 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
                 const TgpRole *fr = role_of(ctx, f, 0);
                 if (fr && fr->expert >= 0 && (uint32_t)fr->expert < c.E) traced[fr->expert] = 1;
             }
-            const size_t slot = ((size_t)e->next_step * c.L + o.layer) * c.E;
-            if (ctx->run_counts.size() < slot + c.E) ctx->run_counts.resize(slot + c.E, 0);
             for (uint32_t x = 0; x < c.E; ++x) {
                 e->cnt[x] = (uint32_t)e->ecount_host[x];
                 ctx->run_counts[slot + x] = e->cnt[x];
@@ -992,6 +1061,13 @@ extern "C" int tgp_managed_evict(void *ptr, uint64_t bytes) {
 // the profile a first pass records so that the next trace lists exactly the experts that are used.
 extern "C" int tgp_expert_counts(tgp_ctx *ctx, uint32_t *out, uint64_t *n) {
     if (!ctx || !n) return TGP_E_INVAL;
+    if (out && ctx->eng && !ctx->eng->count_slots.empty()) {             // counts the router kernels wrote to host memory
+        TgpEngine *e = ctx->eng;
+        CU(ctx, cudaDeviceSynchronize());
+        for (size_t slot : e->count_slots)
+            for (uint32_t k = 0; k < ctx->cfg.E && slot + k < ctx->run_counts.size(); ++k) ctx->run_counts[slot + k] = (uint32_t)e->count_log[slot + k];
+        e->count_slots.clear();
+    }
     if (out) { if (*n < ctx->run_counts.size()) return TGP_E_INVAL; memcpy(out, ctx->run_counts.data(), ctx->run_counts.size() * 4); }
     *n = ctx->run_counts.size();
     return TGP_OK;

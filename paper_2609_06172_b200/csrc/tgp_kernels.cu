@@ -1158,6 +1158,21 @@ __global__ void __launch_bounds__(256) tgp_argmax_kernel(const float *logits, in
 // logits[e] = sum_k h[m,k] * Wr[e,k] + bias[e] in fp32; the two largest (ties: lower expert id); gates = softmax
 // over those two logits.
 template <int E>
+__device__ __forceinline__ void route_pick(const float (&acc)[E], uint32_t topk, int &i0, int &i1, float &g0, float &g1) {
+    i0 = 0;                                            // strict > while visiting ascending ids keeps the lower id on ties
+#pragma unroll
+    for (int e = 1; e < E; ++e) if (acc[e] > acc[i0]) i0 = e;
+    i1 = -1; g0 = 1.0f; g1 = 0.0f;
+    if (E == 1 || topk == 1) return;
+    i1 = i0 == 0 ? 1 : 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) if (e != i0 && acc[e] > acc[i1]) i1 = e;
+    const float e1 = expf(acc[i1] - acc[i0]);
+    g0 = 1.0f / (1.0f + e1);
+    g1 = e1 / (1.0f + e1);
+}
+
+template <int E>
 __global__ void __launch_bounds__(256) tgp_router_kernel(const bf16 *__restrict__ h, const bf16 *__restrict__ Wr, const float *__restrict__ bias,
                                                      int32_t *__restrict__ idx, float *__restrict__ gate, uint32_t M, uint32_t d, uint32_t topk) {
     const uint32_t m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -1179,20 +1194,63 @@ __global__ void __launch_bounds__(256) tgp_router_kernel(const bf16 *__restrict_
 #pragma unroll
     for (int e = 0; e < E; ++e) acc[e] = warp_sum(acc[e]) + bias[e];
     if (lane == 0) {
-        int i0 = 0;                                    // strict > while visiting ascending ids keeps the lower id on ties
+        int i0, i1; float g0, g1;
+        route_pick<E>(acc, topk, i0, i1, g0, g1);
+        idx[2 * m] = i0; idx[2 * m + 1] = i1;
+        gate[2 * m] = g0; gate[2 * m + 1] = g1;
+    }
+}
+
+// Up to ROUTE_SMALL tokens: router and token lists in one CTA and one launch (below), with the arithmetic of tgp_router_kernel.  Warp w
+// takes tokens w, w + 32; then warp e lists the tokens of expert e in ascending order.  pos[2 m + s]: the place of token m in the
+// list of its s-th expert.  counts_host (may be NULL): mapped host memory that receives the counts too.
+constexpr uint32_t ROUTE_SMALL = 64;
+
+template <int E>
+__global__ void __launch_bounds__(1024) tgp_route_small_kernel(const bf16 *h, const bf16 *__restrict__ Wr, const float *__restrict__ bias, int32_t *idx, float *gate, int32_t *rows,
+                                                             float *gates, int32_t *counts, int32_t *pos, int32_t *counts_host, uint32_t M, uint32_t stride, uint32_t d, uint32_t topk) {
+    pdl_enter();
+    __shared__ int32_t si[2 * ROUTE_SMALL];
+    __shared__ float sg[2 * ROUTE_SMALL];
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (uint32_t m = warp; m < M; m += 32) {
+        float acc[E];
 #pragma unroll
-        for (int e = 1; e < E; ++e) if (acc[e] > acc[i0]) i0 = e;
-        if (E == 1 || topk == 1) {
-            idx[2 * m] = i0; idx[2 * m + 1] = -1;
-            gate[2 * m] = 1.0f; gate[2 * m + 1] = 0.0f;
-        } else {
-            int i1 = i0 == 0 ? 1 : 0;
+        for (int e = 0; e < E; ++e) acc[e] = 0.f;
+#pragma unroll 2
+        for (uint32_t k = lane * 8; k < d; k += 256) {
+            float xf[8];
+            unpack8(ld_act(reinterpret_cast<const uint4 *>(h + (size_t)m * d + k)), xf);
 #pragma unroll
-            for (int e = 0; e < E; ++e) if (e != i0 && acc[e] > acc[i1]) i1 = e;
-            const float e1 = expf(acc[i1] - acc[i0]);
-            idx[2 * m] = i0; idx[2 * m + 1] = i1;
-            gate[2 * m] = 1.0f / (1.0f + e1); gate[2 * m + 1] = e1 / (1.0f + e1);
+            for (int e = 0; e < E; ++e) {
+                float wf[8];
+                unpack8(__ldg(reinterpret_cast<const uint4 *>(Wr + (size_t)e * d + k)), wf);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[e] = fmaf(xf[i], wf[i], acc[e]);
+            }
         }
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[e] = warp_sum(acc[e]) + bias[e];
+        if (lane == 0) {
+            int i0, i1; float g0, g1;
+            route_pick<E>(acc, topk, i0, i1, g0, g1);
+            si[2 * m] = i0; si[2 * m + 1] = i1;
+            sg[2 * m] = g0; sg[2 * m + 1] = g1;
+        }
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < 2 * M; i += 1024) { idx[i] = si[i]; gate[i] = sg[i]; }
+    if (warp < (uint32_t)E) {
+        uint32_t base = 0;
+        for (uint32_t m0 = 0; m0 < M; m0 += 32) {
+            const uint32_t m = m0 + lane;
+            int slot = -1;
+            if (m < M) slot = si[2 * m] == (int)warp ? 0 : topk > 1 && si[2 * m + 1] == (int)warp ? 1 : -1;
+            const uint32_t bal = __ballot_sync(0xffffffffu, slot >= 0), at = base + __popc(bal & ((1u << lane) - 1));
+            if (slot >= 0) { rows[(size_t)warp * stride + at] = (int32_t)m; gates[(size_t)warp * stride + at] = sg[2 * m + slot]; pos[2 * m + slot] = (int32_t)at; }
+            base += __popc(bal);
+        }
+        if (lane == 0) { counts[warp] = (int32_t)base; if (counts_host) *(volatile int32_t *)(counts_host + warp) = (int32_t)base; }
     }
 }
 
@@ -1248,21 +1306,27 @@ __global__ void tgp_scatter_add_kernel(float *__restrict__ x, const float *__res
 }
 
 // ============================ launchers (internal) ===================================================
-int tgpk_router(const void *h, const void *Wr, const float *bias, int32_t *idx, float *gate, int32_t *rows, float *gates, int32_t *counts,
-                uint32_t M, uint32_t stride, uint32_t d, uint32_t E, uint32_t topk, cudaStream_t st) {
+int tgpk_router(const void *h, const void *Wr, const float *bias, int32_t *idx, float *gate, int32_t *rows, float *gates, int32_t *counts, int32_t *pos,
+                int32_t *counts_host, uint32_t M, uint32_t stride, uint32_t d, uint32_t E, uint32_t topk, cudaStream_t st) {
     if (!M) return TGP_OK;
     if (d % 8 || topk < 1 || topk > 2) return TGP_E_INVAL;
+    const bool small = M <= ROUTE_SMALL;
+    if (counts_host && !small) return TGP_E_INVAL;
     const uint32_t blocks = (M + 7) / 8;
+#define TGP_ROUTE(E_) do { \
+        if (small) launch_pdl(tgp_route_small_kernel<E_>, dim3(1), dim3(1024), 0, st, (const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, rows, gates, counts, pos, counts_host, M, stride, d, topk); \
+        else tgp_router_kernel<E_><<<blocks, 256, 0, st>>>((const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, M, d, topk); } while (0)
     switch (E) {
-    case 1: tgp_router_kernel<1><<<blocks, 256, 0, st>>>((const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, M, d, topk); break;
-    case 2: tgp_router_kernel<2><<<blocks, 256, 0, st>>>((const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, M, d, topk); break;
-    case 4: tgp_router_kernel<4><<<blocks, 256, 0, st>>>((const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, M, d, topk); break;
-    case 8: tgp_router_kernel<8><<<blocks, 256, 0, st>>>((const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, M, d, topk); break;
-    case 16: tgp_router_kernel<16><<<blocks, 256, 0, st>>>((const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, M, d, topk); break;
+    case 1: TGP_ROUTE(1); break;
+    case 2: TGP_ROUTE(2); break;
+    case 4: TGP_ROUTE(4); break;
+    case 8: TGP_ROUTE(8); break;
+    case 16: TGP_ROUTE(16); break;
     default: return TGP_E_INVAL;
     }
-    tgp_route_fill_kernel<<<E, 1024, 0, st>>>(idx, gate, rows, gates, counts, M, stride, topk);
-    LAUNCH_CHECK(2);
+#undef TGP_ROUTE
+    if (!small) tgp_route_fill_kernel<<<E, 1024, 0, st>>>(idx, gate, rows, gates, counts, M, stride, topk);
+    LAUNCH_CHECK(small ? 1 : 2);
     return TGP_OK;
 }
 
@@ -1304,6 +1368,7 @@ static int g_skinny_impl = 0;    // 0: tensor-core skinny kernels for 3 <= M <= 
 static int g_gemm_impl = 0;      // 0: tensor cores for M > 16; 1: CUDA-core tiles (kept as an on-device cross-check)
 static int g_gemv_splitk = 1;    // small-n blocks at M <= 2: CTA per RB rows with K split over its warps (0: one warp per row)
 static int g_gemm_group = 1;     // products over the same activations: one launch where the parts allow it (0: always one launch each)
+bool tgpk_gemm_grouping() { return g_gemm_group != 0; }
 static int g_gemv_balance = 1;   // grouped skinny launches: rows per group chosen so that every persistent CTA gets the same number of groups
 static int g_gemv_pdl = 1;       // consecutive weight-streaming launches may overlap (programmatic dependent launch)
 bool tgpk_launch_overlap() { return g_gemv_pdl != 0; }
@@ -1763,6 +1828,261 @@ static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows,
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, tgp_wstream_group_kernel<MT, 8>, A, p, Mrows, n_total, K, acc, src);
     tgpk_last_gemm_kernel = "tgp_wstream_group_kernel";
+}
+
+// ---- all experts of a layer in one launch ------------------------------------------------------------------------------------
+// A decode step of a mixture routes a few tokens to each of several experts.  One launch per expert and matrix, sized by counts that
+// the host has to wait for, left the GPU idle most of the time (16 users, 8 experts of 3 x 3584 x 1024: 190 us per layer, of which
+// the weights in use take 18 us); here one launch covers the gate and up projections with SwiGLU of every expert that has
+// tokens, a second one the down projections, and a third adds a token's two results to its residual row.  The counts
+// are read on the device: work items are (expert, up to 8 NB of its tokens, 16 rows of gate and of up, or two groups of `rpc`
+// rows of down), and the CTAs walk the list of those that exist.
+//   The arithmetic of an item is that of tgp_wstream_mma_group_kernel<NB, EXP_U, EXP_NW, 16, 2>: which warp adds which k in which order
+// depends on K alone, so the bits are those of the expert's own products (tgpk_gemm_rows).
+struct ExpertParts {
+    const bf16 *w[2][TGP_MOE_EXPERTS][TGP_MOE_BLOCKS];       // GLU: gate and up; else [0]: down; in blocks of `per` rows
+    const bf16 *A;                                           // GLU: [M, K], rows picked by `rows`; else one row per routed slot
+    const int32_t *rows, *counts;                            // token lists, `stride` apart
+    void *out;                                               // GLU: bf16 [slots, n]; else fp32 [slots, n]
+    uint32_t n, K, per, E, stride, rpc;
+};
+
+// Eight warps of four load steps: a chunk of 1024 columns, so that the K of a small expert keeps every warp at work; two CTAs per
+// SM have 64 KB of loads under way, as many as HBM needs.
+constexpr int EXP_U = 4, EXP_NW = 8;
+
+template <int NB, bool GLU>
+__global__ void __launch_bounds__(EXP_NW * 32, 2) tgp_expert_mma_kernel(const ExpertParts p) {
+    constexpr int U = EXP_U, NW = EXP_NW, G = 2, SK = U / (2 * G), T = NB * 8;       // T: tokens per item
+    __shared__ float part[NW][G * NB * 4][32];
+    __shared__ uint32_t s_first[TGP_MOE_EXPERTS + 1], s_slot[TGP_MOE_EXPERTS], s_cnt[TGP_MOE_EXPERTS];
+    pdl_enter();
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, c = lane & 3, K = p.K;
+    const uint32_t span = GLU ? p.rpc : 2 * p.rpc, groups = (p.n + span - 1) / span;     // items per expert and token chunk
+    if (threadIdx.x == 0) {
+        uint32_t items = 0, slot = 0;
+        for (uint32_t e = 0; e < p.E; ++e) {
+            const uint32_t cnt = (uint32_t)p.counts[e];
+            s_first[e] = items; s_slot[e] = slot; s_cnt[e] = cnt;
+            items += (cnt + T - 1) / T * groups;
+            slot += cnt;
+        }
+        s_first[p.E] = items;
+    }
+    __syncthreads();
+    const uint32_t total = s_first[p.E];
+    if (blockIdx.x >= total) return;
+    const bf16 *wlo[G], *whi[G], *arow[NB];                  // of the item that is being loaded
+    uint4 lo[2][G][SK], hi[2][G][SK], xs[2][SK][NB];
+    float acc[G][NB][4];
+    auto find = [&](uint32_t item, uint32_t &e, uint32_t &chunk, uint32_t &row0) {
+        e = 0;
+        while (item >= s_first[e + 1]) ++e;
+        const uint32_t local = item - s_first[e];
+        chunk = local / groups;
+        row0 = local % groups * span;
+    };
+    auto locate = [&](uint32_t item) {
+        uint32_t e, chunk, row0;
+        find(item, e, chunk, row0);
+#pragma unroll
+        for (int r = 0; r < G; ++r) {
+            const uint32_t first = GLU ? row0 : min(row0 + r * p.rpc, p.n - 1), last = min(first + p.rpc, p.n) - 1;
+            const uint32_t a = min(first + g, last), b = min(first + g + 8, last);       // rows a group lacks re-read its last one
+            const bf16 *const *blocks = p.w[GLU ? r : 0][e];
+            wlo[r] = blocks[a / p.per] + (size_t)(a % p.per) * K + c * 8;
+            whi[r] = blocks[b / p.per] + (size_t)(b % p.per) * K + c * 8;
+        }
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const uint32_t i = chunk * T + b * 8 + g;
+            arow[b] = i >= s_cnt[e] ? nullptr : p.A + (size_t)(GLU ? (uint32_t)p.rows[(size_t)e * p.stride + i] : s_slot[e] + i) * K + c * 8;
+        }
+    };
+    auto issue = [&](auto set, uint32_t kb) {
+        constexpr int S = decltype(set)::value;
+#pragma unroll
+        for (int s = 0; s < SK; ++s) {
+            const uint32_t k = kb + 32 * s;
+#pragma unroll
+            for (int r = 0; r < G; ++r) {
+                lo[S][r][s] = k < K ? __ldcs(reinterpret_cast<const uint4 *>(wlo[r] + k)) : make_uint4(0, 0, 0, 0);
+                hi[S][r][s] = k < K ? __ldcs(reinterpret_cast<const uint4 *>(whi[r] + k)) : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int b = 0; b < NB; ++b) xs[S][s][b] = k < K && arow[b] ? ld_act(reinterpret_cast<const uint4 *>(arow[b] + k)) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    auto consume = [&](auto set) {
+        constexpr int S = decltype(set)::value;
+#pragma unroll
+        for (int s = 0; s < SK; ++s)
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const uint4 xv = xs[S][s][b];
+#pragma unroll
+                for (int r = 0; r < G; ++r) {
+                    mma_bf16_16816(acc[r][b], lo[S][r][s].x, hi[S][r][s].x, lo[S][r][s].y, hi[S][r][s].y, xv.x, xv.y);
+                    mma_bf16_16816(acc[r][b], lo[S][r][s].z, hi[S][r][s].z, lo[S][r][s].w, hi[S][r][s].w, xv.z, xv.w);
+                }
+            }
+    };
+    auto clear = [&]() {
+#pragma unroll
+        for (int r = 0; r < G; ++r)
+#pragma unroll
+            for (int b = 0; b < NB; ++b) { acc[r][b][0] = acc[r][b][1] = acc[r][b][2] = acc[r][b][3] = 0.f; }
+    };
+    const std::integral_constant<int, 0> set0;
+    const std::integral_constant<int, 1> set1;
+    // one stream of loads over all items of this CTA, two register sets, as in tgp_wstream_mma_group_kernel
+    uint32_t cur = blockIdx.x, item = cur, k0 = warp * 32 * U, pr = 0;
+    auto advance = [&]() -> bool {
+        if (++pr == (uint32_t)G) { pr = 0; k0 += NW * 32 * U; }
+        if (k0 < K) return false;
+        item += gridDim.x;
+        k0 = warp * 32 * U;
+        pr = 0;
+        if (item < total) locate(item);
+        return true;
+    };
+    locate(item);
+    issue(set0, k0);
+    issue(set1, k0 + 32 * SK);
+    bool cur_last = advance();
+    clear();
+    for (;;) {
+        const bool have_next = item < total;
+        const uint32_t kb = k0 + pr * 64 * SK;
+        consume(set0);
+        if (have_next) issue(set0, kb);
+        consume(set1);
+        if (have_next) issue(set1, kb + 32 * SK);
+        const bool next_last = have_next ? advance() : false;
+        const bool ended = cur_last;
+        cur_last = next_last;
+        if (!ended) continue;
+#pragma unroll
+        for (int r = 0; r < G; ++r)
+#pragma unroll
+            for (int b = 0; b < NB; ++b)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) part[warp][(r * NB + b) * 4 + i][lane] = acc[r][b][i];
+        __syncthreads();
+        uint32_t e, chunk, row0;
+        find(cur, e, chunk, row0);
+        for (uint32_t v = threadIdx.x; v < (GLU ? 1 : G) * NB * 4 * 32; v += NW * 32) {
+            const uint32_t slot = v >> 5, ln = v & 31, r = slot / (NB * 4), b = (slot >> 2) % NB, i = slot & 3;
+            float sum = 0.f, up = 0.f;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) sum += part[w][slot][ln];
+            if constexpr (GLU) {
+#pragma unroll
+                for (int w = 0; w < NW; ++w) up += part[w][NB * 4 + slot][ln];
+            }
+            const uint32_t first = row0 + r * p.rpc, row = first + (ln >> 2) + 8 * (i >> 1), t = chunk * T + b * 8 + 2 * (ln & 3) + (i & 1);
+            if (t < s_cnt[e] && row < min(first + p.rpc, p.n)) {
+                const size_t at = (size_t)(s_slot[e] + t) * p.n + row;
+                if constexpr (GLU) reinterpret_cast<bf16 *>(p.out)[at] = __float2bfloat16_rn(sum / (1.0f + expf(-sum)) * up);
+                else reinterpret_cast<float *>(p.out)[at] = sum;
+            }
+        }
+        cur += gridDim.x;
+        if (cur >= total) break;
+        __syncthreads();
+        clear();
+    }
+}
+
+// x[m, :] += gate * y[slot of m in its expert, :], experts in ascending order: the sums of tgp_scatter_add_kernel expert by expert.
+__global__ void __launch_bounds__(256) tgp_expert_combine_kernel(float *x, const float *y, const int32_t *idx, const float *gate, const int32_t *pos, const int32_t *counts, uint32_t d) {
+    pdl_enter();
+    const uint32_t m = blockIdx.x;
+    int e[2] = {idx[2 * m], idx[2 * m + 1]}, s[2] = {0, 1};
+    if (e[1] >= 0 && e[1] < e[0]) { s[0] = 1; s[1] = 0; }
+    const float4 *src[2] = {nullptr, nullptr};
+    float g[2] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int ex = e[s[i]];
+        if (ex < 0) continue;
+        uint32_t slot = (uint32_t)pos[2 * m + s[i]];
+        for (int q = 0; q < ex; ++q) slot += (uint32_t)counts[q];
+        src[i] = reinterpret_cast<const float4 *>(y + (size_t)slot * d);
+        g[i] = gate[2 * m + s[i]];
+    }
+    float4 *o = reinterpret_cast<float4 *>(x + (size_t)m * d);
+    for (uint32_t i = blockIdx.y * 256 + threadIdx.x; i < d / 4; i += gridDim.y * 256) {
+        float4 a = o[i];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            if (src[q]) {
+                const float4 b = src[q][i];
+                a.x += g[q] * b.x; a.y += g[q] * b.y; a.z += g[q] * b.z; a.w += g[q] * b.w;
+            }
+        o[i] = a;
+    }
+}
+
+// Whether the products of a step's experts take tgpk_gemm_rows() and may run all in one launch: the step has at most 32 tokens.
+bool tgpk_expert_rows(uint32_t M, uint32_t K) { return M <= 32 && K % 32 == 0 && g_skinny_impl == 0 && g_gemm_impl == 0; }
+
+// Blocks over the same `me` activation rows with the arithmetic of the expert kernels of a step of M tokens, in one launch per
+// 8 (M <= 8) or 16 rows.
+int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t me, uint32_t M, uint32_t K, cudaStream_t st) {
+    if (!count || count > TGP_GEMM_GROUP_MAX || K % 32) return TGP_E_INVAL;
+    const uint32_t T = M <= 8 ? 8 : 16;
+    for (uint32_t m0 = 0; m0 < me; m0 += T) {
+        GemvParts p;
+        memset(&p, 0, sizeof(p));
+        for (uint32_t s = 0; s < count; ++s) { p.W[s] = (const bf16 *)W[s]; p.C[s] = C[s] + (size_t)m0 * ldc[s]; p.n[s] = n[s]; p.ldc[s] = ldc[s]; }
+        p.count = count;
+        uint32_t groups = 0;
+        for (uint32_t s = 0; s < count; ++s) groups += p.groups[s] = (n[s] + 15) / 16;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(std::min((groups + 1) / 2, 2 * (uint32_t)device_sms())); cfg.blockDim = dim3(EXP_NW * 32); cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const bf16 *am = (const bf16 *)A + (size_t)m0 * K;
+        const uint32_t mr = std::min(T, me - m0);
+        if (T == 8) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<1, EXP_U, EXP_NW, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
+        else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<2, EXP_U, EXP_NW, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
+        tgpk_last_gemm_kernel = "tgp_wstream_mma_group_kernel";
+        LAUNCH_CHECK(1);
+    }
+    return TGP_OK;
+}
+
+int tgpk_experts(const TgpExperts &x, cudaStream_t st) {
+    if (x.E > TGP_MOE_EXPERTS || !tgpk_expert_rows(x.M, x.d) || x.F % 32) return TGP_E_INVAL;
+    const uint32_t sms = (uint32_t)device_sms(), T = x.M <= 8 ? 8 : 16;
+    ExpertParts p;
+    memset(&p, 0, sizeof(p));
+    p.rows = x.rows; p.counts = x.counts; p.E = x.E; p.stride = x.stride;
+    for (uint32_t e = 0; e < x.E; ++e)
+        for (uint32_t b = 0; b < TGP_MOE_BLOCKS; ++b) { p.w[0][e][b] = (const bf16 *)x.w[0][e][b]; p.w[1][e][b] = (const bf16 *)x.w[1][e][b]; }
+    p.A = (const bf16 *)x.h; p.out = x.a; p.n = x.F; p.K = x.d; p.per = x.per_f; p.rpc = 16;
+    if (T == 8) launch_pdl(tgp_expert_mma_kernel<1, true>, dim3(2 * sms), dim3(EXP_NW * 32), 0, st, p);
+    else launch_pdl(tgp_expert_mma_kernel<2, true>, dim3(2 * sms), dim3(EXP_NW * 32), 0, st, p);
+    for (uint32_t e = 0; e < x.E; ++e)
+        for (uint32_t b = 0; b < TGP_MOE_BLOCKS; ++b) { p.w[0][e][b] = (const bf16 *)x.w[2][e][b]; p.w[1][e][b] = nullptr; }
+    p.A = (const bf16 *)x.a; p.out = x.y; p.n = x.d; p.K = x.F; p.per = x.per_d;
+    // rows per group: the fewest rounds of the busiest CTA, weighted with its loads (rows a group lacks still take load slots), if three
+    // quarters of the experts that could have tokens do
+    const uint32_t busy = std::max(1u, std::min(x.E, x.M * x.topk) * 3 / 4);
+    uint64_t best = ~0ull;
+    for (uint32_t r = 16; r >= 5; --r) {
+        const uint64_t items = (uint64_t)busy * ((x.d + 2 * r - 1) / (2 * r)), cost = (items + 2 * sms - 1) / (2 * sms) * (r + 16 + 4);
+        if (cost < best) { best = cost; p.rpc = r; }
+    }
+    if (T == 8) launch_pdl(tgp_expert_mma_kernel<1, false>, dim3(2 * sms), dim3(EXP_NW * 32), 0, st, p);
+    else launch_pdl(tgp_expert_mma_kernel<2, false>, dim3(2 * sms), dim3(EXP_NW * 32), 0, st, p);
+    launch_pdl(tgp_expert_combine_kernel, dim3(x.M, x.d > 2048 ? 2 : 1), dim3(256), 0, st, x.x, (const float *)x.y, x.idx, x.gate, x.pos, x.counts, x.d);
+    LAUNCH_CHECK(3);
+    return TGP_OK;
 }
 
 // Which products may share a launch: those with the same non-zero key.  A key names the kernel a block takes on its own

@@ -43,9 +43,27 @@ int tgpk_attn_prefill_tc5(const void *qb, const TgpTilePtrs &tiles, void *ob, co
 // mma.sync flash-style causal attention for q_len > 1 (tgp_attn_prefill.cu); Dh 64 or 128
 int tgpk_attn_prefill_tc(const void *qb, const TgpTilePtrs &tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0, cudaStream_t st);
 int tgpk_swiglu(const float *g, const float *u, void *ab, uint64_t n, cudaStream_t st);
-// MoE: router logits + top-k (1 or 2) + gates, then per-expert token lists rows[e*stride + i], gates[e*stride + i], counts[e]
-int tgpk_router(const void *h, const void *Wr, const float *bias, int32_t *idx, float *gate, int32_t *rows, float *gates, int32_t *counts,
-                uint32_t M, uint32_t stride, uint32_t d, uint32_t E, uint32_t topk, cudaStream_t st);
+// MoE: router logits + top-k (1 or 2) + gates, then per-expert token lists rows[e*stride + i], gates[e*stride + i], counts[e].  Up to 64
+// tokens: one launch, which also writes pos[2 m + s] (place of token m in the list of its s-th expert) and, if given, the
+// counts to mapped host memory
+int tgpk_router(const void *h, const void *Wr, const float *bias, int32_t *idx, float *gate, int32_t *rows, float *gates, int32_t *counts, int32_t *pos,
+                int32_t *counts_host, uint32_t M, uint32_t stride, uint32_t d, uint32_t E, uint32_t topk, cudaStream_t st);
+// all experts of a layer for a step of at most 32 tokens, from the router's lists on the device: a = SwiGLU of the gate and up
+// projections of the routed rows of h (one row per slot), y = their down projections, x += gate * y.  w[0..2]: gate, up, down of
+// each expert in blocks of per_f (gate, up) or per_d (down) rows.  Bit-identical to the experts one by one (tgpk_gemm_rows)
+#define TGP_MOE_EXPERTS 16
+#define TGP_MOE_BLOCKS 4
+struct TgpExperts {
+    const void *w[3][TGP_MOE_EXPERTS][TGP_MOE_BLOCKS], *h;
+    void *a; float *y, *x;
+    const int32_t *rows, *counts, *idx, *pos; const float *gate;
+    uint32_t E, topk, M, d, F, per_f, per_d, stride;
+};
+int tgpk_experts(const TgpExperts &x, cudaStream_t st);
+bool tgpk_expert_rows(uint32_t M, uint32_t K);
+int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t me, uint32_t M, uint32_t K, cudaStream_t st);
+// products over the same activations may share a launch (tgp_k_gemm_group_select)
+bool tgpk_gemm_grouping();
 int tgpk_gather_rows(const void *src, const int32_t *rows, void *dst, uint32_t m, uint32_t d, cudaStream_t st);
 int tgpk_scatter_add(float *x, const float *y, const int32_t *rows, const float *gates, uint32_t m, uint32_t d, cudaStream_t st);
 int tgpk_argmax(const float *logits, int32_t *out, uint32_t B, uint32_t V, cudaStream_t st);

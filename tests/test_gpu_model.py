@@ -502,6 +502,49 @@ def test_llama_8b_widths_at_two_layers_lockstep_parity():
     assert tb.k_attn_status() == 0 and tb.k_gemm_status() == 0
 
 
+@pytest.mark.parametrize("B,topk,d,F,cap", [(1, 2, 256, 512, 64 << 10), (8, 2, 256, 480, 128 << 10), (9, 1, 256, 512, 1 << 20), (16, 2, 512, 1056, 1 << 20),
+                                            (17, 2, 256, 512, 1 << 20), (32, 2, 256, 544, 1 << 20), (33, 2, 256, 512, 1 << 20)])
+def test_moe_decode_runs_all_experts_of_a_layer_together_with_the_same_bits(B, topk, d, F, cap):
+    """Decode steps of up to 32 tokens with every expert traced and on the device: one launch for the gate and up projections of all
+    experts, one for the down projections, one that adds them up, and the host does not wait for the router.  Against the same
+    step with grouping off (one launch per block, sized by the host): token counts at the edges of the 8- and 16-token
+    chunks, one and several blocks per matrix, ragged row groups - the same bits, the same expert counts, the oracle's logits."""
+    cfg = replace(MOE, B=B, S=7, T=3, d=d, F=F, Hq=d // 64, Hkv=d // 128, Dh=64, topk=topk)
+    lay = si.build_layout(cfg, budget=64 << 20, cap=cap)
+    bias = si.router_bias(cfg)
+    pool = pinned_pool(lay.pool_bytes)
+    si.fill_pool(lay, pool.numpy())
+    om = forward.OracleModel(cfg, si.weights_as_bits(lay), bias, dtype=np.float32)
+    prompt = si.prompt_tokens(cfg)
+    ref, toks = om.generate(prompt, cfg.T)
+    s = Session(lay, MACHINE, pool_base=pool.data_ptr(), pool_flags=tb.POOL_PINNED, router_bias=bias)
+    s.plan(expert_counts=np.ones((1 + cfg.T, cfg.L, cfg.E), dtype=np.uint32))
+    r = Runner(s, cfg.B * cfg.S)
+    runs = []
+    for enable in (1, 0):
+        tb.k_gemm_group_select(enable)
+        logits, launches = [], []
+        r.reset()
+        r.step(tb.PREFILL, prompt, cfg.S, want_stats=True)
+        logits.append(r.logits.cpu().numpy().copy())
+        for t in range(cfg.T):
+            st = r.step(tb.DECODE, np.ascontiguousarray(toks[:, t:t + 1]), 1, want_stats=True)
+            launches.append(st.n_launches)
+            assert st.n_mismatch == 0
+            logits.append(r.logits.cpu().numpy().copy())
+        runs.append((logits, s.ctx.expert_counts(cfg.L, cfg.E).copy(), launches))
+    tb.k_gemm_group_select(1)
+    s.close()
+    for a, b in zip(runs[0][0], runs[1][0]):
+        assert np.array_equal(a, b)
+    assert np.array_equal(runs[0][1], runs[1][1]) and (runs[0][1].sum(axis=2)[1:] == B * topk).all()
+    if B <= 32:
+        # per layer 2 norms, the q k v list, rope, attention, its merge at most, o, router, 3 for the experts; embed, norm, head blocks, argmax
+        assert max(runs[0][2]) <= 11 * cfg.L + 3 + len(lay.blocks(si.K_LM, -1, -1)), runs[0][2]
+    if B == 16:
+        check_logits([runs[0][0][0]], [ref[0]])
+
+
 def test_mixtral_widths_at_one_layer_match_oracle_batch_of_eight():
     """Full widths of the Mixtral shape (8 experts of 14336, top-2) at one layer, batch 8, free-running: the expert
     products run at the handful of tokens each expert receives (skinny tensor-core GEMV on blocks of few rows), planned
