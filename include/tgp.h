@@ -302,8 +302,9 @@ int  tgp_k_gemm(const void *A_dev, const void *W_dev, float *C_dev, uint32_t M, 
  * returns.  Blocks whose tgp_k_gemm_group_key() is the same non-zero value are served by one launch - a block of few
  * rows alone leaves most SMs without work - anything else by one launch per part; the results are bit-identical to
  * tgp_k_gemm() per part either way, because the key names the kernel the block takes on its own (M <= 2: fewer than
- * 4736 rows and K < 8192; 3 <= M <= 32 with K % 32 == 0: blocks of fewer 16-row groups than the GPU has SMs, which pick
- * the same split-K kernel instance).
+ * 4736 rows of W and K < 8192; to 16 rows with K % 32 == 0: blocks that the persistent list kernel serves, which pick the
+ * same instance of it; to 32 rows: blocks that the tcgen05 kernel serves with the same split of K).  Above 32 rows the
+ * key is 0, but neighbours in the list that one tcgen05 kernel serves share a launch all the same.
  * tgp_k_gemm_group_select(0) makes every key 0 (process-wide; default 1), also inside tgp_step(), which groups
  * consecutive weight-block products of a decode step that read the same activations this way when their copies have
  * all been enqueued and no tap is set, except blocks under 2 MiB whose arena slot a later copy waits for (with op timing
@@ -329,32 +330,31 @@ int  tgp_k_swiglu_epilogue(int enable);
  * Results are identical either way.  Process-wide; default off: on the tiny configuration it takes a decode step from 50
  * launches to 32, but a fused span waits for the copies of all its blocks, and the step got no faster (measured). */
 int  tgp_k_decode_fuse(int enable);
-/* Which kernel serves M > 16: 0 (default) the tcgen05 tensor-core GEMM, 1 the CUDA-core tile kernel (an on-device
- * cross-check).  M <= 16 always takes the weight-streaming GEMV.  Process-wide. */
+/* Which kernel serves M > 16 (and, on blocks of 8065 or more rows, M > 8): 0 (default) the tcgen05 tensor-core kernels, 1 the
+ * CUDA-core tile kernel (an on-device cross-check; M <= 16 then takes the weight-streaming kernels).  Process-wide. */
 int  tgp_k_gemm_select(int impl);
-/* Which kernel serves 3 <= M <= 32 (K % 32 == 0; and, as two launches of half the rows, 33 <= M <= 64 on blocks of fewer
- * than 4096 rows): 0 (default) the weight-streaming tensor-core kernel, 1 the
- * CUDA-core GEMV (M <= 16) / GEMM paths (an on-device cross-check).  Process-wide. */
+/* Which kernel serves 3 <= M <= 16 (K % 32 == 0): 0 (default) the weight-streaming mma.sync kernels, 1 the CUDA-core GEMV (an
+ * on-device cross-check).  Process-wide. */
 int  tgp_k_skinny_select(int impl);
-/* Weight-streaming launches (M <= 32) and the small kernels of a step (embedding gather, RMSNorm, RoPE + KV append, decode
- * attention and its merge, SwiGLU, argmax) use programmatic dependent launch: a launch lets its successor be scheduled
- * at once; a weight-streaming kernel starts reading its weights while the previous kernel of the stream drains and
- * waits for it only before it touches activations or output, a small kernel waits first thing, so that only its launch
- * latency overlaps.  0 switches that off (each launch then starts after the previous one has completed).  Results are
+/* Products, attention and the small kernels of a step (embedding gather, RMSNorm, RoPE + KV append, SwiGLU, argmax, router and
+ * experts of a small step) use programmatic dependent launch: a launch lets its successor be scheduled at once; a
+ * weight-streaming kernel of up to 16 rows starts reading its weights while the previous kernel of the stream drains and
+ * waits for it only before it touches activations or output, every other kernel waits before it reads anything, so that
+ * only its launch latency and set-up overlap.  0 switches that off (each launch then starts after the previous one has completed).  Results are
  * identical either way.  Process-wide; default on. */
 int  tgp_k_gemv_overlap(int enable);
 /* A promise by a caller of the kernel entry points, for the calling thread: between consecutive tgp_k_gemm() /
  * tgp_k_gemm_group() calls on one stream nothing but this library's kernels (launched by this thread) is enqueued on that
- * stream.  A product of 3 - 32 activation rows that directly follows another one over the same activation pointer then
+ * stream.  A product of 3 - 16 activation rows that directly follows another one over the same activation pointer then
  * requests its activations together with its weights, before the previous launch has finished (they are older than that
  * launch); results are identical.  tgp_step() works this way by itself.  Default off: a caller that rewrites the
  * activations between two calls by other means must leave it off. */
 int  tgp_k_gemm_chain(int enable);
-/* Tensor-core GEMM variant: 0 (default) picks by problem size, 1 forces the 128x128 one-tile-per-CTA kernel,
- * 2 the persistent 128x256 kernel with double-buffered accumulators, 3 the paired kernel (256x256 tiles on the two SMs
- * of a CTA pair, each loading half of the weight tile), 4 the one-tile-per-CTA kernel with the operands swapped (the
- * weights are the 128-row operand, the tile is stored transposed; for M <= 128, else as 0; picked by size for M <= 64 on
- * blocks of many rows).  Process-wide; for tests and timing. */
+/* Tensor-core GEMM variant: 0 (default) picks by problem size between the paired kernel (tiles of 256 weight rows x up to 256
+ * activation rows on the two SMs of a CTA pair) and the one of one 128-row weight tile per CTA, with K in one, two or four
+ * slices; 1 forces the 128x128 one-tile-per-CTA kernel, 2 the persistent 128x256 kernel with double-buffered accumulators,
+ * 3 the paired kernel with its largest tiles, 4 the one-tile-per-CTA kernel of variant 1 with the operands swapped (the weights
+ * are the 128-row operand, the tile is stored transposed; for M <= 128, else as 0).  Process-wide; for tests and timing. */
 int  tgp_k_gemm_tc_variant(int variant);
 /* Which kernel serves attention with q_len >= 16: 0 (default) by problem size - the tcgen05 kernel (S and O in TMEM,
  * K/V fed by TMA) for q_len >= 128, else the mma.sync flash-style kernel;
@@ -362,11 +362,11 @@ int  tgp_k_gemm_tc_variant(int variant);
  * kernel needs KV tiles of a multiple of 64 keys whose base addresses differ by whole rows of Dh elements (and
  * 16-byte aligned q); any other geometry is served by the mma.sync kernel even when 3 is forced.  Process-wide. */
 int  tgp_k_attn_select(int impl);
-/* Which kernel serves decode attention (q_len == 1 with scratch): 0 (default) by size - the tensor-core kernel (the G query
- * heads of a KV head as rows of an mma.sync tile, K and V staged through shared memory with cp.async three chunks of 16
- * keys deep, P rounded to bf16 for the second product) when KV tiles hold a multiple of 16 keys, G is 1, 2, 4 or 8 and
- * the batch's context adds up to 256 chunks or more, else the CUDA-core kernels (one pass per KV tile and group of query
- * heads); 1 forces the CUDA-core kernels, 2 the tensor-core kernel wherever its geometry allows.  Process-wide. */
+/* Which kernel serves decode attention (q_len == 1 with scratch): 0 (default) and 2 the tensor-core kernel (the G query heads of
+ * a KV head as rows of an mma.sync tile, K and V staged through shared memory with cp.async three chunks of 16 keys deep)
+ * when KV tiles hold a multiple of 16 keys and G is 1, 2, 4 or 8, else the CUDA-core kernels (one pass per KV tile and group
+ * of query heads); 1 forces the CUDA-core kernels.  The tensor-core kernel rounds P to bf16 for the second product; while the
+ * batch's context adds up to less than 256 chunks it multiplies the remainder with V too.  Process-wide. */
 int  tgp_k_attn_decode_select(int impl);
 /* Error word of the tcgen05 attention kernel: 0, or which bounded wait ran out first (1 for S, 2 for P V, 3 for a K/V
  * load, 4 for the hand-over between the softmax warps and the MMA warp), or 5 if shared memory was not 1024-byte

@@ -879,8 +879,7 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
             else rc = tgpk_swiglu(e->g32, e->u32, e->ab, (uint64_t)M * c.F, cs);
             break;
         case TGP_OP_ARGMAX:
-            rc = tgpk_argmax(logits_dev, e->amax, B, c.V, cs);
-            if (!rc && argmax_dev) CU(ctx, cudaMemcpyAsync(argmax_dev, e->amax, (size_t)B * 4, cudaMemcpyDeviceToDevice, cs));
+            rc = tgpk_argmax(logits_dev, e->amax, argmax_dev, B, c.V, cs);
             break;
         default:
             return tgp_fail(ctx, TGP_E_MISMATCH, "op kind the bound model cannot run");

@@ -542,6 +542,10 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
 // their weights in no faster than HBM delivers them), and there are four times as many tiles to share out.
 //   K slices: a block of few tiles is split along K over the SL CTAs of a cluster; their partial tiles meet in shared memory
 // and are summed pairwise.  The split depends on M, n and K alone: a block computes the same bits alone or in a list.
+//   Accumulators: consecutive MMAs go to different ones (eight up to 32 activation rows, four up to 64, else two), summed at the end.
+// The tensor core adds into fp32 without rounding to nearest, so the error of a sum grows with the number of additions in a
+// row, and MMAs into one accumulator or into several take the same time (M=61, n=4096, K=4096: distance from 64 bits 1.0e-6 with
+// one, 2.4e-7 with four; n=14336 unsplit 4.4e-6, 1.0e-6).
 //   Ring: 200 KB where the launch gives an SM one CTA (M=61, n=14336, K=4096: 24.9 us; 28.4 us with 100 KB), else 100 KB, so that
 // an SM holds two (28672 rows: 43.0 us; 50.3 us with 200 KB).
 constexpr uint32_t S_RING = 100 * 1024, S_RING_LONE = 200 * 1024, S_STAGES = 12;
@@ -599,7 +603,8 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t slice = SL > 1 ? cluster_ctarank() : 0, tile = blockIdx.x / SL;
     const uint32_t kblocks = (p.K + BK - 1) / BK, kb_lo = kblocks * slice / SL, num_k = kblocks * (slice + 1) / SL - kb_lo;
-    const uint32_t cols = N <= 32 ? 32u : N <= 64 ? 64u : 128u;                     // TMEM columns
+    const uint32_t acc_cols = N <= 32 ? 32u : N <= 64 ? 64u : 128u, cols = 256;     // TMEM: up to 256 / acc_cols accumulators
+    const uint32_t accs = N > 64 ? 2u : N > 32 || num_k < 2 ? 4u : 8u;
     const uint32_t m0 = tile % p.tiles_m * N, rows = min(N, p.M - m0);              // this tile's activation rows
     uint32_t part = 0, wt = tile / p.tiles_m;
     while (part + 1 < p.count && wt >= p.tiles[part]) wt -= p.tiles[part++];
@@ -655,7 +660,7 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint64_t dw = umma_desc(smem_u32(ring + s * STAGE)), dx = umma_desc(smem_u32(ring + s * STAGE + W_BYTES));
 #pragma unroll
-                for (uint32_t k = 0; k < BK / 16; ++k) umma(tmem_base, dw + 2 * k, dx + 2 * k, idesc, (kb | k) != 0);
+                for (uint32_t k = 0; k < BK / 16; ++k) umma(tmem_base + ((4 * kb + k) & (accs - 1)) * acc_cols, dw + 2 * k, dx + 2 * k, idesc, 4 * kb + k >= accs);
                 umma_commit(&empty[s]);
                 if (++s == ST) { s = 0; ph ^= 1; }
             }
@@ -673,8 +678,18 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
             const bool mine = row < p.n[part];
 #pragma unroll 1
             for (uint32_t c = 0; c < N; c += 32) {
-                float v[32];
-                tmem_ld32(tmem_base + ((quarter * 32) << 16) + c, v);          // (N = 16, 48, ...: the columns past N are not used)
+                const uint32_t at_t = tmem_base + ((quarter * 32) << 16) + c;  // (N = 16, 48, ...: the columns past N are not used)
+                float v[32], w[32], y[32];
+                tmem_ld32(at_t, v);
+                tmem_ld32(at_t + acc_cols, w);
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] += w[j];
+                for (uint32_t i = 2; i < accs; i += 2) {
+                    tmem_ld32(at_t + i * acc_cols, w);
+                    tmem_ld32(at_t + (i + 1) * acc_cols, y);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] += w[j] + y[j];
+                }
                 if (SL > 1) {                                      // this slice's partial over the idle ring
                     float *part_s = reinterpret_cast<float *>(ring) + wrow;
 #pragma unroll

@@ -249,8 +249,7 @@ __device__ __forceinline__ float rms_scale_as_kernel(const float *xrow, uint32_t
     return 1.0f / sqrtf(t / (float)d + eps);
 }
 
-__device__ __forceinline__ void act8(const ASrc &s, const bf16 *A, uint32_t m, uint32_t K, uint32_t k, float r, float *xf) {
-    if (s.mode == 0) { unpack8(ld_act(reinterpret_cast<const uint4 *>(A + (size_t)m * K + k)), xf); return; }
+__device__ __forceinline__ void act8(const ASrc &s, uint32_t m, uint32_t K, uint32_t k, float r, float *xf) {
     if (s.mode == 1) {
         const float4 *xr = reinterpret_cast<const float4 *>(s.x + (size_t)m * s.ldx + k);
         const float4 v0 = xr[0], v1 = xr[1];
@@ -268,7 +267,9 @@ __device__ __forceinline__ void act8(const ASrc &s, const bf16 *A, uint32_t m, u
     for (int i = 0; i < 8; ++i) xf[i] = __bfloat162float(__float2bfloat16_rn(gv[i] / (1.0f + expf(-gv[i])) * uv[i]));
 }
 
-template <int MT, int U>
+// FUSED: src.mode is 1 or 2.  The plain form has its own instance: with the choice of source between them the activation loads of a
+// row's U chunks waited for one another (M=1, three blocks of 3072 rows in all, K=2048: 6.0 us, 2.9 us without).
+template <int MT, int U, bool FUSED>
 __global__ void __launch_bounds__(256) tgp_wstream_group_kernel(const bf16 *A, const GemvParts p, uint32_t Mrows, uint32_t n_total, uint32_t K, int accumulate, const ASrc src) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarp = (gridDim.x * blockDim.x) >> 5;
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(256) tgp_wstream_group_kernel(const bf16 *A, c
             if (!synced) {
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 synced = true;
-                if (src.mode == 1) {
+                if (FUSED && src.mode == 1) {
 #pragma unroll
                     for (int m = 0; m < MT; ++m) if (m < (int)Mrows) rs[m] = rms_scale_as_kernel(src.x + (size_t)m * src.ldx, K, src.eps, lane);
                 }
@@ -312,7 +313,8 @@ __global__ void __launch_bounds__(256) tgp_wstream_group_kernel(const bf16 *A, c
 #pragma unroll
                 for (int m = 0; m < MT; ++m) {
                     float xf[8];
-                    if (k < K && m < (int)Mrows) act8(src, A, m, K, k, rs[m], xf);
+                    if constexpr (!FUSED) unpack8((k < K && m < (int)Mrows) ? ld_act(reinterpret_cast<const uint4 *>(A + (size_t)m * K + k)) : make_uint4(0, 0, 0, 0), xf);
+                    else if (k < K && m < (int)Mrows) act8(src, m, K, k, rs[m], xf);
                     else {
 #pragma unroll
                         for (int i = 0; i < 8; ++i) xf[i] = 0.f;
@@ -907,7 +909,9 @@ __global__ void __launch_bounds__(DH) tgp_attn_decode_merge_kernel(AttnArgs a) {
 //   online softmax per row       (the running maximum moves rarely: O is rescaled only when a row's maximum grew);
 //   O[16 x Dh] += P V            Dh/8 MMAs, P straight from the S accumulators as the A fragment, V fragments by
 //                                ldmatrix.trans (V rows are keys: the transposed load makes keys the contraction index).
-// P is rounded to bf16 for the second product, as in the prefill kernels.  A CTA of four warps owns a contiguous range of
+// P is rounded to bf16 for the second product, as in the prefill kernels; in short contexts (SPLIT_P) what that leaves over is
+// multiplied with V too, so P counts with 16 bits (the distance from 64-bit attention is then that of the CUDA-core kernels to
+// six digits, 9 - 1500 keys).  A CTA of four warps owns a contiguous range of
 // chunks of one (sequence, KV head); its warps take every fourth chunk, merge their four partials through shared memory
 // and write one (max, sum, unnormalised O) per query head and CTA to the scratch array tgp_attn_decode_merge_kernel reads.
 // Stage layout: row = key, 2*DH bytes, 16-byte chunk j of row r at chunk position j ^ (r & 7): conflict-free for the
@@ -929,7 +933,7 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
 }
 __device__ __forceinline__ float fast_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
-template <int DH, int G>
+template <int DH, int G, bool SPLIT_P>
 __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(AttnArgs a, uint32_t chunks_per_cta) {
     pdl_enter();
     extern __shared__ __align__(128) uint8_t dec_sm[];
@@ -1028,6 +1032,11 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
         l_run += ls;
         __nv_bfloat162 plo = __floats2bfloat162_rn(p[0], p[1]), phi = __floats2bfloat162_rn(p[2], p[3]);
         const uint32_t pa0 = *reinterpret_cast<uint32_t *>(&plo), pa2 = *reinterpret_cast<uint32_t *>(&phi);
+        uint32_t pb0 = 0, pb2 = 0;                                        // what the rounding of P left over
+        if constexpr (SPLIT_P) {
+            __nv_bfloat162 rlo = __floats2bfloat162_rn(p[0] - __low2float(plo), p[1] - __high2float(plo)), rhi = __floats2bfloat162_rn(p[2] - __low2float(phi), p[3] - __high2float(phi));
+            pb0 = *reinterpret_cast<uint32_t *>(&rlo); pb2 = *reinterpret_cast<uint32_t *>(&rhi);
+        }
         // ---- O += P V: Dh/8 n-tiles, two per ldmatrix ----
 #pragma unroll
         for (int jp = 0; jp < DH / 16; ++jp) {
@@ -1036,6 +1045,7 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
             ldsm_x4_t(vb + row * ROW + ((j ^ (row & 7)) << 4), v0, v1, v2, v3);
             mma_bf16(o[2 * jp], pa0, 0u, pa2, 0u, v0, v1);
             mma_bf16(o[2 * jp + 1], pa0, 0u, pa2, 0u, v2, v3);
+            if constexpr (SPLIT_P) { mma_bf16(o[2 * jp], pb0, 0u, pb2, 0u, v0, v1); mma_bf16(o[2 * jp + 1], pb0, 0u, pb2, 0u, v2, v3); }
         }
         __syncwarp();                                                 // the stage may be refilled two iterations from now
     }
@@ -1091,7 +1101,7 @@ __global__ void tgp_swiglu_kernel(const float4 *g, const float4 *u, __nv_bfloat1
 // A row is shared by the CTAs of a cluster (8 for long rows): each scans a contiguous part with four independent 16-byte loads per
 // thread under way, and the parts' winners meet in the first CTA's shared memory (8 rows of 32000: 9.5 us with one CTA of 1024
 // threads and one dependent element per thread and round, 3.4 us now, from the end of the kernel before).
-__global__ void __launch_bounds__(256) tgp_argmax_kernel(const float *logits, int32_t *out, uint32_t V, int vec) {
+__global__ void __launch_bounds__(256) tgp_argmax_kernel(const float *logits, int32_t *out, int32_t *out2, uint32_t V, int vec) {
     pdl_enter();
     __shared__ float bv[8], cv[8];
     __shared__ uint32_t bi[8], ci[8];
@@ -1132,7 +1142,7 @@ __global__ void __launch_bounds__(256) tgp_argmax_kernel(const float *logits, in
         for (int o = 4; o; o >>= 1) merge(best, idx, __shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, idx, o));
     }
     if (parts == 1) {
-        if (threadIdx.x == 0) out[blockIdx.x] = (int32_t)idx;
+        if (threadIdx.x == 0) { out[blockIdx.x] = (int32_t)idx; if (out2) out2[blockIdx.x] = (int32_t)idx; }
         return;
     }
     if (threadIdx.x == 0) {                                    // to slot `rank` of the cluster's first CTA
@@ -1150,7 +1160,7 @@ __global__ void __launch_bounds__(256) tgp_argmax_kernel(const float *logits, in
         idx = lane < parts ? ci[lane] : 0u;
 #pragma unroll
         for (int o = 4; o; o >>= 1) merge(best, idx, __shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, idx, o));
-        if (lane == 0) out[blockIdx.x / parts] = (int32_t)idx;
+        if (lane == 0) { out[blockIdx.x / parts] = (int32_t)idx; if (out2) out2[blockIdx.x / parts] = (int32_t)idx; }
     }
 }
 
@@ -1806,14 +1816,14 @@ static void launch_gemv_rows(const bf16 *A, const bf16 *W, float *C, uint32_t Mr
     }
 }
 
-template <int MT>
+template <int MT, bool FUSED>
 static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows, uint32_t n_total, uint32_t K, int acc, cudaStream_t st, const ASrc &src = ASrc{}) {
     static int blocks_per_sm = 0, sms = 0;
     if (!blocks_per_sm) {
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, tgp_wstream_group_kernel<MT, 8>, 256, 0) != cudaSuccess || blocks_per_sm < 1) blocks_per_sm = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, tgp_wstream_group_kernel<MT, 8, FUSED>, 256, 0) != cudaSuccess || blocks_per_sm < 1) blocks_per_sm = 1;
         if (sms < 1) sms = 148;
     }
     uint32_t need = (n_total + 7) / 8, full = (uint32_t)(sms * blocks_per_sm);
@@ -1826,7 +1836,7 @@ static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows,
     attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, tgp_wstream_group_kernel<MT, 8>, A, p, Mrows, n_total, K, acc, src);
+    cudaLaunchKernelEx(&cfg, tgp_wstream_group_kernel<MT, 8, FUSED>, A, p, Mrows, n_total, K, acc, src);
     tgpk_last_gemm_kernel = "tgp_wstream_group_kernel";
 }
 
@@ -1837,7 +1847,7 @@ static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows,
 // tokens, a second one the down projections, and a third adds a token's two results to its residual row.  The counts
 // are read on the device: work items are (expert, up to 8 NB of its tokens, 16 rows of gate and of up, or two groups of `rpc`
 // rows of down), and the CTAs walk the list of those that exist.
-//   The arithmetic of an item is that of tgp_wstream_mma_group_kernel<NB, EXP_U, EXP_NW, 16, 2>: which warp adds which k in which order
+//   The arithmetic of an item is that of tgp_wstream_mma_group_kernel<NB, EXP_U, NW, 16, 2>: which warp adds which k in which order
 // depends on K alone, so the bits are those of the expert's own products (tgpk_gemm_rows).
 struct ExpertParts {
     const bf16 *w[2][TGP_MOE_EXPERTS][TGP_MOE_BLOCKS];       // GLU: gate and up; else [0]: down; in blocks of `per` rows
@@ -1847,13 +1857,15 @@ struct ExpertParts {
     uint32_t n, K, per, E, stride, rpc;
 };
 
-// Eight warps of four load steps: a chunk of 1024 columns, so that the K of a small expert keeps every warp at work; two CTAs per
-// SM have 64 KB of loads under way, as many as HBM needs.
-constexpr int EXP_U = 4, EXP_NW = 8;
+// 16 warps of four load steps, or up to K=2047 twice as many CTAs of eight: a chunk of 1024 columns, so that the K of a small expert
+// keeps every warp at work.  Either way an SM has 64 KB of loads under way, as many as HBM needs.  More warps mean fewer
+// additions in a row per warp: a warp adds K / (16 NW) MMAs, no more than in the products of 3 - 16 rows above.
+constexpr int EXP_U = 4;
+static int expert_warps(uint32_t K) { return K >= 2048 ? 16 : 8; }
 
-template <int NB, bool GLU>
-__global__ void __launch_bounds__(EXP_NW * 32, 2) tgp_expert_mma_kernel(const ExpertParts p) {
-    constexpr int U = EXP_U, NW = EXP_NW, G = 2, SK = U / (2 * G), T = NB * 8;       // T: tokens per item
+template <int NB, int NW, bool GLU>
+__global__ void __launch_bounds__(NW * 32, 16 / NW) tgp_expert_mma_kernel(const ExpertParts p) {
+    constexpr int U = EXP_U, G = 2, SK = U / (2 * G), T = NB * 8;       // T: tokens per item
     __shared__ float part[NW][G * NB * 4][32];
     __shared__ uint32_t s_first[TGP_MOE_EXPERTS + 1], s_slot[TGP_MOE_EXPERTS], s_cnt[TGP_MOE_EXPERTS];
     pdl_enter();
@@ -2024,8 +2036,9 @@ __global__ void __launch_bounds__(256) tgp_expert_combine_kernel(float *x, const
     }
 }
 
-// Whether the products of a step's experts take tgpk_gemm_rows() and may run all in one launch: the step has at most 32 tokens.
-bool tgpk_expert_rows(uint32_t M, uint32_t K) { return M <= 32 && K % 32 == 0 && g_skinny_impl == 0 && g_gemm_impl == 0; }
+// Whether the products of a step's experts take tgpk_gemm_rows() and may run all in one launch: the step has 3 to 32 tokens (one or two
+// stay with the CUDA-core kernels, whose sums are closer to 64 bits).
+bool tgpk_expert_rows(uint32_t M, uint32_t K) { return M >= 3 && M <= 32 && K % 32 == 0 && g_skinny_impl == 0 && g_gemm_impl == 0; }
 
 // Blocks over the same `me` activation rows with the arithmetic of the expert kernels of a step of M tokens, in one launch per
 // 8 (M <= 8) or 16 rows.
@@ -2040,7 +2053,8 @@ int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *c
         uint32_t groups = 0;
         for (uint32_t s = 0; s < count; ++s) groups += p.groups[s] = (n[s] + 15) / 16;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(std::min((groups + 1) / 2, 2 * (uint32_t)device_sms())); cfg.blockDim = dim3(EXP_NW * 32); cfg.stream = st;
+        const uint32_t nw = (uint32_t)expert_warps(K);
+        cfg.gridDim = dim3(std::min((groups + 1) / 2, 16 / nw * (uint32_t)device_sms())); cfg.blockDim = dim3(nw * 32); cfg.stream = st;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
@@ -2048,12 +2062,26 @@ int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *c
         cfg.numAttrs = 1;
         const bf16 *am = (const bf16 *)A + (size_t)m0 * K;
         const uint32_t mr = std::min(T, me - m0);
-        if (T == 8) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<1, EXP_U, EXP_NW, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
-        else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<2, EXP_U, EXP_NW, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
+        if (T == 8 && nw == 8) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<1, EXP_U, 8, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
+        else if (T == 8) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<1, EXP_U, 16, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
+        else if (nw == 8) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<2, EXP_U, 8, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
+        else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<2, EXP_U, 16, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
         tgpk_last_gemm_kernel = "tgp_wstream_mma_group_kernel";
         LAUNCH_CHECK(1);
     }
     return TGP_OK;
+}
+
+template <bool GLU>
+static void launch_experts(const ExpertParts &p, uint32_t T, cudaStream_t st) {
+    const uint32_t sms = (uint32_t)device_sms();
+    if (expert_warps(p.K) == 8) {
+        if (T == 8) launch_pdl(tgp_expert_mma_kernel<1, 8, GLU>, dim3(2 * sms), dim3(256), 0, st, p);
+        else launch_pdl(tgp_expert_mma_kernel<2, 8, GLU>, dim3(2 * sms), dim3(256), 0, st, p);
+    } else {
+        if (T == 8) launch_pdl(tgp_expert_mma_kernel<1, 16, GLU>, dim3(sms), dim3(512), 0, st, p);
+        else launch_pdl(tgp_expert_mma_kernel<2, 16, GLU>, dim3(sms), dim3(512), 0, st, p);
+    }
 }
 
 int tgpk_experts(const TgpExperts &x, cudaStream_t st) {
@@ -2065,21 +2093,19 @@ int tgpk_experts(const TgpExperts &x, cudaStream_t st) {
     for (uint32_t e = 0; e < x.E; ++e)
         for (uint32_t b = 0; b < TGP_MOE_BLOCKS; ++b) { p.w[0][e][b] = (const bf16 *)x.w[0][e][b]; p.w[1][e][b] = (const bf16 *)x.w[1][e][b]; }
     p.A = (const bf16 *)x.h; p.out = x.a; p.n = x.F; p.K = x.d; p.per = x.per_f; p.rpc = 16;
-    if (T == 8) launch_pdl(tgp_expert_mma_kernel<1, true>, dim3(2 * sms), dim3(EXP_NW * 32), 0, st, p);
-    else launch_pdl(tgp_expert_mma_kernel<2, true>, dim3(2 * sms), dim3(EXP_NW * 32), 0, st, p);
+    launch_experts<true>(p, T, st);
     for (uint32_t e = 0; e < x.E; ++e)
         for (uint32_t b = 0; b < TGP_MOE_BLOCKS; ++b) { p.w[0][e][b] = (const bf16 *)x.w[2][e][b]; p.w[1][e][b] = nullptr; }
     p.A = (const bf16 *)x.a; p.out = x.y; p.n = x.d; p.K = x.F; p.per = x.per_d;
     // rows per group: the fewest rounds of the busiest CTA, weighted with its loads (rows a group lacks still take load slots), if three
     // quarters of the experts that could have tokens do
-    const uint32_t busy = std::max(1u, std::min(x.E, x.M * x.topk) * 3 / 4);
+    const uint32_t slots = 16 / (uint32_t)expert_warps(x.F) * sms, busy = std::max(1u, std::min(x.E, x.M * x.topk) * 3 / 4);
     uint64_t best = ~0ull;
     for (uint32_t r = 16; r >= 5; --r) {
-        const uint64_t items = (uint64_t)busy * ((x.d + 2 * r - 1) / (2 * r)), cost = (items + 2 * sms - 1) / (2 * sms) * (r + 16 + 4);
+        const uint64_t items = (uint64_t)busy * ((x.d + 2 * r - 1) / (2 * r)), cost = (items + slots - 1) / slots * (r + 16 + 4);
         if (cost < best) { best = cost; p.rpc = r; }
     }
-    if (T == 8) launch_pdl(tgp_expert_mma_kernel<1, false>, dim3(2 * sms), dim3(EXP_NW * 32), 0, st, p);
-    else launch_pdl(tgp_expert_mma_kernel<2, false>, dim3(2 * sms), dim3(EXP_NW * 32), 0, st, p);
+    launch_experts<false>(p, T, st);
     launch_pdl(tgp_expert_combine_kernel, dim3(x.M, x.d > 2048 ? 2 : 1), dim3(256), 0, st, x.x, (const float *)x.y, x.idx, x.gate, x.pos, x.counts, x.d);
     LAUNCH_CHECK(3);
     return TGP_OK;
@@ -2124,8 +2150,8 @@ int tgpk_gemm_group(const void *A, uint32_t count, const void *const *W, float *
     uint32_t total = 0;
     for (uint32_t s = 0; s < count; ++s) { p.W[s] = (const bf16 *)W[s]; p.C[s] = C[s]; p.n[s] = n[s]; p.ldc[s] = ldc[s]; total += n[s]; }
     p.count = count;
-    if (M == 1) launch_gemv_group<1>((const bf16 *)A, p, M, total, K, accumulate, st);
-    else if (M == 2) launch_gemv_group<2>((const bf16 *)A, p, M, total, K, accumulate, st);
+    if (M == 1) launch_gemv_group<1, false>((const bf16 *)A, p, M, total, K, accumulate, st);
+    else if (M == 2) launch_gemv_group<2, false>((const bf16 *)A, p, M, total, K, accumulate, st);
     else launch_skinny_pick((const bf16 *)A, p, pick_skinny(M, n[0], K), M, K, accumulate, st);
     LAUNCH_CHECK(1);
     return TGP_OK;
@@ -2144,8 +2170,8 @@ int tgpk_gemm_group_fused(int mode, const float *x, uint32_t ldx, const void *ga
     for (uint32_t s = 0; s < count; ++s) { p.W[s] = (const bf16 *)W[s]; p.C[s] = C[s]; p.n[s] = n[s]; p.ldc[s] = ldc[s]; total += n[s]; }
     p.count = count;
     const ASrc src{mode, x, ldx, (const bf16 *)gain, eps, g32, u32};
-    if (M == 1) launch_gemv_group<1>(nullptr, p, M, total, K, accumulate, st, src);
-    else launch_gemv_group<2>(nullptr, p, M, total, K, accumulate, st, src);
+    if (M == 1) launch_gemv_group<1, true>(nullptr, p, M, total, K, accumulate, st, src);
+    else launch_gemv_group<2, true>(nullptr, p, M, total, K, accumulate, st, src);
     LAUNCH_CHECK(1);
     return TGP_OK;
 }
@@ -2200,7 +2226,7 @@ int tgpk_rope_kv(const float *q32, const float *k32, const float *v32, void *qb,
 }
 
 static int g_attn_decode_grouped = 1;   // decode: one pass over a KV tile serves all query heads of the group (0: one pass per head)
-static int g_attn_decode_impl = 0;      // decode: 0 by size, 1 the CUDA-core per-tile kernels only, 2 the tensor-core kernel wherever its geometry allows
+static int g_attn_decode_impl = 0;      // decode: 0 and 2 the tensor-core kernel wherever its geometry allows, 1 the CUDA-core per-tile kernels only
 static int g_attn_impl = 0;      // q_len >= 16: 0 by problem size, 3 tcgen05 kernel, 2 mma.sync flash kernel, 1 warp-per-row CUDA-core kernel
 
 int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0,
@@ -2216,12 +2242,13 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
         if (split < 1) split = 1;
         dim3 grid(nt, c->Hkv, B);
         const bool grouped = g_attn_decode_grouped && (G == 1 || G == 2 || G == 4 || G == 8) && c->Hq % c->Hkv == 0;
-        // tensor-core decode kernel: whole 16-key chunks inside a tile, 16-byte aligned rows; the context must be long enough
-        // to give its warps a few chunks each (below that the per-tile kernel's single pass is as fast)
+        // tensor-core decode kernel: whole 16-key chunks inside a tile, 16-byte aligned rows.  It is ahead at any length (us with
+        // the merge, against the per-tile kernels: 40 keys of 4 heads 1.8 / 4.3, which is one CTA per head and no merge; one sequence
+        // of 32 over 8 heads x 64, 130 keys 4.2 / 5.8, 700 keys 4.9 / 6.6; 1500 keys of 8 heads over 1 x 128: 6.7 / 13.3)
         const uint32_t nchunks = (pos0 + 1 + DEC_KEYS - 1) / DEC_KEYS;
         bool aligned16 = (reinterpret_cast<uintptr_t>(qb) & 3u) == 0;
         for (uint32_t t = 0; t < nt && aligned16; ++t) aligned16 = ((reinterpret_cast<uintptr_t>(tiles.k[t]) | reinterpret_cast<uintptr_t>(tiles.v[t])) & 15u) == 0;
-        if (grouped && g_attn_decode_impl != 1 && c->TK % DEC_KEYS == 0 && aligned16 && (g_attn_decode_impl == 2 || nchunks * B * c->Hkv >= 256)) {
+        if (grouped && g_attn_decode_impl != 1 && c->TK % DEC_KEYS == 0 && aligned16) {
             static int sms = 0;
             if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
             const uint32_t units = B * c->Hkv, per_sm = c->Dh == 64 ? 4 : 2;             // CTAs that fit an SM (96 / 48 KB of shared memory each)
@@ -2230,17 +2257,21 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
             const uint32_t per_cta = (nchunks + parts - 1) / parts;
             parts = (nchunks + per_cta - 1) / per_cta;                                    // no CTA without a chunk
             a.n_parts = parts;
+            // below 256 chunks in all the kernel is bound by latency and the second product for the rest of P is free
+            const bool split_p = nchunks * B * c->Hkv < 256;
             const size_t smem = (size_t)DEC_WARPS * DEC_STAGES * 2 * DEC_KEYS * c->Dh * 2;        // 96 KB at Dh = 128, 48 KB at 64
             dim3 g2(parts, c->Hkv, B);
-#define TGP_DECODE_MMA(DH_, G_) do { \
+#define TGP_DECODE_MMA_P(DH_, G_, SP_) do { \
                 static bool attr_set = false; \
-                if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_decode_mma_kernel<DH_, G_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TGP_E_CUDA; attr_set = true; } \
-                launch_pdl(tgp_attn_decode_mma_kernel<DH_, G_>, g2, dim3(DEC_WARPS * 32), smem, st, a, per_cta); } while (0)
+                if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_decode_mma_kernel<DH_, G_, SP_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TGP_E_CUDA; attr_set = true; } \
+                launch_pdl(tgp_attn_decode_mma_kernel<DH_, G_, SP_>, g2, dim3(DEC_WARPS * 32), smem, st, a, per_cta); } while (0)
+#define TGP_DECODE_MMA(DH_, G_) do { if (split_p) TGP_DECODE_MMA_P(DH_, G_, true); else TGP_DECODE_MMA_P(DH_, G_, false); } while (0)
 #define TGP_DECODE_MMA_G(DH_) do { if (G == 1) TGP_DECODE_MMA(DH_, 1); else if (G == 2) TGP_DECODE_MMA(DH_, 2); else if (G == 4) TGP_DECODE_MMA(DH_, 4); else TGP_DECODE_MMA(DH_, 8); } while (0)
             if (c->Dh == 64) { TGP_DECODE_MMA_G(64); if (parts > 1) launch_pdl(tgp_attn_decode_merge_kernel<64>, dim3(c->Hq, B), dim3(64), 0, st, a); }
             else { TGP_DECODE_MMA_G(128); if (parts > 1) launch_pdl(tgp_attn_decode_merge_kernel<128>, dim3(c->Hq, B), dim3(128), 0, st, a); }
 #undef TGP_DECODE_MMA_G
 #undef TGP_DECODE_MMA
+#undef TGP_DECODE_MMA_P
             LAUNCH_CHECK(parts > 1 ? 2 : 1);
             return TGP_OK;
         }
@@ -2287,7 +2318,7 @@ int tgpk_swiglu(const float *g, const float *u, void *ab, uint64_t n, cudaStream
     return TGP_OK;
 }
 
-int tgpk_argmax(const float *logits, int32_t *out, uint32_t B, uint32_t V, cudaStream_t st) {
+int tgpk_argmax(const float *logits, int32_t *out, int32_t *out2, uint32_t B, uint32_t V, cudaStream_t st) {
     if (!B) return TGP_OK;
     // rows of up to 4096 logits are one round of one CTA
     const uint32_t parts = V > 4096 ? 8 : 1;
@@ -2301,7 +2332,7 @@ int tgpk_argmax(const float *logits, int32_t *out, uint32_t B, uint32_t V, cudaS
     attr[1].val.clusterDim.x = parts; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaLaunchKernelEx(&cfg, tgp_argmax_kernel, logits, out, V, vec);
+    cudaLaunchKernelEx(&cfg, tgp_argmax_kernel, logits, out, out2, V, vec);
     LAUNCH_CHECK(1);
     return TGP_OK;
 }
@@ -2480,7 +2511,7 @@ int tgp_k_swiglu(const float *g32, const float *u32, void *ab, uint64_t n_elems,
 
 int tgp_k_argmax(const float *logits, int32_t *out, uint32_t B, uint32_t V, void *stream) {
     if (!logits || !out || !V) return TGP_E_INVAL;
-    return tgpk_argmax(logits, out, B, V, (cudaStream_t)stream);
+    return tgpk_argmax(logits, out, nullptr, B, V, (cudaStream_t)stream);
 }
 
 }  // extern "C"

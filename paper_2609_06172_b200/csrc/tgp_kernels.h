@@ -48,7 +48,7 @@ int tgpk_swiglu(const float *g, const float *u, void *ab, uint64_t n, cudaStream
 // counts to mapped host memory
 int tgpk_router(const void *h, const void *Wr, const float *bias, int32_t *idx, float *gate, int32_t *rows, float *gates, int32_t *counts, int32_t *pos,
                 int32_t *counts_host, uint32_t M, uint32_t stride, uint32_t d, uint32_t E, uint32_t topk, cudaStream_t st);
-// all experts of a layer for a step of at most 32 tokens, from the router's lists on the device: a = SwiGLU of the gate and up
+// all experts of a layer for a step of 3 to 32 tokens, from the router's lists on the device: a = SwiGLU of the gate and up
 // projections of the routed rows of h (one row per slot), y = their down projections, x += gate * y.  w[0..2]: gate, up, down of
 // each expert in blocks of per_f (gate, up) or per_d (down) rows.  Bit-identical to the experts one by one (tgpk_gemm_rows)
 #define TGP_MOE_EXPERTS 16
@@ -66,7 +66,8 @@ int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *c
 bool tgpk_gemm_grouping();
 int tgpk_gather_rows(const void *src, const int32_t *rows, void *dst, uint32_t m, uint32_t d, cudaStream_t st);
 int tgpk_scatter_add(float *x, const float *y, const int32_t *rows, const float *gates, uint32_t m, uint32_t d, cudaStream_t st);
-int tgpk_argmax(const float *logits, int32_t *out, uint32_t B, uint32_t V, cudaStream_t st);
+// the result also goes to out2 if that is not NULL
+int tgpk_argmax(const float *logits, int32_t *out, int32_t *out2, uint32_t B, uint32_t V, cudaStream_t st);
 // cos/sin tables [max_len, Dh/2] fp32 (angle = pos * base^(-2i/Dh), evaluated in double) written to device memory
 int tgp_rope_tables_upload(uint32_t Dh, uint32_t max_len, float base, float *cos_dev, float *sin_dev);
 // reset of the tensor-core kernels' error words (tgp_gemm_sm100.cu, tgp_attn_sm100.cu)

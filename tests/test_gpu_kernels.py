@@ -857,3 +857,25 @@ def test_argmax_parts_ties_and_special_values(V):
     a = lg.cpu().numpy()
     want = [0 if not np.any(r > -np.inf) else int(np.flatnonzero(r == np.nanmax(r))[0]) for r in a]
     assert out.cpu().tolist() == want
+
+
+@pytest.mark.parametrize("Dh,Hq,Hkv,TK,kvlen,B", [(64, 4, 4, 16, 1, 1), (64, 8, 2, 16, 16, 2), (128, 8, 1, 32, 17, 1), (64, 16, 8, 64, 33, 3), (128, 4, 2, 16, 65, 1)])
+def test_decode_attention_of_short_contexts(Dh, Hq, Hkv, TK, kvlen, B):
+    """The automatic choice at contexts of one key to a few chunks (one CTA per head writes the result itself, warps without a
+    chunk, chunks that end in a tile's middle) against double precision."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(kvlen)
+    nt = (kvlen + TK - 1) // TK
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=kvlen, T=0, B=B, d=Hq * Dh)
+    mc = model_cfg(cfg)
+    kt, vt = ([torch.randn((B * Hkv * TK, Dh), device=DEV, generator=gen).bfloat16() for _ in range(nt)] for _ in range(2))
+    q = torch.randn((B, Hq * Dh), device=DEV, generator=gen).bfloat16()
+    o = torch.zeros_like(q)
+    scratch = torch.empty(tb.k_attn_scratch_bytes(mc) // 4, dtype=torch.float32, device=DEV)
+    tb.k_attn(q, kt, vt, o, mc, B, 1, kvlen - 1, scratch)
+    torch.cuda.synchronize()
+    K, V = (torch.stack([t.view(B, Hkv, TK, Dh) for t in tiles], dim=2).reshape(B, Hkv, nt * TK, Dh)[:, :, :kvlen].double().repeat_interleave(Hq // Hkv, dim=1) for tiles in (kt, vt))
+    p = torch.softmax((K @ q.double().view(B, Hq, Dh, 1)).squeeze(-1) / Dh ** 0.5, dim=-1)
+    want = (p.unsqueeze(2) @ V).view(B, Hq * Dh)
+    # P counts with 16 bits (2^-16 of averages of V); the result is rounded to bf16: half a step
+    assert float(((o.double() - want).abs() - 2.0 ** -8 * want.abs()).max()) < 2.0 ** -14 * float(V.abs().max())
