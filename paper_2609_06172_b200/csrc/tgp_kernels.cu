@@ -1108,6 +1108,8 @@ __global__ void __launch_bounds__(256) tgp_argmax_kernel(const float *logits, in
     uint32_t rank, parts;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(parts));
+    // (the wait stands before the first access to the first CTA's memory: only then is that CTA known to run, however short this part is)
+    if (parts > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float *row = logits + (size_t)(blockIdx.x / parts) * V;
     const uint32_t per = ((V + parts - 1) / parts + 3) / 4 * 4, lo = min(V, rank * per), hi = min(V, lo + per);
@@ -1145,6 +1147,7 @@ __global__ void __launch_bounds__(256) tgp_argmax_kernel(const float *logits, in
         if (threadIdx.x == 0) { out[blockIdx.x] = (int32_t)idx; if (out2) out2[blockIdx.x] = (int32_t)idx; }
         return;
     }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (threadIdx.x == 0) {                                    // to slot `rank` of the cluster's first CTA
         uint32_t rv, ri;
         asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(rv) : "r"((uint32_t)__cvta_generic_to_shared(&cv[rank])));

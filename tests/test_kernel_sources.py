@@ -1,0 +1,46 @@
+"""Orders inside the CUDA kernels that no run can show: a kernel that breaks one of them works almost always and is undefined,
+or hangs, when the scheduler does something unusual.  Read from the sources, without a GPU."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_06172_b200", "csrc")
+
+
+def kernels():
+    """(file, kernel name, body without comments) of every __global__ function."""
+    out = []
+    for f in sorted(os.listdir(CSRC)):
+        if not f.endswith((".cu", ".cuh")):
+            continue
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, f)).read())
+        text = re.sub(r"__launch_bounds__\([^()]*\)", "", text)
+        for m in re.finditer(r"__global__\s+void\s+(\w+)\s*\([^{;]*\)\s*\{", text):
+            depth, at = 1, m.end()
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[at], 0)
+                at += 1
+            out.append((f, m.group(1), text[m.end():at]))
+    return out
+
+
+KERNELS = kernels()
+
+
+def test_every_kernel_is_found():
+    names = {k for _, k, _ in KERNELS}
+    assert {"tgp_argmax_kernel", "tgp_wstream_tc_kernel", "tgp_matmul_tc_pair_kernel", "tgp_attn_prefill_tc_kernel", "tgp_expert_mma_kernel"} <= names
+
+
+REMOTE = r"mapa\.shared::cluster|ld_remote_|sum_slices<|mbar_arrive_remote|tma_load_2d_pair|umma_pair|umma_commit_pair"
+CLUSTER_WAIT = r"cluster_sync_all\(\)|barrier\.cluster\.wait"
+
+
+@pytest.mark.parametrize("f,name,body", [k for k in KERNELS if re.search(REMOTE, k[2])], ids=lambda v: v if isinstance(v, str) and len(v) < 60 else "")
+def test_shared_memory_of_another_cta_is_touched_only_after_a_cluster_barrier(f, name, body):
+    """Another CTA's shared memory may be accessed only when that CTA is known to run, and it may leave only when nobody will touch its
+    memory any more: one cluster barrier before the first access, one after the last."""
+    waits = [m.start() for m in re.finditer(CLUSTER_WAIT, body)]
+    uses = [m.start() for m in re.finditer(REMOTE, body)]
+    assert waits and waits[0] < uses[0] and waits[-1] > uses[-1], (f, name)
