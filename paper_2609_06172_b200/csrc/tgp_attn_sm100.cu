@@ -88,7 +88,6 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
     volatile uint32_t *failed = tmem_slot + 1;
 
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (smem_u32(smem) & 1023u) {                            // the swizzle assumes 1024-byte aligned tiles
         if (tid == 0) atomicCAS(&g_attn_tc_error, 0, 5);
         return;
@@ -137,6 +136,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
     if (warp == 4) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(256u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");     // not before the allocation: see tgp_sm100.cuh
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();                                         // (after the TMA thread's wait for the previous kernel: nothing below runs before it)

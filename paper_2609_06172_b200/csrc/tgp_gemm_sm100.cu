@@ -413,7 +413,6 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
     const uint32_t tiles = p.tiles_m * p.tiles_n;
     const uint32_t buf_cols = N <= 64 ? 64u : N <= 128 ? 128u : 256u;               // TMEM columns of one accumulator
 
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (threadIdx.x == 0) {
         for (uint32_t s = 0; s < 8; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * Q_EPI); }
@@ -423,6 +422,7 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
     if (warp == 2) {                                  // the same warp in both CTAs of the pair
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2 * buf_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");     // not before the allocation: see tgp_sm100.cuh
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     cluster_sync_all();                               // barriers of all CTAs initialised, TMEM allocated
@@ -611,7 +611,6 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
     const uint32_t w0 = wt * BM;
     const CUtensorMap *mw = &p.w[part];
 
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (threadIdx.x == 0) {
         for (uint32_t s = 0; s < S_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         mbar_init(acc_full, 1);
@@ -623,6 +622,7 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
     if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");     // not before the allocation: see tgp_sm100.cuh
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();

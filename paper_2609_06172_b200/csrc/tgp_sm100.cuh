@@ -1,5 +1,10 @@
 // PTX helpers shared by the sm_100a tensor-core kernels: bounded mbarrier waits, TMA loads, tcgen05 descriptors,
 // MMA issue / commit and TMEM loads / stores.
+//
+// Order in a kernel that is launched with programmatic dependents: tcgen05.alloc first, griddepcontrol.launch_dependents after it, by the
+// warp that allocated (the first thread that asks releases for its whole CTA).  Every CTA of the grid then holds its columns
+// before a CTA of the next kernel can be scheduled.  The other way round a CTA could wait for columns that a dependent on
+// its SM holds until this grid has ended.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>

@@ -44,3 +44,12 @@ def test_shared_memory_of_another_cta_is_touched_only_after_a_cluster_barrier(f,
     waits = [m.start() for m in re.finditer(CLUSTER_WAIT, body)]
     uses = [m.start() for m in re.finditer(REMOTE, body)]
     assert waits and waits[0] < uses[0] and waits[-1] > uses[-1], (f, name)
+
+
+@pytest.mark.parametrize("f,name,body", [k for k in KERNELS if "tcgen05.alloc" in k[2] and "launch_dependents" in k[2]], ids=lambda v: v if isinstance(v, str) and len(v) < 60 else "")
+def test_a_kernel_holds_its_tensor_memory_before_it_releases_its_dependents(f, name, body):
+    """A CTA that releases the next kernel before it has allocated tensor memory may find a CTA of that kernel on its SM with the columns
+    it needs, which gives them back only after this kernel has ended.  The first thread that asks releases for the whole CTA, so
+    the one place that asks stands behind the allocation, in the warp that made it."""
+    assert body.count("launch_dependents") == 1, (f, name)
+    assert re.search(r"tcgen05\.alloc[^;]*;[^}]*tcgen05\.relinquish_alloc_permit[^;]*;[^}]*griddepcontrol\.launch_dependents", body), (f, name)
