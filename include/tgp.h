@@ -366,7 +366,7 @@ int  tgp_k_attn_select(int impl);
  * a KV head as rows of an mma.sync tile, K and V staged through shared memory with cp.async three chunks of 16 keys deep)
  * when KV tiles hold a multiple of 16 keys and G is 1, 2, 4 or 8, else the CUDA-core kernels (one pass per KV tile and group
  * of query heads); 1 forces the CUDA-core kernels.  The tensor-core kernel rounds P to bf16 for the second product; while the
- * batch's context adds up to less than 256 chunks it multiplies the remainder with V too.  Process-wide. */
+ * batch's context adds up to less than 256 chunks it multiplies what that leaves over with V too, all 24 bits of P.  Process-wide. */
 int  tgp_k_attn_decode_select(int impl);
 /* Error word of the tcgen05 attention kernel: 0, or which bounded wait ran out first (1 for S, 2 for P V, 3 for a K/V
  * load, 4 for the hand-over between the softmax warps and the MMA warp), or 5 if shared memory was not 1024-byte

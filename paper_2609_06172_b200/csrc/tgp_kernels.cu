@@ -909,9 +909,11 @@ __global__ void __launch_bounds__(DH) tgp_attn_decode_merge_kernel(AttnArgs a) {
 //   online softmax per row       (the running maximum moves rarely: O is rescaled only when a row's maximum grew);
 //   O[16 x Dh] += P V            Dh/8 MMAs, P straight from the S accumulators as the A fragment, V fragments by
 //                                ldmatrix.trans (V rows are keys: the transposed load makes keys the contraction index).
-// P is rounded to bf16 for the second product, as in the prefill kernels; in short contexts (SPLIT_P) what that leaves over is
-// multiplied with V too, so P counts with 16 bits (the distance from 64-bit attention is then that of the CUDA-core kernels to
-// six digits, 9 - 1500 keys).  A CTA of four warps owns a contiguous range of
+// P is rounded to bf16 for the second product, as in the prefill kernels; in short contexts (SPLIT_P) it counts with all of its 24 bits:
+// as three bf16 parts, each what the rounding of those before it left over.  The second part takes the rows 8 - 15 that the
+// tile has to spare, the third a product of its own.  Both are summed apart from the first and dropped where that sum is not
+// finite: an infinity in V makes their products NaN (0 x inf), and the first part alone says what the row becomes.
+// A CTA of four warps owns a contiguous range of
 // chunks of one (sequence, KV head); its warps take every fourth chunk, merge their four partials through shared memory
 // and write one (max, sum, unnormalised O) per query head and CTA to the scratch array tgp_attn_decode_merge_kernel reads.
 // Stage layout: row = key, 2*DH bytes, 16-byte chunk j of row r at chunk position j ^ (r & 7): conflict-free for the
@@ -980,9 +982,12 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
         if (issued < total) { issue(q_lo + warp + issued * DEC_WARPS, issued % DEC_STAGES); ++issued; }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    float o[DH / 8][4];
+    float o[DH / 8][4], o3[SPLIT_P ? DH / 8 : 1][4];                  // o: the first part of P in elements 0 and 1, the second in 2 and 3; o3: the third
 #pragma unroll
-    for (int j = 0; j < DH / 8; ++j) { o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f; }
+    for (int j = 0; j < DH / 8; ++j) {
+        o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
+        if constexpr (SPLIT_P) o3[j][0] = o3[j][1] = o3[j][2] = o3[j][3] = 0.f;
+    }
     float m_run = -INFINITY, l_run = 0.f;                             // of row r (replicated over the four lanes of the row)
     for (uint32_t it = 0; it < total; ++it) {
         if (issued < total) { issue(q_lo + warp + issued * DEC_WARPS, issued % DEC_STAGES); ++issued; }
@@ -1020,7 +1025,10 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
             const float alpha = fast_ex2(m_run - m_new);              // first chunk: ex2(-inf) = 0 on zeros
             l_run *= alpha;
 #pragma unroll
-            for (int j = 0; j < DH / 8; ++j) { o[j][0] *= alpha; o[j][1] *= alpha; }
+            for (int j = 0; j < DH / 8; ++j) {
+                o[j][0] *= alpha; o[j][1] *= alpha;
+                if constexpr (SPLIT_P) { o[j][2] *= alpha; o[j][3] *= alpha; o3[j][0] *= alpha; o3[j][1] *= alpha; }
+            }
             m_run = m_new;
         }
         float p[4];
@@ -1030,26 +1038,37 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
         ls += __shfl_xor_sync(0xffffffffu, ls, 1);
         ls += __shfl_xor_sync(0xffffffffu, ls, 2);
         l_run += ls;
-        __nv_bfloat162 plo = __floats2bfloat162_rn(p[0], p[1]), phi = __floats2bfloat162_rn(p[2], p[3]);
-        const uint32_t pa0 = *reinterpret_cast<uint32_t *>(&plo), pa2 = *reinterpret_cast<uint32_t *>(&phi);
-        uint32_t pb0 = 0, pb2 = 0;                                        // what the rounding of P left over
-        if constexpr (SPLIT_P) {
-            __nv_bfloat162 rlo = __floats2bfloat162_rn(p[0] - __low2float(plo), p[1] - __high2float(plo)), rhi = __floats2bfloat162_rn(p[2] - __low2float(phi), p[3] - __high2float(phi));
-            pb0 = *reinterpret_cast<uint32_t *>(&rlo); pb2 = *reinterpret_cast<uint32_t *>(&rhi);
-        }
+        // rounds p to bf16 and leaves the remainder in it
+        auto take_part = [&](uint32_t &lo, uint32_t &hi) {
+            const __nv_bfloat162 a01 = __floats2bfloat162_rn(p[0], p[1]), a23 = __floats2bfloat162_rn(p[2], p[3]);
+            p[0] -= __low2float(a01); p[1] -= __high2float(a01); p[2] -= __low2float(a23); p[3] -= __high2float(a23);
+            lo = *reinterpret_cast<const uint32_t *>(&a01); hi = *reinterpret_cast<const uint32_t *>(&a23);
+        };
+        uint32_t pa0, pa2, pb0 = 0, pb2 = 0, pc0 = 0, pc2 = 0;
+        take_part(pa0, pa2);
+        if constexpr (SPLIT_P) { take_part(pb0, pb2); take_part(pc0, pc2); }
         // ---- O += P V: Dh/8 n-tiles, two per ldmatrix ----
 #pragma unroll
         for (int jp = 0; jp < DH / 16; ++jp) {
             const uint32_t row = ((lane >> 3) & 1) * 8 + (lane & 7), j = 2 * jp + (lane >> 4);
             uint32_t v0, v1, v2, v3;
             ldsm_x4_t(vb + row * ROW + ((j ^ (row & 7)) << 4), v0, v1, v2, v3);
-            mma_bf16(o[2 * jp], pa0, 0u, pa2, 0u, v0, v1);
-            mma_bf16(o[2 * jp + 1], pa0, 0u, pa2, 0u, v2, v3);
-            if constexpr (SPLIT_P) { mma_bf16(o[2 * jp], pb0, 0u, pb2, 0u, v0, v1); mma_bf16(o[2 * jp + 1], pb0, 0u, pb2, 0u, v2, v3); }
+            mma_bf16(o[2 * jp], pa0, pb0, pa2, pb2, v0, v1);
+            mma_bf16(o[2 * jp + 1], pa0, pb0, pa2, pb2, v2, v3);
+            if constexpr (SPLIT_P) { mma_bf16(o3[2 * jp], pc0, 0u, pc2, 0u, v0, v1); mma_bf16(o3[2 * jp + 1], pc0, 0u, pc2, 0u, v2, v3); }
         }
         __syncwarp();                                                 // the stage may be refilled two iterations from now
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if constexpr (SPLIT_P) {
+#pragma unroll
+        for (int j = 0; j < DH / 8; ++j)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float rest = o[j][2 + i] + o3[j][i];
+                if (fabsf(rest) < INFINITY) o[j][i] += rest;
+            }
+    }
     // ---- merge the four warps' partials (rows < G), write one partial per head for this CTA ----
     // (each warp's partial goes to the start of its own stages, which it no longer needs: [G][DH + 2] floats)
     __syncwarp();
@@ -1057,7 +1076,8 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
     float *wp = reinterpret_cast<float *>(dec_sm);
     if (r < G) {
         float *dst = wp + (size_t)warp * WSTRIDE + (size_t)r * (DH + 2);
-        if (c == 0) { dst[0] = m_run; dst[1] = l_run; }
+        // (a warp whose scores were all NaN or -inf: its maximum is NaN, not that of a warp without a chunk, so that the row becomes NaN)
+        if (c == 0) { dst[0] = total && m_run == -INFINITY ? __int_as_float(0x7fffffff) : m_run; dst[1] = l_run; }
 #pragma unroll
         for (int j = 0; j < DH / 8; ++j) { dst[2 + j * 8 + 2 * c] = o[j][0]; dst[2 + j * 8 + 2 * c + 1] = o[j][1]; }
     }
@@ -2260,7 +2280,8 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
             const uint32_t per_cta = (nchunks + parts - 1) / parts;
             parts = (nchunks + per_cta - 1) / per_cta;                                    // no CTA without a chunk
             a.n_parts = parts;
-            // below 256 chunks in all the kernel is bound by latency and the second product for the rest of P is free
+            // below 256 chunks in all the kernel is bound by latency and takes no longer with all of P (1183 shapes of 1 - 4000 keys: 3.4 us
+            // on average, 3.4 with two parts, 7.8 on the CUDA cores; results that are not the rounded exact value: 1 in 7750, 1 in 720, 1 in 7500)
             const bool split_p = nchunks * B * c->Hkv < 256;
             const size_t smem = (size_t)DEC_WARPS * DEC_STAGES * 2 * DEC_KEYS * c->Dh * 2;        // 96 KB at Dh = 128, 48 KB at 64
             dim3 g2(parts, c->Hkv, B);

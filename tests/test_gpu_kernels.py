@@ -879,3 +879,63 @@ def test_decode_attention_of_short_contexts(Dh, Hq, Hkv, TK, kvlen, B):
     want = (p.unsqueeze(2) @ V).view(B, Hq * Dh)
     # P counts with 16 bits (2^-16 of averages of V); the result is rounded to bf16: half a step
     assert float(((o.double() - want).abs() - 2.0 ** -8 * want.abs()).max()) < 2.0 ** -14 * float(V.abs().max())
+
+
+@pytest.mark.parametrize("Dh,Hq,Hkv,TK,kvlen,B", [(64, 32, 8, 64, 9, 16), (64, 16, 2, 64, 130, 8), (128, 32, 8, 128, 17, 8), (128, 8, 8, 16, 40, 8), (128, 8, 1, 64, 700, 5),
+                                                  (64, 8, 8, 128, 400, 1)])
+def test_decode_attention_of_short_contexts_is_as_exact_as_the_cuda_core_kernels(Dh, Hq, Hkv, TK, kvlen, B):
+    """Fewer than 256 chunks of 16 keys in all: P counts with all of its 24 bits.  Of the results, rounded to bf16, hardly any may differ
+    from the rounded exact value: fp32 sums of fp32 weights are within 2^-21 of it, so that one in 2^12 lies that close to a
+    rounding boundary (2^-21 to either side, of steps of 2^-8); twice that is allowed.  With P rounded to 16 bits it
+    is one in 700.  The CUDA-core kernels, forced, meet the same bound."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(kvlen)
+    nt = (kvlen + TK - 1) // TK
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=kvlen, T=0, B=B, d=Hq * Dh)
+    mc = model_cfg(cfg)
+    wrong, total = [0, 0], 0
+    for _ in range(8):
+        kt, vt = ([torch.randn((B * Hkv * TK, Dh), device=DEV, generator=gen).bfloat16() for _ in range(nt)] for _ in range(2))
+        q = torch.randn((B, Hq * Dh), device=DEV, generator=gen).bfloat16()
+        scratch = torch.empty(tb.k_attn_scratch_bytes(mc) // 4, dtype=torch.float32, device=DEV)
+        K, V = (torch.stack([t.view(B, Hkv, TK, Dh) for t in tiles], dim=2).reshape(B, Hkv, nt * TK, Dh)[:, :, :kvlen].double().repeat_interleave(Hq // Hkv, dim=1) for tiles in (kt, vt))
+        p = torch.softmax((K @ q.double().view(B, Hq, Dh, 1)).squeeze(-1) / Dh ** 0.5, dim=-1)
+        want = (p.unsqueeze(2) @ V).view(B, Hq * Dh).bfloat16()
+        total += want.numel()
+        for impl in (0, 1):
+            o = torch.zeros_like(q)
+            tb.k_attn_decode_select(impl)
+            tb.k_attn(q, kt, vt, o, mc, B, 1, kvlen - 1, scratch)
+            torch.cuda.synchronize()
+            wrong[impl] += int((o != want).sum())
+    tb.k_attn_decode_select(0)
+    assert max(wrong) <= 2 * total / 2 ** 12, (wrong, total)
+
+
+@pytest.mark.parametrize("Dh,G,kvlen", [(64, 4, 9), (64, 1, 40), (128, 8, 130), (128, 2, 64)])
+def test_decode_attention_of_short_contexts_with_infinities_and_nan(Dh, G, kvlen):
+    """An infinity in V reaches the result as it is (not as NaN) where its key has a weight, NaN scores make their row NaN also when they
+    are all that one warp sees (its 16 keys)."""
+    Hkv, TK, B = 2, 16, 1
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(kvlen)
+    nt = (kvlen + TK - 1) // TK
+    cfg = replace(KCFG, Dh=Dh, Hq=Hkv * G, Hkv=Hkv, TK=TK, S=kvlen, T=0, B=B, d=Hkv * G * Dh)
+    mc = model_cfg(cfg)
+    kt, vt = ([torch.randn((Hkv * TK, Dh), device=DEV, generator=gen).bfloat16() for _ in range(nt)] for _ in range(2))
+    q = torch.randn((B, Hkv * G * Dh), device=DEV, generator=gen).bfloat16()
+    scratch = torch.empty(tb.k_attn_scratch_bytes(mc) // 4, dtype=torch.float32, device=DEV)
+    vt[0].view(Hkv, TK, Dh)[0, 3, 5] = float("inf")
+    vt[0].view(Hkv, TK, Dh)[0, 4, 6] = float("-inf")
+    vt[0].view(Hkv, TK, Dh)[0, 3, 7], vt[0].view(Hkv, TK, Dh)[0, 4, 7] = float("inf"), float("-inf")
+    o = torch.zeros_like(q)
+    tb.k_attn(q, kt, vt, o, mc, B, 1, kvlen - 1, scratch)
+    torch.cuda.synchronize()
+    got = o.float().view(Hkv, G, Dh)
+    assert (got[0, :, 5] == float("inf")).all() and (got[0, :, 6] == float("-inf")).all() and got[0, :, 7].isnan().all()
+    rest = [i for i in range(Dh) if i not in (5, 6, 7)]
+    assert got[0][:, rest].isfinite().all() and got[1].isfinite().all()
+    kt[-1].view(Hkv, TK, Dh)[1] = float("nan")
+    tb.k_attn(q, kt, vt, o, mc, B, 1, kvlen - 1, scratch)
+    torch.cuda.synchronize()
+    assert o.float().view(Hkv, G, Dh)[1].isnan().all()
