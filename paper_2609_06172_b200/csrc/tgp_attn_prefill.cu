@@ -5,7 +5,8 @@
 // for the second product; that is the one rounding of this path the CPU oracle does not mirror.  Where no row has more
 // than 64 keys (SPLIT_P, one key block) what that rounding leaves over is multiplied with V too, so P counts with 16 bits: with
 // few keys nothing averages the rounding out (one layer of the Mixtral widths, 16 keys: largest logit error 0.033 -> 0.020),
-// and one block costs 0.2 us more (3.1 -> 3.3 us); with 1600 keys it would be 67 -> 80 us and gain nothing.
+// and one block costs up to 0.5 us more (four sequences of 33 queries, 32 heads x 128: 4.7 -> 5.2 us; x 64: 3.3 -> 3.1 us with the launch
+// overlap); with 1600 keys it would be 67 -> 80 us and gain nothing.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cstdint>
@@ -55,8 +56,7 @@ template <int DH> __device__ __forceinline__ uint32_t tile_off(uint32_t r, uint3
 template <int DH, bool SPLIT_P>
 __global__ void __launch_bounds__(128) tgp_attn_prefill_mma_kernel(PArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");       // a programmatic dependent launch: the next one's latency overlaps this kernel,
-    asm volatile("griddepcontrol.wait;" ::: "memory");                    // which reads nothing before the previous one has finished
+    asm volatile("griddepcontrol.wait;" ::: "memory");       // a programmatic dependent launch: nothing is read before the previous kernel has finished
     constexpr int CH = DH / 8;                              // 16-byte chunks per row
     constexpr int TILE = BN * DH * 2;
     uint8_t *Qs = smem, *Ks = smem + BM * DH * 2, *Vs = Ks + 2 * TILE;
@@ -149,33 +149,59 @@ __global__ void __launch_bounds__(128) tgp_attn_prefill_mma_kernel(PArgs a) {
                 s[t][i] = p;
                 lrow[i >> 1] += p;
             }
+        if constexpr (!SPLIT_P)                             // (one key block: o is still zero)
 #pragma unroll
         for (int t = 0; t < DH / 8; ++t) { o[t][0] *= alpha[0]; o[t][1] *= alpha[0]; o[t][2] *= alpha[1]; o[t][3] *= alpha[1]; }
         // ---- O += P V ----
+        auto load_v = [&](int kk, int nt, uint32_t (&b)[4]) {
+            ldsm4t(smem_u32(Vst + tile_off<DH>(kk * 16 + (lane & 7) + 8 * ((lane >> 3) & 1), nt + (lane >> 4))), b[0], b[1], b[2], b[3]);
+        };
+        if constexpr (SPLIT_P) {
+            // What the rounding of P leaves over has sums of its own, which are dropped where they are not finite: an infinity in V
+            // makes these products NaN (0 x inf), and the rounded P alone says what the row becomes.
+            uint32_t pf[BN / 16][4], pl[BN / 16][4];
 #pragma unroll
-        for (int kk = 0; kk < BN / 16; ++kk) {
-            uint32_t pf[4] = {pack2(s[2 * kk][0], s[2 * kk][1]), pack2(s[2 * kk][2], s[2 * kk][3]),
-                              pack2(s[2 * kk + 1][0], s[2 * kk + 1][1]), pack2(s[2 * kk + 1][2], s[2 * kk + 1][3])};
-            uint32_t pl[4];
-            if constexpr (SPLIT_P) {                        // what the rounding of P left over
+            for (int kk = 0; kk < BN / 16; ++kk)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float2 h = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162 *>(&pf[i]));
                     const float *sv = &s[2 * kk + (i >> 1)][(i & 1) * 2];
-                    pl[i] = pack2(sv[0] - h.x, sv[1] - h.y);
+                    pf[kk][i] = pack2(sv[0], sv[1]);
+                    const float2 h = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162 *>(&pf[kk][i]));
+                    pl[kk][i] = pack2(sv[0] - h.x, sv[1] - h.y);
                 }
-            }
 #pragma unroll
             for (int nt = 0; nt < DH / 8; nt += 2) {
-                uint32_t b0, b1, b2, b3;
-                ldsm4t(smem_u32(Vst + tile_off<DH>(kk * 16 + (lane & 7) + 8 * ((lane >> 3) & 1), nt + (lane >> 4))), b0, b1, b2, b3);
-                mma16816(o[nt], pf, b0, b1);
-                mma16816(o[nt + 1], pf, b2, b3);
-                if constexpr (SPLIT_P) { mma16816(o[nt], pl, b0, b1); mma16816(o[nt + 1], pl, b2, b3); }
+                float rest[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+                for (int kk = 0; kk < BN / 16; ++kk) {
+                    uint32_t b[4];
+                    load_v(kk, nt, b);
+                    mma16816(o[nt], pf[kk], b[0], b[1]);
+                    mma16816(o[nt + 1], pf[kk], b[2], b[3]);
+                    mma16816(rest[0], pl[kk], b[0], b[1]);
+                    mma16816(rest[1], pl[kk], b[2], b[3]);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) if (fabsf(rest[i >> 2][i & 3]) < INFINITY) o[nt + (i >> 2)][i & 3] += rest[i >> 2][i & 3];
+            }
+        } else {
+#pragma unroll
+            for (int kk = 0; kk < BN / 16; ++kk) {
+                const uint32_t pf[4] = {pack2(s[2 * kk][0], s[2 * kk][1]), pack2(s[2 * kk][2], s[2 * kk][3]),
+                                        pack2(s[2 * kk + 1][0], s[2 * kk + 1][1]), pack2(s[2 * kk + 1][2], s[2 * kk + 1][3])};
+#pragma unroll
+                for (int nt = 0; nt < DH / 8; nt += 2) {
+                    uint32_t b[4];
+                    load_v(kk, nt, b);
+                    mma16816(o[nt], pf, b[0], b[1]);
+                    mma16816(o[nt + 1], pf, b[2], b[3]);
+                }
             }
         }
         __syncthreads();                                    // everyone is done with this stage before it is refilled
     }
+    // (released here and not first thing: the next kernel's CTAs, back to back with this one, took 0.6 - 1.1 us of 3 - 9 from it)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // ---- normalise and store ----
 #pragma unroll
     for (int h = 0; h < 2; ++h) {

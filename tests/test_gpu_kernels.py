@@ -939,3 +939,26 @@ def test_decode_attention_of_short_contexts_with_infinities_and_nan(Dh, G, kvlen
     tb.k_attn(q, kt, vt, o, mc, B, 1, kvlen - 1, scratch)
     torch.cuda.synchronize()
     assert o.float().view(Hkv, G, Dh)[1].isnan().all()
+
+
+@pytest.mark.parametrize("Dh,S,pos0", [(64, 16, 0), (64, 40, 20), (128, 33, 0), (128, 17, 47)])
+def test_attention_of_short_prompts_with_infinities_in_v(Dh, S, pos0):
+    """Up to 64 keys what the rounding of P leaves over is multiplied with V too; an infinity in V still reaches the queries that see its
+    key as it is, and every other dimension is finite."""
+    Hq, Hkv, TK, B = 4, 2, 16, 1
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(S)
+    nt = (pos0 + S + TK - 1) // TK
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=pos0 + S, T=0, B=B, d=Hq * Dh)
+    mc = model_cfg(cfg)
+    kt, vt = ([torch.randn((Hkv * TK, Dh), device=DEV, generator=gen).bfloat16() for _ in range(nt)] for _ in range(2))
+    q = torch.randn((B * S, Hq * Dh), device=DEV, generator=gen).bfloat16()
+    key = 6
+    vt[0].view(Hkv, TK, Dh)[0, key, 5], vt[0].view(Hkv, TK, Dh)[0, key, 6] = float("inf"), float("-inf")
+    o = torch.zeros_like(q)
+    tb.k_attn(q, kt, vt, o, mc, B, S, pos0, None)
+    torch.cuda.synchronize()
+    got = o.float().view(S, Hq, Dh)
+    sees = [i for i in range(S) if pos0 + i >= key]
+    assert (got[sees, :2, 5] == float("inf")).all() and (got[sees, :2, 6] == float("-inf")).all()
+    assert got[:, :, [i for i in range(Dh) if i not in (5, 6)]].isfinite().all() and got[:, 2:].isfinite().all()
