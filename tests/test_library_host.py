@@ -449,3 +449,9 @@ def test_aliased_host_pool_shares_pages_between_layer_groups_only():
     a[emb.pool_off + 5] = 3
     assert int((a[:emb.size] == 3).sum()) == 1 and all(int(a[t.pool_off + 5]) != 3 for t in w)
     p.close()
+
+
+@pytest.mark.parametrize("M,n,K,family", [(12, 12000, 1000, 0), (16, 8065, 520, 0), (9, 32000, 4104, 0), (12, 12000, 1024, 2), (16, 8065, 512, 2), (16, 8064, 4096, 1), (17, 64, 1000, 2)])
+def test_products_of_9_to_16_rows_take_the_tcgen05_kernel_only_where_k_is_a_multiple_of_32(M, n, K, family):
+    """Other K stay with the CUDA cores (key 0, launched alone), whose sums are closer to 64 bits."""
+    assert tb.k_gemm_group_key(M, n, K) >> 24 == family
