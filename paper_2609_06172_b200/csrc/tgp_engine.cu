@@ -498,7 +498,7 @@ static int run_expert_block(tgp_ctx *ctx, const TgpRole &r, const void *W, uint3
     int rc = TGP_OK;
     auto product = [&](const void *A, float *C, uint32_t ldc) {
         C += r.row0;
-        if (tgpk_expert_rows(e->step_tokens, K)) return tgpk_gemm_rows(A, 1, &W, &C, &r.rows, &ldc, me, e->step_tokens, K, cs);
+        if (tgpk_expert_rows(e->step_tokens, K)) return tgpk_gemm_rows(A, 1, &W, &C, &r.rows, &ldc, me, K, cs);
         return tgpk_gemm(A, W, C, me, r.rows, K, ldc, 0, 0, cs);
     };
     switch (r.kind) {
@@ -788,7 +788,7 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
                     e->cur_expert = g_expert;
                     const int32_t *rows = e->erow + (size_t)g_expert * e->max_tokens;
                     if (g_gather && (rc = tgpk_gather_rows(e->h, rows, e->hg, g0.Mrows, c.d, cs))) break;
-                    rc = tgpk_expert_rows(M, gK) ? tgpk_gemm_rows(g0.A, span, gW, gC, gn, gld, g0.Mrows, M, gK, cs) : tgpk_gemm_group(g0.A, span, gW, gC, gn, gld, g0.Mrows, gK, 0, cs);
+                    rc = tgpk_expert_rows(M, gK) ? tgpk_gemm_rows(g0.A, span, gW, gC, gn, gld, g0.Mrows, gK, cs) : tgpk_gemm_group(g0.A, span, gW, gC, gn, gld, g0.Mrows, gK, 0, cs);
                     if (rc) break;
                     if (g_scatter) rc = tgpk_scatter_add(e->x, e->y32, rows, e->egate + (size_t)g_expert * e->max_tokens, g0.Mrows, c.d, cs);
                     break;

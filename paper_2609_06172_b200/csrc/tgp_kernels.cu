@@ -1498,15 +1498,24 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const b
 // as one list, RG consecutive groups at a time, whose MMAs share each activation fragment - every CTA reads its K
 // slices of all activation rows from L2, so at 16 rows per CTA that traffic equals the weights'; RG row groups divide
 // it by RG.  K is split over the CTA's NW warps in interleaved chunks of 32*U columns and the partial tiles are summed
-// in warp order.  A group's arithmetic (which warp adds which k, in which order) depends on NB, U, NW and K alone -
+// in warp order.  A group's arithmetic (which warp adds which k, in which order) depends on the width of these chunks, NW and K alone -
 // not on RG, the rows per group or the list: a block gives the same bits alone or in any list.
-template <int NB, int U, int NW, int ROWS, int RG>
+// CS: load steps per chunk, U unless a warp's U steps under way are to cover several of its chunks.
+template <int NB, int U, int NW, int ROWS, int RG, int CS = ROWS == 8 ? 2 * U : U>
 __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf16 *A, const GemvParts p, uint32_t Mrows, uint32_t groups_total,
                                                               uint32_t K, int accumulate, uint32_t rpc, int acts_early) {
     constexpr int UL = ROWS == 8 ? 2 * U : U;             // half a tile per load step: twice the steps in flight
     constexpr int G = RG, SK = UL / (2 * G);              // a register set holds SK load steps of G groups: two sets are as many loads as UL steps of one group
     static_assert(UL % (2 * G) == 0 && SK >= 1, "row groups per CTA must divide half the load steps");
-    __shared__ float part[NW][G * NB * 4][32];            // the warps' partial tiles
+    static_assert(UL % CS == 0 && CS % SK == 0, "a register set lies in one chunk");
+    // the warps' partial tiles: static where they fit the 48 KB a kernel may declare, else the launch's dynamic shared memory
+    constexpr bool PART_DYNAMIC = NW * G * NB * 4 * 32 * 4 > 48 * 1024;
+    __shared__ float part_static[PART_DYNAMIC ? 1 : NW * G * NB * 4 * 32];
+    extern __shared__ float part_dynamic[];
+    auto part = [&](uint32_t w, uint32_t slot, uint32_t ln) -> float & {
+        const uint32_t at = (w * (G * NB * 4) + slot) * 32 + ln;
+        if constexpr (PART_DYNAMIC) return part_dynamic[at]; else return part_static[at];
+    };
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, c = lane & 3;
     uint32_t grp0 = blockIdx.x * G;
     if (grp0 >= groups_total) return;
@@ -1599,37 +1608,42 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
     // meets in shared memory to sum and store the group it has finished, and the memory pipe never drains.  Per group
     // the k order of a warp's additions is that of its chunks, ascending: the bits do not depend on the pairing.  A warp
     // whose first chunk lies beyond K runs one pair of zeros (the sums do not change).
-    uint32_t grp = grp0, k0 = warp * 32 * UL, pr = 0;       // the pair that is loaded next: group, chunk, pair within the chunk
+    uint32_t grp = grp0, k0 = warp * 32 * CS, pr = 0;       // the pair that is loaded next: group, first chunk, pair within its chunks
+    constexpr uint32_t SET1 = CS == SK ? NW * 32 * CS : 32 * SK;       // from a pair's first set to its second
+    auto column = [&]() -> uint32_t {                       // first column of that pair
+        if constexpr (CS == UL) return k0 + pr * 64 * SK;
+        else return k0 + 2 * pr * SK / CS * (NW * 32 * CS) + 2 * pr * SK % CS * 32;
+    };
     auto advance = [&]() -> bool {                         // moves on by one pair; true: the pair just passed ended its group
         if (++pr == (uint32_t)G) { pr = 0; k0 += NW * 32 * UL; }
-        if (k0 < K) return false;
+        if (CS == UL ? k0 < K : column() < K) return false;
         grp += gridDim.x * G;
-        k0 = warp * 32 * UL;
+        k0 = warp * 32 * CS;
         pr = 0;
         if (grp < groups_total) locate(grp);
         return true;
     };
     locate(grp);
-    uint32_t kb_cur = k0;
+    uint32_t kb_cur = column();
     issue(set0, kb_cur);
-    issue(set1, kb_cur + 32 * SK);
+    issue(set1, kb_cur + SET1);
     bool cur_last = advance();
     // Weights are never written by a kernel, so they are requested before the previous launch of the stream has finished.
     // The activations are read after it has - unless the launcher knows that they are older than that launch (it read the
     // same activations): then they are requested with the weights.  The next launch is released only here, after the wait:
     // when it starts, everything before this launch is complete, which is what lets it read its activations early in turn.
-    if (acts_early) { issue_act(set0, kb_cur); issue_act(set1, kb_cur + 32 * SK); }
+    if (acts_early) { issue_act(set0, kb_cur); issue_act(set1, kb_cur + SET1); }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!acts_early) { issue_act(set0, kb_cur); issue_act(set1, kb_cur + 32 * SK); }
+    if (!acts_early) { issue_act(set0, kb_cur); issue_act(set1, kb_cur + SET1); }
     clear();
     for (;;) {
         const bool have_next = grp < groups_total;
-        const uint32_t kb_next = k0 + pr * 64 * SK;
+        const uint32_t kb_next = column();
         consume(set0, kb_cur);
         if (have_next) { issue(set0, kb_next); issue_act(set0, kb_next); }
-        consume(set1, kb_cur + 32 * SK);
-        if (have_next) { issue(set1, kb_next + 32 * SK); issue_act(set1, kb_next + 32 * SK); }
+        consume(set1, kb_cur + SET1);
+        if (have_next) { issue(set1, kb_next + SET1); issue_act(set1, kb_next + SET1); }
         const bool next_last = have_next ? advance() : false;
         kb_cur = kb_next;
         if (!cur_last) { cur_last = next_last; continue; }
@@ -1640,7 +1654,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
 #pragma unroll
             for (int b = 0; b < NB; ++b)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) part[warp][(r * NB + b) * 4 + i][lane] = acc[r][b][i];
+                for (int i = 0; i < 4; ++i) part(warp, (r * NB + b) * 4 + i, lane) = acc[r][b][i];
         __syncthreads();
         for (uint32_t v = threadIdx.x; v < G * NB * 4 * 32; v += NW * 32) {
             const uint32_t slot = v >> 5, ln = v & 31, r = slot / (NB * 4), b = (slot >> 2) % NB, i = slot & 3;
@@ -1648,7 +1662,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
             if (gi >= groups_total) continue;
             float sum = 0.f;
 #pragma unroll
-            for (int w = 0; w < NW; ++w) sum += part[w][slot][ln];
+            for (int w = 0; w < NW; ++w) sum += part(w, slot, ln);
             float *C = p.C[0];
             uint32_t ldc = p.ldc[0], n = p.n[0], row0 = gi * rpc;
             {
@@ -1871,8 +1885,10 @@ static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows,
 // tokens, a second one the down projections, and a third adds a token's two results to its residual row.  The counts
 // are read on the device: work items are (expert, up to 8 NB of its tokens, 16 rows of gate and of up, or two groups of `rpc`
 // rows of down), and the CTAs walk the list of those that exist.
-//   The arithmetic of an item is that of tgp_wstream_mma_group_kernel<NB, EXP_U, NW, 16, 2>: which warp adds which k in which order
+//   The arithmetic of an item is that of tgp_wstream_mma_group_kernel<NB, EXP_U, NW, 16, RG>: which warp adds which k in which order
 // depends on K alone, so the bits are those of the expert's own products (tgpk_gemm_rows).
+//   Experts of one or two tokens have no items: their rows follow, a warp each, on the CUDA cores, whose sums are closer to 64 bits
+// (K=1024: 7.1e-8 against 1.3e-7 through mma.sync, K=14336: 9.3e-8 against 8.7e-7), as in the products of one and two rows.
 struct ExpertParts {
     const bf16 *w[2][TGP_MOE_EXPERTS][TGP_MOE_BLOCKS];       // GLU: gate and up; else [0]: down; in blocks of `per` rows
     const bf16 *A;                                           // GLU: [M, K], rows picked by `rows`; else one row per routed slot
@@ -1887,27 +1903,92 @@ struct ExpertParts {
 constexpr int EXP_U = 4;
 static int expert_warps(uint32_t K) { return K >= 2048 ? 16 : 8; }
 
+// From this K on the products of one or two tokens of an expert have the sums of tgp_wstream_splitk_kernel, below it those of tgp_wstream_kernel.
+constexpr uint32_t EXP_SPLIT_K = 8192;
+
+// The rows of the `ns` experts listed in `small` (at most two tokens each), one warp per row (GLU: per row of gate and of up), eight 16-byte
+// loads of weights under way.
+template <bool GLU>
+__device__ __forceinline__ void expert_rows_fma(const ExpertParts &p, const uint32_t *small, uint32_t ns, const uint32_t *s_slot, const uint32_t *s_cnt, uint32_t warp0, uint32_t warps) {
+    constexpr int R = GLU ? 2 : 1, U = 8 / R;
+    const uint32_t lane = threadIdx.x & 31, K = p.K, parts = K >= EXP_SPLIT_K ? 8 : 1;
+    for (uint32_t i = warp0; i < ns * p.n; i += warps) {
+        const uint32_t e = small[i / p.n], row = i % p.n, cnt = s_cnt[e];
+        const bf16 *w[R], *x[2];
+#pragma unroll
+        for (int r = 0; r < R; ++r) w[r] = p.w[r][e][row / p.per] + (size_t)(row % p.per) * K;
+#pragma unroll
+        for (uint32_t m = 0; m < 2; ++m) x[m] = p.A + (size_t)(GLU ? (uint32_t)p.rows[(size_t)e * p.stride + min(m, cnt - 1)] : s_slot[e] + min(m, cnt - 1)) * K;
+        float sum[R][2];
+        for (uint32_t v = 0; v < parts; ++v) {              // (the eight warps of the split-K kernel, one after the other)
+            float acc[R][2];
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r][0] = acc[r][1] = 0.f;
+            for (uint32_t k0 = v * 256 + lane * 8; k0 < K; k0 += parts * 256 * U) {
+                uint4 wv[U][R];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const uint32_t k = k0 + parts * 256 * u;
+                        wv[u][r] = k < K ? __ldcs(reinterpret_cast<const uint4 *>(w[r] + k)) : make_uint4(0, 0, 0, 0);
+                    }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const uint32_t k = k0 + parts * 256 * u;
+#pragma unroll
+                    for (uint32_t m = 0; m < 2; ++m) {
+                        float xf[8];
+                        unpack8(k < K && m < cnt ? ld_act(reinterpret_cast<const uint4 *>(x[m] + k)) : make_uint4(0, 0, 0, 0), xf);
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            float wf[8];
+                            unpack8(wv[u][r], wf);
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) acc[r][m] = fmaf(wf[j], xf[j], acc[r][m]);
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int m = 0; m < 2; ++m) { const float t = warp_sum(acc[r][m]); sum[r][m] = v ? sum[r][m] + t : t; }
+        }
+        if (lane < cnt) {
+            const size_t at = (size_t)(s_slot[e] + lane) * p.n + row;
+            const float a = lane ? sum[0][1] : sum[0][0];
+            if constexpr (GLU) { const float up = lane ? sum[1][1] : sum[1][0]; reinterpret_cast<bf16 *>(p.out)[at] = __float2bfloat16_rn(a / (1.0f + expf(-a)) * up); }
+            else reinterpret_cast<float *>(p.out)[at] = a;
+        }
+    }
+}
+
 template <int NB, int NW, bool GLU>
 __global__ void __launch_bounds__(NW * 32, 16 / NW) tgp_expert_mma_kernel(const ExpertParts p) {
     constexpr int U = EXP_U, G = 2, SK = U / (2 * G), T = NB * 8;       // T: tokens per item
     __shared__ float part[NW][G * NB * 4][32];
-    __shared__ uint32_t s_first[TGP_MOE_EXPERTS + 1], s_slot[TGP_MOE_EXPERTS], s_cnt[TGP_MOE_EXPERTS];
+    __shared__ uint32_t s_first[TGP_MOE_EXPERTS + 1], s_slot[TGP_MOE_EXPERTS], s_cnt[TGP_MOE_EXPERTS], s_small[TGP_MOE_EXPERTS], s_ns;
     pdl_enter();
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, c = lane & 3, K = p.K;
     const uint32_t span = GLU ? p.rpc : 2 * p.rpc, groups = (p.n + span - 1) / span;     // items per expert and token chunk
     if (threadIdx.x == 0) {
-        uint32_t items = 0, slot = 0;
+        uint32_t items = 0, slot = 0, ns = 0;
         for (uint32_t e = 0; e < p.E; ++e) {
             const uint32_t cnt = (uint32_t)p.counts[e];
             s_first[e] = items; s_slot[e] = slot; s_cnt[e] = cnt;
-            items += (cnt + T - 1) / T * groups;
+            if (cnt > 2) items += (cnt + T - 1) / T * groups;
+            else if (cnt) s_small[ns++] = e;
             slot += cnt;
         }
         s_first[p.E] = items;
+        s_ns = ns;
     }
     __syncthreads();
     const uint32_t total = s_first[p.E];
-    if (blockIdx.x >= total) return;
+    // (the last CTAs, which have the fewest items, begin with the rows of the small experts)
+    auto small = [&]() { expert_rows_fma<GLU>(p, s_small, s_ns, s_slot, s_cnt, (gridDim.x - 1 - blockIdx.x) * NW + warp, gridDim.x * NW); };
+    if (blockIdx.x >= total) { small(); return; }
     const bf16 *wlo[G], *whi[G], *arow[NB];                  // of the item that is being loaded
     uint4 lo[2][G][SK], hi[2][G][SK], xs[2][SK][NB];
     float acc[G][NB][4];
@@ -2028,6 +2109,7 @@ __global__ void __launch_bounds__(NW * 32, 16 / NW) tgp_expert_mma_kernel(const 
         __syncthreads();
         clear();
     }
+    small();
 }
 
 // x[m, :] += gate * y[slot of m in its expert, :], experts in ascending order: the sums of tgp_scatter_add_kernel expert by expert.
@@ -2060,39 +2142,78 @@ __global__ void __launch_bounds__(256) tgp_expert_combine_kernel(float *x, const
     }
 }
 
-// Whether the products of a step's experts take tgpk_gemm_rows() and may run all in one launch: the step has 3 to 32 tokens (one or two
-// stay with the CUDA-core kernels, whose sums are closer to 64 bits).
+// Whether the products of a step's experts take tgpk_gemm_rows() and may run all in one launch: the step has 3 to 32 tokens.
 bool tgpk_expert_rows(uint32_t M, uint32_t K) { return M >= 3 && M <= 32 && K % 32 == 0 && g_skinny_impl == 0 && g_gemm_impl == 0; }
 
-// Blocks over the same `me` activation rows with the arithmetic of the expert kernels of a step of M tokens, in one launch per
-// 8 (M <= 8) or 16 rows.
-int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t me, uint32_t M, uint32_t K, cudaStream_t st) {
-    if (!count || count > TGP_GEMM_GROUP_MAX || K % 32) return TGP_E_INVAL;
-    const uint32_t T = M <= 8 ? 8 : 16;
-    for (uint32_t m0 = 0; m0 < me; m0 += T) {
-        GemvParts p;
-        memset(&p, 0, sizeof(p));
-        for (uint32_t s = 0; s < count; ++s) { p.W[s] = (const bf16 *)W[s]; p.C[s] = C[s] + (size_t)m0 * ldc[s]; p.n[s] = n[s]; p.ldc[s] = ldc[s]; }
-        p.count = count;
-        uint32_t groups = 0;
-        for (uint32_t s = 0; s < count; ++s) groups += p.groups[s] = (n[s] + 15) / 16;
-        cudaLaunchConfig_t cfg = {};
-        const uint32_t nw = (uint32_t)expert_warps(K);
-        cfg.gridDim = dim3(std::min((groups + 1) / 2, 16 / nw * (uint32_t)device_sms())); cfg.blockDim = dim3(nw * 32); cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const bf16 *am = (const bf16 *)A + (size_t)m0 * K;
-        const uint32_t mr = std::min(T, me - m0);
-        if (T == 8 && nw == 8) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<1, EXP_U, 8, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
-        else if (T == 8) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<1, EXP_U, 16, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
-        else if (nw == 8) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<2, EXP_U, 8, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
-        else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<2, EXP_U, 16, 16, 2>, am, p, mr, groups, K, 0, 16u, 0);
-        tgpk_last_gemm_kernel = "tgp_wstream_mma_group_kernel";
-        LAUNCH_CHECK(1);
+// EXP_U load steps per chunk everywhere; 16 warps on up to 8 activation rows have registers for twice as many steps under way, from one
+// chunk of two row groups or two chunks of one.
+template <int NB, int NW, int RG>
+static void launch_expert_rows(cudaLaunchConfig_t &cfg, const bf16 *A, const GemvParts &p, uint32_t me, uint32_t groups, uint32_t K, uint32_t rpc) {
+    auto launch = [&](auto steps) {
+        constexpr int U = decltype(steps)::value;
+        constexpr size_t smem = (size_t)NW * RG * NB * 4 * 32 * 4;
+        if constexpr (smem > 48 * 1024) {
+            static bool attr_set = false;
+            if (!attr_set) { cudaFuncSetAttribute(tgp_wstream_mma_group_kernel<NB, U, NW, 16, RG, EXP_U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); attr_set = true; }
+            cfg.dynamicSmemBytes = smem;
+        }
+        cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, NW, 16, RG, EXP_U>, A, p, me, groups, K, 0, rpc, 0);
+    };
+    if constexpr (NB == 1 && NW == 16)
+        if (RG == 2 || K > NW * 32 * EXP_U) return launch(std::integral_constant<int, 2 * EXP_U>());
+    launch(std::integral_constant<int, EXP_U>());
+}
+
+// Blocks over the same `me` activation rows (at most 32) with the arithmetic of the expert kernels, in one launch: the row groups and rows per
+// group of launch_skinny(), which the bits do not depend on.  One or two rows: the CUDA cores' products, one launch per block from EXP_SPLIT_K on.
+int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t me, uint32_t K, cudaStream_t st) {
+    if (!count || count > TGP_GEMM_GROUP_MAX || K % 32 || me > 32) return TGP_E_INVAL;
+    if (!me) return TGP_OK;
+    const bf16 *a = (const bf16 *)A;
+    if (me <= 2 && K >= EXP_SPLIT_K) {
+        for (uint32_t s = 0; s < count; ++s) {
+            if (n[s] <= 1024) { if (me == 1) launch_gemv_splitk<1, 1, 4>(a, (const bf16 *)W[s], C[s], me, n[s], K, ldc[s], 0, 0, st); else launch_gemv_splitk<2, 1, 4>(a, (const bf16 *)W[s], C[s], me, n[s], K, ldc[s], 0, 0, st); }
+            else { if (me == 1) launch_gemv_splitk<1, 2, 4>(a, (const bf16 *)W[s], C[s], me, n[s], K, ldc[s], 0, 0, st); else launch_gemv_splitk<2, 2, 4>(a, (const bf16 *)W[s], C[s], me, n[s], K, ldc[s], 0, 0, st); }
+        }
+        LAUNCH_CHECK(count);
+        return TGP_OK;
     }
+    GemvParts p;
+    memset(&p, 0, sizeof(p));
+    uint32_t total = 0;
+    for (uint32_t s = 0; s < count; ++s) { p.W[s] = (const bf16 *)W[s]; p.C[s] = C[s]; p.n[s] = n[s]; p.ldc[s] = ldc[s]; total += n[s]; }
+    p.count = count;
+    if (me <= 2) {
+        if (count == 1) { if (me == 1) launch_gemv_rows<1>(a, p.W[0], p.C[0], me, n[0], K, ldc[0], 0, 0, st); else launch_gemv_rows<2>(a, p.W[0], p.C[0], me, n[0], K, ldc[0], 0, 0, st); }
+        else if (me == 1) launch_gemv_group<1, false>(a, p, me, total, K, 0, st);
+        else launch_gemv_group<2, false>(a, p, me, total, K, 0, st);
+        LAUNCH_CHECK(1);
+        return TGP_OK;
+    }
+    const uint32_t nb = me <= 8 ? 1 : me <= 16 ? 2 : 4, nw = (uint32_t)expert_warps(K), full = 16 / nw * (uint32_t)device_sms();
+    uint32_t best = 0xffffffffu, rpc = 16, RG = 1, groups = 0;
+    for (uint32_t G = 2; G >= 1; --G)
+        for (uint32_t r = 9; r <= 16; ++r) {
+            uint32_t g = 0;
+            for (uint32_t s = 0; s < count; ++s) g += (n[s] + r - 1) / r;
+            const uint32_t rounds = ((g + G - 1) / G + full - 1) / full, cost = rounds * (G * (r + 16) + 8 * nb);
+            if (cost < best) { best = cost; rpc = r; RG = G; groups = g; }
+        }
+    for (uint32_t s = 0; s < count; ++s) p.groups[s] = (n[s] + rpc - 1) / rpc;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::min((groups + RG - 1) / RG, full)); cfg.blockDim = dim3(nw * 32); cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+#define TGP_EXPERT_ROWS(NB_) do { \
+        if (nw == 8) { if (RG == 2) launch_expert_rows<NB_, 8, 2>(cfg, a, p, me, groups, K, rpc); else launch_expert_rows<NB_, 8, 1>(cfg, a, p, me, groups, K, rpc); } \
+        else { if (RG == 2) launch_expert_rows<NB_, 16, 2>(cfg, a, p, me, groups, K, rpc); else launch_expert_rows<NB_, 16, 1>(cfg, a, p, me, groups, K, rpc); } } while (0)
+    if (nb == 1) TGP_EXPERT_ROWS(1); else if (nb == 2) TGP_EXPERT_ROWS(2); else TGP_EXPERT_ROWS(4);
+#undef TGP_EXPERT_ROWS
+    tgpk_last_gemm_kernel = "tgp_wstream_mma_group_kernel";
+    LAUNCH_CHECK(1);
     return TGP_OK;
 }
 

@@ -61,7 +61,7 @@ struct TgpExperts {
 };
 int tgpk_experts(const TgpExperts &x, cudaStream_t st);
 bool tgpk_expert_rows(uint32_t M, uint32_t K);
-int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t me, uint32_t M, uint32_t K, cudaStream_t st);
+int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t me, uint32_t K, cudaStream_t st);
 // products over the same activations may share a launch (tgp_k_gemm_group_select)
 bool tgpk_gemm_grouping();
 int tgpk_gather_rows(const void *src, const int32_t *rows, void *dst, uint32_t m, uint32_t d, cudaStream_t st);

@@ -503,7 +503,7 @@ def test_llama_8b_widths_at_two_layers_lockstep_parity():
 
 
 @pytest.mark.parametrize("B,topk,d,F,cap", [(1, 2, 256, 512, 64 << 10), (3, 2, 256, 2112, 1 << 20), (8, 2, 256, 480, 128 << 10), (9, 1, 256, 512, 1 << 20), (16, 2, 512, 1056, 1 << 20),
-                                            (17, 2, 256, 2080, 1 << 20), (32, 2, 256, 544, 1 << 20), (33, 2, 256, 512, 1 << 20)])
+                                            (17, 2, 256, 2080, 1 << 20), (32, 2, 256, 544, 1 << 20), (33, 2, 256, 512, 1 << 20), (3, 2, 128, 8224, 1 << 20)])
 def test_moe_decode_runs_all_experts_of_a_layer_together_with_the_same_bits(B, topk, d, F, cap):
     """Decode steps of 3 to 32 tokens with every expert traced and on the device: one launch for the gate and up projections of all
     experts, one for the down projections, one that adds them up, and the host does not wait for the router.  Against the same
@@ -543,6 +543,53 @@ def test_moe_decode_runs_all_experts_of_a_layer_together_with_the_same_bits(B, t
         assert max(runs[0][2]) <= 11 * cfg.L + 3 + len(lay.blocks(si.K_LM, -1, -1)), runs[0][2]
     if B == 16:
         check_logits([runs[0][0][0]], [ref[0]])
+
+
+@pytest.mark.parametrize("B,F", [(3, 512), (5, 8192)])
+def test_experts_of_one_or_two_tokens_have_the_sums_of_the_products_of_one_row(B, F):
+    """A step of 3 to 32 tokens: what an expert with one or two of them computes is, bit for bit, what k_gemm() and k_swiglu() give for
+    each token alone - the CUDA cores' sums, which are closer to 64 bits than those of the kernels that serve more rows.
+    Seen at the activation tap (the step runs expert by expert then, with the bits of the joint launch, see above)."""
+    cfg = replace(MOE, B=B, S=7, T=2, d=256, F=F)
+    lay = si.build_layout(cfg, budget=64 << 20, cap=1 << 20)
+    pool = pinned_pool(lay.pool_bytes)
+    si.fill_pool(lay, pool.numpy())
+    s = Session(lay, MACHINE, pool_base=pool.data_ptr(), pool_flags=tb.POOL_PINNED, router_bias=si.router_bias(cfg))
+    s.plan(expert_counts=np.ones((1 + cfg.T, cfg.L, cfg.E), dtype=np.uint32))
+    r = Runner(s, cfg.B * cfg.S)
+    tap = torch.zeros(64 << 20, dtype=torch.uint8, device="cuda:0")
+    weights = lambda kind, l, e, cols: torch.cat([pool[t.pool_off:t.pool_off + t.rows * cols * 2].view(torch.bfloat16) for t in lay.blocks(kind, l, e)]).to("cuda:0").view(-1, cols)
+    ops = s.ctx.trace_ops()
+    small = 0
+    r.reset()
+    r.step(tb.PREFILL, si.prompt_tokens(cfg), cfg.S)
+    for _ in range(cfg.T):
+        s.ctx.set_tap(tap, tap.numel())
+        r.step(tb.DECODE, None, 1)
+        r.sync()
+        h = {}                                             # per layer the last normed state before the experts
+        for (op, tag, sub, off, nbytes) in s.ctx.tap_index().tolist():
+            l = ops[op][2]
+            if tag == tb.TAP_H:
+                h[l] = tap[off:off + nbytes].view(torch.bfloat16).view(B, cfg.d).clone()
+            if tag != tb.TAP_A or nbytes > 2 * F * 2:
+                continue
+            rows = tap[off:off + nbytes].view(torch.bfloat16).view(-1, F)
+            wg, wu = weights(si.K_WG, l, sub, cfg.d), weights(si.K_WU, l, sub, cfg.d)
+            alone = []
+            for t in range(B):
+                g, u, a = torch.zeros((1, F), device="cuda:0"), torch.zeros((1, F), device="cuda:0"), torch.zeros((1, F), dtype=torch.bfloat16, device="cuda:0")
+                tb.k_gemm(h[l][t:t + 1].contiguous(), wg, g, 1, F, cfg.d, F, 0, 0)
+                tb.k_gemm(h[l][t:t + 1].contiguous(), wu, u, 1, F, cfg.d, F, 0, 0)
+                tb.k_swiglu(g, u, a, F)
+                alone.append(a)
+            torch.cuda.synchronize()
+            for row in rows:
+                assert any(torch.equal(row, a[0]) for a in alone), (l, sub)
+            small += 1
+    s.ctx.set_tap(None, 0)
+    s.close()
+    assert small
 
 
 def test_mixtral_widths_at_one_layer_match_oracle_batch_of_eight():
