@@ -230,7 +230,8 @@ int  tgp_copies_issued(tgp_ctx *ctx, uint64_t *n);
  * routed to each expert, per step and layer, in the run since the last tgp_run_reset(): uint32 [steps, L, E].
  * Two-call form: out == NULL returns the element count in *n.  Feed it to tgp_model_trace() to trace exactly the
  * experts in use.  At run time an expert the router picks but the trace does not list is fetched synchronously
- * into a spill buffer and counted in tgp_step_stats.n_mismatch. */
+ * into a spill buffer and counted in tgp_step_stats.n_mismatch.  With out given the call waits for the routers of the steps that
+ * have been issued (and for nothing else on the device). */
 int  tgp_expert_counts(tgp_ctx *ctx, uint32_t *out, uint64_t *n);
 
 /* Managed-memory helpers for the two managed variants (Section II-A: cudaMallocManaged pools that migrate on

@@ -44,8 +44,10 @@ struct TgpEngine {
     int32_t *ecount_host = nullptr;                      // pinned mirror of the per-expert counts
     int32_t *epos = nullptr;                             // place of a token in the lists of its experts
     // counts of the steps whose experts ran without the host looking at them, written by the router kernel: [steps, L, E] of the
-    // plan in mapped host memory (sized by tgp_run_reset()); the slots to fold into run_counts when someone asks
+    // plan in mapped host memory (sized by tgp_run_reset()); the slots to fold into run_counts when someone asks, and what to
+    // wait for first: recorded on the compute stream behind the last of them
     int32_t *count_log = nullptr;
+    cudaEvent_t count_ev = nullptr;
     size_t count_log_words = 0;
     std::vector<size_t> count_slots;
     uint32_t step_tokens = 0;                            // tokens of the step being executed
@@ -156,6 +158,7 @@ void tgp_engine_free(tgp_ctx *ctx) {
     if (e->wb_stream) cudaStreamDestroy(e->wb_stream);
     if (e->ecount_host) cudaFreeHost(e->ecount_host);
     if (e->count_log) cudaFreeHost(e->count_log);
+    if (e->count_ev) cudaEventDestroy(e->count_ev);
     delete e;
     ctx->eng = nullptr;
 }
@@ -275,6 +278,7 @@ int tgp_run_reset(tgp_ctx *ctx) {
         if (e->count_log) CU(ctx, cudaFreeHost(e->count_log));
         e->count_log = nullptr;
         e->count_log_words = 0;
+        if (!e->count_ev) CU(ctx, cudaEventCreateWithFlags(&e->count_ev, cudaEventDisableTiming));
         CU(ctx, cudaHostAlloc((void **)&e->count_log, words * 4, cudaHostAllocMapped));
         e->count_log_words = words;
     }
@@ -644,6 +648,11 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
     // every kernel of the step is launched from here on the compute stream: consecutive products over the same activations
     // may read them before their predecessor has finished
     struct ChainScope { bool was; ChainScope() : was(tgpk_chain_ok) { tgpk_chain_ok = true; } ~ChainScope() { tgpk_chain_ok = was; } } chain_scope;
+    // however the step ends, tgp_expert_counts() waits for the router kernels it has launched
+    struct CountScope {
+        TgpEngine *e; cudaStream_t cs; size_t before;
+        ~CountScope() { if (e->count_slots.size() > before) cudaEventRecord(e->count_ev, cs); }
+    } count_scope{e, cs, e->count_slots.size()};
     uint32_t n_cmds = 0, n_mismatch = 0;
     e->cur_expert = -1;
     e->step_tokens = M;
@@ -1062,7 +1071,7 @@ extern "C" int tgp_expert_counts(tgp_ctx *ctx, uint32_t *out, uint64_t *n) {
     if (!ctx || !n) return TGP_E_INVAL;
     if (out && ctx->eng && !ctx->eng->count_slots.empty()) {             // counts the router kernels wrote to host memory
         TgpEngine *e = ctx->eng;
-        CU(ctx, cudaDeviceSynchronize());
+        CU(ctx, cudaEventSynchronize(e->count_ev));                      // (whichever device is current; nothing else that runs on it)
         for (size_t slot : e->count_slots)
             for (uint32_t k = 0; k < ctx->cfg.E && slot + k < ctx->run_counts.size(); ++k) ctx->run_counts[slot + k] = (uint32_t)e->count_log[slot + k];
         e->count_slots.clear();

@@ -592,6 +592,35 @@ def test_experts_of_one_or_two_tokens_have_the_sums_of_the_products_of_one_row(B
     assert small
 
 
+def test_expert_counts_wait_for_the_run_and_for_nothing_else():
+    """Counts that router kernels write to host memory: complete when the call returns, right behind steps that nobody has waited for,
+    while another stream of the device is still busy."""
+    cfg = replace(MOE, B=8, S=7, T=6)
+    lay = si.build_layout(cfg, budget=64 << 20, cap=1 << 20)
+    pool = pinned_pool(lay.pool_bytes)
+    si.fill_pool(lay, pool.numpy())
+    s = Session(lay, MACHINE, pool_base=pool.data_ptr(), pool_flags=tb.POOL_PINNED, router_bias=si.router_bias(cfg))
+    s.plan(expert_counts=np.ones((1 + cfg.T, cfg.L, cfg.E), dtype=np.uint32))
+    r = Runner(s, cfg.B * cfg.S)
+    prompt = si.prompt_tokens(cfg)
+    for _ in range(2):                                       # (the first run also sets the kernels up)
+        r.sync()
+        r.reset()
+        r.step(tb.PREFILL, prompt, cfg.S)
+        side, done = torch.cuda.Stream(), torch.cuda.Event()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(1_000_000_000)                 # half a second or so, one thread
+            done.record()
+        for _ in range(cfg.T):
+            r.step(tb.DECODE, None, 1)
+        counts = s.ctx.expert_counts(cfg.L, cfg.E)
+        busy = not done.query()
+        assert counts.shape == (1 + cfg.T, cfg.L, cfg.E) and (counts[1:].sum(axis=2) == cfg.B * cfg.topk).all()
+    assert busy
+    r.sync()
+    s.close()
+
+
 def test_mixtral_widths_at_one_layer_match_oracle_batch_of_eight():
     """Full widths of the Mixtral shape (8 experts of 14336, top-2) at one layer, batch 8, free-running: the expert
     products run at the handful of tokens each expert receives (skinny tensor-core GEMV on blocks of few rows), planned
