@@ -1206,8 +1206,9 @@ __device__ __forceinline__ void route_pick(const float (&acc)[E], uint32_t topk,
 }
 
 template <int E>
-__global__ void __launch_bounds__(256) tgp_router_kernel(const bf16 *__restrict__ h, const bf16 *__restrict__ Wr, const float *__restrict__ bias,
-                                                     int32_t *__restrict__ idx, float *__restrict__ gate, uint32_t M, uint32_t d, uint32_t topk) {
+__global__ void __launch_bounds__(256) tgp_router_kernel(const bf16 *h, const bf16 *__restrict__ Wr, const float *__restrict__ bias,
+                                                     int32_t *idx, float *gate, uint32_t M, uint32_t d, uint32_t topk) {
+    pdl_enter();
     const uint32_t m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (m >= M) return;
     float acc[E];
@@ -1215,7 +1216,7 @@ __global__ void __launch_bounds__(256) tgp_router_kernel(const bf16 *__restrict_
     for (int e = 0; e < E; ++e) acc[e] = 0.f;
     for (uint32_t k = lane * 8; k < d; k += 256) {
         float xf[8];
-        unpack8(*reinterpret_cast<const uint4 *>(h + (size_t)m * d + k), xf);
+        unpack8(ld_act(reinterpret_cast<const uint4 *>(h + (size_t)m * d + k)), xf);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             float wf[8];
@@ -1234,19 +1235,26 @@ __global__ void __launch_bounds__(256) tgp_router_kernel(const bf16 *__restrict_
     }
 }
 
-// Up to ROUTE_SMALL tokens: router and token lists in one CTA and one launch (below), with the arithmetic of tgp_router_kernel.  Warp w
-// takes tokens w, w + 32; then warp e lists the tokens of expert e in ascending order.  pos[2 m + s]: the place of token m in the
-// list of its s-th expert.  counts_host (may be NULL): mapped host memory that receives the counts too.
+// Up to ROUTE_SMALL tokens: router and token lists in one launch, with the arithmetic of tgp_router_kernel.  A cluster takes the tokens, a warp
+// each, eight per CTA (one CTA reads the router's weights for all of them through one SM: 16 experts, d=8192, 32 tokens 68 us, 37 us in
+// four; with 64 tokens 135 and 37); the picks meet in its first CTA, whose warps list the tokens of the experts in ascending order.  pos[2 m + s]: the place of
+// token m in the list of its s-th expert.  counts_host (may be NULL): mapped host memory that receives the counts too.
 constexpr uint32_t ROUTE_SMALL = 64;
 
 template <int E>
-__global__ void __launch_bounds__(1024) tgp_route_small_kernel(const bf16 *h, const bf16 *__restrict__ Wr, const float *__restrict__ bias, int32_t *idx, float *gate, int32_t *rows,
+__global__ void __launch_bounds__(256) tgp_route_small_kernel(const bf16 *h, const bf16 *__restrict__ Wr, const float *__restrict__ bias, int32_t *idx, float *gate, int32_t *rows,
                                                              float *gates, int32_t *counts, int32_t *pos, int32_t *counts_host, uint32_t M, uint32_t stride, uint32_t d, uint32_t topk) {
     pdl_enter();
-    __shared__ int32_t si[2 * ROUTE_SMALL];
-    __shared__ float sg[2 * ROUTE_SMALL];
+    __shared__ __align__(8) int32_t si[2 * ROUTE_SMALL];     // the first CTA's: the picks of all tokens
+    __shared__ __align__(8) float sg[2 * ROUTE_SMALL];
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (uint32_t m = warp; m < M; m += 32) {
+    uint32_t rank, parts;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(parts));
+    if (parts > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    const uint32_t m = rank * 8 + warp;
+    int i0 = 0, i1 = -1; float g0 = 0.f, g1 = 0.f;
+    if (m < M) {
         float acc[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) acc[e] = 0.f;
@@ -1264,26 +1272,34 @@ __global__ void __launch_bounds__(1024) tgp_route_small_kernel(const bf16 *h, co
         }
 #pragma unroll
         for (int e = 0; e < E; ++e) acc[e] = warp_sum(acc[e]) + bias[e];
-        if (lane == 0) {
-            int i0, i1; float g0, g1;
-            route_pick<E>(acc, topk, i0, i1, g0, g1);
-            si[2 * m] = i0; si[2 * m + 1] = i1;
-            sg[2 * m] = g0; sg[2 * m + 1] = g1;
-        }
+        route_pick<E>(acc, topk, i0, i1, g0, g1);
     }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < 2 * M; i += 1024) { idx[i] = si[i]; gate[i] = sg[i]; }
-    if (warp < (uint32_t)E) {
+    __syncwarp();
+    if (parts > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");         // (the first CTA is known to run)
+    if (m < M && lane == 0) {
+        idx[2 * m] = i0; idx[2 * m + 1] = i1;
+        gate[2 * m] = g0; gate[2 * m + 1] = g1;
+        uint32_t ri, rg;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(ri) : "r"((uint32_t)__cvta_generic_to_shared(&si[2 * m])));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(rg) : "r"((uint32_t)__cvta_generic_to_shared(&sg[2 * m])));
+        asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(ri), "r"(i0), "r"(i1) : "memory");
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(rg), "f"(g0), "f"(g1) : "memory");
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank) return;
+    for (uint32_t e = warp; e < (uint32_t)E; e += 8) {
         uint32_t base = 0;
         for (uint32_t m0 = 0; m0 < M; m0 += 32) {
-            const uint32_t m = m0 + lane;
+            const uint32_t t = m0 + lane;
             int slot = -1;
-            if (m < M) slot = si[2 * m] == (int)warp ? 0 : topk > 1 && si[2 * m + 1] == (int)warp ? 1 : -1;
+            if (t < M) slot = si[2 * t] == (int)e ? 0 : topk > 1 && si[2 * t + 1] == (int)e ? 1 : -1;
             const uint32_t bal = __ballot_sync(0xffffffffu, slot >= 0), at = base + __popc(bal & ((1u << lane) - 1));
-            if (slot >= 0) { rows[(size_t)warp * stride + at] = (int32_t)m; gates[(size_t)warp * stride + at] = sg[2 * m + slot]; pos[2 * m + slot] = (int32_t)at; }
+            if (slot >= 0) { rows[(size_t)e * stride + at] = (int32_t)t; gates[(size_t)e * stride + at] = sg[2 * t + slot]; pos[2 * t + slot] = (int32_t)at; }
             base += __popc(bal);
         }
-        if (lane == 0) { counts[warp] = (int32_t)base; if (counts_host) *(volatile int32_t *)(counts_host + warp) = (int32_t)base; }
+        if (lane == 0) { counts[e] = (int32_t)base; if (counts_host) *(volatile int32_t *)(counts_host + e) = (int32_t)base; }
     }
 }
 
@@ -1346,9 +1362,18 @@ int tgpk_router(const void *h, const void *Wr, const float *bias, int32_t *idx, 
     const bool small = M <= ROUTE_SMALL;
     if (counts_host && !small) return TGP_E_INVAL;
     const uint32_t blocks = (M + 7) / 8;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks <= 2 ? blocks : blocks <= 4 ? 4 : 8); cfg.blockDim = dim3(256); cfg.stream = st;       // one cluster
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cfg.gridDim.x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
 #define TGP_ROUTE(E_) do { \
-        if (small) launch_pdl(tgp_route_small_kernel<E_>, dim3(1), dim3(1024), 0, st, (const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, rows, gates, counts, pos, counts_host, M, stride, d, topk); \
-        else tgp_router_kernel<E_><<<blocks, 256, 0, st>>>((const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, M, d, topk); } while (0)
+        if (small) cudaLaunchKernelEx(&cfg, tgp_route_small_kernel<E_>, (const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, rows, gates, counts, pos, counts_host, M, stride, d, topk); \
+        else launch_pdl(tgp_router_kernel<E_>, dim3(blocks), dim3(256), 0, st, (const bf16 *)h, (const bf16 *)Wr, bias, idx, gate, M, d, topk); } while (0)
     switch (E) {
     case 1: TGP_ROUTE(1); break;
     case 2: TGP_ROUTE(2); break;

@@ -621,6 +621,31 @@ def test_expert_counts_wait_for_the_run_and_for_nothing_else():
     s.close()
 
 
+@pytest.mark.parametrize("B", [8, 9, 16, 17, 32, 33, 64, 65])
+def test_router_and_lists_in_one_cluster_and_in_many_ctas(B):
+    """Decode steps on either side of the lines between the router's forms: one cluster of one, two, four or eight CTAs up to 64 tokens, above
+    a launch each for router and lists; against the oracle's logits."""
+    cfg = replace(MOE, L=1, B=B, S=5, T=1)
+    lay = si.build_layout(cfg, budget=64 << 20, cap=1 << 20)
+    bias = si.router_bias(cfg)
+    pool = pinned_pool(lay.pool_bytes)
+    si.fill_pool(lay, pool.numpy())
+    om = forward.OracleModel(cfg, si.weights_as_bits(lay), bias, dtype=np.float32)
+    prompt = si.prompt_tokens(cfg)
+    ref, toks = om.generate(prompt, cfg.T)
+    s = Session(lay, MACHINE, pool_base=pool.data_ptr(), pool_flags=tb.POOL_PINNED, router_bias=bias)
+    s.plan(expert_counts=np.ones((1 + cfg.T, cfg.L, cfg.E), dtype=np.uint32))
+    r = Runner(s, cfg.B * cfg.S)
+    r.reset()
+    r.step(tb.PREFILL, prompt, cfg.S, want_stats=True)
+    r.step(tb.DECODE, np.ascontiguousarray(toks[:, :1]), 1, want_stats=True)
+    got = r.logits.cpu().numpy().copy()
+    counts = s.ctx.expert_counts(cfg.L, cfg.E)
+    s.close()
+    assert (counts[1].sum(axis=1) == B * cfg.topk).all()
+    check_logits([got], [ref[1]])
+
+
 def test_mixtral_widths_at_one_layer_match_oracle_batch_of_eight():
     """Full widths of the Mixtral shape (8 experts of 14336, top-2) at one layer, batch 8, free-running: the expert
     products run at the handful of tokens each expert receives (skinny tensor-core GEMV on blocks of few rows), planned
