@@ -1118,7 +1118,7 @@ __global__ void tgp_swiglu_kernel(const float4 *g, const float4 *u, __nv_bfloat1
 }
 
 // ---- argmax, lowest index on ties -----------------------------------------------------------------
-// A row is shared by the CTAs of a cluster (8 for long rows): each scans a contiguous part with four independent 16-byte loads per
+// A row is shared by the CTAs of a cluster (up to 8 for long rows): each scans a contiguous part with four independent 16-byte loads per
 // thread under way, and the parts' winners meet in the first CTA's shared memory (8 rows of 32000: 9.5 us with one CTA of 1024
 // threads and one dependent element per thread and round, 3.4 us now, from the end of the kernel before).
 __global__ void __launch_bounds__(256) tgp_argmax_kernel(const float *logits, int32_t *out, int32_t *out2, uint32_t V, int vec) {
@@ -2491,8 +2491,12 @@ int tgpk_swiglu(const float *g, const float *u, void *ab, uint64_t n, cudaStream
 
 int tgpk_argmax(const float *logits, int32_t *out, int32_t *out2, uint32_t B, uint32_t V, cudaStream_t st) {
     if (!B) return TGP_OK;
-    // rows of up to 4096 logits are one round of one CTA
-    const uint32_t parts = V > 4096 ? 8 : 1;
+    // Rows of up to 8192 logits are two rounds of one CTA, faster than a cluster at any B (8192 x 1: 2.0 us, 2.3 in eight parts).  Longer ones
+    // have eight parts, fewer where the CTAs are one and a half waves and more and a part would be short: the clusters' launches add up (us in
+    // 1 / 2 / 4 / 8 parts: 32000 x 8 3.8 / 3.3 / 2.8 / 2.5, x 61 4.0 / 3.5 / 3.7 / 3.8, x 1024 24 / 25 / 26 / 34; 16384 x 256 4.2 / 4.7 / 5.6 / 8.5;
+    // 128256 x 96 10.9 / 9.4 / 8.0 / 6.5)
+    uint32_t parts = V > 8192 ? 8 : 1;
+    while (parts > 1 && 2ull * B * parts > 3ull * (uint32_t)device_sms() && V / parts < 12288) parts /= 2;
     const int vec = V % 4 == 0 && (reinterpret_cast<uintptr_t>(logits) & 15u) == 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(B * parts); cfg.blockDim = dim3(256); cfg.stream = st;

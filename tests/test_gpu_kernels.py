@@ -962,3 +962,17 @@ def test_attention_of_short_prompts_with_infinities_in_v(Dh, S, pos0):
     sees = [i for i in range(S) if pos0 + i >= key]
     assert (got[sees, :2, 5] == float("inf")).all() and (got[sees, :2, 6] == float("-inf")).all()
     assert got[:, :, [i for i in range(Dh) if i not in (5, 6)]].isfinite().all() and got[:, 2:].isfinite().all()
+
+
+@pytest.mark.parametrize("B,V", [(27, 8192), (27, 8193), (28, 8193), (56, 8196), (112, 12000), (60, 32000), (300, 8200), (300, 24577), (97, 65537)])
+def test_argmax_in_eight_four_two_and_one_parts(B, V):
+    """Batches and row lengths on either side of the lines between eight parts per row and one; equal maxima in different parts."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(B + V)
+    lg = torch.randn((B, V), device=DEV, generator=gen)
+    at = torch.randint(0, V, (B, 2), device=DEV, generator=gen)
+    lg.scatter_(1, at, 9.0)
+    out = torch.full((B,), -7, dtype=torch.int32, device=DEV)
+    tb.k_argmax(lg, out, B, V)
+    torch.cuda.synchronize()
+    assert torch.equal(out.long(), at.min(dim=1).values)
