@@ -331,7 +331,7 @@ int  tgp_k_swiglu_epilogue(int enable);
  * Results are identical either way.  Process-wide; default off: on the tiny configuration it takes a decode step from 50
  * launches to 32, but a fused span waits for the copies of all its blocks, and the step got no faster (measured). */
 int  tgp_k_decode_fuse(int enable);
-/* Which kernel serves M > 16 (and, on blocks of 8065 or more rows with K % 32 == 0, M > 8): 0 (default) the tcgen05 tensor-core kernels, 1 the
+/* Which kernel serves M > 16 (and, on blocks of 8065 or more rows with K % 32 == 0 and a K of 1536 or more than 148 tiles, M > 8): 0 (default) the tcgen05 tensor-core kernels, 1 the
  * CUDA-core tile kernel (an on-device cross-check; M <= 16 then takes the weight-streaming kernels).  Process-wide. */
 int  tgp_k_gemm_select(int impl);
 /* Which kernel serves 3 <= M <= 16 (K % 32 == 0): 0 (default) the weight-streaming mma.sync kernels, 1 the CUDA-core GEMV (an

@@ -1472,9 +1472,11 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const b
         const uint32_t rlast = min(row0 + RPC, n) - 1;
         const bf16 *wlo = W + (size_t)min(row0 + g, rlast) * K + c * 8;
         const bf16 *whi = W + (size_t)min(row0 + g + 8, rlast) * K + c * 8;
-        float acc[NB][4];
+        float acc[2][NB][4];                               // a load step's two MMAs have sums of their own: half as many additions in a row
 #pragma unroll
-        for (int b = 0; b < NB; ++b) { acc[b][0] = acc[b][1] = acc[b][2] = acc[b][3] = 0.f; }
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[0][b][i] = acc[1][b][i] = 0.f;
         for (uint32_t k0 = warp * 32 * UL; k0 < K; k0 += NW * 32 * UL) {
             uint4 lo[UL], hi[UL];
 #pragma unroll
@@ -1491,8 +1493,8 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const b
                 for (int b = 0; b < NB; ++b) {
                     const uint32_t m = b * 8 + g;
                     const uint4 xv = (k < K && m < Mrows) ? ld_act(reinterpret_cast<const uint4 *>(A + (size_t)m * K + k + c * 8)) : make_uint4(0, 0, 0, 0);
-                    mma_bf16_16816(acc[b], lo[u].x, hi[u].x, lo[u].y, hi[u].y, xv.x, xv.y);
-                    mma_bf16_16816(acc[b], lo[u].z, hi[u].z, lo[u].w, hi[u].w, xv.z, xv.w);
+                    mma_bf16_16816(acc[0][b], lo[u].x, hi[u].x, lo[u].y, hi[u].y, xv.x, xv.y);
+                    mma_bf16_16816(acc[1][b], lo[u].z, hi[u].z, lo[u].w, hi[u].w, xv.z, xv.w);
                 }
             }
         }
@@ -1500,7 +1502,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const b
 #pragma unroll
         for (int b = 0; b < NB; ++b)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) part[warp][b * 4 + i][lane] = acc[b][i];
+            for (int i = 0; i < 4; ++i) part[warp][b * 4 + i][lane] = acc[0][b][i] + acc[1][b][i];
         __syncthreads();
         for (uint32_t v = threadIdx.x; v < NB * 4 * 32; v += NW * 32) {
             const uint32_t slot = v >> 5, ln = v & 31, b = slot >> 2, i = slot & 3;
@@ -1727,8 +1729,14 @@ constexpr uint32_t TILES_WIN_ROWS = 8065;
 // a product that the tcgen05 kernels serve (tgpk_gemm_tc)
 static bool takes_tiles(uint32_t M, uint32_t n, uint32_t K) {
     if (g_gemm_impl || K % 8) return false;
+    if (M > 16) return true;
     // (K not a multiple of 32: the CUDA cores' sums are closer to 64 bits, 6.9e-8 against 1.24e-7 at n=12000, K=1000)
-    return M > 16 || (M >= 9 && n >= TILES_WIN_ROWS && K % 32 == 0 && g_skinny_impl == 0 && !tgpk_gemm_tc_forced());
+    if (M < 9 || n < TILES_WIN_ROWS || K % 32 || g_skinny_impl || tgpk_gemm_tc_forced()) return false;
+    // A short K on fewer tiles than SMs is over before the ring is under way (M=9, K=1024: n=8192 4.6 us in tgp_wstream_mma_splitk_kernel against
+    // 7.0, n=12288 5.5 against 8.1; K=1536, n=16384 12.8 against 10.7; n=32000, K=1024 17.1 against 9.4).  From K=1536 on lists
+    // decide: two blocks of 8192 rows as above, though one alone takes 9.9 - 11.0 us against 11.2 at K=2048, and one of 12288 rows (96
+    // tiles) 10.9 - 11.9 against 14.3.
+    return K >= 1536 || (n + 127) / 128 > (uint32_t)device_sms();
 }
 
 static SkinnyPick pick_skinny(uint32_t M, uint32_t n, uint32_t K) {

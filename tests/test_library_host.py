@@ -451,7 +451,9 @@ def test_aliased_host_pool_shares_pages_between_layer_groups_only():
     p.close()
 
 
-@pytest.mark.parametrize("M,n,K,family", [(12, 12000, 1000, 0), (16, 8065, 520, 0), (9, 32000, 4104, 0), (12, 12000, 1024, 2), (16, 8065, 512, 2), (16, 8064, 4096, 1), (17, 64, 1000, 2)])
-def test_products_of_9_to_16_rows_take_the_tcgen05_kernel_only_where_k_is_a_multiple_of_32(M, n, K, family):
-    """Other K stay with the CUDA cores (key 0, launched alone), whose sums are closer to 64 bits."""
+@pytest.mark.parametrize("M,n,K,family", [(12, 12000, 1000, 0), (16, 8065, 2056, 0), (9, 32000, 4104, 0), (12, 12000, 2048, 2), (16, 8065, 2048, 2), (16, 8064, 4096, 1), (17, 64, 1000, 2),
+                                          (12, 12000, 1024, 0), (9, 18944, 1504, 0), (9, 8065, 1536, 2), (9, 18945, 64, 2)])
+def test_products_of_9_to_16_rows_take_the_tcgen05_kernel_only_where_it_is_ahead_and_as_exact(M, n, K, family):
+    """K not a multiple of 32 stays with the CUDA cores (key 0, launched alone), whose sums are closer to 64 bits; K below 1536 on fewer
+    tiles of 128 rows than SMs (148) with the split-K kernel, which is faster."""
     assert tb.k_gemm_group_key(M, n, K) >> 24 == family
