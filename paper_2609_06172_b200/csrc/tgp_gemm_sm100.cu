@@ -888,6 +888,16 @@ int tgpk_gemm_tc_list(const void *A, uint32_t count, const void *const *W, float
     return TGP_OK;
 }
 
+// Weight rows per tile if the one-tile-per-CTA kernel serves a block of more than 128 activation rows that is launched alone, else 0.  A pair
+// takes 128 cycles an MMA however few its tiles are, one CTA 75 (N <= 128), so where narrow tiles give every CTA one the length of K
+// counts less (us: M=256, K=4096 n=512 16.2 against 18.2 in pairs, n=1024 17.0 / 18.7; M=509, K=6144, n=2048 24.5 / 27.2, n=1024
+// 23.0 / 26.6, but K=2048, n=2048 even).  Both kernels add K in one order into one accumulator: the bits are those of the pairs, which a list takes.
+static uint32_t lone_tile(uint32_t M, uint32_t n, uint32_t K) {
+    if (M <= BM || n > 2048 || (n > 1024 && K < 4096) || cta_slices(M, n, K)) return 0;
+    const uint32_t bn = n > 1024 ? 64 : 32;
+    return (M + BM - 1) / BM * ((n + bn - 1) / bn) <= tc_sms() ? bn : 0;
+}
+
 int tgpk_gemm_tc(const void *A, const void *W, float *C, uint32_t M, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int accumulate, cudaStream_t st,
                  const float *gate, void *aout) {
     constexpr int BN = 128;
@@ -895,6 +905,15 @@ int tgpk_gemm_tc(const void *A, const void *W, float *C, uint32_t M, uint32_t n,
     if (ep.aout && accumulate) return TGP_E_INVAL;
     if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W)) & 15u) return TGP_E_INVAL;     // TMA needs 16-byte aligned bases
     if (K % 8) return TGP_E_INVAL;                                                                       // and 16-byte row strides
+    if (const uint32_t bn = g_tc_variant == 0 && !ep.aout ? lone_tile(M, n, K) : 0) {
+        CUtensorMap ma, mb;
+        if (!make_map(&ma, A, M, K, BM) || !make_map(&mb, W, n, K, bn)) return TGP_E_CUDA;
+        if (!(bn == 32 ? launch_tile<32, 3, 3>(ma, mb, C, M, n, K, ldc, col0, accumulate, st) : launch_tile<64, 3, 3>(ma, mb, C, M, n, K, ldc, col0, accumulate, st))) return TGP_E_CUDA;
+        if (cudaGetLastError() != cudaSuccess) return TGP_E_CUDA;
+        tgpk_launches += 1;
+        tgpk_last_gemm_kernel = "tgp_matmul_tc_kernel";
+        return TGP_OK;
+    }
     if (g_tc_variant == 0 || g_tc_variant == 3 || (g_tc_variant == 4 && (ep.aout || M > 128))) {
         float *Cb = C + col0;
         return tgpk_gemm_tc_list(A, 1, &W, &Cb, &n, &ldc, M, K, accumulate, st, gate ? gate + col0 : nullptr, aout ? (__nv_bfloat16 *)aout + col0 : nullptr);

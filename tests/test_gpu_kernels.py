@@ -976,3 +976,27 @@ def test_argmax_in_eight_four_two_and_one_parts(B, V):
     tb.k_argmax(lg, out, B, V)
     torch.cuda.synchronize()
     assert torch.equal(out.long(), at.min(dim=1).values)
+
+
+@pytest.mark.parametrize("M,n,K,alone", [(129, 1, 64, True), (200, 1023, 1032, True), (512, 1024, 520, True), (513, 1024, 520, False), (512, 1025, 4096, True), (300, 1025, 4088, False),
+                                         (512, 2048, 4104, True), (513, 2048, 4104, False), (256, 2049, 4096, False), (1100, 257, 72, True)])
+def test_products_of_few_tiles_alone_have_the_bits_of_the_pairs(M, n, K, alone):
+    """More than 128 activation rows on either side of the lines between the one-tile-per-CTA kernel, which a block launched alone takes
+    where its tiles are few, and the pairs, which a list takes: the same bits, and the fp64 product."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(M + n + K)
+    A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
+    W = (torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16()
+    want = A.double() @ W.double().T
+    for acc in (False, True):
+        c0 = torch.randn((M, n + 4), device=DEV, generator=gen)
+        one, pair = c0.clone(), [c0.clone(), c0.clone()]
+        tb.k_gemm(A, W, one, M, n, K, n + 4, 0, acc)
+        assert tb.k_gemm_last_kernel() == ("tgp_matmul_tc_kernel" if alone else "tgp_matmul_tc_pair_kernel")
+        tb.k_gemm_group(A, [W, W], pair, M, [n, n], K, [n + 4, n + 4], acc)
+        assert tb.k_gemm_last_kernel() == "tgp_matmul_tc_pair_kernel"
+        torch.cuda.synchronize()
+        assert tb.k_gemm_status() == 0
+        assert torch.equal(one, pair[0]) and torch.equal(one, pair[1]) and torch.equal(one[:, n:], c0[:, n:])
+        exact = want + (c0[:, :n].double() if acc else 0)
+        assert float((one[:, :n].double() - exact).abs().max()) < 2e-5 * float(exact.abs().max())
