@@ -260,7 +260,8 @@ int  tgp_tap_index(tgp_ctx *ctx, uint64_t *out, uint64_t *n_words);
 
 /* Per-op timestamps (Section IV-E "Runtime Monitor": lightweight timestamping).  While enabled, tgp_step()
  * brackets every op with CUDA events on the compute stream (after the op's copies have been waited for, so
- * the figure is kernel time, not stall time).  tgp_op_times() waits for the last timed step and returns one
+ * the figure is kernel time, not stall time).  Steps of a mixture run expert by expert meanwhile (the same bits; untimed steps of 3
+ * to 32 tokens may run all experts of a layer in joint launches).  tgp_op_times() waits for the last timed step and returns one
  * duration in ms per op of that step, ops [*first_op, *first_op + *n_ops) of the trace; ms == NULL asks
  * for the count only. */
 int  tgp_set_op_timing(tgp_ctx *ctx, int enable);
@@ -293,7 +294,8 @@ int  tgp_k_status_clear(void);
 int  tgp_k_rmsnorm(const float *x_dev, uint32_t ldx, const void *g_dev, void *h_dev, uint32_t M, uint32_t d,
                    float eps, void *stream);
 /* C[m, col0 + j] (=|+=) sum_k A[m, k] * W[j, k]: A bf16 [M, K] row-major, W bf16 [n, K] row-major (one out-row
- * block), C fp32 with row stride ldc.  accumulate != 0 adds to C (fused residual).  K % 8 == 0. */
+ * block), C fp32 with row stride ldc.  accumulate != 0 adds to C (fused residual; most kernels add with red.add.f32, which takes
+ * and gives subnormal numbers, below 2^-126, as zeros).  K % 8 == 0. */
 int  tgp_k_gemm(const void *A_dev, const void *W_dev, float *C_dev, uint32_t M, uint32_t n, uint32_t K,
                 uint32_t ldc, uint32_t col0, int accumulate, void *stream);
 /* Several products over the same activations in one call (Section II-B's kernel sequence: the q, k and v projections of a
@@ -331,8 +333,9 @@ int  tgp_k_swiglu_epilogue(int enable);
  * Results are identical either way.  Process-wide; default off: on the tiny configuration it takes a decode step from 50
  * launches to 32, but a fused span waits for the copies of all its blocks, and the step got no faster (measured). */
 int  tgp_k_decode_fuse(int enable);
-/* Which kernel serves M > 16 (and, on blocks of 8065 or more rows with K % 32 == 0 and a K of 1536 or more than 148 tiles, M > 8): 0 (default) the tcgen05 tensor-core kernels, 1 the
- * CUDA-core tile kernel (an on-device cross-check; M <= 16 then takes the weight-streaming kernels).  Process-wide. */
+/* Which kernel serves M > 16 (and M > 8 on blocks of 8065 or more rows with K % 32 == 0 and K >= 1536, or of more 128-row tiles
+ * than the GPU has SMs): 0 (default) the tcgen05 tensor-core kernels, 1 the CUDA-core tile kernel (an on-device cross-check;
+ * M <= 16 then takes the weight-streaming kernels).  Process-wide. */
 int  tgp_k_gemm_select(int impl);
 /* Which kernel serves 3 <= M <= 16 (K % 32 == 0): 0 (default) the weight-streaming mma.sync kernels, 1 the CUDA-core GEMV (an
  * on-device cross-check).  Process-wide. */
@@ -353,7 +356,8 @@ int  tgp_k_gemv_overlap(int enable);
 int  tgp_k_gemm_chain(int enable);
 /* Tensor-core GEMM variant: 0 (default) picks by problem size between the paired kernel (tiles of 256 weight rows x up to 256
  * activation rows on the two SMs of a CTA pair) and the one of one 128-row weight tile per CTA, with K in one, two or four
- * slices; 1 forces the 128x128 one-tile-per-CTA kernel, 2 the persistent 128x256 kernel with double-buffered accumulators,
+ * slices, and for blocks of few tiles launched alone above 128 activation rows one narrow tile per CTA (the bits of the pairs);
+ * 1 forces the 128x128 one-tile-per-CTA kernel, 2 the persistent 128x256 kernel with double-buffered accumulators,
  * 3 the paired kernel with its largest tiles, 4 the one-tile-per-CTA kernel of variant 1 with the operands swapped (the weights
  * are the 128-row operand, the tile is stored transposed; for M <= 128, else as 0).  Process-wide; for tests and timing. */
 int  tgp_k_gemm_tc_variant(int variant);

@@ -1105,7 +1105,7 @@ extern "C" int tgp_run_capture_begin(tgp_ctx *ctx, void *compute_stream, void *c
     TgpEngine *e = ctx->eng;
     if (!ctx->plan.valid) return TGP_E_NO_PLAN;
     if (ctx->variant != TGP_VAR_EXPLICIT_RING) return tgp_fail(ctx, TGP_E_STATE, "only the explicit engine can be captured");
-    if (ctx->cfg.E) return tgp_fail(ctx, TGP_E_STATE, "an MoE step reads routing counts on the host and cannot be captured");
+    if (ctx->cfg.E) return tgp_fail(ctx, TGP_E_STATE, "an MoE run cannot be captured: steps whose experts run one by one read routing counts on the host");
     if (e->capturing || e->next_step != 0 || e->next_cmd != 0) return tgp_fail(ctx, TGP_E_STATE, "call tgp_run_reset() first");
     if (e->op_timing || e->tap) return tgp_fail(ctx, TGP_E_STATE, "switch timing and tap off before capturing");
     if (!compute_stream || !copy_stream || compute_stream == copy_stream) return tgp_fail(ctx, TGP_E_INVAL, "two distinct non-default streams are required");

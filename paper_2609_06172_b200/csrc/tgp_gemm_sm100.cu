@@ -1,8 +1,13 @@
-// Prefill GEMM on the 5th-generation tensor cores (sm_100a): C[M, n] (=|+=) A[M, K] * W[n, K]^T,
-// bf16 operands, fp32 accumulation in tensor memory.  Three kernels, chosen by problem size in tgpk_gemm_tc(): one
-// tile per CTA (below), a persistent kernel with 128 x 256 tiles and double-buffered accumulators, and - for the large
-// products of a prefill - a kernel in which the two CTAs of a cluster share 256 x 256 tiles through the two-SM MMA.
+// GEMM on the 5th-generation tensor cores (sm_100a): C[M, n] (=|+=) A[M, K] * W[n, K]^T,
+// bf16 operands, fp32 accumulation in tensor memory.  tgpk_gemm_tc() and tgpk_gemm_tc_list() choose between
+//   tgp_wstream_tc_kernel         one tile of 128 weight rows x up to 128 activation rows per CTA, K in 1, 2 or 4 slices: up to 128
+//                                 activation rows, and more of them on few tiles with a long K;
+//   tgp_matmul_tc_pair_kernel     tiles of 256 weight rows x up to 256 activation rows on the two SMs of a CTA pair: the rest;
+//   tgp_matmul_tc_kernel          one narrow tile per CTA (below): more than 128 activation rows on few tiles, launched alone.
+// tgp_matmul_tc_persistent_kernel and the other forms of tgp_matmul_tc_kernel run by request only (tgp_k_gemm_tc_variant): they
+// cross-check the others.
 //
+// tgp_matmul_tc_kernel:
 // One CTA computes a 128 x BN tile.  Warp 0 (one lane) feeds a shared-memory ring of ST stages with TMA
 // (128-byte swizzle, 64 bf16 of K per stage); warp 1 (one lane) issues tcgen05.mma (M=128, N=BN, K=16,
 // four per stage) into a TMEM accumulator and releases stages with tcgen05.commit; warps 2-5 wait for the
@@ -541,7 +546,7 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
 // per MMA and not a pair: an MMA costs 75 cycles for N <= 128, a pair's 128 for any N <= 256 (112 SMs of pairs would take
 // their weights in no faster than HBM delivers them), and there are four times as many tiles to share out.
 //   K slices: a block of few tiles is split along K over the SL CTAs of a cluster; their partial tiles meet in shared memory
-// and are summed pairwise.  The split depends on M, n and K alone: a block computes the same bits alone or in a list.
+// and are summed pairwise.  The split depends on M, n, K and the number of SMs: a block computes the same bits alone or in a list.
 //   Accumulators: consecutive MMAs go to different ones (eight up to 32 activation rows, four up to 64, else two), summed at the end.
 // The tensor core adds into fp32 without rounding to nearest, so the error of a sum grows with the number of additions in a
 // row, and MMAs into one accumulator or into several take the same time (M=61, n=4096, K=4096: distance from 64 bits 1.0e-6 with
@@ -755,8 +760,8 @@ static bool launch_tile(const CUtensorMap &ma, const CUtensorMap &mb, float *C, 
     return true;
 }
 
-static int g_tc_variant = 0;     // 0 and 3 the paired kernel, 1 force the 128x128 per-tile kernel, 2 the persistent 128x256 kernel,
-                                 // 4 the per-tile kernel with the weights as the 128-row operand (M <= 128 only; else as 0)
+static int g_tc_variant = 0;     // 0 by size (see the top of this file), 1 force the 128x128 per-tile kernel, 2 the persistent 128x256 kernel, 3 the paired
+                                 // kernel with its largest tiles, 4 the per-tile kernel with the weights as the 128-row operand (M <= 128 only; else as 0)
 
 bool tgpk_gemm_tc_forced() { return g_tc_variant != 0; }
 
@@ -766,8 +771,8 @@ static uint32_t tc_sms() {
     return (uint32_t)sms;
 }
 
-// K slices of a block in the one-tile-per-CTA kernel, 0: the paired kernel serves it.  The choice depends on M, n and K of the block
-// alone.  Measured (us; M=61 unless stated):
+// K slices of a block in the one-tile-per-CTA kernel, 0: the paired kernel serves it.  The choice depends on M, n and K of the block and
+// on the number of SMs (the bits of a sliced product may differ between devices of different sizes), not on a list.  Measured (us; M=61 unless stated):
 //   n=4096, K=4096        22.4 unsplit, 15.3 in two slices, 11.9 in four, 12.4 in eight
 //   n=2048, K=8192        41.6, 24.7, 15.4, 21.1 (few clusters of eight fit the GPU at a time: no eight anywhere)
 //   n=8192, K=8192        42.4, 28.1, 26.4 (256 CTAs, two per SM)

@@ -2285,6 +2285,7 @@ int tgpk_experts(const TgpExperts &x, cudaStream_t st) {
     }
     launch_experts<false>(p, T, st);
     launch_pdl(tgp_expert_combine_kernel, dim3(x.M, x.d > 2048 ? 2 : 1), dim3(256), 0, st, x.x, (const float *)x.y, x.idx, x.gate, x.pos, x.counts, x.d);
+    tgpk_last_gemm_kernel = "tgp_expert_mma_kernel";
     LAUNCH_CHECK(3);
     return TGP_OK;
 }

@@ -47,9 +47,9 @@ def bf16_close(got_f32, want_f32, frac=0.01):
                                    # few rows, long K at M <= 2: the split-K GEMV (two rows per CTA; one row per CTA up to 1024 rows),
                                    # odd row counts, K not a multiple of the 256-element chunk, more CTAs than resident slots
                                    (1, 2048, 8192), (2, 2051, 8200), (1, 513, 8192), (2, 1, 16384), (1, 4735, 8192),
-                                   # 33 - 64 activation rows on a block of few rows: two weight-streaming launches of half the rows
+                                   # 33 - 64 activation rows on blocks of few rows: one 128-row weight tile per CTA, K in two or four slices
                                    (33, 1030, 512), (48, 2049, 4096), (64, 130, 96), (40, 4090, 64),
-                                   # ... and on blocks of many rows the tiled GEMM with the weights as its 128-row operand
+                                   # ... and on blocks of many rows
                                    (40, 4720, 64), (64, 4096, 1032), (20, 8200, 128)])
 @pytest.mark.parametrize("accumulate", [0, 1])
 def test_gemm_matches_oracle(M, n, K, accumulate):
@@ -122,12 +122,10 @@ def test_tensor_core_gemm_with_the_weights_as_the_128_row_operand(M, n, K, acc):
     ldc, col0 = n + 12, 4
     c0 = np.random.default_rng(9).standard_normal((M, ldc)).astype(np.float32) * 0.01
     tb.k_gemm_tc_variant(4)
-    tb.k_skinny_select(1)            # 17 - 32 rows reach the tiled GEMM only with the weight-streaming kernel switched off
     Cd = torch.from_numpy(c0.copy()).to(DEV)
     tb.k_gemm(A, W, Cd, M, n, K, ldc, col0, acc)
     torch.cuda.synchronize()
     tb.k_gemm_tc_variant(0)
-    tb.k_skinny_select(0)
     assert tb.k_gemm_status() == 0
     got = Cd.cpu().numpy()
     want = oracle().linear(si.bf16_bits_to_f32(a_bits), si.bf16_bits_to_f32(w_bits).astype(np.float64)).astype(np.float64)
@@ -690,14 +688,17 @@ def test_skinny_tensor_core_gemv_matches_oracle_and_cuda_core_path(M, n, K, accu
     a_bits, w_bits = rnd_bits(41, M * K).reshape(M, K), rnd_bits(42, n * K).reshape(n, K)
     A, W = bf16_dev(a_bits), bf16_dev(w_bits)
     c0 = np.random.default_rng(M + n).standard_normal((M, n + 8)).astype(np.float32) * 0.01
-    outs = []
+    outs, names = [], []
     for impl in (0, 1):
-        tb.k_skinny_select(impl)
+        (tb.k_skinny_select if M <= 16 else tb.k_gemm_select)(impl)          # (17 rows and more are the tcgen05 kernels', 1: the CUDA-core tiles)
         Cd = torch.from_numpy(c0.copy()).to(DEV)
         tb.k_gemm(A, W, Cd, M, n, K, n + 8, 4, accumulate)
         torch.cuda.synchronize()
         outs.append(Cd.cpu().numpy())
+        names.append(tb.k_gemm_last_kernel())
     tb.k_skinny_select(0)
+    tb.k_gemm_select(0)
+    assert names[0] != names[1]
     want = c0.astype(np.float64).copy()
     prod = oracle().linear(si.bf16_bits_to_f32(a_bits), si.bf16_bits_to_f32(w_bits).astype(np.float64)).astype(np.float64)
     want[:, 4:4 + n] = prod + (c0[:, 4:4 + n] if accumulate else 0)
@@ -708,11 +709,12 @@ def test_skinny_tensor_core_gemv_matches_oracle_and_cuda_core_path(M, n, K, accu
         assert np.array_equal(out[:, :4], c0[:, :4]) and np.array_equal(out[:, 4 + n:], c0[:, 4 + n:])
 
 
-# blocks on either side of the lines that send a product of 3 - 32 rows to the persistent list kernel: K below / at 2048 and 3072
-# (M <= 8) and 4096 (M <= 32), row counts around five 16-row groups per SM, a ragged last group, a K that ends inside a warp's chunk
-@pytest.mark.parametrize("M,ns,K", [(3, (4737,), 3072), (8, (4800, 4737), 3104), (8, (11840, 12000), 2048), (5, (11800,), 2080), (9, (4737, 5000), 4096),
-                                    (16, (9001,), 4128), (17, (4737, 8064), 4096), (32, (8065,), 4096)])
-def test_blocks_of_many_rows_take_the_list_kernel_with_the_same_bits_alone_and_in_a_list(M, ns, K):
+# blocks on either side of the lines that send a product of 3 - 16 rows to the persistent list kernel: K below / at 2048 and 3072
+# (M <= 8) and 4096 (M <= 16), row counts around five 16-row groups per SM, a ragged last group, a K that ends inside a warp's chunk
+@pytest.mark.parametrize("M,ns,K,listed_family", [(3, (4737,), 3072, 1), (8, (4800, 4737), 3104, 1), (8, (11840, 12000), 2048, 1), (5, (11800,), 2080, 0), (9, (4737, 5000), 4096, 1),
+                                                  (16, (4737, 8064), 4128, 1), (13, (8064,), 4096, 1), (12, (4737, 8064), 4064, 0)])
+def test_blocks_of_many_rows_take_the_list_kernel_with_the_same_bits_alone_and_in_a_list(M, ns, K, listed_family):
+    assert all(tb.k_gemm_group_key(M, n, K) >> 24 == listed_family for n in ns)      # 1: the list kernel, 0: alone in another one
     gen = torch.Generator(device=DEV)
     gen.manual_seed(M * K + len(ns))
     A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
