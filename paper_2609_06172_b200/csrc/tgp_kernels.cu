@@ -1550,8 +1550,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
     uint4 lo[2][G][SK], hi[2][G][SK];                     // two register sets of SK load steps of every group
     // the activation fragments of a set are loaded with its weights (they come from L2 more often than from L1 -
     // a long K does not fit there - and would otherwise be waited for inside the MMA sequence)
-    constexpr bool XPRE = !(NB >= 2 && G == 1);           // (those instances have no registers left for them)
-    uint4 xs[2][XPRE ? SK : 1][XPRE ? NB : 1];
+    uint4 xs[2][SK][NB];
     float acc[G][NB][4];
     // which block a group belongs to: looked up here for the weights and again after the K loop for the output, so
     // that the output's pointer and stride do not occupy registers while the loads are in flight
@@ -1592,27 +1591,21 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
     };
     auto issue_act = [&](auto set, uint32_t kb) {          // the activation fragments that go with a set; only after griddepcontrol.wait
         constexpr int S = decltype(set)::value;
-        if constexpr (XPRE) {
-#pragma unroll
-            for (int u = 0; u < SK; ++u) {
-                const uint32_t k = kb + 32 * u;
-#pragma unroll
-                for (int b = 0; b < NB; ++b)
-                    xs[S][u][b] = (k < K && b * 8 + g < Mrows) ? ld_act(reinterpret_cast<const uint4 *>(A + (size_t)(b * 8 + g) * K + k + c * 8)) : make_uint4(0, 0, 0, 0);
-            }
-        }
-    };
-    auto consume = [&](auto set, uint32_t kb) {
-        constexpr int S = decltype(set)::value;
 #pragma unroll
         for (int u = 0; u < SK; ++u) {
             const uint32_t k = kb + 32 * u;
 #pragma unroll
+            for (int b = 0; b < NB; ++b)
+                xs[S][u][b] = (k < K && b * 8 + g < Mrows) ? ld_act(reinterpret_cast<const uint4 *>(A + (size_t)(b * 8 + g) * K + k + c * 8)) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    auto consume = [&](auto set) {
+        constexpr int S = decltype(set)::value;
+#pragma unroll
+        for (int u = 0; u < SK; ++u) {
+#pragma unroll
             for (int b = 0; b < NB; ++b) {
-                const uint32_t m = b * 8 + g;
-                uint4 xv;
-                if constexpr (XPRE) xv = xs[S][u][b];
-                else xv = (k < K && m < Mrows) ? ld_act(reinterpret_cast<const uint4 *>(A + (size_t)m * K + k + c * 8)) : make_uint4(0, 0, 0, 0);
+                const uint4 xv = xs[S][u][b];
 #pragma unroll
                 for (int r = 0; r < G; ++r) {
                     mma_bf16_16816(acc[r][b], lo[S][r][u].x, hi[S][r][u].x, lo[S][r][u].y, hi[S][r][u].y, xv.x, xv.y);
@@ -1651,28 +1644,27 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
         return true;
     };
     locate(grp);
-    uint32_t kb_cur = column();
-    issue(set0, kb_cur);
-    issue(set1, kb_cur + SET1);
+    const uint32_t kb_first = column();
+    issue(set0, kb_first);
+    issue(set1, kb_first + SET1);
     bool cur_last = advance();
     // Weights are never written by a kernel, so they are requested before the previous launch of the stream has finished.
     // The activations are read after it has - unless the launcher knows that they are older than that launch (it read the
     // same activations): then they are requested with the weights.  The next launch is released only here, after the wait:
     // when it starts, everything before this launch is complete, which is what lets it read its activations early in turn.
-    if (acts_early) { issue_act(set0, kb_cur); issue_act(set1, kb_cur + SET1); }
+    if (acts_early) { issue_act(set0, kb_first); issue_act(set1, kb_first + SET1); }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!acts_early) { issue_act(set0, kb_cur); issue_act(set1, kb_cur + SET1); }
+    if (!acts_early) { issue_act(set0, kb_first); issue_act(set1, kb_first + SET1); }
     clear();
     for (;;) {
         const bool have_next = grp < groups_total;
         const uint32_t kb_next = column();
-        consume(set0, kb_cur);
+        consume(set0);
         if (have_next) { issue(set0, kb_next); issue_act(set0, kb_next); }
-        consume(set1, kb_cur + SET1);
+        consume(set1);
         if (have_next) { issue(set1, kb_next + SET1); issue_act(set1, kb_next + SET1); }
         const bool next_last = have_next ? advance() : false;
-        kb_cur = kb_next;
         if (!cur_last) { cur_last = next_last; continue; }
         cur_last = next_last;
         // this warp has finished the group(s) at grp0
@@ -1753,20 +1745,22 @@ static SkinnyPick pick_skinny(uint32_t M, uint32_t n, uint32_t K) {
     // One choice per class of M for all of them, so that the pieces of a matrix share a launch whatever the rows of its
     // last piece:
     //   M <= 8   16 warps, 8 load steps per warp and chunk
-    //   M <= 16  8 warps of twice the registers, 16 load steps: room for the activation fragments of a register set
+    //   M <= 16  16 warps, 4 load steps: a chunk of 2048 columns, so that a K of 1024 still occupies half of the warps, and registers for the
+    //            activation fragments of both sets (M=16, from the end of the norm before: n=1024, K=1024 8.5 us with 8 warps of 16 steps,
+    //            2.0 us; n=2048, K=2048 9.9 / 3.8; n=2048, K=8192 20.5 / 10.1; n=4096, K=14336 31.4 / 26.8.  Twice as many CTAs
+    //            of 8 warps are no faster: 2.1, 3.8.  Half the additions in a row, too: 1.4e-7 from 64 bits at K=2048, 4.8e-7 before)
     const bool few = k.split && groups16 < 2u * sms;
     const bool deep = k.nb == 1 ? K >= 3072 || (K >= 2048 && groups16 >= 5u * sms) : K >= 4096;
     k.persistent = few || deep;
     if (k.persistent) k.split = true;
     if (k.persistent) {
-        k.nw = k.nb == 1 ? 16 : 8;
-        k.u = k.nb == 1 ? 8 : 16;
-        k.rows = 16;
+        k.nw = 16;
+        k.u = k.nb == 1 ? 8 : 4;
     } else {
         k.nw = 8;
         k.u = 4;
-        k.rows = 16;
     }
+    k.rows = 16;
     return k;
 }
 
@@ -1795,7 +1789,7 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
         // 40 SMs one round short, 293 of 14 do not) - but the rows a tile lacks still occupy its load slots (their lanes
         // re-read the group's last row; fewer than 9 rows per group measured no faster for blocks of few rows).  G and r are the
         // pair with the least estimated time of the busiest CTA: rounds x (G x (r + tile rows) / 2 + 4 NB), in rows read.
-        const uint32_t tile = (uint32_t)k.rows, gmax = NB == 1 ? 2 : 4;
+        const uint32_t tile = (uint32_t)k.rows, gmax = 2;
         uint32_t best = 0xffffffffu, best_r = tile;
         for (uint32_t G = gmax; G >= 1; G >>= 1)
             for (uint32_t r = g_gemv_balance ? tile / 2 + 1 : tile; r <= tile; ++r) {
@@ -1831,10 +1825,14 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
         if constexpr (NB == 1 && U == 8) {
             if (per_cta == 2) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>, A, p, Mrows, total, K, acc, rpc, early);
             else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 16, 16, 1>, A, p, Mrows, total, K, acc, rpc, early);
-        } else if constexpr (NB == 2 && U == 16) {
-            if (per_cta == 4) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 8, 16, 4>, A, p, Mrows, total, K, acc, rpc, early);
-            else if (per_cta == 2) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 8, 16, 2>, A, p, Mrows, total, K, acc, rpc, early);
-            else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 8, 16, 1>, A, p, Mrows, total, K, acc, rpc, early);
+        } else if constexpr (NB == 2) {
+            if (per_cta == 2) {
+                constexpr size_t smem = 16 * 2 * NB * 4 * 32 * 4;      // the partial tiles of 16 warps, two row groups each
+                static bool attr_set = false;
+                if (!attr_set) { cudaFuncSetAttribute(tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); attr_set = true; }
+                cfg.dynamicSmemBytes = smem;
+                cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>, A, p, Mrows, total, K, acc, rpc, early);
+            } else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 16, 16, 1>, A, p, Mrows, total, K, acc, rpc, early);
         }
     } else if constexpr (STREAMS) {
         if (!k.split) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_kernel<NB, U>, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);
@@ -1844,7 +1842,7 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
 
 static void launch_skinny_pick(const bf16 *A, const GemvParts &p, const SkinnyPick &k, uint32_t Mrows, uint32_t K, int acc, cudaStream_t st) {
     if (k.nb == 1) { if (k.u == 8) launch_skinny<1, 8>(A, p, k, Mrows, K, acc, st); else launch_skinny<1, 4>(A, p, k, Mrows, K, acc, st); }
-    else { if (k.u == 16) launch_skinny<2, 16>(A, p, k, Mrows, K, acc, st); else launch_skinny<2, 4>(A, p, k, Mrows, K, acc, st); }
+    else launch_skinny<2, 4>(A, p, k, Mrows, K, acc, st);
 }
 
 template <int MT, int RB, int U>
@@ -2304,38 +2302,42 @@ uint32_t tgpk_gemm_group_key(uint32_t M, uint32_t n, uint32_t K) {
     return k.persistent ? (0x1000000u | (uint32_t)k.nb | (uint32_t)k.u << 4 | (uint32_t)k.nw << 8 | (uint32_t)k.rows << 16) : 0;
 }
 
-int tgpk_gemm_group(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t M, uint32_t K,
-                    int accumulate, cudaStream_t st) {
-    if (!count || !M) return TGP_OK;
-    const uint32_t key = tgpk_gemm_group_key(M, n[0], K);
-    bool same = key != 0 && key < 0x2000000u && count >= 2 && count <= TGP_GEMM_GROUP_MAX;
-    for (uint32_t s = 1; s < count && same; ++s) same = tgpk_gemm_group_key(M, n[s], K) == key;
-    if (!same) {
-        // neighbours that one tcgen05 kernel serves with one split of K share a launch, at any M; other parts are launched alone
-        auto tc_class = [&](uint32_t s) { return g_gemm_group && n[s] && takes_tiles(M, n[s], K) && !tgpk_gemm_tc_forced() ? tgpk_gemm_tc_class(M, n[s], K) : 0u; };
-        for (uint32_t s = 0; s < count;) {
-            const uint32_t cls = tc_class(s);
-            uint32_t e = s + 1;
-            while (cls && e < count && e - s < TGP_GEMM_GROUP_MAX && tc_class(e) == cls) ++e;
-            const int rc = e - s > 1 ? tgpk_gemm_tc_list(A, e - s, W + s, C + s, n + s, ldc + s, M, K, accumulate, st)
-                                     : tgpk_gemm(A, W[s], C[s], M, n[s], K, ldc[s], 0, accumulate, st);
-            if (rc) return rc;
-            s = e;
-        }
-        return TGP_OK;
-    }
+// Blocks of one key below 0x2000000 over the same activations, in one launch.
+static int gemm_list(const bf16 *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t M, uint32_t K, int accumulate, cudaStream_t st) {
     GemvParts p;
     memset(&p, 0, sizeof(p));
     uint32_t total = 0;
     for (uint32_t s = 0; s < count; ++s) { p.W[s] = (const bf16 *)W[s]; p.C[s] = C[s]; p.n[s] = n[s]; p.ldc[s] = ldc[s]; total += n[s]; }
     p.count = count;
-    if (M == 1) launch_gemv_group<1, false>((const bf16 *)A, p, M, total, K, accumulate, st);
-    else if (M == 2) launch_gemv_group<2, false>((const bf16 *)A, p, M, total, K, accumulate, st);
-    else launch_skinny_pick((const bf16 *)A, p, pick_skinny(M, n[0], K), M, K, accumulate, st);
+    if (M == 1) launch_gemv_group<1, false>(A, p, M, total, K, accumulate, st);
+    else if (M == 2) launch_gemv_group<2, false>(A, p, M, total, K, accumulate, st);
+    else launch_skinny_pick(A, p, pick_skinny(M, n[0], K), M, K, accumulate, st);
     LAUNCH_CHECK(1);
     return TGP_OK;
 }
 
+int tgpk_gemm_group(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t M, uint32_t K,
+                    int accumulate, cudaStream_t st) {
+    if (!count || !M) return TGP_OK;
+    // Neighbours with one key share a launch, the others are launched alone (q of a large model takes the tcgen05 kernel at 16 rows, its k and v
+    // the list kernel: each in a launch of its own 62 us at d=8192, 1024 rows of k and of v, 37 with k and v in one).  From 33 rows on the key is that of the tcgen05 kernels.
+    auto key_of = [&](uint32_t s) -> uint32_t {
+        if (M <= 32) return tgpk_gemm_group_key(M, n[s], K);
+        return g_gemm_group && n[s] && takes_tiles(M, n[s], K) && !tgpk_gemm_tc_forced() ? 0x2000000u | tgpk_gemm_tc_class(M, n[s], K) : 0u;
+    };
+    for (uint32_t s = 0; s < count;) {
+        const uint32_t key = key_of(s);
+        uint32_t e = s + 1;
+        while (key && e < count && e - s < TGP_GEMM_GROUP_MAX && key_of(e) == key) ++e;
+        int rc;
+        if (e - s == 1) rc = tgpk_gemm(A, W[s], C[s], M, n[s], K, ldc[s], 0, accumulate, st);
+        else if (key >= 0x2000000u) rc = tgpk_gemm_tc_list(A, e - s, W + s, C + s, n + s, ldc + s, M, K, accumulate, st);
+        else rc = gemm_list((const bf16 *)A, e - s, W + s, C + s, n + s, ldc + s, M, K, accumulate, st);
+        if (rc) return rc;
+        s = e;
+    }
+    return TGP_OK;
+}
 
 // Products of M <= 2 activation rows whose activations are computed on the fly (see ASrc): the RMSNorm of x, or SwiGLU of
 // (g32, u32).  Every block must carry the M <= 2 group key (tgpk_gemm_group_key(M, n, K) == M); K % 8 == 0.

@@ -732,6 +732,30 @@ def test_blocks_of_many_rows_take_the_list_kernel_with_the_same_bits_alone_and_i
         assert float((a.double() - want).abs().max()) < 2e-5 * float(want.abs().max())
 
 
+# the list kernel at 9 - 16 rows around a chunk of 16 warps x 128 columns (one column block, a warp's chunk more or less, many chunks), ragged
+# row groups, one and two row groups per CTA; and lists of which only neighbours share a kernel
+@pytest.mark.parametrize("M,ns,K", [(9, (1, 17), 32), (16, (1024, 1000), 1024), (12, (300,), 2016), (16, (2048, 4100), 2048), (11, (33, 640), 2080), (16, (500,), 14368),
+                                    (16, (8200, 1024, 1000), 4096), (10, (1000, 4800, 4736, 7), 2048), (9, (16, 8065, 8070, 16, 24), 4096)])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_products_of_9_to_16_rows_alone_and_in_lists_of_several_kernels(M, ns, K, accumulate):
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(M * K + len(ns))
+    A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
+    Ws = [(torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16() for n in ns]
+    lds = [n + 4 * (s % 3) for s, n in enumerate(ns)]
+    c0 = [torch.randn((M, ld), device=DEV, generator=gen) for ld in lds]
+    alone, listed = [c.clone() for c in c0], [c.clone() for c in c0]
+    for W, C, n, ld in zip(Ws, alone, ns, lds):
+        tb.k_gemm(A, W, C, M, n, K, ld, 0, accumulate)
+    tb.k_gemm_group(A, Ws, listed, M, list(ns), K, lds, accumulate)
+    torch.cuda.synchronize()
+    for W, a, b, c, n in zip(Ws, alone, listed, c0, ns):
+        assert torch.equal(a, b) and torch.equal(a[:, n:], c[:, n:])
+        want = A.double() @ W.double().T + (c[:, :n].double() if accumulate else 0)
+        # fp32 sums of K products of N(0, 1) x N(0, 0.02): errors of a few 2^-24 of the partial sums' size, bounded as in the tests above
+        assert float((a[:, :n].double() - want).abs().max()) < 2e-5 * float(want.abs().max()) + 1e-7
+
+
 # the tcgen05 kernels on either side of their dispatch lines: one tile per CTA unsplit / in 2 / in 4 slices of K (ragged row tiles, K that
 # ends inside a 64-wide block or leaves slices of unequal length), the line at 8192 columns above 128 activation rows, the paired
 # kernel's activation tiles (one of 160 rows, three of 224, the last one ragged), lists of ragged parts
