@@ -636,6 +636,10 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
 
     if (warp == 0) {
         if (lane == 0) {
+            // The weights of the first ring come into L2 while the previous kernel still runs; loading them here would be wrong where that
+            // kernel writes them (M=61: n=4096, K=4096 13.3 -> 12.3 us, the list of 2 x 14336 45.7 -> 43.6, with 16 rows 42.4 -> 40.6; from the
+            // end of the norm before).  Requests ahead of the ring further on make it slower.
+            for (uint32_t kb = 0; kb < min(num_k, ST); ++kb) tma_prefetch_2d(mw, (int)((kb_lo + kb) * BK), (int)w0);
             asm volatile("griddepcontrol.wait;" ::: "memory");
             uint32_t s = 0, ph = 0, armed = 0;
             const uint32_t withhold = blockIdx.x == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;     // test hook: this stage is never loaded
