@@ -1235,48 +1235,69 @@ __global__ void __launch_bounds__(256) tgp_router_kernel(const bf16 *h, const bf
     }
 }
 
-// Up to ROUTE_SMALL tokens: router and token lists in one launch, with the arithmetic of tgp_router_kernel.  A cluster takes the tokens, a warp
-// each, eight per CTA (one CTA reads the router's weights for all of them through one SM: 16 experts, d=8192, 32 tokens 68 us, 37 us in
-// four; with 64 tokens 135 and 37); the picks meet in its first CTA, whose warps list the tokens of the experts in ascending order.  pos[2 m + s]: the place of
+// Up to ROUTE_SMALL tokens: router and token lists in one launch of a cluster, with the arithmetic of tgp_router_kernel.  It is a chain of
+// latencies, so the tokens are spread over up to eight CTAs and a warp computes one logit at a time, up to eight loads of each operand under way; the weights of
+// its first one, which no kernel writes, are requested before the previous kernel has finished (8 experts, d=1024, 16 tokens: a warp per token and
+// all its experts, eight tokens per CTA 6.3 us, 3.7 us now; 8 experts, d=4096, 32 tokens 15.9, 7.2).  The picks meet in the first CTA, whose warps
+// list the tokens of the experts in ascending order.  pos[2 m + s]: the place of
 // token m in the list of its s-th expert.  counts_host (may be NULL): mapped host memory that receives the counts too.
-constexpr uint32_t ROUTE_SMALL = 64;
+constexpr uint32_t ROUTE_SMALL = 64, ROUTE_WARPS = 16;
 
 template <int E>
-__global__ void __launch_bounds__(256) tgp_route_small_kernel(const bf16 *h, const bf16 *__restrict__ Wr, const float *__restrict__ bias, int32_t *idx, float *gate, int32_t *rows,
+__global__ void __launch_bounds__(ROUTE_WARPS * 32) tgp_route_small_kernel(const bf16 *h, const bf16 *__restrict__ Wr, const float *__restrict__ bias, int32_t *idx, float *gate, int32_t *rows,
                                                              float *gates, int32_t *counts, int32_t *pos, int32_t *counts_host, uint32_t M, uint32_t stride, uint32_t d, uint32_t topk) {
-    pdl_enter();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ __align__(8) int32_t si[2 * ROUTE_SMALL];     // the first CTA's: the picks of all tokens
     __shared__ __align__(8) float sg[2 * ROUTE_SMALL];
+    __shared__ float logit[ROUTE_SMALL / 8][E];              // of this CTA's tokens
+    constexpr int U = 8;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t rank, parts;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(parts));
     if (parts > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    const uint32_t m = rank * 8 + warp;
-    int i0 = 0, i1 = -1; float g0 = 0.f, g1 = 0.f;
-    if (m < M) {
-        float acc[E];
+    const uint32_t per = (M + parts - 1) / parts, m0 = rank * per, mine = m0 < M ? min(per, M - m0) : 0u;       // this CTA's tokens
+    uint4 w[U];
+    auto load_w = [&](uint32_t e, uint32_t k0) {
 #pragma unroll
-        for (int e = 0; e < E; ++e) acc[e] = 0.f;
-#pragma unroll 2
-        for (uint32_t k = lane * 8; k < d; k += 256) {
-            float xf[8];
-            unpack8(ld_act(reinterpret_cast<const uint4 *>(h + (size_t)m * d + k)), xf);
+        for (int u = 0; u < U; ++u) w[u] = k0 + 256 * u < d ? __ldg(reinterpret_cast<const uint4 *>(Wr + (size_t)e * d + k0 + 256 * u)) : make_uint4(0, 0, 0, 0);
+    };
+    load_w(warp % E, lane * 8);
+    const float b0 = bias[warp % E];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (uint32_t q = warp; q < mine * E; q += ROUTE_WARPS) {        // logit q % E of token m0 + q / E
+        const uint32_t e = q % E;
+        const bf16 *x = h + (size_t)(m0 + q / E) * d;
+        float acc = 0.f;
+        for (uint32_t k0 = lane * 8; k0 < d; k0 += 256 * U) {
+            uint4 xv[U];
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                float wf[8];
-                unpack8(__ldg(reinterpret_cast<const uint4 *>(Wr + (size_t)e * d + k)), wf);
+            for (int u = 0; u < U; ++u) xv[u] = k0 + 256 * u < d ? ld_act(reinterpret_cast<const uint4 *>(x + k0 + 256 * u)) : make_uint4(0, 0, 0, 0);
+            if (q != warp || k0 != lane * 8) load_w(e, k0);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) acc[e] = fmaf(xf[i], wf[i], acc[e]);
+            for (int u = 0; u < U; ++u) {
+                float xf[8], wf[8];
+                unpack8(xv[u], xf);
+                unpack8(w[u], wf);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc = fmaf(xf[i], wf[i], acc);
             }
         }
+        acc = warp_sum(acc) + (q == warp ? b0 : bias[e]);
+        if (lane == 0) logit[q / E][e] = acc;
+    }
+    __syncthreads();
+    int i0 = 0, i1 = -1; float g0 = 0.f, g1 = 0.f;
+    if (threadIdx.x < mine) {
+        float acc[E];
 #pragma unroll
-        for (int e = 0; e < E; ++e) acc[e] = warp_sum(acc[e]) + bias[e];
+        for (int e = 0; e < E; ++e) acc[e] = logit[threadIdx.x][e];
         route_pick<E>(acc, topk, i0, i1, g0, g1);
     }
     __syncwarp();
     if (parts > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");         // (the first CTA is known to run)
-    if (m < M && lane == 0) {
+    if (threadIdx.x < mine) {
+        const uint32_t m = m0 + threadIdx.x;
         idx[2 * m] = i0; idx[2 * m + 1] = i1;
         gate[2 * m] = g0; gate[2 * m + 1] = g1;
         uint32_t ri, rg;
@@ -1289,7 +1310,7 @@ __global__ void __launch_bounds__(256) tgp_route_small_kernel(const bf16 *h, con
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (rank) return;
-    for (uint32_t e = warp; e < (uint32_t)E; e += 8) {
+    for (uint32_t e = warp; e < (uint32_t)E; e += ROUTE_WARPS) {
         uint32_t base = 0;
         for (uint32_t m0 = 0; m0 < M; m0 += 32) {
             const uint32_t t = m0 + lane;
@@ -1363,7 +1384,7 @@ int tgpk_router(const void *h, const void *Wr, const float *bias, int32_t *idx, 
     if (counts_host && !small) return TGP_E_INVAL;
     const uint32_t blocks = (M + 7) / 8;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks <= 2 ? blocks : blocks <= 4 ? 4 : 8); cfg.blockDim = dim3(256); cfg.stream = st;       // one cluster
+    cfg.gridDim = dim3(M <= 2 ? M : M <= 4 ? 4 : 8); cfg.blockDim = dim3(ROUTE_WARPS * 32); cfg.stream = st;        // one cluster
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;

@@ -545,6 +545,38 @@ def test_moe_decode_runs_all_experts_of_a_layer_together_with_the_same_bits(B, t
         check_logits([runs[0][0][0]], [ref[0]])
 
 
+@pytest.mark.parametrize("tokens,E,topk,d", [(1, 8, 2, 256), (2, 4, 2, 256), (3, 16, 2, 256), (9, 8, 1, 512), (17, 8, 2, 2304), (33, 16, 2, 256), (64, 4, 2, 512), (65, 8, 2, 256)])
+def test_router_counts_of_few_tokens(tokens, E, topk, d):
+    """Tokens per expert against the routing that 64-bit logits of the same normed states give: every size of the cluster, CTAs with several
+    tokens, one and none, more and fewer logits than warps, rows longer than the loads under way, and one token more than the cluster takes."""
+    cfg = replace(MOE, B=1, S=tokens, T=1, E=E, topk=topk, d=d, F=512, Hq=d // 64, Hkv=d // 128, Dh=64)
+    lay = si.build_layout(cfg, budget=256 << 20, cap=1 << 20)
+    pool = pinned_pool(lay.pool_bytes)
+    si.fill_pool(lay, pool.numpy())
+    bias = si.router_bias(cfg)
+    s = Session(lay, MACHINE, pool_base=pool.data_ptr(), pool_flags=tb.POOL_PINNED, router_bias=bias)
+    s.plan(expert_counts=np.ones((1 + cfg.T, cfg.L, cfg.E), dtype=np.uint32))
+    r = Runner(s, tokens)
+    tap = torch.zeros(128 << 20, dtype=torch.uint8, device="cuda:0")
+    ops = s.ctx.trace_ops()
+    r.reset()
+    s.ctx.set_tap(tap, tap.numel())
+    r.step(tb.PREFILL, si.prompt_tokens(cfg), tokens)
+    r.sync()
+    h = {ops[op][2]: tap[off:off + nbytes].view(torch.bfloat16).view(tokens, d).double().cpu()
+         for (op, tag, sub, off, nbytes) in s.ctx.tap_index().tolist() if tag == tb.TAP_H}          # the later of a layer's two: what the router reads
+    counts = s.ctx.expert_counts(cfg.L, E)[0]
+    for l in range(cfg.L):
+        t, = lay.blocks(si.K_ROUTER, l, -1)
+        logits = h[l] @ pool[t.pool_off:t.pool_off + E * d * 2].view(torch.bfloat16).view(E, d).double().T + torch.from_numpy(bias[l]).double()
+        top = logits.sort(dim=1, descending=True)
+        margin = (top.values[:, topk - 1] - top.values[:, topk]).min()
+        assert margin > 1e-5                               # (fp32 sums of d products: no pick hangs on their rounding)
+        assert counts[l].tolist() == torch.bincount(top.indices[:, :topk].reshape(-1), minlength=E).tolist()
+    s.ctx.set_tap(None, 0)
+    s.close()
+
+
 @pytest.mark.parametrize("B,F", [(3, 512), (5, 8192)])
 def test_experts_of_one_or_two_tokens_have_the_sums_of_the_products_of_one_row(B, F):
     """A step of 3 to 32 tokens: what an expert with one or two of them computes is, bit for bit, what k_gemm() and k_swiglu() give for
