@@ -1452,6 +1452,17 @@ static int g_gemv_balance = 1;   // grouped skinny launches: rows per group chos
 static int g_gemv_pdl = 1;       // consecutive weight-streaming launches may overlap (programmatic dependent launch)
 bool tgpk_launch_overlap() { return g_gemv_pdl != 0; }
 
+// Launches a kernel that streams weights through registers.  Its loads under way take up L1, 64 KB of them and more per SM, and a kernel without a
+// preference of its own runs on the split of L1 and shared memory that the SM has: next to nothing is left of L1 behind an attention or tcgen05
+// kernel that overlaps it (n=32000, K=4096 at 3 rows behind the products of a prefill: 68 us, 42 with half of it kept for
+// L1; a decode step of 8 users at d=4096 249 us, 233; a quarter or all of it for L1 is the same).
+template <auto KERNEL, typename... Args>
+static void launch_weights(const cudaLaunchConfig_t &cfg, Args... args) {
+    static const cudaError_t hint = cudaFuncSetAttribute(KERNEL, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
+    (void)hint;
+    cudaLaunchKernelEx(&cfg, KERNEL, args...);
+}
+
 template <int MT, int R, int U>
 static void launch_gemv(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int acc, cudaStream_t st) {
     static int blocks_per_sm = 0, sms = 0;
@@ -1472,7 +1483,7 @@ static void launch_gemv(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, 
     attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, tgp_wstream_kernel<MT, R, U>, A, W, C, Mrows, n, K, ldc, col0, acc);
+    launch_weights<tgp_wstream_kernel<MT, R, U>>(cfg, A, W, C, Mrows, n, K, ldc, col0, acc);
     tgpk_last_gemm_kernel = "tgp_wstream_kernel";
 }
 
@@ -1844,20 +1855,20 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
     tgpk_last_gemm_kernel = !k.split ? "tgp_wstream_mma_kernel" : persistent ? "tgp_wstream_mma_group_kernel" : "tgp_wstream_mma_splitk_kernel";
     if (persistent) {
         if constexpr (NB == 1 && U == 8) {
-            if (per_cta == 2) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>, A, p, Mrows, total, K, acc, rpc, early);
-            else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 16, 16, 1>, A, p, Mrows, total, K, acc, rpc, early);
+            if (per_cta == 2) launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
+            else launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 1>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
         } else if constexpr (NB == 2) {
             if (per_cta == 2) {
                 constexpr size_t smem = 16 * 2 * NB * 4 * 32 * 4;      // the partial tiles of 16 warps, two row groups each
                 static bool attr_set = false;
                 if (!attr_set) { cudaFuncSetAttribute(tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); attr_set = true; }
                 cfg.dynamicSmemBytes = smem;
-                cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>, A, p, Mrows, total, K, acc, rpc, early);
-            } else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, 16, 16, 1>, A, p, Mrows, total, K, acc, rpc, early);
+                launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
+            } else launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 1>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
         }
     } else if constexpr (STREAMS) {
-        if (!k.split) cudaLaunchKernelEx(&cfg, tgp_wstream_mma_kernel<NB, U>, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);
-        else cudaLaunchKernelEx(&cfg, tgp_wstream_mma_splitk_kernel<NB, U, 8, 16>, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);
+        if (!k.split) launch_weights<tgp_wstream_mma_kernel<NB, U>>(cfg, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);
+        else launch_weights<tgp_wstream_mma_splitk_kernel<NB, U, 8, 16>>(cfg, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);
     }
 }
 
@@ -1886,7 +1897,7 @@ static void launch_gemv_splitk(const bf16 *A, const bf16 *W, float *C, uint32_t 
     attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, tgp_wstream_splitk_kernel<MT, RB, U>, A, W, C, Mrows, n, K, ldc, col0, acc);
+    launch_weights<tgp_wstream_splitk_kernel<MT, RB, U>>(cfg, A, W, C, Mrows, n, K, ldc, col0, acc);
     tgpk_last_gemm_kernel = "tgp_wstream_splitk_kernel";
 }
 
@@ -1926,7 +1937,7 @@ static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows,
     attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, tgp_wstream_group_kernel<MT, 8, FUSED>, A, p, Mrows, n_total, K, acc, src);
+    launch_weights<tgp_wstream_group_kernel<MT, 8, FUSED>>(cfg, A, p, Mrows, n_total, K, acc, src);
     tgpk_last_gemm_kernel = "tgp_wstream_group_kernel";
 }
 
@@ -2209,7 +2220,7 @@ static void launch_expert_rows(cudaLaunchConfig_t &cfg, const bf16 *A, const Gem
             if (!attr_set) { cudaFuncSetAttribute(tgp_wstream_mma_group_kernel<NB, U, NW, 16, RG, EXP_U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); attr_set = true; }
             cfg.dynamicSmemBytes = smem;
         }
-        cudaLaunchKernelEx(&cfg, tgp_wstream_mma_group_kernel<NB, U, NW, 16, RG, EXP_U>, A, p, me, groups, K, 0, rpc, 0);
+        launch_weights<tgp_wstream_mma_group_kernel<NB, U, NW, 16, RG, EXP_U>>(cfg, A, p, me, groups, K, 0, rpc, 0);
     };
     if constexpr (NB == 1 && NW == 16)
         if (RG == 2 || K > NW * 32 * EXP_U) return launch(std::integral_constant<int, 2 * EXP_U>());
@@ -2271,14 +2282,16 @@ int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *c
 
 template <bool GLU>
 static void launch_experts(const ExpertParts &p, uint32_t T, cudaStream_t st) {
-    const uint32_t sms = (uint32_t)device_sms();
-    if (expert_warps(p.K) == 8) {
-        if (T == 8) launch_pdl(tgp_expert_mma_kernel<1, 8, GLU>, dim3(2 * sms), dim3(256), 0, st, p);
-        else launch_pdl(tgp_expert_mma_kernel<2, 8, GLU>, dim3(2 * sms), dim3(256), 0, st, p);
-    } else {
-        if (T == 8) launch_pdl(tgp_expert_mma_kernel<1, 16, GLU>, dim3(sms), dim3(512), 0, st, p);
-        else launch_pdl(tgp_expert_mma_kernel<2, 16, GLU>, dim3(sms), dim3(512), 0, st, p);
-    }
+    const uint32_t warps = (uint32_t)expert_warps(p.K);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16 / warps * (uint32_t)device_sms()); cfg.blockDim = dim3(32 * warps); cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (warps == 8) { if (T == 8) launch_weights<tgp_expert_mma_kernel<1, 8, GLU>>(cfg, p); else launch_weights<tgp_expert_mma_kernel<2, 8, GLU>>(cfg, p); }
+    else { if (T == 8) launch_weights<tgp_expert_mma_kernel<1, 16, GLU>>(cfg, p); else launch_weights<tgp_expert_mma_kernel<2, 16, GLU>>(cfg, p); }
 }
 
 int tgpk_experts(const TgpExperts &x, cudaStream_t st) {
