@@ -914,11 +914,13 @@ __global__ void __launch_bounds__(DH) tgp_attn_decode_merge_kernel(AttnArgs a) {
 // tile has to spare, the third a product of its own.  Both are summed apart from the first and dropped where that sum is not
 // finite: an infinity in V makes their products NaN (0 x inf), and the first part alone says what the row becomes.
 // A CTA of four warps owns a contiguous range of
-// chunks of one (sequence, KV head); its warps take every fourth chunk, merge their four partials through shared memory
-// and write one (max, sum, unnormalised O) per query head and CTA to the scratch array tgp_attn_decode_merge_kernel reads.
+// chunks of one (sequence, KV head); its warps take every fourth chunk and merge their four partials through shared memory.  The CTAs of
+// one (sequence, KV head) are a cluster where they are few and merge theirs through distributed shared memory (one sequence of 32 heads over
+// 8 x 64, 400 keys: 4.6 -> 3.4 us); else each writes one (max, sum, unnormalised O) per query head to the scratch array
+// that tgp_attn_decode_merge_kernel reads.
 // Stage layout: row = key, 2*DH bytes, 16-byte chunk j of row r at chunk position j ^ (r & 7): conflict-free for the
 // ldmatrix reads (eight rows, same j) and for the cp.async writes.
-constexpr int DEC_STAGES = 3, DEC_WARPS = 4, DEC_KEYS = 16;
+constexpr int DEC_STAGES = 3, DEC_WARPS = 4, DEC_KEYS = 16, DEC_CLUSTER = 8;
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
@@ -935,7 +937,8 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
 }
 __device__ __forceinline__ float fast_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
-template <int DH, int G, bool SPLIT_P>
+// (CLUSTER is an instance of its own: what only clusters need makes the others 5 - 14 % slower)
+template <int DH, int G, bool SPLIT_P, bool CLUSTER>
 __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(AttnArgs a, uint32_t chunks_per_cta) {
     pdl_enter();
     extern __shared__ __align__(128) uint8_t dec_sm[];
@@ -1082,6 +1085,8 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
         for (int j = 0; j < DH / 8; ++j) { dst[2 + j * 8 + 2 * c] = o[j][0]; dst[2 + j * 8 + 2 * c + 1] = o[j][1]; }
     }
     __syncthreads();
+    constexpr uint32_t CLUSTER_AT = 16 * DH;                              // floats: behind the partial of warp 0, in stages nobody reads any more
+    static_assert(CLUSTER_AT >= G * (DH + 2) && CLUSTER_AT + G * (DH + 2) <= WSTRIDE, "the CTA's partial lies in warp 0's stages");
     for (uint32_t e = threadIdx.x; e < G * DH; e += blockDim.x) {
         const uint32_t g = e / DH, d = e % DH;
         float M = -INFINITY;
@@ -1095,14 +1100,50 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
             l += wgt * src[1];
             acc += wgt * src[2 + d];
         }
-        if (a.n_parts == 1) {                                              // the CTA saw the whole context: this is the result
+        if (!CLUSTER && a.n_parts == 1) {                                  // the CTA saw the whole context: this is the result
             a.ob[((size_t)b * a.Hq + hk * G + g) * DH + d] = __float2bfloat16_rn(acc / l);
+            continue;
+        }
+        if constexpr (CLUSTER) {
+            float *cp = wp + CLUSTER_AT + (size_t)g * (DH + 2);
+            if (d == 0) { cp[0] = M; cp[1] = l; }
+            cp[2 + d] = acc;
             continue;
         }
         float *out = a.scratch + ((size_t)(b * a.Hq + hk * G + g) * a.n_tiles + part) * (DH + 2);
         if (d == 0) { out[0] = M * 0.6931471805599453f; out[1] = l; }      // the merge kernel works in natural-log units
         out[2 + d] = acc;
     }
+    if constexpr (!CLUSTER) return;
+    // The CTAs of a cluster are the parts of one sequence and KV head: every CTA takes a share of the outputs and reads all partials of it.
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const uint32_t cp_u = (uint32_t)__cvta_generic_to_shared(wp + CLUSTER_AT), rank = part, ctas = gridDim.x;
+    auto remote = [&](uint32_t part_at, uint32_t offset) {
+        uint32_t at;
+        float v;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(cp_u + offset * 4), "r"(part_at));
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+        return v;
+    };
+    for (uint32_t e = G * DH * rank / ctas + threadIdx.x; e < G * DH * (rank + 1) / ctas; e += blockDim.x) {
+        const uint32_t g = e / DH, d = e % DH;
+        float m[DEC_CLUSTER], l[DEC_CLUSTER], o_p[DEC_CLUSTER], M = -INFINITY;
+#pragma unroll
+        for (uint32_t q = 0; q < DEC_CLUSTER; ++q)
+            if (q < ctas) { m[q] = remote(q, g * (DH + 2)); l[q] = remote(q, g * (DH + 2) + 1); o_p[q] = remote(q, g * (DH + 2) + 2 + d); }
+#pragma unroll
+        for (uint32_t q = 0; q < DEC_CLUSTER; ++q) if (q < ctas) M = fmaxf(M, m[q]);
+        float lsum = 0.f, acc = 0.f;
+#pragma unroll
+        for (uint32_t q = 0; q < DEC_CLUSTER; ++q)
+            if (q < ctas) { const float w = fast_ex2(m[q] - M); lsum += w * l[q]; acc += w * o_p[q]; }
+        a.ob[((size_t)b * a.Hq + hk * G + g) * DH + d] = __float2bfloat16_rn(acc / lsum);
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");        // no CTA leaves while another may still read its partial
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // ---- SwiGLU -----------------------------------------------------------------------------------------
@@ -2468,27 +2509,45 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
             if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
             const uint32_t units = B * c->Hkv, per_sm = c->Dh == 64 ? 4 : 2;             // CTAs that fit an SM (96 / 48 KB of shared memory each)
             uint32_t parts = (uint32_t)sms * per_sm / units;                              // CTAs per (sequence, KV head): one wave at most
-            parts = std::max(1u, std::min(parts, std::min(n_tiles, (nchunks + DEC_WARPS - 1) / DEC_WARPS)));
+            // Up to DEC_CLUSTER parts can be a cluster, which merges them itself; more parts meet in the scratch array and a second kernel.
+            // Up to four parts always are one.  A context that would have more is worth eight where it is short or its clusters are few: eight
+            // CTAs need one GPC to hold them, and 32 such clusters wait for one another in a step, though not back to back (eight parts against
+            // all, us: 32 heads over 8 x 64, B=1, 700 keys 3.7 / 5.2, 2112 keys 5.3 / 8.8, 4000 6.8 / 6.9, 9000 11.8 / 10.6; x 128, 2112 keys
+            // 7.1 / 9.5, 4000 9.5 / 8.3; a step of two layers, B=4, 16000 keys 356 / 321)
+            parts = std::max(1u, std::min(parts, (nchunks + DEC_WARPS - 1) / DEC_WARPS));
+            // (the scratch array holds a partial per KV tile: where that is four or fewer, a cluster of four is at least as many)
+            const bool eight = nchunks <= 64 || (units <= 16 && (nchunks <= 192 || n_tiles <= DEC_CLUSTER)), clustered = eight || parts <= 4 || n_tiles <= 4;
+            parts = std::min(parts, eight ? (uint32_t)DEC_CLUSTER : clustered ? 4u : n_tiles);
             const uint32_t per_cta = (nchunks + parts - 1) / parts;
             parts = (nchunks + per_cta - 1) / per_cta;                                    // no CTA without a chunk
+            const bool cluster = clustered && parts > 1, merge = !clustered && parts > 1;
             a.n_parts = parts;
             // below 256 chunks in all the kernel is bound by latency and takes no longer with all of P (1183 shapes of 1 - 4000 keys: 3.4 us
             // on average, 3.4 with two parts, 7.8 on the CUDA cores; results that are not the rounded exact value: 1 in 7750, 1 in 720, 1 in 7500)
             const bool split_p = nchunks * B * c->Hkv < 256;
             const size_t smem = (size_t)DEC_WARPS * DEC_STAGES * 2 * DEC_KEYS * c->Dh * 2;        // 96 KB at Dh = 128, 48 KB at 64
-            dim3 g2(parts, c->Hkv, B);
-#define TGP_DECODE_MMA_P(DH_, G_, SP_) do { \
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(parts, c->Hkv, B); cfg.blockDim = dim3(DEC_WARPS * 32); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+            cudaLaunchAttribute attr[2];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;
+            attr[1].id = cudaLaunchAttributeClusterDimension;
+            attr[1].val.clusterDim.x = parts; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = cluster ? 2 : 1;
+#define TGP_DECODE_MMA_P(DH_, G_, SP_, CL_) do { \
                 static bool attr_set = false; \
-                if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_decode_mma_kernel<DH_, G_, SP_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TGP_E_CUDA; attr_set = true; } \
-                launch_pdl(tgp_attn_decode_mma_kernel<DH_, G_, SP_>, g2, dim3(DEC_WARPS * 32), smem, st, a, per_cta); } while (0)
-#define TGP_DECODE_MMA(DH_, G_) do { if (split_p) TGP_DECODE_MMA_P(DH_, G_, true); else TGP_DECODE_MMA_P(DH_, G_, false); } while (0)
+                if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_decode_mma_kernel<DH_, G_, SP_, CL_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TGP_E_CUDA; attr_set = true; } \
+                cudaLaunchKernelEx(&cfg, tgp_attn_decode_mma_kernel<DH_, G_, SP_, CL_>, a, per_cta); } while (0)
+#define TGP_DECODE_MMA(DH_, G_) do { if (cluster) { if (split_p) TGP_DECODE_MMA_P(DH_, G_, true, true); else TGP_DECODE_MMA_P(DH_, G_, false, true); } \
+                else { if (split_p) TGP_DECODE_MMA_P(DH_, G_, true, false); else TGP_DECODE_MMA_P(DH_, G_, false, false); } } while (0)
 #define TGP_DECODE_MMA_G(DH_) do { if (G == 1) TGP_DECODE_MMA(DH_, 1); else if (G == 2) TGP_DECODE_MMA(DH_, 2); else if (G == 4) TGP_DECODE_MMA(DH_, 4); else TGP_DECODE_MMA(DH_, 8); } while (0)
-            if (c->Dh == 64) { TGP_DECODE_MMA_G(64); if (parts > 1) launch_pdl(tgp_attn_decode_merge_kernel<64>, dim3(c->Hq, B), dim3(64), 0, st, a); }
-            else { TGP_DECODE_MMA_G(128); if (parts > 1) launch_pdl(tgp_attn_decode_merge_kernel<128>, dim3(c->Hq, B), dim3(128), 0, st, a); }
+            if (c->Dh == 64) { TGP_DECODE_MMA_G(64); if (merge) launch_pdl(tgp_attn_decode_merge_kernel<64>, dim3(c->Hq, B), dim3(64), 0, st, a); }
+            else { TGP_DECODE_MMA_G(128); if (merge) launch_pdl(tgp_attn_decode_merge_kernel<128>, dim3(c->Hq, B), dim3(128), 0, st, a); }
 #undef TGP_DECODE_MMA_G
 #undef TGP_DECODE_MMA
 #undef TGP_DECODE_MMA_P
-            LAUNCH_CHECK(parts > 1 ? 2 : 1);
+            LAUNCH_CHECK(merge ? 2 : 1);
             return TGP_OK;
         }
         if (grouped) {                                      // K and V read once for the whole group of query heads

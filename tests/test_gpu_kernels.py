@@ -529,6 +529,30 @@ def test_tensor_core_decode_attention_matches_oracle_and_cuda_core_kernel(Dh, Hq
         assert np.mean(np.abs(got - bf16_round(att))) < 3e-3 * np.abs(att).mean(), impl
 
 
+# parts of a context in a cluster or through the scratch array: the last length that eight parts take and the first that more do, few KV tiles (one
+# and two, which the scratch array would limit; five), numbers of parts that are not a power of two, eight query heads per KV head
+@pytest.mark.parametrize("Dh,Hq,Hkv,TK,kvlen,B,launches", [(64, 4, 4, 64, 3072, 1, 1), (64, 4, 4, 64, 3073, 1, 2), (128, 8, 1, 1024, 5000, 1, 1), (128, 32, 8, 256, 4000, 4, 2),
+                                                           (64, 8, 8, 64, 330, 2, 1), (128, 64, 8, 64, 900, 4, 1), (128, 16, 8, 64, 3100, 2, 2), (128, 8, 8, 64, 1500, 8, 1),
+                                                           (128, 32, 8, 2048, 4000, 4, 1), (64, 40, 40, 4096, 1100, 2, 1), (128, 32, 8, 800, 4000, 4, 2)])
+def test_parts_of_a_decode_context_in_clusters_and_in_the_scratch_array(Dh, Hq, Hkv, TK, kvlen, B, launches):
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=kvlen, T=0, B=B, d=Hq * Dh)
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(kvlen + B)
+    n = (kvlen + TK - 1) // TK
+    kt, vt = ([torch.randn((B * Hkv * TK, Dh), device=DEV, generator=gen).bfloat16() for _ in range(n)] for _ in range(2))
+    q = torch.randn((B, Hq * Dh), device=DEV, generator=gen).bfloat16()
+    scratch = torch.full((tb.k_attn_scratch_bytes(model_cfg(cfg)) // 4,), 7.0, device=DEV)
+    ob = torch.full((B, Hq * Dh), float("nan"), dtype=torch.bfloat16, device=DEV)
+    tb.k_attn(q, kt, vt, ob, model_cfg(cfg), B, 1, kvlen - 1, scratch)
+    torch.cuda.synchronize()
+    assert bool((scratch == 7.0).all()) == (launches == 1)         # parts of a cluster do not touch it
+    K, V = (torch.stack([t.view(B, Hkv, TK, Dh) for t in ts], dim=2).reshape(B, Hkv, n * TK, Dh)[:, :, :kvlen].double().repeat_interleave(Hq // Hkv, dim=1) for ts in (kt, vt))
+    want = (torch.softmax(q.double().view(B, Hq, 1, Dh) @ K.transpose(-1, -2) / Dh ** 0.5, -1) @ V).reshape(B, Hq * Dh)
+    # half a bf16 step of the output and of each of the probabilities, whose roundings average out: 2^-9 of the largest V, as in the tests above
+    assert float((ob.double() - want).abs().max()) < 2.0 ** -7 * float(want.abs().max()) + 1e-6
+    assert float((ob.double() - want).abs().mean()) < 5e-3 * float(want.abs().mean())
+
+
 def test_attention_single_key_returns_v():
     cfg = replace(KCFG, B=1, S=1, T=0)
     mc = model_cfg(cfg)
