@@ -457,3 +457,28 @@ def test_products_of_9_to_16_rows_take_the_tcgen05_kernel_only_where_it_is_ahead
     """K not a multiple of 32 stays with the CUDA cores (key 0, launched alone), whose sums are closer to 64 bits; K below 1536 on fewer
     tiles of 128 rows than SMs (148) with the split-K kernel, which is faster."""
     assert tb.k_gemm_group_key(M, n, K) >> 24 == family
+
+
+def test_addresses_of_every_kind_of_argument_alone_and_in_arrays():
+    import torch
+
+    class Stream:
+        cuda_stream = 77
+
+    class Holder:
+        def __init__(self, **kw):
+            self.__dict__.update(kw)
+
+    a, t = np.arange(12, dtype=np.float32), torch.zeros(5)
+    cases = [(None, None), (4096, 4096), (True, True), (a, a.ctypes.data), (a[3:], a.ctypes.data + 12), (t, t.data_ptr()), (t[2:], t.data_ptr() + 8),
+             (torch.nn.Parameter(t), t.data_ptr()), (Stream(), 77), (Holder(cuda_stream=5), 5), (Holder(data_ptr=lambda: 9, cuda_stream=5), 9), (Holder(cuda_stream=6), 6)]
+    for _ in range(2):                                     # the first use of a type and the next
+        for x, want in cases:
+            assert tb._ptr(x) == want
+    for bad in ("x", 1.5, Holder(), [1]):
+        for _ in range(2):
+            with pytest.raises(TypeError):
+                tb._ptr(bad)
+    assert [v for v in tb._pointers([x for x, _ in cases])] == [w if w is None else int(w) for _, w in cases]
+    assert list(tb._pointers([t[1:], t])) == [t.data_ptr() + 4, t.data_ptr()] and len(tb._pointers([])) == 1
+    assert list(tb._pointers((Holder(cuda_stream=3), Holder(data_ptr=lambda: 4)))) == [3, 4]
