@@ -1942,18 +1942,25 @@ static void launch_gemv_splitk(const bf16 *A, const bf16 *W, float *C, uint32_t 
     tgpk_last_gemm_kernel = "tgp_wstream_splitk_kernel";
 }
 
+// From this many rows on a block of one or two activation rows gives every SM two rows for each of its warps.
+constexpr uint32_t GEMV_MANY_ROWS = 2 * 148 * 16;
+
+// One activation row on a block of many rows whose K is two to four times the 2048 columns of eight load steps: a row per warp with all eight under
+// way is ahead of two rows with four each (n=14336, K=4096 18.3 us against 19.7, n=32000, K=8192 76 / 81; with K=1024 25 / 16, K=28672 78 / 72).
+static bool one_row_deep(uint32_t M, uint32_t K) { return M == 1 && K % 2048 == 0 && K >= 4096 && K <= 8192; }
+
 // rows per warp: fewer when the block has few rows, so that every SM still gets warps
 template <int MT>
 static void launch_gemv_rows(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int acc, cudaStream_t st) {
     if constexpr (MT <= 2) {
-        if (n >= 2 * 148 * 16) return launch_gemv<MT, 2, 4>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
-        if (g_gemv_splitk && K >= 8192) {                    // at least four 256-element chunks per warp and row
+        if (n >= GEMV_MANY_ROWS && !one_row_deep(MT, K)) return launch_gemv<MT, 2, 4>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
+        if (n < GEMV_MANY_ROWS && g_gemv_splitk && K >= 8192) {                    // at least four 256-element chunks per warp and row
             if (n <= 1024) return launch_gemv_splitk<MT, 1, 4>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
             return launch_gemv_splitk<MT, 2, 4>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
         }
         return launch_gemv<MT, 1, 8>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
     } else {
-        if (n >= 2 * 148 * 16) return launch_gemv<MT, 2, 2>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
+        if (n >= GEMV_MANY_ROWS) return launch_gemv<MT, 2, 2>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
         return launch_gemv<MT, 1, 4>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
     }
 }
@@ -2364,12 +2371,15 @@ int tgpk_experts(const TgpExperts &x, cudaStream_t st) {
 }
 
 // Which products may share a launch: those with the same non-zero key.  A key names the kernel a block takes on its own
-// (M <= 2: tgp_wstream_kernel<MT, 1, 8>; 3 <= M <= 32: one instance of the persistent list kernel, or the tcgen05 kernel and
+// (M <= 2: tgp_wstream_kernel<MT, 1, 8>, or a kernel with its sums; 3 <= M <= 32: one instance of the persistent list kernel, or the tcgen05 kernel and
 // split of K); blocks of so many rows that they fill the machine alone, and the shapes served by other kernels, have key 0 and
 // are launched alone.
 uint32_t tgpk_gemm_group_key(uint32_t M, uint32_t n, uint32_t K) {
     if (!g_gemm_group || !M || !n || !K || K % 8) return 0;
-    if (M <= 2) return (n < 2 * 148 * 16 && !(g_gemv_splitk && K >= 8192)) ? M : 0;
+    // Blocks of many rows at M <= 2 run one behind the other at little cost, but a list of them has one ramp instead of several: 2 x 14336, K=4096 at
+    // one row 39.0 -> 34.9 us; at two rows 2 x 8192, K=2048 18.0 / 15.4, 3 x 8192, K=8192 87 / 72, while 2 x 14336 are even and 2 x 28672 slower (145 / 161)
+    if (M <= 2 && n >= GEMV_MANY_ROWS) return one_row_deep(M, K) || (M == 2 && n <= 8704) ? 0x100u | M : 0;
+    if (M <= 2) return !(g_gemv_splitk && K >= 8192) ? M : 0;
     if (M > 32) return 0;
     if (takes_tiles(M, n, K)) return tgpk_gemm_tc_forced() ? 0 : 0x2000000u | tgpk_gemm_tc_class(M, n, K);
     if (M > 16 || K % 32 || g_skinny_impl) return 0;

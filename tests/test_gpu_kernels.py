@@ -756,6 +756,30 @@ def test_blocks_of_many_rows_take_the_list_kernel_with_the_same_bits_alone_and_i
         assert float((a.double() - want).abs().max()) < 2e-5 * float(want.abs().max())
 
 
+# one and two rows on blocks of many rows, on either side of what is listed (K of two to four times 2048 columns at one row, up to 8704 weight rows at two)
+@pytest.mark.parametrize("M,ns,K,listed", [(1, (4736, 5001), 4096, True), (1, (9000, 4737), 8192, True), (1, (4800, 4736), 6144, True), (1, (5000, 4736), 4104, False),
+                                           (1, (5000, 4736), 10240, False), (2, (8704, 4736, 8192), 520, True), (2, (4740, 8705), 264, False), (2, (4736, 4736), 8192, True)])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_blocks_of_many_rows_at_one_and_two_activation_rows(M, ns, K, listed, accumulate):
+    keys = {tb.k_gemm_group_key(M, n, K) for n in ns}
+    assert (len(keys) == 1 and 0 not in keys) == listed
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(M * K + len(ns))
+    A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
+    Ws = [(torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16() for n in ns]
+    c0 = [torch.randn((M, n + 4), device=DEV, generator=gen) for n in ns]
+    alone, listed_c = [c.clone() for c in c0], [c.clone() for c in c0]
+    for W, C, n in zip(Ws, alone, ns):
+        tb.k_gemm(A, W, C, M, n, K, n + 4, 0, accumulate)
+    tb.k_gemm_group(A, Ws, listed_c, M, list(ns), K, [n + 4 for n in ns], accumulate)
+    torch.cuda.synchronize()
+    for W, a, b, c, n in zip(Ws, alone, listed_c, c0, ns):
+        assert torch.equal(a, b) and torch.equal(a[:, n:], c[:, n:])
+        want = A.double() @ W.double().T + (c[:, :n].double() if accumulate else 0)
+        # lane-strided fp32 sums of K products: a few 2^-24 of the partial sums' size, as in the tests below
+        assert float((a[:, :n].double() - want).abs().max()) < 2e-5 * float(want.abs().max())
+
+
 # the list kernel at 9 - 16 rows around a chunk of 16 warps x 128 columns (one column block, a warp's chunk more or less, many chunks), ragged
 # row groups, one and two row groups per CTA; and lists of which only neighbours share a kernel
 @pytest.mark.parametrize("M,ns,K", [(9, (1, 17), 32), (16, (1024, 1000), 1024), (12, (300,), 2016), (16, (2048, 4100), 2048), (11, (33, 640), 2080), (16, (500,), 14368),
