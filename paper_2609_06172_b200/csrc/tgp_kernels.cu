@@ -2377,8 +2377,9 @@ int tgpk_experts(const TgpExperts &x, cudaStream_t st) {
 uint32_t tgpk_gemm_group_key(uint32_t M, uint32_t n, uint32_t K) {
     if (!g_gemm_group || !M || !n || !K || K % 8) return 0;
     // Blocks of many rows at M <= 2 run one behind the other at little cost, but a list of them has one ramp instead of several: 2 x 14336, K=4096 at
-    // one row 39.0 -> 34.9 us; at two rows 2 x 8192, K=2048 18.0 / 15.4, 3 x 8192, K=8192 87 / 72, while 2 x 14336 are even and 2 x 28672 slower (145 / 161)
-    if (M <= 2 && n >= GEMV_MANY_ROWS) return one_row_deep(M, K) || (M == 2 && n <= 8704) ? 0x100u | M : 0;
+    // one row 39.0 -> 34.9 us; at two rows 2 x 8192, K=2048 18.0 / 15.4, 3 x 8192, K=8192 87 / 72, while 2 x 14336 are even and 2 x 28672 slower (145 / 161).
+    // (a K that is no multiple of the 2048 columns of its eight load steps leaves them partly empty: a step of 2 users at d=2560 93 / 98)
+    if (M <= 2 && n >= GEMV_MANY_ROWS) return one_row_deep(M, K) || (M == 2 && n <= 8704 && K % 2048 == 0) ? 0x100u | M : 0;
     if (M <= 2) return !(g_gemv_splitk && K >= 8192) ? M : 0;
     if (M > 32) return 0;
     if (takes_tiles(M, n, K)) return tgpk_gemm_tc_forced() ? 0 : 0x2000000u | tgpk_gemm_tc_class(M, n, K);

@@ -756,9 +756,10 @@ def test_blocks_of_many_rows_take_the_list_kernel_with_the_same_bits_alone_and_i
         assert float((a.double() - want).abs().max()) < 2e-5 * float(want.abs().max())
 
 
-# one and two rows on blocks of many rows, on either side of what is listed (K of two to four times 2048 columns at one row, up to 8704 weight rows at two)
+# one and two rows on blocks of many rows, on either side of what is listed (K of two to four times 2048 columns at one row, up to 8704 weight rows and K a multiple of 2048 at two)
 @pytest.mark.parametrize("M,ns,K,listed", [(1, (4736, 5001), 4096, True), (1, (9000, 4737), 8192, True), (1, (4800, 4736), 6144, True), (1, (5000, 4736), 4104, False),
-                                           (1, (5000, 4736), 10240, False), (2, (8704, 4736, 8192), 520, True), (2, (4740, 8705), 264, False), (2, (4736, 4736), 8192, True)])
+                                           (1, (5000, 4736), 10240, False), (2, (8704, 4736, 8192), 2048, True), (2, (4740, 8705), 2048, False), (2, (8704, 4736), 520, False),
+                                           (2, (4736, 4736), 8192, True)])
 @pytest.mark.parametrize("accumulate", [False, True])
 def test_blocks_of_many_rows_at_one_and_two_activation_rows(M, ns, K, listed, accumulate):
     keys = {tb.k_gemm_group_key(M, n, K) for n in ns}
