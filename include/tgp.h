@@ -342,8 +342,9 @@ int  tgp_k_gemm_select(int impl);
 int  tgp_k_skinny_select(int impl);
 /* Products, attention and the small kernels of a step (embedding gather, RMSNorm, RoPE + KV append, SwiGLU, argmax, router and
  * experts of a small step) use programmatic dependent launch: a launch lets its successor be scheduled at once; a
- * weight-streaming kernel of up to 16 rows starts reading its weights while the previous kernel of the stream drains and
- * waits for it only before it touches activations or output, every other kernel waits before it reads anything, so that
+ * weight-streaming kernel of up to 16 rows, and the router of up to 64 tokens, starts reading its weights while the previous
+ * kernel of the stream drains and waits for it only before it touches activations or output; the product of one weight tile per CTA
+ * asks L2 for its first weights then, which reads nothing; every other kernel waits before it reads anything, so that
  * only its launch latency and set-up overlap.  0 switches that off (each launch then starts after the previous one has completed).  Results are
  * identical either way.  Process-wide; default on. */
 int  tgp_k_gemv_overlap(int enable);

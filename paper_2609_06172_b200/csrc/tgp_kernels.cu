@@ -1786,8 +1786,8 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
 struct SkinnyPick { int nb, u, nw, rows; bool split, persistent; };
 
 // 9 - 16 activation rows on a block of at least this many weight rows (64 tiles of 128): the tcgen05 kernel is ahead of the
-// mma.sync ones (M=16: n=28672, K=8192 76 us against 85 us; two blocks of 8192 rows, K=2048 15 us against 22 us; n=32000, K=4096
-// 46 us either way; below, n=4096, K=4096: 11.3 us against 8.4 us).  From 17 rows on it is ahead on blocks of any size (M=32:
+// mma.sync ones (M=16, from the end of the norm before: two blocks of 28672 rows, K=8192 144 us against 160; two of 8192 rows, K=2048 14.8 / 15.8;
+// n=32000, K=4096 43.2 / 48.3; below, n=4096, K=4096 about 11 against 9.7).  From 17 rows on it is ahead on blocks of any size (M=32:
 // n=6144 in three blocks, K=4096 14.7 us against 18.4 us; n=4096, K=14336 24 us against 35 us).
 constexpr uint32_t TILES_WIN_ROWS = 8065;
 
@@ -1810,9 +1810,9 @@ static SkinnyPick pick_skinny(uint32_t M, uint32_t n, uint32_t K) {
     k.nb = M <= 8 ? 1 : 2;
     k.split = n < 16u * 8u * sms;                         // too few 16-row groups to give every SM eight warps
     // One persistent CTA per SM walks the row groups of the block, or of a list of such blocks (tgp_wstream_mma_group_kernel).
-    // It is bound by HBM: its loads never drain between row groups (n=14336, K=4096: 18.5 us = 6.36 TB/s at M=8, 23.2 us at
-    // M=16; one CTA per row group took 22.7 and 31.6 us.  n=32000, K=4096, M=8: 40.1 us against 55.3 us of one warp per 16
-    // rows).  Its warps share K in chunks of 4096 columns, so a short K leaves most of them without work: with two or more
+    // It is bound by HBM: its loads never drain between row groups (n=14336, K=4096: 18.5 us = 6.36 TB/s at M=8;
+    // one CTA per row group took 22.7 us.  n=32000, K=4096, M=8: 40.1 us against 55.3 us of one warp per 16
+    // rows).  Its warps share K in chunks of 4096 columns (2048 above 8 rows), so a short K leaves most of them without work: with two or more
     // row groups per SM it is taken from K=3072 on at M <= 8 (K=2048: ahead from five row groups per SM on - n=32000: 23.1 us
     // against 29.5 us, n=6144: 6.3 us against 5.6 us) and from K=4096 on at M <= 16 (K=2048, M=16, n=12288: 15.1 us against 11.5 us).
     // One choice per class of M for all of them, so that the pieces of a matrix share a launch whatever the rows of its
