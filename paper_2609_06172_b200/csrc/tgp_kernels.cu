@@ -2,6 +2,7 @@
 // Precision contract: bf16 weights / KV / GEMM inputs, fp32 accumulation and residual stream.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <cfloat>
 #include <cstdint>
 #include <type_traits>
 #include <algorithm>
@@ -991,7 +992,9 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
         o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
         if constexpr (SPLIT_P) o3[j][0] = o3[j][1] = o3[j][2] = o3[j][3] = 0.f;
     }
-    float m_run = -INFINITY, l_run = 0.f;                             // of row r (replicated over the four lanes of the row)
+    // The maximum starts at the least number, not at -inf: keys of score -inf weigh nothing then (ex2(-inf - it) = 0) wherever a warp's chunks
+    // begin, while from -inf the first of them would be ex2(-inf + inf) = NaN, and which keys those are depends on the number of parts
+    float m_run = -FLT_MAX, l_run = 0.f;                              // of row r (replicated over the four lanes of the row)
     for (uint32_t it = 0; it < total; ++it) {
         if (issued < total) { issue(q_lo + warp + issued * DEC_WARPS, issued % DEC_STAGES); ++issued; }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -1023,9 +1026,9 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
         float mx = fmaxf(fmaxf(sv[0], sv[1]), fmaxf(sv[2], sv[3]));
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float m_new = fmaxf(m_run, mx);                          // finite: every chunk holds a valid key
+        const float m_new = fmaxf(m_run, mx);
         if (__any_sync(0xffffffffu, m_new > m_run)) {
-            const float alpha = fast_ex2(m_run - m_new);              // first chunk: ex2(-inf) = 0 on zeros
+            const float alpha = fast_ex2(m_run - m_new);              // first chunk: on zeros
             l_run *= alpha;
 #pragma unroll
             for (int j = 0; j < DH / 8; ++j) {
@@ -1079,8 +1082,8 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
     float *wp = reinterpret_cast<float *>(dec_sm);
     if (r < G) {
         float *dst = wp + (size_t)warp * WSTRIDE + (size_t)r * (DH + 2);
-        // (a warp whose scores were all NaN or -inf: its maximum is NaN, not that of a warp without a chunk, so that the row becomes NaN)
-        if (c == 0) { dst[0] = total && m_run == -INFINITY ? __int_as_float(0x7fffffff) : m_run; dst[1] = l_run; }
+        // (NaN scores: the sum is NaN and makes the row NaN with any weight; a row of nothing but -inf: 0 / 0)
+        if (c == 0) { dst[0] = m_run; dst[1] = l_run; }
 #pragma unroll
         for (int j = 0; j < DH / 8; ++j) { dst[2 + j * 8 + 2 * c] = o[j][0]; dst[2 + j * 8 + 2 * c + 1] = o[j][1]; }
     }
@@ -1089,14 +1092,14 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
     static_assert(CLUSTER_AT >= G * (DH + 2) && CLUSTER_AT + G * (DH + 2) <= WSTRIDE, "the CTA's partial lies in warp 0's stages");
     for (uint32_t e = threadIdx.x; e < G * DH; e += blockDim.x) {
         const uint32_t g = e / DH, d = e % DH;
-        float M = -INFINITY;
+        float M = -FLT_MAX;
 #pragma unroll
         for (int w = 0; w < DEC_WARPS; ++w) M = fmaxf(M, wp[(size_t)w * WSTRIDE + (size_t)g * (DH + 2)]);
         float l = 0.f, acc = 0.f;
 #pragma unroll
         for (int w = 0; w < DEC_WARPS; ++w) {
             const float *src = wp + (size_t)w * WSTRIDE + (size_t)g * (DH + 2);
-            const float wgt = src[0] == -INFINITY ? 0.f : fast_ex2(src[0] - M);       // a warp without a chunk: weight 0
+            const float wgt = fast_ex2(src[0] - M);                        // (a warp without a chunk: any weight of zeros)
             l += wgt * src[1];
             acc += wgt * src[2 + d];
         }
@@ -1129,7 +1132,7 @@ __global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(Att
     };
     for (uint32_t e = G * DH * rank / ctas + threadIdx.x; e < G * DH * (rank + 1) / ctas; e += blockDim.x) {
         const uint32_t g = e / DH, d = e % DH;
-        float m[DEC_CLUSTER], l[DEC_CLUSTER], o_p[DEC_CLUSTER], M = -INFINITY;
+        float m[DEC_CLUSTER], l[DEC_CLUSTER], o_p[DEC_CLUSTER], M = -FLT_MAX;
 #pragma unroll
         for (uint32_t q = 0; q < DEC_CLUSTER; ++q)
             if (q < ctas) { m[q] = remote(q, g * (DH + 2)); l[q] = remote(q, g * (DH + 2) + 1); o_p[q] = remote(q, g * (DH + 2) + 2 + d); }

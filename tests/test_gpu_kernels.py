@@ -1016,6 +1016,46 @@ def test_decode_attention_of_short_contexts_with_infinities_and_nan(Dh, G, kvlen
     assert o.float().view(Hkv, G, Dh)[1].isnan().all()
 
 
+# one part, clusters with and without all bits of P, the scratch array; keys that begin a warp's chunks in one of the splits and not in another
+@pytest.mark.parametrize("Dh,Hq,Hkv,TK,kvlen,B", [(64, 8, 8, 4096, 400, 1), (64, 4, 4, 64, 64, 1), (64, 32, 8, 128, 700, 1), (128, 32, 8, 1024, 1000, 1),
+                                                  (128, 8, 1, 256, 3000, 2), (128, 32, 8, 256, 4000, 4), (64, 16, 2, 64, 40, 2)])
+def test_decode_attention_with_keys_of_score_minus_infinity(Dh, Hq, Hkv, TK, kvlen, B):
+    """Keys whose scores are -inf (an infinity in K against a negative query) weigh nothing, wherever they lie; a row of nothing else, or with
+    one NaN score, is NaN; an infinity in V reaches the result as it is.  As 64 bits have it."""
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=kvlen, T=0, B=B, d=Hq * Dh)
+    mc, G, n = model_cfg(cfg), Hq // Hkv, (kvlen + TK - 1) // TK
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(kvlen)
+    K, V = (torch.zeros((n * TK, B, Hkv, Dh), device=DEV, dtype=torch.bfloat16) for _ in range(2))
+    K[:kvlen], V[:kvlen] = (torch.randn((kvlen, B, Hkv, Dh), device=DEV, generator=gen).bfloat16() for _ in range(2))
+    q = torch.randn((B, Hq, Dh), device=DEV, generator=gen).bfloat16()
+    q[:, :, 0] = -1
+    scratch = torch.zeros(tb.k_attn_scratch_bytes(mc) // 4, device=DEV)
+
+    def check(K, V):
+        kt, vt = ([t.permute(1, 2, 0, 3).contiguous() for t in T.split(TK)] for T in (K, V))
+        ob = torch.zeros((B, Hq, Dh), device=DEV, dtype=torch.bfloat16)
+        tb.k_attn(q, kt, vt, ob, mc, B, 1, kvlen - 1, scratch)
+        k64, v64 = (T[:kvlen].permute(1, 2, 0, 3).double() for T in (K, V))
+        want = (torch.softmax(q.double().view(B, Hkv, G, Dh) @ k64.transpose(-1, -2) / Dh ** 0.5, -1) @ v64).view(B, Hq, Dh)
+        got, fin = ob.double(), want.isfinite()
+        assert torch.equal(got.isfinite(), fin) and torch.equal(got[~fin].nan_to_num(0.0), want[~fin].nan_to_num(0.0))
+        # half a bf16 step of the output and of each of the probabilities, whose roundings average out: 2^-9 of the largest V, as in the tests above
+        assert not fin.any() or float((got - want)[fin].abs().max()) < 2.0 ** -7 * float(want[fin].abs().max()) + 1e-6
+
+    for lo, hi in [(0, 16), (16, 32), (0, 32), (64, 80), (kvlen // 32 * 16, kvlen // 32 * 16 + 16), (128, 256), ((kvlen - 1) // 16 * 16, kvlen), (1, kvlen), (0, kvlen)]:
+        if lo < kvlen:
+            Ki = K.clone()
+            Ki[lo:min(hi, kvlen), :, :, 0] = float("inf")
+            check(Ki, V)
+    for key in (0, kvlen // 2, kvlen - 1):
+        Kn, Vi = K.clone(), V.clone()
+        Kn[key, B - 1, Hkv - 1] = float("nan")
+        check(Kn, V)
+        Vi[key, 0, 0, 5], Vi[key, 0, 0, 6] = float("inf"), float("-inf")
+        check(K, Vi)
+
+
 @pytest.mark.parametrize("Dh,S,pos0", [(64, 16, 0), (64, 40, 20), (128, 33, 0), (128, 17, 47)])
 def test_attention_of_short_prompts_with_infinities_in_v(Dh, S, pos0):
     """Up to 64 keys what the rounding of P leaves over is multiplied with V too; an infinity in V still reaches the queries that see its
