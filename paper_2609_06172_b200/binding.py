@@ -421,8 +421,10 @@ def model_workspace_bytes(cfg: ModelCfg, max_tokens: int) -> int:
 _POINTER_ARRAYS = {}                                       # ctypes array types by length (building the name of one costs more than filling it)
 
 
-def _pointers(xs):
-    n = len(xs)
+def _pointers(xs, n):
+    """An array of n addresses, n being what the library is told: NULL where xs (any iterable) has fewer, IndexError where it has more."""
+    if not hasattr(xs, "__len__"):
+        xs = list(xs)
     t = _POINTER_ARRAYS.get(n)
     if t is None:
         t = _POINTER_ARRAYS[n] = _P * max(1, n)
@@ -431,7 +433,8 @@ def _pointers(xs):
 
 
 def _tile_arrays(k_tiles, v_tiles):
-    return _pointers(k_tiles), _pointers(v_tiles), len(k_tiles)
+    n = len(k_tiles)
+    return _pointers(k_tiles, n), _pointers(v_tiles, n), n
 
 
 def _k(rc, where):
@@ -469,7 +472,7 @@ def k_gemm(A, W, Cout, M, n, K, ldc, col0, accumulate, stream=None):
 def k_gemm_group(A, Ws, Couts, M, ns, K, ldcs, accumulate=False, stream=None):
     """Products of the same activations A [M, K] with several weight blocks Ws[s] [ns[s], K] into Couts[s] (row stride ldcs[s])."""
     c = len(Ws)
-    _k(lib().tgp_k_gemm_group(_ptr(A), c, _pointers(Ws), _pointers(Couts),
+    _k(lib().tgp_k_gemm_group(_ptr(A), c, _pointers(Ws, c), _pointers(Couts, c),
                               (_U32 * c)(*ns), (_U32 * c)(*ldcs), M, K, int(accumulate), _ptr(stream)), "tgp_k_gemm_group")
 
 

@@ -482,3 +482,21 @@ def test_addresses_of_every_kind_of_argument_alone_and_in_arrays():
     assert [v for v in tb._pointers([x for x, _ in cases])] == [w if w is None else int(w) for _, w in cases]
     assert list(tb._pointers([t[1:], t])) == [t.data_ptr() + 4, t.data_ptr()] and len(tb._pointers([])) == 1
     assert list(tb._pointers((Holder(cuda_stream=3), Holder(data_ptr=lambda: 4)))) == [3, 4]
+
+
+def test_pointer_lists_have_the_length_the_library_is_told():
+    """Lists of another length than the first of a call: NULL for what is missing, which the library refuses where it would use it, an
+    IndexError for more; any iterable will do."""
+    for ka, va, n in (tb._tile_arrays([16, 32, 48], [64, 80]), tb._tile_arrays((16, 32, 48), (v for v in (64, 80)))):
+        assert n == 3 and list(ka) == [16, 32, 48] and list(va) == [64, 80, None]
+    with pytest.raises(IndexError):
+        tb._tile_arrays([16], [64, 80])
+    # (no rows, or a call that is refused: nothing is launched)
+    group = lambda outs: tb.k_gemm_group(16, [16, 32, 48], outs, 0, [8, 8, 8], 64, [8, 8, 8])
+    group([64, 80, 96])
+    group(v for v in (64, 80, 96))
+    with pytest.raises(tb.TgpError) as e:
+        group([64, 80])
+    assert e.value.code == tb.E_INVAL
+    with pytest.raises(IndexError):
+        group([64, 80, 96, 112])
