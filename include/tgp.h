@@ -394,7 +394,8 @@ int  tgp_k_wait_test(uint64_t limit_ns, int withhold_step);
 int  tgp_k_rope_tables(uint32_t Dh, uint32_t max_len, float base, float *cos_dev, float *sin_dev);
 /* Rotary embedding (rotate-half pairs (i, i+Dh/2)) on q and k, bf16 rounding, and append of k, v to the KV
  * tiles.  q32/k32/v32 fp32 [B*q_len, H*Dh]; qb bf16 out; k_tiles/v_tiles: HOST arrays of n_tiles (<= 64)
- * device pointers, tile layout [B, Hkv, TK, Dh] bf16; token (b, p) sits at position pos0 + p. */
+ * device pointers, tile layout [B, Hkv, TK, Dh] bf16; token (b, p) sits at position pos0 + p.  Tiles that hold none of
+ * the call's positions may be NULL, any other NULL is TGP_E_INVAL (so in the calls below). */
 int  tgp_k_rope_kv(const float *q32, const float *k32, const float *v32, void *qb, void *const *k_tiles,
                    void *const *v_tiles, uint32_t n_tiles, const float *cos_dev, const float *sin_dev,
                    const tgp_model_cfg *cfg, uint32_t B, uint32_t q_len, uint32_t pos0, void *stream);

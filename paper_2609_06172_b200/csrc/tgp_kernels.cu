@@ -2631,10 +2631,14 @@ int tgpk_argmax(const float *logits, int32_t *out, int32_t *out2, uint32_t B, ui
 }
 
 // ============================ C entry points ===========================================================
-static int fill_tiles(TgpTilePtrs &t, void *const *k, void *const *v, uint32_t n) {
+// The tiles of a call whose kernels access tiles first <= i < end <= n: those may not be NULL.
+static int fill_tiles(TgpTilePtrs &t, void *const *k, void *const *v, uint32_t n, uint32_t first, uint32_t end) {
     if (n > TGP_MAX_TILES) return TGP_E_TOO_LARGE;
     if (!k || !v) return TGP_E_INVAL;
-    for (uint32_t i = 0; i < n; ++i) { t.k[i] = k[i]; t.v[i] = v[i]; }
+    for (uint32_t i = 0; i < n; ++i) {
+        t.k[i] = k[i]; t.v[i] = v[i];
+        if (i >= first && i < end && (!k[i] || !v[i])) return TGP_E_INVAL;
+    }
     return TGP_OK;
 }
 
@@ -2747,9 +2751,9 @@ int tgp_k_gemm(const void *A_dev, const void *W_dev, float *C_dev, uint32_t M, u
 int tgp_k_rope_kv(const float *q32, const float *k32, const float *v32, void *qb, void *const *k_tiles, void *const *v_tiles, uint32_t n_tiles,
                   const float *cos_dev, const float *sin_dev, const tgp_model_cfg *cfg, uint32_t B, uint32_t q_len, uint32_t pos0, void *stream) {
     if (!q32 || !k32 || !v32 || !qb || !cfg || !cos_dev || !sin_dev) return TGP_E_INVAL;
-    if (pos0 + q_len > cfg->max_len || (uint64_t)n_tiles * cfg->TK < pos0 + q_len || cfg->Dh % 2) return TGP_E_INVAL;
+    if ((uint64_t)pos0 + q_len > cfg->max_len || (uint64_t)n_tiles * cfg->TK < (uint64_t)pos0 + q_len || cfg->Dh % 2) return TGP_E_INVAL;
     TgpTilePtrs t;
-    int rc = fill_tiles(t, k_tiles, v_tiles, n_tiles);
+    int rc = fill_tiles(t, k_tiles, v_tiles, n_tiles, cfg->TK ? pos0 / cfg->TK : 0, B && q_len ? (pos0 + q_len - 1) / cfg->TK + 1 : 0);
     if (rc) return rc;
     return tgpk_rope_kv(q32, k32, v32, qb, t, cos_dev, sin_dev, cfg, B, q_len, pos0, (cudaStream_t)stream);
 }
@@ -2757,9 +2761,9 @@ int tgp_k_rope_kv(const float *q32, const float *k32, const float *v32, void *qb
 int tgp_k_attn(const void *qb, void *const *k_tiles, void *const *v_tiles, uint32_t n_tiles, void *ob, const tgp_model_cfg *cfg, uint32_t B, uint32_t q_len,
                uint32_t pos0, float *scratch_dev, void *stream) {
     if (!qb || !ob || !cfg || !cfg->Hkv || cfg->Hq % cfg->Hkv) return TGP_E_INVAL;
-    if ((uint64_t)n_tiles * cfg->TK < pos0 + q_len) return TGP_E_INVAL;
+    if ((uint64_t)n_tiles * cfg->TK < (uint64_t)pos0 + q_len) return TGP_E_INVAL;
     TgpTilePtrs t;
-    int rc = fill_tiles(t, k_tiles, v_tiles, n_tiles);
+    int rc = fill_tiles(t, k_tiles, v_tiles, n_tiles, 0, B && q_len ? (pos0 + q_len - 1) / cfg->TK + 1 : 0);
     if (rc) return rc;
     return tgpk_attn(qb, t, n_tiles, ob, cfg, B, q_len, pos0, scratch_dev, (cudaStream_t)stream);
 }
@@ -2777,7 +2781,7 @@ int tgp_k_attn_decode_static(const void *qb, void *const *k_tiles, void *const *
     const uint64_t need = (uint64_t)B * cfg->Hq * n_tiles * (cfg->Dh + 2) * sizeof(float);
     if (need > TGP_STATIC_SCRATCH_BYTES) return TGP_E_TOO_LARGE;
     TgpTilePtrs t;
-    int rc = fill_tiles(t, k_tiles, v_tiles, n_tiles);
+    int rc = fill_tiles(t, k_tiles, v_tiles, n_tiles, 0, pos0 / cfg->TK + 1);
     if (rc) return rc;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return TGP_E_CUDA;

@@ -500,3 +500,19 @@ def test_pointer_lists_have_the_length_the_library_is_told():
     assert e.value.code == tb.E_INVAL
     with pytest.raises(IndexError):
         group([64, 80, 96, 112])
+
+
+def test_null_tiles_are_refused_where_the_call_uses_them():
+    mc = tb.ModelCfg()
+    mc.B, mc.Hq, mc.Hkv, mc.Dh, mc.TK, mc.max_len = 1, 2, 1, 64, 16, 48
+    calls = [lambda k, v, B, q, p: tb.k_rope_kv(16, 16, 16, 16, k, v, 16, 16, mc, B, q, p), lambda k, v, B, q, p: tb.k_attn(16, k, v, 16, mc, B, q, p)]
+    for call in calls:
+        for k, v, q, p in (([16, None, 48], [16, 32, 48], 32, 10), ([16, 32, 48], [16, 32], 1, 47), ([16, 32, 48], [16, None, 48], 1, 16), ([16, 32, 48], [], 48, 0)):
+            with pytest.raises(tb.TgpError) as e:
+                call(k, v, 1, q, p)
+            assert e.value.code == tb.E_INVAL
+        call([None, 32], [None, None], 0, 1, 16)            # (no sequence: nothing is used, nothing launched)
+    for k, v, p in (([16], [None], 0), ([16, 32], [16], 16), ([None, 32], [16, 32], 20)):
+        with pytest.raises(tb.TgpError) as e:
+            tb.k_attn_decode_static(16, k, v, 16, mc, 1, p)
+        assert e.value.code == tb.E_INVAL
