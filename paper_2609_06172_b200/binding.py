@@ -421,10 +421,13 @@ def model_workspace_bytes(cfg: ModelCfg, max_tokens: int) -> int:
 _POINTER_ARRAYS = {}                                       # ctypes array types by length (building the name of one costs more than filling it)
 
 
-def _pointers(xs, n):
-    """An array of n addresses, n being what the library is told: NULL where xs (any iterable) has fewer, IndexError where it has more."""
+def _pointers(xs, n=None):
+    """An array of n addresses, n being what the library is told (else as many as there are): NULL where xs, any iterable, has fewer, IndexError
+    where it has more."""
     if not hasattr(xs, "__len__"):
         xs = list(xs)
+    if n is None:
+        n = len(xs)
     t = _POINTER_ARRAYS.get(n)
     if t is None:
         t = _POINTER_ARRAYS[n] = _P * max(1, n)
