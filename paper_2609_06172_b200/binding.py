@@ -184,10 +184,10 @@ def _accessor(x):
         f = getattr(t, "data_ptr", None)
         if not isinstance(f, types.MethodDescriptorType):  # not a tensor
             return operator.methodcaller("data_ptr")
-    elif hasattr(t, "cuda_stream"):
-        f = operator.attrgetter("cuda_stream")
     elif hasattr(x, "cuda_stream"):
-        return operator.attrgetter("cuda_stream")
+        f = operator.attrgetter("cuda_stream")
+        if not isinstance(getattr(t, "cuda_stream", None), (types.GetSetDescriptorType, types.MemberDescriptorType)):
+            return f                                       # not a torch stream: another object of the type may be read in another way
     else:
         raise TypeError(t)
     _ACCESSORS[t] = f

@@ -484,6 +484,17 @@ def test_addresses_of_every_kind_of_argument_alone_and_in_arrays():
     assert list(tb._pointers((Holder(cuda_stream=3), Holder(data_ptr=lambda: 4)))) == [3, 4]
 
 
+def test_the_address_of_an_object_is_its_own_not_that_of_its_type():
+    class Arg:                                             # a stream, and a buffer where it has one
+        cuda_stream = 7
+
+    buffer = Arg()
+    buffer.data_ptr = lambda: 9
+    for x, want in ((Arg(), 7), (buffer, 9), (Arg(), 7)):
+        assert tb._ptr(x) == want
+    assert list(tb._pointers([Arg(), buffer])) == [7, 9]
+
+
 def test_pointer_lists_have_the_length_the_library_is_told():
     """Lists of another length than the first of a call: NULL for what is missing, which the library refuses where it would use it, an
     IndexError for more; any iterable will do."""
