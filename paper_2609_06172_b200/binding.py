@@ -171,6 +171,7 @@ def parse_trace(blob):
     return ops
 
 
+CACHED_MAX = 64                                            # entries the two tables below may hold: KV tiles a call can address, and few types
 _ACCESSORS = {}                                            # how the address of an object is read, by its type
 
 
@@ -190,7 +191,8 @@ def _accessor(x):
             return f                                       # not a torch stream: another object of the type may be read in another way
     else:
         raise TypeError(t)
-    _ACCESSORS[t] = f
+    if len(_ACCESSORS) < CACHED_MAX:
+        _ACCESSORS[t] = f
     return f
 
 
@@ -430,7 +432,9 @@ def _pointers(xs, n=None):
         n = len(xs)
     t = _POINTER_ARRAYS.get(n)
     if t is None:
-        t = _POINTER_ARRAYS[n] = _P * max(1, n)
+        t = _P * max(1, n)
+        if len(_POINTER_ARRAYS) < CACHED_MAX:
+            _POINTER_ARRAYS[n] = t
     kinds = set(map(type, xs))
     return t(*map(_ACCESSORS.get(kinds.pop(), _ptr) if len(kinds) == 1 else _ptr, xs))
 

@@ -495,6 +495,13 @@ def test_the_address_of_an_object_is_its_own_not_that_of_its_type():
     assert list(tb._pointers([Arg(), buffer])) == [7, 9]
 
 
+def test_what_is_kept_for_addresses_and_arrays_is_bounded():
+    for i in range(200):
+        assert tb._ptr(type("Number", (int,), {})(i)) == i
+        assert len(tb._pointers([8] * i)) == max(1, i) and tb._pointers([8] * i)[0] == (8 if i else None)
+    assert len(tb._ACCESSORS) <= 64 and len(tb._POINTER_ARRAYS) <= 64
+
+
 def test_pointer_lists_have_the_length_the_library_is_told():
     """Lists of another length than the first of a call: NULL for what is missing, which the library refuses where it would use it, an
     IndexError for more; any iterable will do."""
