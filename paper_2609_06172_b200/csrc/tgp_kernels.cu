@@ -1898,17 +1898,9 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
     else g_chain.A = nullptr;
     tgpk_last_gemm_kernel = !k.split ? "tgp_wstream_mma_kernel" : persistent ? "tgp_wstream_mma_group_kernel" : "tgp_wstream_mma_splitk_kernel";
     if (persistent) {
-        if constexpr (NB == 1 && U == 8) {
+        if constexpr (NB == 2 || U == 8) {                  // (their partial tiles, 32 KB at most, are static)
             if (per_cta == 2) launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
             else launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 1>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
-        } else if constexpr (NB == 2) {
-            if (per_cta == 2) {
-                constexpr size_t smem = 16 * 2 * NB * 4 * 32 * 4;      // the partial tiles of 16 warps, two row groups each
-                static bool attr_set = false;
-                if (!attr_set) { cudaFuncSetAttribute(tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); attr_set = true; }
-                cfg.dynamicSmemBytes = smem;
-                launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
-            } else launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 1>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
         }
     } else if constexpr (STREAMS) {
         if (!k.split) launch_weights<tgp_wstream_mma_kernel<NB, U>>(cfg, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);

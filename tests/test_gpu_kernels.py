@@ -1,5 +1,6 @@
 """Kernel parity on the GPU: every kernel of the path, called through the C ABI, against the CPU oracle
 on the same seeded inputs; sizes span several tiles and ragged tails, plus the degenerate cases."""
+import json
 from dataclasses import replace
 
 import numpy as np
@@ -754,6 +755,29 @@ def test_blocks_of_many_rows_take_the_list_kernel_with_the_same_bits_alone_and_i
         want = A.double() @ W.double().T + c.double()
         # fp32 sums of K products of N(0, 1) x N(0, 0.02): errors of a few 2^-24 of the partial sums' size, bounded as in the tests above
         assert float((a.double() - want).abs().max()) < 2e-5 * float(want.abs().max())
+
+
+def kernels_of(call, tmp_path):
+    """Names and shared memory (static and dynamic, bytes) of the kernels a call launches, in order."""
+    call()                                                 # (function attributes, first-use allocations)
+    torch.cuda.synchronize()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    path = tmp_path / "trace.json"
+    prof.export_chrome_trace(str(path))
+    events = [e for e in json.loads(path.read_text())["traceEvents"] if e.get("cat") == "kernel"]
+    return [(e["name"], e["args"]["shared memory"]) for e in sorted(events, key=lambda e: e["ts"])]
+
+
+# two row groups per CTA (4096 and 2 x 2048 rows on 148 SMs: 128 CTAs of 32 rows) and one
+@pytest.mark.parametrize("M,ns,K", [(16, (4096,), 4096), (9, (2048, 2048), 1024), (16, (1024, 1000), 1024)])
+def test_products_of_9_to_16_rows_take_no_more_shared_memory_than_their_partial_tiles(M, ns, K, tmp_path):
+    A = torch.ones((M, K), device=DEV, dtype=torch.bfloat16)
+    Ws, Cs = [torch.ones((n, K), device=DEV, dtype=torch.bfloat16) for n in ns], [torch.empty((M, n), device=DEV) for n in ns]
+    launched = kernels_of(lambda: tb.k_gemm_group(A, Ws, Cs, M, list(ns), K, list(ns)), tmp_path)
+    assert len(launched) == 1 and "tgp_wstream_mma_group_kernel" in launched[0][0]
+    assert launched[0][1] in (16 << 10, 32 << 10)          # 16 warps x 1 or 2 groups x 16 x 16 sums, which a kernel may declare
 
 
 # one and two rows on blocks of many rows, on either side of what is listed (K of two to four times 2048 columns at one row, up to 8704 weight rows and K a multiple of 2048 at two)
