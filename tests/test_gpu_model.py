@@ -217,6 +217,7 @@ def test_prefill_swiglu_in_the_up_projection_epilogue_gives_the_same_bits():
             logits = [r.logits.cpu().numpy().copy()]
             for t in range(T):
                 r.step(tb.DECODE, np.ascontiguousarray(forced[:, t:t + 1]), 1)
+                r.sync()                                            # (a step without statistics is not waited for)
                 logits.append(r.logits.cpu().numpy().copy())
             runs[(variant, enable)] = (logits, st.n_launches)
     tb.k_gemm_tc_variant(0)
