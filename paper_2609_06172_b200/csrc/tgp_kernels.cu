@@ -938,9 +938,12 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
 }
 __device__ __forceinline__ float fast_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
-// (CLUSTER is an instance of its own: what only clusters need makes the others 5 - 14 % slower)
+// (CLUSTER is an instance of its own: what only clusters need makes the others 5 - 14 % slower.  The second bound is the number of CTAs that
+// shared memory leaves room for: told so, the compiler keeps its loads apart with 177 - 179 registers at DH = 128; left to itself it takes 141 to 165,
+// by what the instance holds besides, and is up to 20 % slower: 8 heads over one, 9000 keys of one sequence 19.1 -> 15.0 us with the norm before, in clusters 3 - 6 %.  All bits of P
+// take 151 registers at DH = 64, and the few CTAs they are for fit an SM in threes.)
 template <int DH, int G, bool SPLIT_P, bool CLUSTER>
-__global__ void __launch_bounds__(DEC_WARPS * 32) tgp_attn_decode_mma_kernel(AttnArgs a, uint32_t chunks_per_cta) {
+__global__ void __launch_bounds__(DEC_WARPS * 32, DH == 128 ? 2 : SPLIT_P ? 3 : 4) tgp_attn_decode_mma_kernel(AttnArgs a, uint32_t chunks_per_cta) {
     pdl_enter();
     extern __shared__ __align__(128) uint8_t dec_sm[];
     constexpr uint32_t ROW = DH * 2, CPR = ROW / 16;                  // bytes and 16-byte chunks per key row
