@@ -2518,15 +2518,23 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
             if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
             const uint32_t units = B * c->Hkv, per_sm = c->Dh == 64 ? 4 : 2;             // CTAs that fit an SM (96 / 48 KB of shared memory each)
             uint32_t parts = (uint32_t)sms * per_sm / units;                              // CTAs per (sequence, KV head): one wave at most
-            // Up to DEC_CLUSTER parts can be a cluster, which merges them itself; more parts meet in the scratch array and a second kernel.
-            // Up to four parts always are one.  A context that would have more is worth eight where it is short or its clusters are few: eight
-            // CTAs need one GPC to hold them, and 32 such clusters wait for one another in a step, though not back to back (eight parts against
-            // all, us: 32 heads over 8 x 64, B=1, 700 keys 3.7 / 5.2, 2112 keys 5.3 / 8.8, 4000 6.8 / 6.9, 9000 11.8 / 10.6; x 128, 2112 keys
-            // 7.1 / 9.5, 4000 9.5 / 8.3; a step of two layers, B=4, 16000 keys 356 / 321)
+            const uint32_t slots = (uint32_t)sms * per_sm;
             parts = std::max(1u, std::min(parts, (nchunks + DEC_WARPS - 1) / DEC_WARPS));
+            // A short context stays in one CTA, whose chain of a few chunks per warp is over sooner than a cluster has met, the longer a chain the
+            // more CTAs there are (one part against four, us with the norm before: 32 heads over 8 x 64, one sequence, 100 keys 4.7 / 5.3, 200 keys
+            // 5.8 / 5.3; 16 sequences, 200 keys 5.3 / 6.8, 400 keys 6.8 / 7.4 but 14.5 / 13.0 with a product on either side; x 128 against two, 400 keys 9.4 / 10.4).
+            const bool one = nchunks <= std::max(12u, 8 + (units * c->Dh + 511) / 512);
+            // Up to DEC_CLUSTER parts can be a cluster, which merges them itself; more parts meet in the scratch array and a second kernel.
+            // Eight CTAs need one GPC to hold them: a context takes eight only while its clusters leave half of the GPU free, and beyond 1024 keys only if they are few
+            // (eight parts against all, us: 32 heads over 8 x 64, B=1, 700 keys 3.7 / 5.2, 2112 keys 5.3 / 8.8, 4000 6.8 / 6.9, 9000 11.8 / 10.6; x 128, 2112 keys
+            // 7.1 / 9.5, 4000 9.5 / 8.3; a step of two layers, B=4, 16000 keys 356 / 321; 32 units x 128, 700 keys with a product on either side:
+            // 17.7 in eight parts, 14.5 in four).
+            const bool eight = (nchunks <= 64 && 16 * units <= slots) || (units <= 16 && (nchunks <= 192 || n_tiles <= DEC_CLUSTER));
+            // Up to four parts are one if seven eighths of the GPU hold all clusters: in the rest there is room for CTAs, but not for clusters, and the last of
+            // them run alone (a layer of d=512, 24 sequences of 8 heads x 64, 6000 keys, three parts each for 592 places: 94.5 us in clusters, 80.5 through the scratch array).
             // (the scratch array holds a partial per KV tile: where that is four or fewer, a cluster of four is at least as many)
-            const bool eight = nchunks <= 64 || (units <= 16 && (nchunks <= 192 || n_tiles <= DEC_CLUSTER)), clustered = eight || parts <= 4 || n_tiles <= 4;
-            parts = std::min(parts, eight ? (uint32_t)DEC_CLUSTER : clustered ? 4u : n_tiles);
+            const bool clustered = eight || ((nchunks <= 64 || parts <= 4 || n_tiles <= 4) && 8 * units * std::min(parts, 4u) <= 7 * slots);
+            parts = one ? 1u : std::min(parts, eight ? (uint32_t)DEC_CLUSTER : clustered ? 4u : n_tiles);
             const uint32_t per_cta = (nchunks + parts - 1) / parts;
             parts = (nchunks + per_cta - 1) / per_cta;                                    // no CTA without a chunk
             const bool cluster = clustered && parts > 1, merge = !clustered && parts > 1;

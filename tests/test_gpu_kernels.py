@@ -27,6 +27,19 @@ def rnd_bits(role, n):
     return si.normal_bf16_bits(1234, role, 0, n)
 
 
+def kernels_of(call, tmp_path):
+    """Names and launch records ("shared memory": static and dynamic, bytes; "grid") of the kernels a call launches, in order."""
+    call()                                                 # (function attributes, first-use allocations)
+    torch.cuda.synchronize()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    path = tmp_path / "trace.json"
+    prof.export_chrome_trace(str(path))
+    events = [e for e in json.loads(path.read_text())["traceEvents"] if e.get("cat") == "kernel"]
+    return [(e["name"], e["args"]) for e in sorted(events, key=lambda e: e["ts"])]
+
+
 def oracle():
     lay = si.build_layout(KCFG)
     return OracleModel(KCFG, si.weights_as_bits(lay))
@@ -757,19 +770,6 @@ def test_blocks_of_many_rows_take_the_list_kernel_with_the_same_bits_alone_and_i
         assert float((a.double() - want).abs().max()) < 2e-5 * float(want.abs().max())
 
 
-def kernels_of(call, tmp_path):
-    """Names and shared memory (static and dynamic, bytes) of the kernels a call launches, in order."""
-    call()                                                 # (function attributes, first-use allocations)
-    torch.cuda.synchronize()
-    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-        call()
-        torch.cuda.synchronize()
-    path = tmp_path / "trace.json"
-    prof.export_chrome_trace(str(path))
-    events = [e for e in json.loads(path.read_text())["traceEvents"] if e.get("cat") == "kernel"]
-    return [(e["name"], e["args"]["shared memory"]) for e in sorted(events, key=lambda e: e["ts"])]
-
-
 # two row groups per CTA (4096 and 2 x 2048 rows on 148 SMs: 128 CTAs of 32 rows) and one
 @pytest.mark.parametrize("M,ns,K", [(16, (4096,), 4096), (9, (2048, 2048), 1024), (16, (1024, 1000), 1024)])
 def test_products_of_9_to_16_rows_take_no_more_shared_memory_than_their_partial_tiles(M, ns, K, tmp_path):
@@ -777,7 +777,7 @@ def test_products_of_9_to_16_rows_take_no_more_shared_memory_than_their_partial_
     Ws, Cs = [torch.ones((n, K), device=DEV, dtype=torch.bfloat16) for n in ns], [torch.empty((M, n), device=DEV) for n in ns]
     launched = kernels_of(lambda: tb.k_gemm_group(A, Ws, Cs, M, list(ns), K, list(ns)), tmp_path)
     assert len(launched) == 1 and "tgp_wstream_mma_group_kernel" in launched[0][0]
-    assert launched[0][1] in (16 << 10, 32 << 10)          # 16 warps x 1 or 2 groups x 16 x 16 sums, which a kernel may declare
+    assert launched[0][1]["shared memory"] in (16 << 10, 32 << 10)          # 16 warps x 1 or 2 groups x 16 x 16 sums, which a kernel may declare
 
 
 # one and two rows on blocks of many rows, on either side of what is listed (K of two to four times 2048 columns at one row, up to 8704 weight rows and K a multiple of 2048 at two)
@@ -1038,6 +1038,28 @@ def test_decode_attention_of_short_contexts_with_infinities_and_nan(Dh, G, kvlen
     tb.k_attn(q, kt, vt, o, mc, B, 1, kvlen - 1, scratch)
     torch.cuda.synchronize()
     assert o.float().view(Hkv, G, Dh)[1].isnan().all()
+
+
+# either side of each line of the dispatch, on 148 SMs: the last length that stays in one CTA (12 chunks of 16 keys for few sequences, more for many),
+# the last numbers of (sequence, KV head) pairs that take eight parts (18 of 128 dimensions) and four in clusters (64; 148 in twos)
+@pytest.mark.parametrize("Dh,Hq,Hkv,TK,kvlen,B,parts,kernels", [(64, 8, 8, 64, 192, 1, 1, 1), (64, 8, 8, 64, 193, 1, 4, 1), (64, 32, 8, 256, 384, 16, 1, 1), (64, 32, 8, 256, 385, 16, 4, 1),
+                                                                (128, 16, 16, 256, 256, 2, 1, 1), (128, 16, 16, 256, 257, 2, 4, 1), (128, 18, 18, 128, 700, 1, 8, 1), (128, 19, 19, 128, 700, 1, 4, 1),
+                                                                (128, 32, 8, 256, 2000, 8, 4, 1), (128, 32, 8, 256, 2000, 9, 4, 2), (64, 8, 8, 256, 3000, 24, 3, 2), (64, 8, 8, 4096, 3000, 24, 1, 1)])
+def test_parts_of_a_decode_context_on_either_side_of_the_dispatch_lines(Dh, Hq, Hkv, TK, kvlen, B, parts, kernels, tmp_path):
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=kvlen, T=0, B=B, d=Hq * Dh)
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(kvlen + B)
+    n, G = (kvlen + TK - 1) // TK, Hq // Hkv
+    kt, vt = ([torch.randn((B, Hkv, TK, Dh), device=DEV, generator=gen).bfloat16() for _ in range(n)] for _ in range(2))
+    q = torch.randn((B, Hkv, G, Dh), device=DEV, generator=gen).bfloat16()
+    scratch = torch.zeros(tb.k_attn_scratch_bytes(model_cfg(cfg)) // 4, device=DEV)
+    ob = torch.zeros_like(q)
+    launched = kernels_of(lambda: tb.k_attn(q, kt, vt, ob, model_cfg(cfg), B, 1, kvlen - 1, scratch), tmp_path)
+    assert len(launched) == kernels and launched[0][1]["grid"] == [parts, Hkv, B]
+    K, V = (torch.cat(ts, dim=2)[:, :, :kvlen].double() for ts in (kt, vt))
+    want = torch.softmax(q.double() @ K.transpose(-1, -2) / Dh ** 0.5, -1) @ V
+    # half a bf16 step of the output and of each of the probabilities, whose roundings average out: 2^-9 of the largest V, as in the tests above
+    assert float((ob.double() - want).abs().max()) < 2.0 ** -7 * float(want.abs().max()) + 1e-6
 
 
 # one part, clusters with and without all bits of P, the scratch array; keys that begin a warp's chunks in one of the splits and not in another
