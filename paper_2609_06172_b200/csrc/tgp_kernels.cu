@@ -1510,17 +1510,17 @@ static void launch_weights(const cudaLaunchConfig_t &cfg, Args... args) {
     cudaLaunchKernelEx(&cfg, KERNEL, args...);
 }
 
+// CTAs of tgp_wstream_kernel that the GPU holds at a time.
+template <int MT, int R, int U>
+static uint32_t gemv_slots() {
+    static int blocks_per_sm = 0;
+    if (!blocks_per_sm && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, tgp_wstream_kernel<MT, R, U>, 256, 0) != cudaSuccess || blocks_per_sm < 1)) blocks_per_sm = 1;
+    return (uint32_t)(device_sms() * blocks_per_sm);
+}
+
 template <int MT, int R, int U>
 static void launch_gemv(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int acc, cudaStream_t st) {
-    static int blocks_per_sm = 0, sms = 0;
-    if (!blocks_per_sm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, tgp_wstream_kernel<MT, R, U>, 256, 0) != cudaSuccess || blocks_per_sm < 1) blocks_per_sm = 1;
-        if (sms < 1) sms = 148;
-    }
-    uint32_t need = (n + R * 8 - 1) / (R * 8), full = (uint32_t)(sms * blocks_per_sm);
+    const uint32_t need = (n + R * 8 - 1) / (R * 8), full = gemv_slots<MT, R, U>();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(need < full ? need : full);
     cfg.blockDim = dim3(256);
@@ -1947,11 +1947,18 @@ constexpr uint32_t GEMV_MANY_ROWS = 2 * 148 * 16;
 // way is ahead of two rows with four each (n=14336, K=4096 18.3 us against 19.7, n=32000, K=8192 76 / 81; with K=1024 25 / 16, K=28672 78 / 72).
 static bool one_row_deep(uint32_t M, uint32_t K) { return M == 1 && K % 2048 == 0 && K >= 4096 && K <= 8192; }
 
+// ... alone, where its last wave of CTAs of eight rows is no emptier than that of CTAs of sixteen (three and four CTAs per SM: n=8192, K=6144 is 2.3 waves of
+// eight and 0.9 of sixteen rows, 19.1 us and 17.8; n=10240, K=4096 2.9 and 1.1, 15.0 and 17.3); in a list the waves of all blocks are one ramp.
+static bool one_row_fuller(uint32_t n) {
+    auto fill = [n](uint32_t wave) { return (float)n / (float)((n + wave - 1) / wave * wave); };
+    return fill(8 * gemv_slots<1, 1, 8>()) >= fill(16 * gemv_slots<1, 2, 4>());
+}
+
 // rows per warp: fewer when the block has few rows, so that every SM still gets warps
 template <int MT>
 static void launch_gemv_rows(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int acc, cudaStream_t st) {
     if constexpr (MT <= 2) {
-        if (n >= GEMV_MANY_ROWS && !one_row_deep(MT, K)) return launch_gemv<MT, 2, 4>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
+        if (n >= GEMV_MANY_ROWS && !(one_row_deep(MT, K) && one_row_fuller(n))) return launch_gemv<MT, 2, 4>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
         if (n < GEMV_MANY_ROWS && g_gemv_splitk && K >= 8192) {                    // at least four 256-element chunks per warp and row
             if (n <= 1024) return launch_gemv_splitk<MT, 1, 4>(A, W, C, Mrows, n, K, ldc, col0, acc, st);
             return launch_gemv_splitk<MT, 2, 4>(A, W, C, Mrows, n, K, ldc, col0, acc, st);

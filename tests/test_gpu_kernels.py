@@ -805,6 +805,26 @@ def test_blocks_of_many_rows_at_one_and_two_activation_rows(M, ns, K, listed, ac
         assert float((a[:, :n].double() - want).abs().max()) < 2e-5 * float(want.abs().max())
 
 
+# on 148 SMs: waves of 3552 rows (a row per warp) and 9472 (two), the fuller last wave
+@pytest.mark.parametrize("n,K,rows_per_warp", [(7104, 4096, 1), (7105, 8192, 2), (9472, 6144, 2), (9473, 6144, 1), (8192, 2048, 2), (10240, 10240, 2)])
+def test_one_activation_row_takes_the_kernel_whose_last_wave_is_fuller_with_the_same_bits(n, K, rows_per_warp, tmp_path):
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(n + K)
+    A = torch.randn((1, K), device=DEV, generator=gen).bfloat16()
+    W = (torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16()
+    alone, parts = torch.empty((1, n), device=DEV), torch.empty((1, n), device=DEV)
+    (name, _), = kernels_of(lambda: tb.k_gemm(A, W, alone, 1, n, K, n, 0, False), tmp_path)
+    assert f"tgp_wstream_kernel<1, {rows_per_warp}, " in name
+    at = [0, 4000, n]                                      # pieces of fewer than 4736 rows: a row per warp, or K split over warps
+    for lo, hi in zip(at, at[1:]):
+        tb.k_gemm(A, W[lo:hi], parts, 1, hi - lo, K, n, lo, False)
+    want = A.double() @ W.double().T
+    for got in (alone, parts):
+        # lane-strided fp32 sums of K products: a few 2^-24 of the partial sums' size, as in the tests above
+        assert float((got.double() - want).abs().max()) < 2e-5 * float(want.abs().max())
+    assert K >= 8192 or torch.equal(alone[:, :4000], parts[:, :4000])
+
+
 # the list kernel at 9 - 16 rows around a chunk of 16 warps x 128 columns (one column block, a warp's chunk more or less, many chunks), ragged
 # row groups, one and two row groups per CTA; and lists of which only neighbours share a kernel
 @pytest.mark.parametrize("M,ns,K", [(9, (1, 17), 32), (16, (1024, 1000), 1024), (12, (300,), 2016), (16, (2048, 4100), 2048), (11, (33, 640), 2080), (16, (500,), 14368),
