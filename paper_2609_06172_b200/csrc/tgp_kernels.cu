@@ -1954,6 +1954,16 @@ static bool one_row_fuller(uint32_t n) {
     return fill(8 * gemv_slots<1, 1, 8>()) >= fill(16 * gemv_slots<1, 2, 4>());
 }
 
+// Two activation rows on a block of many rows: listed (a row per warp, eight load steps under way) where the block alone leaves the last wave of its CTAs - three of
+// sixteen rows per SM - more than a quarter empty (us in one list / one behind the other: 2 x 4736, K=2048 11.4 / 11.9; 2 x 7168 14.4 / 17.9, 2 x 8192 17.0 / 19.8;
+// K=8192, 3 x 8192 75 / 90; but 2 x 6144, three quarters to all of one wave, 13.3 / 12.6, K=8192 40.1 / 39.0).  K is a multiple of the 2048 columns of the eight load steps, which it
+// otherwise leaves partly empty (2 x 8192: K=2560 26.6 / 24.7, 3072 27.1 / 26.2, 5120 even).  Beyond two waves the ramps count for less (2 x 14336 even, 2 x 20480
+// 36.2 / 33.2); of the second wave's blocks those of up to 8704 rows are listed (54.8 / 63.4 at K=8192; 9216 and 10240 rows would gain 14 - 20 and 4 - 10 %, 12288 nothing).
+static bool two_rows_listed(uint32_t M, uint32_t n, uint32_t K) {
+    const uint32_t wave = 3 * 16 * (uint32_t)device_sms();
+    return M == 2 && K % 2048 == 0 && n <= 8704 && (n > wave || 4 * n <= 3 * wave);
+}
+
 // rows per warp: fewer when the block has few rows, so that every SM still gets warps
 template <int MT>
 static void launch_gemv_rows(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int acc, cudaStream_t st) {
@@ -2382,9 +2392,8 @@ int tgpk_experts(const TgpExperts &x, cudaStream_t st) {
 uint32_t tgpk_gemm_group_key(uint32_t M, uint32_t n, uint32_t K) {
     if (!g_gemm_group || !M || !n || !K || K % 8) return 0;
     // Blocks of many rows at M <= 2 run one behind the other at little cost, but a list of them has one ramp instead of several: 2 x 14336, K=4096 at
-    // one row 39.0 -> 34.9 us; at two rows 2 x 8192, K=2048 18.0 / 15.4, 3 x 8192, K=8192 87 / 72, while 2 x 14336 are even and 2 x 28672 slower (145 / 161).
-    // (a K that is no multiple of the 2048 columns of its eight load steps leaves them partly empty: a step of 2 users at d=2560 93 / 98)
-    if (M <= 2 && n >= GEMV_MANY_ROWS) return one_row_deep(M, K) || (M == 2 && n <= 8704 && K % 2048 == 0) ? 0x100u | M : 0;
+    // one row 39.0 -> 34.9 us
+    if (M <= 2 && n >= GEMV_MANY_ROWS) return one_row_deep(M, K) || two_rows_listed(M, n, K) ? 0x100u | M : 0;
     if (M <= 2) return !(g_gemv_splitk && K >= 8192) ? M : 0;
     if (M > 32) return 0;
     if (takes_tiles(M, n, K)) return tgpk_gemm_tc_forced() ? 0 : 0x2000000u | tgpk_gemm_tc_class(M, n, K);

@@ -805,6 +805,23 @@ def test_blocks_of_many_rows_at_one_and_two_activation_rows(M, ns, K, listed, ac
         assert float((a[:, :n].double() - want).abs().max()) < 2e-5 * float(want.abs().max())
 
 
+# on 148 SMs, one wave being 7104 rows: up to three quarters of one, and the beginning of the second
+@pytest.mark.parametrize("n,K,listed", [(4736, 2048, True), (5328, 4096, True), (5329, 4096, False), (7104, 2048, False), (7105, 2048, True), (8704, 6144, True),
+                                        (8705, 6144, False), (5328, 3072, False)])
+def test_two_activation_rows_share_a_launch_where_the_last_wave_is_emptier(n, K, listed, tmp_path):
+    assert (tb.k_gemm_group_key(2, n, K) != 0) == listed
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(n + K)
+    A = torch.randn((2, K), device=DEV, generator=gen).bfloat16()
+    Ws = [(torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16() for _ in range(2)]
+    alone, together = ([torch.empty((2, n), device=DEV) for _ in Ws] for _ in range(2))
+    for W, C in zip(Ws, alone):
+        tb.k_gemm(A, W, C, 2, n, K, n, 0, False)
+    launched = kernels_of(lambda: tb.k_gemm_group(A, Ws, together, 2, [n, n], K, [n, n]), tmp_path)
+    assert [("group" in name) for name, _ in launched] == ([True] if listed else [False, False])
+    assert all(torch.equal(a, b) for a, b in zip(alone, together))
+
+
 # on 148 SMs: waves of 3552 rows (a row per warp) and 9472 (two), the fuller last wave
 @pytest.mark.parametrize("n,K,rows_per_warp", [(7104, 4096, 1), (7105, 8192, 2), (9472, 6144, 2), (9473, 6144, 1), (8192, 2048, 2), (10240, 10240, 2)])
 def test_one_activation_row_takes_the_kernel_whose_last_wave_is_fuller_with_the_same_bits(n, K, rows_per_warp, tmp_path):
