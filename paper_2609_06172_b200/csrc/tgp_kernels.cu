@@ -1867,7 +1867,9 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
         // block of few rows reaches every SM and no CTA waits for the others' last round (4096 rows: 256 groups of 16 leave
         // 40 SMs one round short, 293 of 14 do not) - but the rows a tile lacks still occupy its load slots (their lanes
         // re-read the group's last row; fewer than 9 rows per group measured no faster for blocks of few rows).  G and r are the
-        // pair with the least estimated time of the busiest CTA: rounds x (G x (r + tile rows) / 2 + 4 NB), in rows read.
+        // pair with the least estimated time of the busiest CTA: rounds x (G x (r + tile rows) / 2 + 4 NB), in rows read; of equal
+        // estimates above 8 activation rows the one of fewer groups and more rows (5120 rows, K=4096 as three rounds of 12 rows 13.2 us at M=9,
+        // 14.3 at M=16, as two of 2 x 9 rows 14.3 and 15.5, from the end of the norm before).
         const uint32_t tile = (uint32_t)k.rows, gmax = 2;
         uint32_t best = 0xffffffffu, best_r = tile;
         for (uint32_t G = gmax; G >= 1; G >>= 1)
@@ -1876,7 +1878,7 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
                 for (uint32_t s = 0; s < p.count; ++s) groups += (p.n[s] + r - 1) / r;
                 const uint32_t ctas = (groups + G - 1) / G, rounds = (ctas + full - 1) / full;
                 const uint32_t cost = rounds * (G * (r + tile) + 8 * NB);           // twice the estimate
-                if (cost < best) { best = cost; best_r = r; per_cta = G; }
+                if (cost < best || (cost == best && NB == 2)) { best = cost; best_r = r; per_cta = G; }
             }
         rpc = best_r;
         need = 0;

@@ -1077,6 +1077,15 @@ def test_decode_attention_of_short_contexts_with_infinities_and_nan(Dh, G, kvlen
     assert o.float().view(Hkv, G, Dh)[1].isnan().all()
 
 
+@pytest.mark.parametrize("M", [9, 16])
+def test_row_groups_of_equal_estimates_are_taken_one_at_a_time(M, tmp_path):
+    """5120 rows on 148 SMs: three rounds of 12 rows, not two of twice 9."""
+    n, K = 5120, 4096
+    A, W, C = torch.ones((M, K), device=DEV, dtype=torch.bfloat16), torch.ones((n, K), device=DEV, dtype=torch.bfloat16), torch.zeros((M, n), device=DEV)
+    (name, args), = kernels_of(lambda: tb.k_gemm(A, W, C, M, n, K, n, 0, False), tmp_path)
+    assert "tgp_wstream_mma_group_kernel" in name and args["shared memory"] == 16 << 10 and bool((C == K).all())
+
+
 # either side of each line of the dispatch, on 148 SMs: the last length that stays in one CTA (12 chunks of 16 keys for few sequences, more for many),
 # the last numbers of (sequence, KV head) pairs that take eight parts (18 of 128 dimensions) and four in clusters (64; 148 in twos)
 @pytest.mark.parametrize("Dh,Hq,Hkv,TK,kvlen,B,parts,kernels", [(64, 8, 8, 64, 192, 1, 1, 1), (64, 8, 8, 64, 193, 1, 4, 1), (64, 32, 8, 256, 384, 16, 1, 1), (64, 32, 8, 256, 385, 16, 4, 1),
