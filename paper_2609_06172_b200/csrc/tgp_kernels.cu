@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <type_traits>
 #include <algorithm>
+#include <atomic>
 #include "tgp.h"
 #include "tgp_kernels.h"
 
@@ -1505,8 +1506,13 @@ bool tgpk_launch_overlap() { return g_gemv_pdl != 0; }
 // L1; a decode step of 8 users at d=4096 249 us, 233; a quarter or all of it for L1 is the same).
 template <auto KERNEL, typename... Args>
 static void launch_weights(const cudaLaunchConfig_t &cfg, Args... args) {
-    static const cudaError_t hint = cudaFuncSetAttribute(KERNEL, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
-    (void)hint;
+    static std::atomic<uint64_t> hinted{0};                  // a bit per device: the attribute is a device's own
+    int dev = 0;
+    const uint64_t bit = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? 1ull << dev : 0;
+    if (bit & ~hinted.load(std::memory_order_relaxed)) {
+        if (cudaFuncSetAttribute(KERNEL, cudaFuncAttributePreferredSharedMemoryCarveout, 50) != cudaSuccess) cudaGetLastError();        // only a hint: it fails no product
+        hinted.fetch_or(bit, std::memory_order_relaxed);
+    }
     cudaLaunchKernelEx(&cfg, KERNEL, args...);
 }
 

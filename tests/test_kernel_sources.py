@@ -53,3 +53,12 @@ def test_a_kernel_holds_its_tensor_memory_before_it_releases_its_dependents(f, n
     the one place that asks stands behind the allocation, in the warp that made it."""
     assert body.count("launch_dependents") == 1, (f, name)
     assert re.search(r"tcgen05\.alloc[^;]*;[^}]*tcgen05\.relinquish_alloc_permit[^;]*;[^}]*griddepcontrol\.launch_dependents", body), (f, name)
+
+
+def test_a_launch_hint_is_given_on_every_device_and_fails_no_product():
+    """Function attributes are a device's own, so a flag of the process alone would leave a second device without them; and the
+    error of a hint that was refused must not be found by the check behind the launch."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "tgp_kernels.cu")).read())
+    body = re.search(r"static void launch_weights\(.*?\n\}\n", text, re.S).group(0)
+    assert not re.search(r"static\s+(const\s+)?(cudaError_t|bool|auto)\b", body) and "cudaGetDevice" in body
+    assert re.search(r"cudaFuncSetAttribute\([^;]*!= cudaSuccess\) cudaGetLastError\(\);", body)
