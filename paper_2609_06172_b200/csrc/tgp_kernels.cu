@@ -1540,21 +1540,19 @@ static void launch_gemv(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, 
     tgpk_last_gemm_kernel = "tgp_wstream_kernel";
 }
 
-// Same product for blocks of a short K with two to eight 16-row groups per SM: one CTA owns ROWS rows of W and its NW warps split K
-// (interleaved chunks of 32*U), so n/ROWS CTAs of NW warps fill the machine where n/16 warps would not.  The partial
-// tiles meet in shared memory and are summed in warp order: deterministic.  RPC <= ROWS: rows a CTA owns (the tile's
-// remaining rows re-read its last row and are not stored; a row's sum does not depend on its place in the tile).
+// Same product for blocks of a short K with two to eight 16-row groups per SM: one CTA owns 16 rows of W and its NW warps split K
+// (interleaved chunks of 32*U), so n/16 CTAs of NW warps fill the machine where n/16 warps would not.  The partial
+// tiles meet in shared memory and are summed in warp order: deterministic.
 // (Blocks of fewer rows or a longer K take tgp_wstream_mma_group_kernel.)
-template <int NB, int U, int NW, int ROWS, int RPC = ROWS>
+template <int NB, int U, int NW>
 __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const bf16 *A, const bf16 *__restrict__ W, float *__restrict__ C,
                                                               uint32_t Mrows, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int accumulate) {
-    constexpr int UL = ROWS == 8 ? 2 * U : U;             // half a tile per load step: twice the steps in flight
     __shared__ float part[NW][NB * 4][32];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, c = lane & 3;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     bool synced = false;
-    for (uint32_t row0 = blockIdx.x * RPC; row0 < n; row0 += gridDim.x * RPC) {
-        const uint32_t rlast = min(row0 + RPC, n) - 1;
+    for (uint32_t row0 = blockIdx.x * 16; row0 < n; row0 += gridDim.x * 16) {
+        const uint32_t rlast = min(row0 + 16, n) - 1;
         const bf16 *wlo = W + (size_t)min(row0 + g, rlast) * K + c * 8;
         const bf16 *whi = W + (size_t)min(row0 + g + 8, rlast) * K + c * 8;
         float acc[2][NB][4];                               // a load step's two MMAs have sums of their own: half as many additions in a row
@@ -1562,17 +1560,17 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const b
         for (int b = 0; b < NB; ++b)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[0][b][i] = acc[1][b][i] = 0.f;
-        for (uint32_t k0 = warp * 32 * UL; k0 < K; k0 += NW * 32 * UL) {
-            uint4 lo[UL], hi[UL];
+        for (uint32_t k0 = warp * 32 * U; k0 < K; k0 += NW * 32 * U) {
+            uint4 lo[U], hi[U];
 #pragma unroll
-            for (int u = 0; u < UL; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const bool in = k0 + 32 * u < K;
                 lo[u] = in ? __ldcs(reinterpret_cast<const uint4 *>(wlo + k0 + 32 * u)) : make_uint4(0, 0, 0, 0);
-                hi[u] = (in && ROWS == 16) ? __ldcs(reinterpret_cast<const uint4 *>(whi + k0 + 32 * u)) : make_uint4(0, 0, 0, 0);   // ROWS == 8: the upper half of the tile stays empty
+                hi[u] = in ? __ldcs(reinterpret_cast<const uint4 *>(whi + k0 + 32 * u)) : make_uint4(0, 0, 0, 0);
             }
             if (!synced) { asm volatile("griddepcontrol.wait;" ::: "memory"); synced = true; }
 #pragma unroll
-            for (int u = 0; u < UL; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const uint32_t k = k0 + 32 * u;
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
@@ -1595,7 +1593,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const b
 #pragma unroll
             for (int w = 0; w < NW; ++w) sum += part[w][slot][ln];
             const uint32_t m = b * 8 + 2 * (ln & 3) + (i & 1), row = row0 + (ln >> 2) + 8 * (i >> 1);
-            if (m < Mrows && row < n && (RPC == ROWS || row < row0 + RPC) && (ROWS == 16 || (i >> 1) == 0)) {
+            if (m < Mrows && row < n) {
                 float *p = C + (size_t)m * ldc + col0 + row;
                 if (accumulate) atomicAdd(p, sum);               // one add per element by one thread, not waited for
                 else *p = sum;
@@ -1613,13 +1611,12 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_splitk_kernel(const b
 // in warp order.  A group's arithmetic (which warp adds which k, in which order) depends on the width of these chunks, NW and K alone -
 // not on RG, the rows per group or the list: a block gives the same bits alone or in any list.
 // CS: load steps per chunk, U unless a warp's U steps under way are to cover several of its chunks.
-template <int NB, int U, int NW, int ROWS, int RG, int CS = ROWS == 8 ? 2 * U : U>
+template <int NB, int U, int NW, int RG, int CS = U>
 __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf16 *A, const GemvParts p, uint32_t Mrows, uint32_t groups_total,
                                                               uint32_t K, int accumulate, uint32_t rpc, int acts_early) {
-    constexpr int UL = ROWS == 8 ? 2 * U : U;             // half a tile per load step: twice the steps in flight
-    constexpr int G = RG, SK = UL / (2 * G);              // a register set holds SK load steps of G groups: two sets are as many loads as UL steps of one group
-    static_assert(UL % (2 * G) == 0 && SK >= 1, "row groups per CTA must divide half the load steps");
-    static_assert(UL % CS == 0 && CS % SK == 0, "a register set lies in one chunk");
+    constexpr int G = RG, SK = U / (2 * G);              // a register set holds SK load steps of G groups: two sets are as many loads as U steps of one group
+    static_assert(U % (2 * G) == 0 && SK >= 1, "row groups per CTA must divide half the load steps");
+    static_assert(U % CS == 0 && CS % SK == 0, "a register set lies in one chunk");
     // the warps' partial tiles: static where they fit the 48 KB a kernel may declare, else the launch's dynamic shared memory
     constexpr bool PART_DYNAMIC = NW * G * NB * 4 * 32 * 4 > 48 * 1024;
     __shared__ float part_static[PART_DYNAMIC ? 1 : NW * G * NB * 4 * 32];
@@ -1654,7 +1651,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
                         start += p.groups[s];
                     }
             }
-            // rpc <= ROWS rows per group, chosen by the launcher so that the persistent CTAs all get the same number of
+            // rpc <= 16 rows per group, chosen by the launcher so that the persistent CTAs all get the same number of
             // groups; the tile's rows beyond rpc re-read the group's last row and are not stored (a row's sum does not
             // depend on its place in the tile)
             const uint32_t rlast = min(local * rpc + rpc, n) - 1;
@@ -1670,7 +1667,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
 #pragma unroll
             for (int r = 0; r < G; ++r) {
                 lo[S][r][u] = k < K ? __ldcs(reinterpret_cast<const uint4 *>(wlo[r] + k)) : make_uint4(0, 0, 0, 0);
-                hi[S][r][u] = (k < K && ROWS == 16) ? __ldcs(reinterpret_cast<const uint4 *>(whi[r] + k)) : make_uint4(0, 0, 0, 0);   // ROWS == 8: the upper half of the tile stays empty
+                hi[S][r][u] = k < K ? __ldcs(reinterpret_cast<const uint4 *>(whi[r] + k)) : make_uint4(0, 0, 0, 0);
             }
         }
     };
@@ -1707,7 +1704,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
     };
     const std::integral_constant<int, 0> set0;
     const std::integral_constant<int, 1> set1;
-    // One stream of loads over all the groups this CTA takes.  A warp's chunk of 32 * UL columns is G pairs of load steps;
+    // One stream of loads over all the groups this CTA takes.  A warp's chunk of 32 * U columns is G pairs of load steps;
     // the two register sets alternate, a set is loaded again as soon as its MMAs are issued, so a warp always has one
     // or two sets in flight - also across the end of a group: the next group's first pair is on its way while the CTA
     // meets in shared memory to sum and store the group it has finished, and the memory pipe never drains.  Per group
@@ -1716,12 +1713,12 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
     uint32_t grp = grp0, k0 = warp * 32 * CS, pr = 0;       // the pair that is loaded next: group, first chunk, pair within its chunks
     constexpr uint32_t SET1 = CS == SK ? NW * 32 * CS : 32 * SK;       // from a pair's first set to its second
     auto column = [&]() -> uint32_t {                       // first column of that pair
-        if constexpr (CS == UL) return k0 + pr * 64 * SK;
+        if constexpr (CS == U) return k0 + pr * 64 * SK;
         else return k0 + 2 * pr * SK / CS * (NW * 32 * CS) + 2 * pr * SK % CS * 32;
     };
     auto advance = [&]() -> bool {                         // moves on by one pair; true: the pair just passed ended its group
-        if (++pr == (uint32_t)G) { pr = 0; k0 += NW * 32 * UL; }
-        if (CS == UL ? k0 < K : column() < K) return false;
+        if (++pr == (uint32_t)G) { pr = 0; k0 += NW * 32 * U; }
+        if (CS == U ? k0 < K : column() < K) return false;
         grp += gridDim.x * G;
         k0 = warp * 32 * CS;
         pr = 0;
@@ -1779,7 +1776,7 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
                     }
             }
             const uint32_t m = b * 8 + 2 * (ln & 3) + (i & 1), row = row0 + (ln >> 2) + 8 * (i >> 1);
-            if (m < Mrows && row < min(row0 + rpc, n) && (ROWS == 16 || (i >> 1) == 0)) {
+            if (m < Mrows && row < min(row0 + rpc, n)) {
                 float *out = C + (size_t)m * ldc + row;
                 if (accumulate) atomicAdd(out, sum);             // one add per element by one thread, not waited for
                 else *out = sum;
@@ -1794,8 +1791,8 @@ __global__ void __launch_bounds__(NW * 32) tgp_wstream_mma_group_kernel(const bf
 
 // Which skinny kernel serves a block of n rows at M activation rows: NB groups of 8 activation rows (M <= 16), U load steps in
 // flight, and for blocks too small to give every SM eight 16-row warps the split-K kernel with NW warps per CTA over
-// ROWS rows.  The choice depends on the block alone, so a block computes the same bits alone or as part of a group.
-struct SkinnyPick { int nb, u, nw, rows; bool split, persistent; };
+// 16 rows.  The choice depends on the block alone, so a block computes the same bits alone or as part of a group.
+struct SkinnyPick { int nb, u, nw; bool split, persistent; };
 
 // 9 - 16 activation rows on a block of at least this many weight rows (64 tiles of 128): the tcgen05 kernel is ahead of the
 // mma.sync ones (M=16, from the end of the norm before: two blocks of 28672 rows, K=8192 144 us against 160; two of 8192 rows, K=2048 14.8 / 15.8;
@@ -1845,7 +1842,6 @@ static SkinnyPick pick_skinny(uint32_t M, uint32_t n, uint32_t K) {
         k.nw = 8;
         k.u = 4;
     }
-    k.rows = 16;
     return k;
 }
 
@@ -1855,15 +1851,16 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
     constexpr bool STREAMS = U <= 4;                         // the load depths of the kernels that are not persistent
     if constexpr (STREAMS) {
         if (!blocks_per_sm && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, tgp_wstream_mma_kernel<NB, U>, 256, 0) != cudaSuccess || blocks_per_sm < 1)) blocks_per_sm = 1;
-        if (!blocks_per_sm_split && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm_split, tgp_wstream_mma_splitk_kernel<NB, U, 8, 16>, 256, 0) != cudaSuccess || blocks_per_sm_split < 1))
+        if (!blocks_per_sm_split && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm_split, tgp_wstream_mma_splitk_kernel<NB, U, 8>, 256, 0) != cudaSuccess || blocks_per_sm_split < 1))
             blocks_per_sm_split = 1;
     }
     const uint32_t sms = (uint32_t)device_sms();
-    uint32_t need = 0, rows_total = 0, rpc = (uint32_t)k.rows;
-    if (k.split) for (uint32_t s = 0; s < p.count; ++s) { p.groups[s] = (p.n[s] + k.rows - 1) / k.rows; need += p.groups[s]; rows_total += p.n[s]; }
+    constexpr uint32_t tile = 16;                           // rows of an MMA
+    uint32_t need = 0, rpc = tile;
+    if (k.split) for (uint32_t s = 0; s < p.count; ++s) { p.groups[s] = (p.n[s] + tile - 1) / tile; need += p.groups[s]; }
     else need = (p.n[0] + 16 * 8 - 1) / (16 * 8);           // whole blocks of many rows are launched alone
     const bool persistent = k.persistent;                   // one block or several: the kernel that walks a list of row groups
-    // (the persistent kernels use the whole register file: one CTA per SM)
+    // (one CTA per SM of the persistent kernels: up to 8 activation rows they take the whole register file, above three quarters of it)
     const uint32_t full = persistent ? sms : sms * (uint32_t)(k.split ? blocks_per_sm_split : blocks_per_sm);
     uint32_t per_cta = 1;
     if (persistent) {
@@ -1876,7 +1873,7 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
         // pair with the least estimated time of the busiest CTA: rounds x (G x (r + tile rows) / 2 + 4 NB), in rows read; of equal
         // estimates above 8 activation rows the one of fewer groups and more rows (5120 rows, K=4096 as three rounds of 12 rows 13.2 us at M=9,
         // 14.3 at M=16, as two of 2 x 9 rows 14.3 and 15.5, from the end of the norm before).
-        const uint32_t tile = (uint32_t)k.rows, gmax = 2;
+        const uint32_t gmax = 2;
         uint32_t best = 0xffffffffu, best_r = tile;
         for (uint32_t G = gmax; G >= 1; G >>= 1)
             for (uint32_t r = g_gemv_balance ? tile / 2 + 1 : tile; r <= tile; ++r) {
@@ -1910,12 +1907,12 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
     tgpk_last_gemm_kernel = !k.split ? "tgp_wstream_mma_kernel" : persistent ? "tgp_wstream_mma_group_kernel" : "tgp_wstream_mma_splitk_kernel";
     if (persistent) {
         if constexpr (NB == 2 || U == 8) {                  // (their partial tiles, 32 KB at most, are static)
-            if (per_cta == 2) launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 2>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
-            else launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 16, 1>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
+            if (per_cta == 2) launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 2>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
+            else launch_weights<tgp_wstream_mma_group_kernel<NB, U, 16, 1>>(cfg, A, p, Mrows, total, K, acc, rpc, early);
         }
     } else if constexpr (STREAMS) {
         if (!k.split) launch_weights<tgp_wstream_mma_kernel<NB, U>>(cfg, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);
-        else launch_weights<tgp_wstream_mma_splitk_kernel<NB, U, 8, 16>>(cfg, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);
+        else launch_weights<tgp_wstream_mma_splitk_kernel<NB, U, 8>>(cfg, A, p.W[0], p.C[0], Mrows, p.n[0], K, p.ldc[0], 0u, acc);
     }
 }
 
@@ -2019,7 +2016,7 @@ static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows,
 // tokens, a second one the down projections, and a third adds a token's two results to its residual row.  The counts
 // are read on the device: work items are (expert, up to 8 NB of its tokens, 16 rows of gate and of up, or two groups of `rpc`
 // rows of down), and the CTAs walk the list of those that exist.
-//   The arithmetic of an item is that of tgp_wstream_mma_group_kernel<NB, EXP_U, NW, 16, RG>: which warp adds which k in which order
+//   The arithmetic of an item is that of tgp_wstream_mma_group_kernel<NB, EXP_U, NW, RG>: which warp adds which k in which order
 // depends on K alone, so the bits are those of the expert's own products (tgpk_gemm_rows).
 //   Experts of one or two tokens have no items: their rows follow, a warp each, on the CUDA cores, whose sums are closer to 64 bits
 // (K=1024: 7.1e-8 against 1.3e-7 through mma.sync, K=14336: 9.3e-8 against 8.7e-7), as in the products of one and two rows.
@@ -2288,10 +2285,10 @@ static void launch_expert_rows(cudaLaunchConfig_t &cfg, const bf16 *A, const Gem
         constexpr size_t smem = (size_t)NW * RG * NB * 4 * 32 * 4;
         if constexpr (smem > 48 * 1024) {
             static bool attr_set = false;
-            if (!attr_set) { cudaFuncSetAttribute(tgp_wstream_mma_group_kernel<NB, U, NW, 16, RG, EXP_U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); attr_set = true; }
+            if (!attr_set) { cudaFuncSetAttribute(tgp_wstream_mma_group_kernel<NB, U, NW, RG, EXP_U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); attr_set = true; }
             cfg.dynamicSmemBytes = smem;
         }
-        launch_weights<tgp_wstream_mma_group_kernel<NB, U, NW, 16, RG, EXP_U>>(cfg, A, p, me, groups, K, 0, rpc, 0);
+        launch_weights<tgp_wstream_mma_group_kernel<NB, U, NW, RG, EXP_U>>(cfg, A, p, me, groups, K, 0, rpc, 0);
     };
     if constexpr (NB == 1 && NW == 16)
         if (RG == 2 || K > NW * 32 * EXP_U) return launch(std::integral_constant<int, 2 * EXP_U>());
@@ -2407,7 +2404,7 @@ uint32_t tgpk_gemm_group_key(uint32_t M, uint32_t n, uint32_t K) {
     if (takes_tiles(M, n, K)) return tgpk_gemm_tc_forced() ? 0 : 0x2000000u | tgpk_gemm_tc_class(M, n, K);
     if (M > 16 || K % 32 || g_skinny_impl) return 0;
     const SkinnyPick k = pick_skinny(M, n, K);
-    return k.persistent ? (0x1000000u | (uint32_t)k.nb | (uint32_t)k.u << 4 | (uint32_t)k.nw << 8 | (uint32_t)k.rows << 16) : 0;
+    return k.persistent ? (0x1100000u | (uint32_t)k.nb | (uint32_t)k.u << 4 | (uint32_t)k.nw << 8) : 0;
 }
 
 // Blocks of one key below 0x2000000 over the same activations, in one launch.
