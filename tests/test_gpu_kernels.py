@@ -866,6 +866,27 @@ def test_products_of_9_to_16_rows_alone_and_in_lists_of_several_kernels(M, ns, K
         assert float((a[:, :n].double() - want).abs().max()) < 2e-5 * float(want.abs().max()) + 1e-7
 
 
+# which neighbours of a list share a launch: those of one key, whatever stands between others (q of a wide model takes the tcgen05 kernel at 16
+# rows, its k and v the list kernel); at most eight blocks
+@pytest.mark.parametrize("M,ns,K,kernels", [(16, (8200, 1024, 1000), 4096, ["wstream_tc", "mma_group"]), (9, (16, 8065, 8070, 16, 24), 4096, ["mma_group", "wstream_tc", "mma_group"]),
+                                            (12, (1000, 8200, 1000), 4096, ["mma_group", "wstream_tc", "mma_group"]), (10, (64,) * 8, 2048, ["mma_group"]),
+                                            (1, (4736, 5000), 4096, ["wstream_group"]), (1, (4736, 64, 4736), 4096, ["wstream_kernel", "wstream_kernel", "wstream_kernel"]),
+                                            (2, (64, 100, 4736, 4736), 4096, ["wstream_group", "wstream_group"]), (1, (5000, 4736), 10240, ["wstream_kernel", "wstream_kernel"]),
+                                            (200, (256, 256), 1024, ["tc"])])
+def test_neighbours_of_one_key_share_a_launch(M, ns, K, kernels, tmp_path):
+    A = torch.ones((M, K), device=DEV, dtype=torch.bfloat16)
+    Ws, Cs = [torch.ones((n, K), device=DEV, dtype=torch.bfloat16) for n in ns], [torch.zeros((M, n), device=DEV) for n in ns]
+    call = lambda: tb.k_gemm_group(A, Ws, Cs, M, list(ns), K, list(ns))
+    launched = [name for name, _ in kernels_of(call, tmp_path)]
+    assert len(launched) == len(kernels) and all(k in name for k, name in zip(kernels, launched)), launched
+    assert all(bool((C == K).all()) for C in Cs)
+    tb.k_gemm_group_select(0)
+    try:
+        assert len(kernels_of(call, tmp_path)) == len(ns)
+    finally:
+        tb.k_gemm_group_select(1)
+
+
 # the tcgen05 kernels on either side of their dispatch lines: one tile per CTA unsplit / in 2 / in 4 slices of K (ragged row tiles, K that
 # ends inside a 64-wide block or leaves slices of unequal length), the line at 8192 columns above 128 activation rows, the paired
 # kernel's activation tiles (one of 160 rows, three of 224, the last one ragged), lists of ragged parts

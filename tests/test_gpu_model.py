@@ -578,6 +578,54 @@ def test_router_counts_of_few_tokens(tokens, E, topk, d):
     s.close()
 
 
+@pytest.mark.parametrize("tokens,E,topk,d", [(3, 16, 2, 256), (9, 8, 2, 512), (17, 8, 2, 2304), (33, 16, 2, 256), (64, 4, 2, 512), (64, 8, 1, 256), (65, 8, 2, 256)])
+def test_router_lists_and_gates_of_few_tokens(tokens, E, topk, d):
+    """The rows every expert of layer 0 works on (the tokens that 64-bit logits send to it, in ascending order) and the gates they come back with
+    (the state that the next layer's norm sees), with one and several tokens per CTA of the router and one more than it takes."""
+    cfg = replace(MOE, B=1, S=tokens, T=1, E=E, topk=topk, d=d, F=512, Hq=d // 64, Hkv=d // 128, Dh=64)
+    lay = si.build_layout(cfg, budget=256 << 20, cap=1 << 20)
+    pool = pinned_pool(lay.pool_bytes)
+    si.fill_pool(lay, pool.numpy())
+    bias = si.router_bias(cfg)
+    s = Session(lay, MACHINE, pool_base=pool.data_ptr(), pool_flags=tb.POOL_PINNED, router_bias=bias)
+    s.plan(expert_counts=np.ones((1 + cfg.T, cfg.L, cfg.E), dtype=np.uint32))
+    r = Runner(s, tokens)
+    tap = torch.zeros(128 << 20, dtype=torch.uint8, device="cuda:0")
+    weight = lambda kind, l, e, cols: torch.cat([pool[t.pool_off:t.pool_off + t.rows * cols * 2].view(torch.bfloat16) for t in lay.blocks(kind, l, e)]).view(-1, cols).double()
+    ops, prompt = s.ctx.trace_ops(), si.prompt_tokens(cfg)
+    r.reset()
+    s.ctx.set_tap(tap, tap.numel())
+    r.step(tb.PREFILL, prompt, tokens)
+    r.sync()
+    h, o, a = {}, {}, {}                                   # norms and attention outputs by layer, SwiGLU outputs by layer and expert
+    for (op, tag, sub, off, nbytes) in s.ctx.tap_index().tolist():
+        t = tap[off:off + nbytes].view(torch.bfloat16).double().cpu()
+        if tag == tb.TAP_H:
+            h.setdefault(ops[op][2], []).append(t.view(tokens, d))
+        elif tag == tb.TAP_O:
+            o[ops[op][2]] = t.view(tokens, -1)
+        elif tag == tb.TAP_A:
+            a[ops[op][2], sub] = t.view(-1, cfg.F)
+    s.ctx.set_tap(None, 0)
+    s.close()
+    x = weight(si.K_EMBED, -1, -1, d)[torch.from_numpy(prompt.reshape(-1).astype(np.int64))] + o[0] @ weight(si.K_WO, 0, -1, cfg.Hq * cfg.Dh).T
+    state = h[0][1]
+    logits = state @ weight(si.K_ROUTER, 0, -1, d).T + torch.from_numpy(bias[0]).double()
+    top = logits.sort(dim=1, descending=True)
+    assert (top.values[:, topk - 1] - top.values[:, topk]).min() > 1e-5        # (fp32 sums of d products: no pick hangs on their rounding)
+    picks, gates = top.indices[:, :topk], torch.softmax(top.values[:, :topk], dim=1)
+    for e in range(E):
+        rows, slot = (picks == e).nonzero(as_tuple=True)
+        assert (0, e) not in a if len(rows) == 0 else a[0, e].shape[0] == len(rows)
+        if not len(rows):
+            continue
+        want = torch.nn.functional.silu(state[rows] @ weight(si.K_WG, 0, e, d).T) * (state[rows] @ weight(si.K_WU, 0, e, d).T)
+        assert float(((a[0, e] - want).abs() - 2.0 ** -8 * want.abs()).max()) < 1e-4 * float(want.abs().max())       # half a bf16 step, and fp32 sums
+        x[rows] += gates[rows, slot][:, None] * (a[0, e] @ weight(si.K_WD, 0, e, cfg.F).T)
+    want = x * torch.rsqrt((x * x).mean(dim=1, keepdim=True) + cfg.eps) * weight(si.K_G1, 1, -1, d)
+    assert float(((h[1][0] - want).abs() - 2.0 ** -8 * want.abs()).max()) < 1e-4 * float(want.abs().max())
+
+
 @pytest.mark.parametrize("B,F", [(3, 512), (5, 8192)])
 def test_experts_of_one_or_two_tokens_have_the_sums_of_the_products_of_one_row(B, F):
     """A step of 3 to 32 tokens: what an expert with one or two of them computes is, bit for bit, what k_gemm() and k_swiglu() give for
