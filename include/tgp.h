@@ -302,12 +302,13 @@ int  tgp_k_gemm(const void *A_dev, const void *W_dev, float *C_dev, uint32_t M, 
  * layer, or the pieces a large matrix was registered as): C_dev[s][m, j] (=|+=) sum_k A[m, k] * W_dev[s][j, k] for
  * s < count <= TGP_GEMM_GROUP_MAX, W_dev[s] bf16 [n[s], K], C_dev[s] fp32 with row stride ldc[s] >= n[s]; accumulate != 0
  * adds to C (fused residual).  The pointer and size arrays are host arrays (of device pointers), read before the call
- * returns.  Blocks whose tgp_k_gemm_group_key() is the same non-zero value are served by one launch - a block of few
- * rows alone leaves most SMs without work - anything else by one launch per part; the results are bit-identical to
- * tgp_k_gemm() per part either way, because the key names the kernel the block takes on its own (M <= 2: fewer than
- * 4736 rows of W and K < 8192; to 16 rows with K % 32 == 0: blocks that the persistent list kernel serves, which pick the
- * same instance of it; to 32 rows: blocks that the tcgen05 kernel serves with the same split of K).  Above 32 rows the
- * key is 0, but neighbours in the list that one tcgen05 kernel serves share a launch all the same.
+ * returns.  Neighbours in the list whose tgp_k_gemm_group_key() is the same non-zero value are served by one launch - a block
+ * of few rows alone leaves most SMs without work - anything else, and blocks of one key with another block between them, by one
+ * launch per part; the results are bit-identical to tgp_k_gemm() per part either way, because the key names the kernel the block takes on
+ * its own or one with its sums (M <= 2: fewer than 4736 rows of W and K < 8192, from 4736 rows on K = 4096, 6144 or 8192 at
+ * one row, K a multiple of 2048 at two rows and 4736 - 5328 or 7105 - 8704 rows of W on 148 SMs; to 16 rows with K % 32 == 0:
+ * blocks that the persistent list kernel serves, which pick the same instance of it; to 32 rows: blocks that the tcgen05 kernel serves
+ * with the same split of K).  Above 32 rows the key is 0, but neighbours in the list that one tcgen05 kernel serves share a launch all the same.
  * tgp_k_gemm_group_select(0) makes every key 0 (process-wide; default 1), also inside tgp_step(), which groups
  * consecutive weight-block products of a decode step that read the same activations this way when their copies have
  * all been enqueued and no tap is set, except blocks under 2 MiB whose arena slot a later copy waits for (with op timing
@@ -342,10 +343,12 @@ int  tgp_k_gemm_select(int impl);
 int  tgp_k_skinny_select(int impl);
 /* Products, attention and the small kernels of a step (embedding gather, RMSNorm, RoPE + KV append, SwiGLU, argmax, router and
  * experts of a small step) use programmatic dependent launch: a launch lets its successor be scheduled at once; a
- * weight-streaming kernel of up to 16 rows, and the router of up to 64 tokens, starts reading its weights while the previous
+ * weight-streaming kernel of up to 16 rows, and the router of up to 64 tokens (inside tgp_step() only), starts reading its weights while the previous
  * kernel of the stream drains and waits for it only before it touches activations or output; the product of one weight tile per CTA
  * asks L2 for its first weights then, which reads nothing; every other kernel waits before it reads anything, so that
- * only its launch latency and set-up overlap.  0 switches that off (each launch then starts after the previous one has completed).  Results are
+ * only its launch latency and set-up overlap.  Weights that are read so early must not be written by a kernel still running on the stream:
+ * tgp_step() gives those kernels what copies have brought that the stream has waited for, and a caller of a product of up to 16 rows does the
+ * same; above 16 rows the weights may be what the previous kernel writes.  0 switches that off (each launch then starts after the previous one has completed).  Results are
  * identical either way.  Process-wide; default on. */
 int  tgp_k_gemv_overlap(int enable);
 /* A promise by a caller of the kernel entry points, for the calling thread: between consecutive tgp_k_gemm() /
@@ -402,7 +405,8 @@ int  tgp_k_rope_kv(const float *q32, const float *k32, const float *v32, void *q
 /* Causal GQA attention of q_len new queries per sequence against the tiles (kvlen = pos0 + q_len valid
  * tokens): o = softmax(q K^T / sqrt(Dh)) V, bf16 out [B*q_len, Hq*Dh].  k_tiles/v_tiles as above (host arrays
  * of device pointers).  Dh must be 64 or 128.  scratch_dev: fp32 workspace of
- * tgp_k_attn_scratch_bytes() used when q_len == 1 (split over KV tiles), else may be NULL. */
+ * tgp_k_attn_scratch_bytes() for q_len == 1 (where a context is split over more CTAs than a cluster merges; without it a
+ * slower kernel serves the call), else may be NULL. */
 int  tgp_k_attn(const void *qb, void *const *k_tiles, void *const *v_tiles, uint32_t n_tiles, void *ob,
                 const tgp_model_cfg *cfg, uint32_t B, uint32_t q_len, uint32_t pos0, float *scratch_dev,
                 void *stream);

@@ -2390,14 +2390,13 @@ int tgpk_experts(const TgpExperts &x, cudaStream_t st) {
     return TGP_OK;
 }
 
-// Which products may share a launch: those with the same non-zero key.  A key names the kernel a block takes on its own
+// Which neighbours of a list may share a launch: those with the same non-zero key.  A key names the kernel a block takes on its own
 // (M <= 2: tgp_wstream_kernel<MT, 1, 8>, or a kernel with its sums; 3 <= M <= 32: one instance of the persistent list kernel, or the tcgen05 kernel and
-// split of K); blocks of so many rows that they fill the machine alone, and the shapes served by other kernels, have key 0 and
-// are launched alone.
+// split of K); blocks that gain nothing from a list, and the shapes served by other kernels, have key 0 and are launched alone.
 uint32_t tgpk_gemm_group_key(uint32_t M, uint32_t n, uint32_t K) {
     if (!g_gemm_group || !M || !n || !K || K % 8) return 0;
-    // Blocks of many rows at M <= 2 run one behind the other at little cost, but a list of them has one ramp instead of several: 2 x 14336, K=4096 at
-    // one row 39.0 -> 34.9 us
+    // Blocks of many rows at M <= 2 run one behind the other at little cost, but a list of them has one ramp instead of several (one row,
+    // with the norm before: 2 x 14336, K=4096 41.0 -> 37.0 us).
     if (M <= 2 && n >= GEMV_MANY_ROWS) return one_row_deep(M, K) || two_rows_listed(M, n, K) ? 0x100u | M : 0;
     if (M <= 2) return !(g_gemv_splitk && K >= 8192) ? M : 0;
     if (M > 32) return 0;

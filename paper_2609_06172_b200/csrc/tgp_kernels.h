@@ -12,7 +12,7 @@ struct TgpTilePtrs { void *k[TGP_MAX_TILES]; void *v[TGP_MAX_TILES]; };
 int tgpk_embed(const void *table, const int32_t *tok, float *x, uint32_t M, uint32_t d, uint32_t V, cudaStream_t st);
 int tgpk_rmsnorm(const float *x, uint32_t ldx, const void *g, void *h, uint32_t M, uint32_t d, float eps, cudaStream_t st);
 int tgpk_gemm(const void *A, const void *W, float *C, uint32_t M, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int accumulate, cudaStream_t st);
-// products over the same activations A [M, K]: C[s][m, j] (=|+=) sum_k A[m, k] * W[s][j, k].  Blocks with the same non-zero
+// products over the same activations A [M, K]: C[s][m, j] (=|+=) sum_k A[m, k] * W[s][j, k].  Neighbours with the same non-zero
 // tgpk_gemm_group_key() are served by one launch (up to TGP_GEMM_GROUP_MAX of them), anything else by one launch per part;
 // the bits are the same either way
 uint32_t tgpk_gemm_group_key(uint32_t M, uint32_t n, uint32_t K);
