@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
         nv += 1;
         if ((v_off += BKV) == a.TK) { v_off = 0; v_tile += 1; }
     };
-    if (warp == 5 && lane == 0) {
+    if (warp == 5 && elect_one()) {
         mbar_init(bar_k, 1); mbar_init(bar_k + 1, 1); mbar_init(bar_v, 1); mbar_init(bar_v + 1, 1);
         mbar_init(bar_s, 1); mbar_init(bar_sfree, 128); mbar_init(bar_p, 128); mbar_init(bar_p + 1, 128); mbar_init(bar_o, 1); mbar_init(bar_o + 1, 1); mbar_init(bar_kfree, 1); mbar_init(bar_kfree + 1, 1);
         failed[0] = 0;
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
         asm volatile("setmaxnreg.dec.sync.aligned.u32 64;" ::: "memory");
         if (warp == 5) {
             // ======================= TMA warp: lane 0 requests the remaining K and V blocks =======================
-            if (lane == 0) {
+            if (elect_one()) {
                 // test hook: the first CTA of the grid never loads this V block, so the wait for it runs out
                 const uint32_t withhold = (blockIdx.x | blockIdx.y | blockIdx.z) == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;
                 for (uint32_t jb = 0; jb + 1 < nblk; ++jb) {
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
             for (uint32_t jb = 0; jb < nblk; ++jb) {
                 if (jb >= 1 && !wait(bar_sfree, (jb - 1) & 1, 4)) break;         // S_jb-1 is in registers
                 if (!wait(bar_k + (jb & 1), (jb >> 1) & 1, 3)) break;            // K_jb (and Q with K_0) has landed
-                if (lane == 0) {
+                if (elect_one()) {
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint8_t *Kj = Ks + (jb & 1) * KV_BYTES;
 #pragma unroll
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                 }
-                if (lane == 0) {
+                if (elect_one()) {
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t dv = umma_desc_mn(smem_u32(Vs + st * KV_BYTES), BKV * 128);
 #pragma unroll

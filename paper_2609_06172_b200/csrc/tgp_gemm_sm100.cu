@@ -113,13 +113,13 @@ __global__ void __launch_bounds__(192) tgp_matmul_tc_kernel(const __grid_constan
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t armed = 0;
             const uint32_t withhold = blockIdx.x == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;     // test hook: this stage is never loaded
             for (uint32_t kb = 0; kb < num_k; ++kb) {
                 const uint32_t s = kb % STAGES, ph = (kb / STAGES) & 1;
                 if (kb == withhold) break;
-                if (*failed || !mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } break; }
+                if (!mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } break; }
                 mbar_expect_tx(&full[s], S::STAGE_BYTES);
 #pragma unroll
                 for (int h = 0; h < KH; ++h) {
@@ -135,12 +135,12 @@ __global__ void __launch_bounds__(192) tgp_matmul_tc_kernel(const __grid_constan
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = umma_idesc(BN);
             bool ok = true;
             for (uint32_t kb = 0; kb < num_k && ok; ++kb) {
                 const uint32_t s = kb % STAGES, ph = (kb / STAGES) & 1;
-                if (*failed || !mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
+                if (!mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
                 for (uint32_t h = 0; h < KH; ++h) {
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(192, 1) tgp_matmul_tc_persistent_kernel(const 
     };
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0, armed = 0;
             bool ok = true;
             const uint32_t withhold = blockIdx.x == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;     // test hook: this stage is never loaded
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(192, 1) tgp_matmul_tc_persistent_kernel(const 
                 for (uint32_t kb = 0; kb < num_k; ++kb, ++it) {
                     const uint32_t s = it % P_STAGES, ph = (it / P_STAGES) & 1;
                     if (it == withhold) { ok = false; break; }
-                    if (*failed || !mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } ok = false; break; }
+                    if (!mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } ok = false; break; }
                     mbar_expect_tx(&full[s], STAGE_BYTES);
                     tma_load_2d(smem + s * STAGE_BYTES, &tmA, (int)(kb * BK), (int)m0, &full[s]);
                     tma_load_2d(smem + s * STAGE_BYTES + A_BYTES, &tmB, (int)(kb * BK), (int)n0, &full[s]);
@@ -272,18 +272,18 @@ __global__ void __launch_bounds__(192, 1) tgp_matmul_tc_persistent_kernel(const 
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = umma_idesc(P_BN);
             uint32_t it = 0, lt = 0;
             bool ok = true;
             for (uint32_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++lt) {
                 const uint32_t buf = lt & 1, use = lt >> 1;
-                if (*failed || !mbar_wait(&acc_empty[buf], (use & 1) ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | 0x80 | (int)buf); } break; }
+                if (!mbar_wait(&acc_empty[buf], (use & 1) ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | 0x80 | (int)buf); } break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t tacc = tmem_base + buf * P_BN;
                 for (uint32_t kb = 0; kb < num_k; ++kb, ++it) {
                     const uint32_t s = it % P_STAGES, ph = (it / P_STAGES) & 1;
-                    if (*failed || !mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
+                    if (!mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t da = umma_desc(smem_u32(smem + s * STAGE_BYTES));
                     const uint64_t db = umma_desc(smem_u32(smem + s * STAGE_BYTES + A_BYTES));
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
     };
 
     if (warp == 0) {
-        if (lane == 0) {                              // TMA thread of this CTA: its 128 weight rows, its half of the activation rows
+        if (elect_one()) {                              // TMA thread of this CTA: its 128 weight rows, its half of the activation rows
             asm volatile("griddepcontrol.wait;" ::: "memory");
             uint32_t it = 0, s = 0, ph = 0;
             const uint32_t withhold = pair == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;     // test hook: both CTAs of the first pair never load this stage
@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
                 const CUtensorMap *mw = &p.w[part];
                 for (uint32_t kb = 0; kb < num_k; ++kb, ++it) {
                     if (it == withhold) { ok = false; break; }
-                    if (*failed || !mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } ok = false; break; }
+                    if (!mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } ok = false; break; }
                     if (rank == 0) mbar_expect_tx(&full[s], 2 * STAGE);
 #pragma unroll
                     for (int h = 0; h < KH; ++h) {
@@ -477,18 +477,18 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {                 // MMA thread of the pair
+        if (rank == 0 && elect_one()) {                 // MMA thread of the pair
             asm volatile("griddepcontrol.wait;" ::: "memory");    // the limit of its waits counts from here
             const uint32_t idesc = umma_idesc_pair(N);
             uint32_t s = 0, ph = 0, lt = 0;
             bool ok = true;
             for (uint32_t tile = pair; tile < tiles && ok; tile += pairs, ++lt) {
                 const uint32_t buf = lt & 1, use = lt >> 1;
-                if (*failed || !mbar_wait(&acc_empty[buf], (use & 1) ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | 0x80 | (int)buf); } break; }
+                if (!mbar_wait(&acc_empty[buf], (use & 1) ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | 0x80 | (int)buf); } break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t tacc = tmem_base + buf * buf_cols;
                 for (uint32_t kb = 0; kb < num_k; ++kb) {
-                    if (*failed || !mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
+                    if (!mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
                     for (uint32_t h = 0; h < KH; ++h) {
@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // The weights of the first ring come into L2 while the previous kernel still runs; loading them here would be wrong where that
             // kernel writes them (M=61: n=4096, K=4096 13.3 -> 12.3 us, the list of 2 x 14336 45.7 -> 43.6, with 16 rows 42.4 -> 40.6; from the
             // end of the norm before).  Requests ahead of the ring further on make it slower.
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
             const uint32_t withhold = blockIdx.x == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;     // test hook: this stage is never loaded
             for (uint32_t kb = 0; kb < num_k; ++kb) {
                 if (kb == withhold) break;
-                if (*failed || !mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } break; }
+                if (!mbar_wait(&empty[s], ph ^ 1, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (1 << 8) | (int)s); } break; }
                 mbar_expect_tx(&full[s], STAGE);
                 tma_load_2d(ring + s * STAGE, mw, (int)((kb_lo + kb) * BK), (int)w0, &full[s]);
                 tma_load_2d(ring + s * STAGE + W_BYTES, &p.x, (int)((kb_lo + kb) * BK), (int)m0, &full[s]);
@@ -659,13 +659,13 @@ __global__ void __launch_bounds__(192, 2) tgp_wstream_tc_kernel(const __grid_con
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             asm volatile("griddepcontrol.wait;" ::: "memory");    // the limit of its waits counts from here
             const uint32_t idesc = umma_idesc((int)N);
             uint32_t s = 0, ph = 0;
             bool ok = true;
             for (uint32_t kb = 0; kb < num_k; ++kb) {
-                if (*failed || !mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
+                if (!mbar_wait(&full[s], ph, failed)) { if (!*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, (2 << 8) | (int)s); } ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint64_t dw = umma_desc(smem_u32(ring + s * STAGE)), dx = umma_desc(smem_u32(ring + s * STAGE + W_BYTES));
 #pragma unroll

@@ -24,6 +24,15 @@ static __device__ int g_withhold_step = -1;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// One thread of a converged warp, the same one every time: for the threads that issue TMA copies and MMAs.  Descriptors, coordinates and barrier
+// addresses of these are warp-uniform operands, and behind an election, unlike behind lane == 0, one running thread is what the compiler
+// may assume (a TMA thread with one 16 KB box per barrier: 47 bytes a clock, 75 elected; with two boxes 81 and 126).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ uint64_t now_ns() { uint64_t t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
