@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(192) tgp_matmul_tc_kernel(const __grid_constan
     if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"((uint32_t)BN) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");     // not before the allocation: see tgp_sm100.cuh
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(192) tgp_matmul_tc_kernel(const __grid_constan
 
     if (warp == 0) {
         if (elect_one()) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
             uint32_t armed = 0;
             const uint32_t withhold = blockIdx.x == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;     // test hook: this stage is never loaded
             for (uint32_t kb = 0; kb < num_k; ++kb) {
@@ -136,6 +138,7 @@ __global__ void __launch_bounds__(192) tgp_matmul_tc_kernel(const __grid_constan
         }
     } else if (warp == 1) {
         if (elect_one()) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");    // the limit of its waits counts from here
             constexpr uint32_t idesc = umma_idesc(BN);
             bool ok = true;
             for (uint32_t kb = 0; kb < num_k && ok; ++kb) {
@@ -154,6 +157,7 @@ __global__ void __launch_bounds__(192) tgp_matmul_tc_kernel(const __grid_constan
             if (ok) umma_commit(acc_full);
         }
     } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");        // what C, the gate and a hold is the previous kernel's work
         bool ready = !*failed && mbar_wait(acc_full, 0, failed);
         if (!ready && !*failed) { *failed = 1; atomicCAS(&g_gemm_tc_error, 0, 3 << 8); }
         ready = __all_sync(0xffffffffu, ready && !*failed);      // tcgen05.ld is warp-collective: decide per warp
@@ -345,14 +349,14 @@ __global__ void __launch_bounds__(192, 1) tgp_matmul_tc_persistent_kernel(const 
 }
 
 // ---- paired variant: tiles of 256 weight rows x up to 256 activation rows per CTA pair (cta_group::2) ----------------
-// What limits the kernel above is not the tensor pipe but what an SM can pull from L2: 48 KB per 64-wide K block is
-// 54 B per clock, and the MMA thread waits for data a third of the time.  Here the two CTAs of a pair sit on the two
-// SMs of a TPC and share one MMA: its 256 rows are WEIGHT rows (128 per CTA), its N columns activation rows, of which each
-// CTA loads half - 32 KB per K block at N = 256 for the same arithmetic per SM.  Weights as rows means that a warp's 32
-// TMEM lanes are 32 consecutive columns of C: every store, residual add and gate load of the epilogue is one full line of
+// What limits the kernel above is what an SM can pull from L2: 48 KB per 64-wide K block of 512 cycles, 96 bytes a clock where a full ring brings in 80.
+// Here the two CTAs of a pair sit on the two SMs of a TPC and share one MMA: its 256 rows are WEIGHT rows (128 per CTA), its N columns activation rows, of
+// which each CTA loads half - 32 KB per K block at N = 256 for the same arithmetic per SM.  An MMA takes N / 2 cycles (43 at least).  Weights as
+// rows means that a warp's 32 TMEM lanes are 32 consecutive columns of C: every store, residual add and gate load of the epilogue is one full line of
 // one output row (with activations as rows each lane walked a row of its own: the SwiGLU epilogue of 32768 x 4096 x 4096
-// took 1280 us against 970 us of the plain one), and N follows the batch: ceil(M / tiles) rounded up to 32, so that M = 603
-// costs 3 x 224 rows and not 3 x 256.
+// took 1280 us against 970 us of the plain one), and N, a multiple of 16, follows the batch: M = 603 costs 3 x 208 rows and not 3 x 256.
+//   Few tiles: what counts is not the tensor pipe but the first load (1.5 us), the K blocks' loads (80 bytes a clock) and the stores (32 bytes a
+// clock and SM, 16 for residual adds), so smaller tiles on more SMs are ahead (M=509, n=2048, K=2048: 64 tiles of N=64 11.4 us, 32 of N=128 13.2).
 //   Parts.  Up to TGP_GEMM_GROUP_MAX weight blocks that read the same activations are walked as one list of tiles.
 //   Pairs are persistent, with two accumulators in TMEM: the epilogue of a tile overlaps the MMAs of the next.
 //   A stage holds two 64-wide K blocks (half the barrier hand-overs of one, 4 % faster), p.stages of them.  Only the
@@ -398,6 +402,20 @@ __device__ __forceinline__ void store32(const ListArgs &p, uint32_t part, size_t
     }
 }
 
+// 32 columns of one TMEM lane, summed over four accumulators 128 columns apart: (0 + 1) + (2 + 3)
+__device__ __forceinline__ void sum_four(uint32_t at, float (&v)[32]) {
+    float w[32], y[32];
+    tmem_ld32_pair(at, at + 128, v, w);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] += w[j];
+    tmem_ld32_pair(at + 256, at + 384, w, y);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] += w[j] + y[j];
+}
+
+// SHARED: a tile (of N <= 128) is shared by the two pairs of a cluster, one half of K each, added into four accumulators by turns; the halves meet
+// through shared memory, and each pair stores half of the activation rows.
+template <bool SHARED>
 __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(const __grid_constant__ ListArgs p) {
     extern __shared__ uint8_t smem_raw[];
     constexpr uint32_t W_BYTES = BM * BK * 2;                     // one K block of this CTA's 128 weight rows
@@ -413,10 +431,14 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
     volatile uint32_t *failed = tmem_slot + 1;
     uint8_t *ring = smem + 1024;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_ctarank(), pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
-    const uint32_t num_k = (p.K + KH * BK - 1) / (KH * BK);                         // stages per tile; a block past K reads zeros
+    constexpr uint32_t SL = SHARED ? 2 : 1;
+    const uint32_t cta = cluster_ctarank(), rank = cta & 1, slice = cta >> 1;      // CTA of the cluster, of its pair; its pair
+    const uint32_t pair = blockIdx.x / (2 * SL), pairs = gridDim.x / (2 * SL);      // (clusters, where two pairs share a tile)
+    const uint32_t stages_k = (p.K + KH * BK - 1) / (KH * BK), half_k = (stages_k + 1) / 2;     // stages of all K and of its first half; a block past K reads zeros
+    const uint32_t kb_lo = slice ? half_k : 0, num_k = SL == 1 ? stages_k : slice ? stages_k - half_k : half_k;
     const uint32_t tiles = p.tiles_m * p.tiles_n;
-    const uint32_t buf_cols = N <= 64 ? 64u : N <= 128 ? 128u : 256u;               // TMEM columns of one accumulator
+    const uint32_t buf_cols = SHARED ? 128u : N <= 64 ? 64u : N <= 128 ? 128u : 256u;           // TMEM columns of one accumulator
+    const uint32_t cols = SHARED ? 4 * buf_cols : 2 * buf_cols;
 
     if (threadIdx.x == 0) {
         for (uint32_t s = 0; s < 8; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -425,7 +447,7 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 2) {                                  // the same warp in both CTAs of the pair
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2 * buf_cols) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");     // not before the allocation: see tgp_sm100.cuh
     }
@@ -448,7 +470,7 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
     };
 
     if (warp == 0) {
-        if (elect_one()) {                              // TMA thread of this CTA: its 128 weight rows, its half of the activation rows
+        if (elect_one()) {                            // TMA thread of this CTA: its 128 weight rows, its half of the activation rows
             asm volatile("griddepcontrol.wait;" ::: "memory");
             uint32_t it = 0, s = 0, ph = 0;
             const uint32_t withhold = pair == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;     // test hook: both CTAs of the first pair never load this stage
@@ -463,7 +485,7 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
                     if (rank == 0) mbar_expect_tx(&full[s], 2 * STAGE);
 #pragma unroll
                     for (int h = 0; h < KH; ++h) {
-                        const int k = (int)((kb * KH + h) * BK);
+                        const int k = (int)(((kb_lo + kb) * KH + h) * BK);
                         tma_load_2d_pair(ring + s * STAGE + h * HALF, mw, k, (int)(w0 + rank * BM), &full[s]);
                         tma_load_2d_pair(ring + s * STAGE + h * HALF + W_BYTES, &p.x, k, (int)(m0 + rank * (N / 2)), &full[s]);
                     }
@@ -477,9 +499,9 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (rank == 0 && elect_one()) {                 // MMA thread of the pair
+        if (rank == 0 && elect_one()) {               // MMA thread of the pair
             asm volatile("griddepcontrol.wait;" ::: "memory");    // the limit of its waits counts from here
-            const uint32_t idesc = umma_idesc_pair(N);
+            const uint32_t idesc = umma_idesc_pair(N), mask = 3u << (cta & 2);
             uint32_t s = 0, ph = 0, lt = 0;
             bool ok = true;
             for (uint32_t tile = pair; tile < tiles && ok; tile += pairs, ++lt) {
@@ -495,19 +517,23 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
                         const uint64_t dw = umma_desc(smem_u32(ring + s * STAGE + h * HALF));
                         const uint64_t dx = umma_desc(smem_u32(ring + s * STAGE + h * HALF + W_BYTES));
 #pragma unroll
-                        for (uint32_t k = 0; k < BK / 16; ++k) umma_pair(tacc, dw + 2 * k, dx + 2 * k, idesc, (kb | h | k) != 0);
+                        for (uint32_t k = 0; k < BK / 16; ++k) {
+                            if (SHARED) umma_pair(tacc + k * 128, dw + 2 * k, dx + 2 * k, idesc, (kb | h) != 0);
+                            else umma_pair(tacc, dw + 2 * k, dx + 2 * k, idesc, (kb | h | k) != 0);
+                        }
                     }
-                    umma_commit_pair(&empty[s]);
+                    umma_commit_pair(&empty[s], mask);
                     if (++s == ST) { s = 0; ph ^= 1; }
                 }
-                if (ok) umma_commit_pair(&acc_full[buf]);
+                if (ok) umma_commit_pair(&acc_full[buf], mask);
             }
         }
         __syncwarp();
     } else {
         asm volatile("griddepcontrol.wait;" ::: "memory");        // what C, the gate and a hold is the previous kernel's work
-        const uint32_t quarter = warp & 3, half = (warp - 2) >> 2, wrow = rank * BM + quarter * 32 + lane;
-        uint32_t lt = 0;
+        const uint32_t quarter = warp & 3, half = (warp - 2) >> 2, wrow = rank * BM + quarter * 32 + lane, tm = tmem_base + ((quarter * 32) << 16);
+        uint32_t lt = 0, out = 0, rows_out = 0;       // (a tile that two pairs share: weight block, activation rows, element of C)
+        size_t at_out = 0;
         for (uint32_t tile = pair; tile < tiles; tile += pairs, ++lt) {
             const uint32_t buf = lt & 1, use = lt >> 1;
             uint32_t part, w0, m0;
@@ -519,32 +545,64 @@ __global__ void __launch_bounds__(Q_WARPS * 32, 1) tgp_matmul_tc_pair_kernel(con
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t row = w0 + wrow, ldc = p.ldc[part], rows = min(N, p.M - m0);      // this lane's column of C; activation rows of the tile
             const bool mine = row < p.n[part];
+            if constexpr (SHARED) {                               // the partial sums of the rows that the other pair stores: over the idle ring
+                for (uint32_t c = half * 32; c < N / 2; c += 64) {
+                    float v[32];
+                    sum_four(tm + (slice ^ 1) * (N / 2) + c, v);
+                    float *part_s = reinterpret_cast<float *>(ring) + quarter * 32 + lane;
+#pragma unroll
+                    for (uint32_t j = 0; j < 32; ++j) if (c + j < N / 2) part_s[(c + j) * BM] = v[j];
+                }
+                out = part; at_out = (size_t)m0 * ldc + row; rows_out = mine ? rows : 0;
+                break;                                            // a cluster has one tile
+            } else {
 #pragma unroll 1
-            for (uint32_t c = half * 32; c < N; c += 64) {        // 32 activation rows at a time
-                float v[32];
-                tmem_ld32(tmem_base + ((quarter * 32) << 16) + buf * buf_cols + c, v);
-                store32(p, part, (size_t)(m0 + c) * ldc + row, ldc, v, mine && c < rows ? rows - c : 0);
+                for (uint32_t c = half * 32; c < N; c += 64) {    // 32 activation rows at a time
+                    float v[32];
+                    tmem_ld32(tm + buf * buf_cols + c, v);
+                    store32(p, part, (size_t)(m0 + c) * ldc + row, ldc, v, mine && c < rows ? rows - c : 0);
+                }
             }
             // this warp has read its share of this CTA's half of the buffer: tell the pair's MMA thread
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive_remote(&acc_empty[buf], 0);
+            if (lane == 0) mbar_arrive_remote(&acc_empty[buf], cta & 2);
+        }
+        if constexpr (SHARED) {
+            __syncwarp();
+            cluster_sync_all();                       // every partial sum is in its CTA's shared memory
+            const uint32_t lo = slice * (N / 2);
+            uint32_t bad = 0;
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) bad |= ld_remote_u32(smem_u32((const void *)failed), q);
+            for (uint32_t c = half * 32; c < N / 2; c += 64) {
+                float v[32], w[32];
+#pragma unroll
+                for (uint32_t j = 0; j < 32; ++j) w[j] = ld_remote_f32(smem_u32(ring) + ((c + j) * BM + quarter * 32 + lane) * 4, cta ^ 2);
+                if (bad) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                sum_four(tm + lo + c, v);
+#pragma unroll
+                for (uint32_t j = 0; j < 32; ++j) v[j] += w[j];
+                const uint32_t ldc = p.ldc[out];
+                store32(p, out, at_out + (size_t)(lo + c) * ldc, ldc, v, lo + c < rows_out ? min(rows_out - lo, N / 2) - c : 0);
+            }
         }
     }
+    if (SHARED && warp < 2) cluster_sync_all();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncwarp();
     cluster_sync_all();                               // neither CTA frees TMEM or leaves while its partner may still touch it
     if (warp == 2) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * buf_cols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(cols) : "memory");
     }
 }
 
 // ---- up to 128 activation rows, and products of few tiles: one tile of 128 weight rows per CTA ----------------------
 // A product of up to 128 activation rows is bound by HBM, one of more rows and few tiles by the length of K.  Every CTA takes 128
 // weight rows (the rows of the MMA; N <= 128 activation rows, a multiple of 16, are its columns) and a slice of K.  One CTA
-// per MMA and not a pair: an MMA costs 75 cycles for N <= 128, a pair's 128 for any N <= 256 (112 SMs of pairs would take
-// their weights in no faster than HBM delivers them), and there are four times as many tiles to share out.
+// per MMA and not a pair: there are four times as many tiles to share out, and the tensor pipe (48 cycles an MMA at N = 64, 64 at 128) waits for HBM.
 //   K slices: a block of few tiles is split along K over the SL CTAs of a cluster; their partial tiles meet in shared memory
 // and are summed pairwise.  The split depends on M, n, K and the number of SMs: a block computes the same bits alone or in a list.
 //   Accumulators: consecutive MMAs go to different ones (eight up to 32 activation rows, four up to 64, else two), summed at the end.
@@ -759,9 +817,13 @@ static bool launch_tile(const CUtensorMap &ma, const CUtensorMap &mb, float *C, 
         if (cudaFuncSetAttribute(tgp_matmul_tc_kernel<BN, ST, KH, SWAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<BN, ST, KH>::TOTAL) != cudaSuccess) return false;
         attr_set = true;
     }
-    dim3 grid(((M + BM - 1) / BM) * ((n + BN - 1) / BN));
-    tgp_matmul_tc_kernel<BN, ST, KH, SWAP><<<grid, 192, Smem<BN, ST, KH>::TOTAL, st>>>(ma, mb, C, M, n, K, ldc, col0, accumulate, ep);
-    return true;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(((M + BM - 1) / BM) * ((n + BN - 1) / BN)); cfg.blockDim = dim3(192); cfg.dynamicSmemBytes = Smem<BN, ST, KH>::TOTAL; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, tgp_matmul_tc_kernel<BN, ST, KH, SWAP>, ma, mb, C, M, n, K, ldc, col0, accumulate, ep) == cudaSuccess;
 }
 
 static int g_tc_variant = 0;     // 0 by size (see the top of this file), 1 force the 128x128 per-tile kernel, 2 the persistent 128x256 kernel, 3 the paired
@@ -775,65 +837,77 @@ static uint32_t tc_sms() {
     return (uint32_t)sms;
 }
 
-// K slices of a block in the one-tile-per-CTA kernel, 0: the paired kernel serves it.  The choice depends on M, n and K of the block and
-// on the number of SMs (the bits of a sliced product may differ between devices of different sizes), not on a list.  Measured (us; M=61 unless stated):
+// Does the paired kernel share the tiles of a block between two pairs?  Blocks of more than 128 activation rows and K >= 8192, more tiles than the one-tile-per-CTA
+// kernel holds in one wave of slices and at most a cluster's tile each in one wave.  The sums are those of half of K in four accumulators each, as near 64 bits as
+// that kernel's four slices with two (M=509, n=2048, K=8192: 29.2 us in slices, 23.9 shared; M=150, n=4096, K=14336: 44.8, 41.8; but n=2048, K=8192
+// 16.8, 18.3).  With a shorter K sharing gains 5 % at best over smaller tiles.  The choice depends on M, n and K of the block and on the
+// number of SMs (the bits may differ between devices of different sizes), not on a list.
+static bool shared_tiles(uint32_t M, uint32_t n, uint32_t K) {
+    const uint64_t rows = (M + BM - 1) / BM, sms = tc_sms();
+    return M > BM && K >= 8192 && rows * ((n + BM - 1) / BM) * 4 > sms && rows * ((n + 2 * BM - 1) / (2 * BM)) * 4 <= sms;
+}
+
+// K slices of a block in the one-tile-per-CTA kernel, 0: the paired kernel serves it.  No list counts here either.  Measured (us; M=61):
 //   n=4096, K=4096        22.4 unsplit, 15.3 in two slices, 11.9 in four, 12.4 in eight
 //   n=2048, K=8192        41.6, 24.7, 15.4, 21.1 (few clusters of eight fit the GPU at a time: no eight anywhere)
 //   n=8192, K=8192        42.4, 28.1, 26.4 (256 CTAs, two per SM)
 //   n=8192 twice, K=2048  14.4, 16.5, 22.2; n=32000, K=4096: 46.2, 51.3, 62.3
-//   M=509, n=2048, K=8192 22.7 in four slices, 33.9 in pairs; M=200, n=4096, K=14336: 35.2, 55.5; M=603, n=4096+1024+1024, K=4096:
-//                         26.5 in pairs, 35 with k and v in slices of their own; M=256, n=4096+1024+1024 and 4096, K=4096: 39.6 in pairs, 45.8
 static uint32_t cta_slices(uint32_t M, uint32_t n, uint32_t K) {
-    const uint32_t tiles = (n + BM - 1) / BM * ((M + BM - 1) / BM), sms = tc_sms();
-    if (tiles * 4 <= 2 * sms && K >= 8192) return 4;
-    if (M > BM) return 0;
-    if (tiles * 4 <= sms && K >= 1024) return 4;
+    const uint64_t tiles = (uint64_t)((n + BM - 1) / BM) * ((M + BM - 1) / BM), sms = tc_sms();
+    if (M > BM) return tiles * 4 <= 2 * sms && K >= 8192 && !shared_tiles(M, n, K) ? 4 : 0;
+    if (tiles * 4 <= (K >= 8192 ? 2 * sms : sms) && K >= 1024) return 4;
     return tiles * 2 <= sms && K >= 1024 ? 2 : 1;
 }
 
-// Estimated cycles of the paired kernel for `wt` tiles of 256 weight rows at M activation rows in tiles of N: a K block of a
-// pair takes 512 cycles of the tensor pipe at any N <= 256, and (16384 + 64 N) bytes per SM from L2 at 40 bytes a clock.
-static uint64_t pair_cost(uint32_t M, uint32_t wt, uint32_t K, uint32_t N, uint32_t pairs) {
-    const uint64_t kblocks = (K + BK - 1) / BK, tiles = (uint64_t)((M + N - 1) / N) * wt;
-    return (tiles + pairs - 1) / pairs * (kblocks * std::max<uint64_t>(512, (16384 + 64 * N) / 40) + 600);
+// Estimated cycles of the paired kernel for `wt` tiles of 256 weight rows at M activation rows in tiles of N, with room for `at_once` tiles.  A 64-wide block of K
+// of a pair takes 2 N cycles of the tensor pipe (172 at least) and (16384 + 64 N) bytes per SM, which arrive at 80 a clock (what a full ring
+// asks for in the 1.4 us a load takes); the first stage arrives after 3000 cycles, and a tile's epilogue writes 512 N bytes per SM at 32 a clock (a few
+// of them are under way when it ends: 1600 cycles), under the MMAs of the next tile.
+static uint64_t pair_cost(uint32_t M, uint32_t wt, uint32_t K, uint32_t N, uint32_t at_once) {
+    const uint64_t tiles = (uint64_t)((M + N - 1) / N) * wt, rounds = (tiles + at_once - 1) / at_once;
+    const uint64_t mma = (uint64_t)((K + BK - 1) / BK) * std::max<uint64_t>(std::max(2 * N, 172u), (16384 + 64 * N) / 80), epi = 16 * N;
+    return 3000 + mma + (rounds - 1) * std::max(mma, epi) + epi + 1600;
 }
 
-// Activation rows per tile: the fewest tiles that hold M rows, or up to two more where smaller tiles fill the pairs better.
-static uint32_t pair_rows(uint32_t M, uint32_t wt, uint32_t K, uint32_t pairs) {
-    const uint32_t t0 = (M + 255) / 256;
+// Activation rows per tile: what the estimate above says is fastest (us with the norm before; estimates rank the choices as the clock does: M=509, n=2048, K=2048
+// N=128 13.9, 96 12.8, 64 12.1; M=603, n=4096 and 1024 twice, K=4096 N=208 30.3, 160 38.1, 112 34.0; M=1024, n=2048, K=2048 N=256 21.1, 176 17.3, 128 14.4).
+static uint32_t pair_rows(uint32_t M, uint32_t wt, uint32_t K, uint32_t at_once, uint32_t most) {
+    const uint32_t t0 = (M + most - 1) / most, unit = most == 256 ? 16 : 32;            // (shared: each pair stores half of them)
     uint32_t best = 0;
     uint64_t cost = 0;
-    for (uint32_t t = t0; t <= (g_tc_variant == 3 ? t0 : t0 + 2); ++t) {                 // (forced: the largest tiles)
-        const uint32_t N = ((M + t - 1) / t + 31) / 32 * 32;
-        const uint64_t c = pair_cost(M, wt, K, N, pairs);
-        if (!best || c < cost) { best = N; cost = c; }
+    for (uint32_t t = t0; t <= (g_tc_variant == 3 ? t0 : t0 + 8); ++t) {                 // (forced: the largest tiles)
+        const uint32_t N = std::max(32u, ((M + t - 1) / t + unit - 1) / unit * unit);
+        const uint64_t c = pair_cost(M, wt, K, N, at_once);
+        if (!best || c * 25 < cost * 24) { best = N; cost = c; }                          // (of equals the largest: less traffic, and less power)
     }
     return best;
 }
 
+constexpr uint32_t Q_RING = 227u * 1024u - 2048u;
+
+template <bool SHARED>
 static int launch_pair(ListArgs &p, cudaStream_t st) {
-    constexpr uint32_t RING = 227u * 1024u - 2048u;
     static bool attr_set = false;
     if (!attr_set) {
-        if (cudaFuncSetAttribute(tgp_matmul_tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, RING + 2048) != cudaSuccess) return TGP_E_CUDA;
+        if (cudaFuncSetAttribute(tgp_matmul_tc_pair_kernel<SHARED>, cudaFuncAttributeMaxDynamicSharedMemorySize, Q_RING + 2048) != cudaSuccess) return TGP_E_CUDA;
         attr_set = true;
     }
     const uint32_t stage = KH * (BM * BK * 2 + p.N / 2 * BK * 2);
-    p.stages = std::min(8u, RING / stage);
-    const uint32_t tiles = p.tiles_m * p.tiles_n, pairs_max = tc_sms() / 2;
+    p.stages = std::min(8u, Q_RING / stage);
+    const uint32_t tiles = p.tiles_m * p.tiles_n;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * std::min(tiles, pairs_max));
+    cfg.gridDim = dim3(SHARED ? 4 * tiles : 2 * std::min(tiles, tc_sms() / 2));
     cfg.blockDim = dim3(Q_WARPS * 32);
     cfg.dynamicSmemBytes = 2048 + p.stages * stage;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[0].val.clusterDim.x = SHARED ? 4 : 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, tgp_matmul_tc_pair_kernel, p) == cudaSuccess ? TGP_OK : TGP_E_CUDA;
+    return cudaLaunchKernelEx(&cfg, tgp_matmul_tc_pair_kernel<SHARED>, p) == cudaSuccess ? TGP_OK : TGP_E_CUDA;
 }
 
 static int launch_stream(ListArgs &p, cudaStream_t st) {
@@ -859,7 +933,8 @@ static int launch_stream(ListArgs &p, cudaStream_t st) {
     return cudaLaunchKernelEx(&cfg, tgp_wstream_tc_kernel, p) == cudaSuccess ? TGP_OK : TGP_E_CUDA;
 }
 
-uint32_t tgpk_gemm_tc_class(uint32_t M, uint32_t n, uint32_t K) { return cta_slices(M, n, K) + 1; }
+// Blocks of one class may share a launch: kernel, slices of K and accumulators are the same.
+uint32_t tgpk_gemm_tc_class(uint32_t M, uint32_t n, uint32_t K) { return cta_slices(M, n, K) + 1 + (shared_tiles(M, n, K) ? 8 : 0); }
 
 // Blocks of equal tgpk_gemm_tc_class() over the same activations, in one launch.
 int tgpk_gemm_tc_list(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t M, uint32_t K,
@@ -884,26 +959,27 @@ int tgpk_gemm_tc_list(const void *A, uint32_t count, const void *const *W, float
         const uint32_t t = (M + BM - 1) / BM;
         p.N = ((M + t - 1) / t + 15) / 16 * 16;
     } else {
-        p.slices = 1;
-        p.N = pair_rows(M, p.tiles_n, K, tc_sms() / 2);
+        p.slices = g_tc_variant != 3 && shared_tiles(M, n[0], K) ? 2 : 1;
+        p.N = p.slices == 2 ? pair_rows(M, p.tiles_n, K / 2, tc_sms() / 4, 128) : pair_rows(M, p.tiles_n, K, tc_sms() / 2, 256);
     }
     p.tiles_m = (M + p.N - 1) / p.N;
     if (!make_map(&p.x, A, M, K, stream ? p.N : p.N / 2)) return TGP_E_CUDA;
     for (uint32_t s = 0; s < count; ++s) if (!make_map(&p.w[s], W[s], n[s], K, BM)) return TGP_E_CUDA;
-    const int rc = stream ? launch_stream(p, st) : launch_pair(p, st);
+    const int rc = stream ? launch_stream(p, st) : p.slices == 2 ? launch_pair<true>(p, st) : launch_pair<false>(p, st);
     if (rc) return rc;
     tgpk_launches += 1;
     tgpk_last_gemm_kernel = stream ? "tgp_wstream_tc_kernel" : "tgp_matmul_tc_pair_kernel";
     return TGP_OK;
 }
 
-// Weight rows per tile if the one-tile-per-CTA kernel serves a block of more than 128 activation rows that is launched alone, else 0.  A pair
-// takes 128 cycles an MMA however few its tiles are, one CTA 75 (N <= 128), so where narrow tiles give every CTA one the length of K
-// counts less (us: M=256, K=4096 n=512 16.2 against 18.2 in pairs, n=1024 17.0 / 18.7; M=509, K=6144, n=2048 24.5 / 27.2, n=1024
-// 23.0 / 26.6, but K=2048, n=2048 even).  Both kernels add K in one order into one accumulator: the bits are those of the pairs, which a list takes.
+// Weight rows per tile if the one-tile-per-CTA kernel serves a block of more than 128 activation rows that is launched alone, else 0: where its narrow
+// tiles are one wave.  Without a cluster's barriers it is level with the pairs or ahead of them for a short K or four tiles of rows and more, up to a
+// tenth behind for a longer K (us with the norm before: M=1024, n=512, K=512 7.1 against 8.3 in pairs, K=2048 10.5 / 11.8; M=509, n=512, K=512
+// 6.5 / 6.5; M=256, n=1024, K=2048 9.4 / 8.9).  Stages of two blocks of K for 32 weight rows (M=129, n=512, K=4096: three blocks 14.9, one 14.3, two 12.5).
+// Both kernels add K in one order into one accumulator: the bits are those of the pairs, which a list takes.
 static uint32_t lone_tile(uint32_t M, uint32_t n, uint32_t K) {
-    if (M <= BM || n > 2048 || (n > 1024 && K < 4096) || cta_slices(M, n, K)) return 0;
-    const uint32_t bn = n > 1024 ? 64 : 32;
+    if (M <= BM || n > 2048 || (n > 1024 && K < 4096) || cta_slices(M, n, K) || shared_tiles(M, n, K)) return 0;
+    const uint32_t bn = n > 1024 && (M + BM - 1) / BM * ((n + 31) / 32) > tc_sms() ? 64 : 32;
     return (M + BM - 1) / BM * ((n + bn - 1) / bn) <= tc_sms() ? bn : 0;
 }
 
@@ -917,7 +993,7 @@ int tgpk_gemm_tc(const void *A, const void *W, float *C, uint32_t M, uint32_t n,
     if (const uint32_t bn = g_tc_variant == 0 && !ep.aout ? lone_tile(M, n, K) : 0) {
         CUtensorMap ma, mb;
         if (!make_map(&ma, A, M, K, BM) || !make_map(&mb, W, n, K, bn)) return TGP_E_CUDA;
-        if (!(bn == 32 ? launch_tile<32, 3, 3>(ma, mb, C, M, n, K, ldc, col0, accumulate, st) : launch_tile<64, 3, 3>(ma, mb, C, M, n, K, ldc, col0, accumulate, st))) return TGP_E_CUDA;
+        if (!(bn == 32 ? launch_tile<32, 5, 2>(ma, mb, C, M, n, K, ldc, col0, accumulate, st) : launch_tile<64, 8, 1>(ma, mb, C, M, n, K, ldc, col0, accumulate, st))) return TGP_E_CUDA;
         if (cudaGetLastError() != cudaSuccess) return TGP_E_CUDA;
         tgpk_launches += 1;
         tgpk_last_gemm_kernel = "tgp_matmul_tc_kernel";

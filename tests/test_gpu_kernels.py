@@ -1228,3 +1228,45 @@ def test_products_of_few_tiles_alone_have_the_bits_of_the_pairs(M, n, K, alone):
         assert torch.equal(one, pair[0]) and torch.equal(one, pair[1]) and torch.equal(one[:, n:], c0[:, n:])
         exact = want + (c0[:, :n].double() if acc else 0)
         assert float((one[:, :n].double() - exact).abs().max()) < 2e-5 * float(exact.abs().max())
+
+
+@pytest.mark.parametrize("M,n,K", [(129, 4097, 8192), (150, 4096, 8200), (257, 2100, 8192), (509, 2048, 8200), (512, 2048, 14336), (1100, 1000, 8328), (256, 4700, 8192)])
+def test_products_of_a_long_k_whose_tiles_two_pairs_share(M, n, K):
+    """More than 128 activation rows, K >= 8192 and few tiles: a block alone and in a list of 2 and of 8 (more clusters than fit the GPU at a time) has
+    the same bits, no other column changes, and it is as near the fp64 product as fp32 sums are."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(M + n + K)
+    A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
+    W = (torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16()
+    want = A.double() @ W.double().T
+    for acc in (False, True):
+        c0 = torch.randn((M, n + 4), device=DEV, generator=gen)
+        one = c0.clone()
+        tb.k_gemm(A, W, one, M, n, K, n + 4, 0, acc)
+        exact = want + (c0[:, :n].double() if acc else 0)
+        for parts in (2, 8):
+            C = [c0.clone() for _ in range(parts)]
+            tb.k_gemm_group(A, [W] * parts, C, M, [n] * parts, K, [n + 4] * parts, acc)
+            torch.cuda.synchronize()
+            assert tb.k_gemm_status() == 0
+            assert all(torch.equal(one, c) for c in C) and torch.equal(one[:, n:], c0[:, n:])
+        # K / 128 additions in each of eight chains, each off by at most a unit of 2^-23 of the running sum (see the real prefill shapes above)
+        assert float((one[:, :n].double() - exact).abs().max()) < 2e-5 * max(1.0, K / 8192) * float(exact.abs().max())
+
+
+@pytest.mark.parametrize("M,n,K", [(129, 4096, 520), (200, 2300, 72), (401, 2048, 1032), (603, 1500, 264), (1030, 1100, 2056)])
+def test_products_in_small_tiles_of_pairs_have_the_bits_of_the_largest(M, n, K):
+    """Activation rows per tile (16 to 256, by the number of tiles) do not change the sums: the automatic choice and the largest tiles, forced."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(M + n + K)
+    A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
+    W = (torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16()
+    out = [torch.full((M, n), 7.0, device=DEV) for _ in range(2)]
+    tb.k_gemm_group(A, [W, W], [out[0], torch.empty_like(out[0])], M, [n, n], K, [n, n], False)
+    tb.k_gemm_tc_variant(3)
+    tb.k_gemm(A, W, out[1], M, n, K, n, 0, 0)
+    tb.k_gemm_tc_variant(0)
+    torch.cuda.synchronize()
+    assert tb.k_gemm_status() == 0 and torch.equal(out[0], out[1])
+    want = A.double() @ W.double().T
+    assert float((out[0].double() - want).abs().max()) < 2e-5 * float(want.abs().max())
