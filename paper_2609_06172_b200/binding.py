@@ -148,7 +148,31 @@ def lib():
         l.tgp_strerror.argtypes, l.tgp_strerror.restype = [C.c_int], C.c_char_p
         l.tgp_last_error.argtypes, l.tgp_last_error.restype = [_P], C.c_char_p
         _lib = l
+        _load_fastcall(l)
     return _lib
+
+
+class _General:
+    """In the place of the extension that calls the kernel entry points without ctypes: until the library is loaded, and where that extension is not built.
+    Its functions do nothing and say so, and the call takes the general path."""
+
+    def __getattr__(self, name):
+        lib()
+        return (lambda *a: None) if _fast is self else getattr(_fast, name)
+
+
+_fast = _General()
+
+
+def _load_fastcall(l):
+    global _fast
+    try:
+        from . import _fastcall
+    except ImportError:
+        return
+    _fastcall.bind(tuple(C.cast(getattr(l, "tgp_k_" + n), C.c_void_p).value for n in ("embed", "rmsnorm", "gemm", "gemm_group", "rope_kv", "attn", "swiglu", "argmax")),
+                   ModelCfg, np.ndarray)
+    _fast = _fastcall
 
 
 def exported_symbols():
@@ -450,7 +474,11 @@ def _k(rc, where):
 
 
 def k_embed(table, tok, x, M, d, V, stream=None):
-    _k(lib().tgp_k_embed(_ptr(table), _ptr(tok), _ptr(x), M, d, V, _ptr(stream)), "tgp_k_embed")
+    rc = _fast.embed(table, tok, x, M, d, V, stream)
+    if rc is None:
+        rc = lib().tgp_k_embed(_ptr(table), _ptr(tok), _ptr(x), M, d, V, _ptr(stream))
+    if rc:
+        raise TgpError(rc, "tgp_k_embed")
 
 
 def k_embed_status():
@@ -469,18 +497,29 @@ def k_status_clear():
 
 
 def k_rmsnorm(x, ldx, g, h, M, d, eps, stream=None):
-    _k(lib().tgp_k_rmsnorm(_ptr(x), ldx, _ptr(g), _ptr(h), M, d, eps, _ptr(stream)), "tgp_k_rmsnorm")
+    rc = _fast.rmsnorm(x, ldx, g, h, M, d, eps, stream)
+    if rc is None:
+        rc = lib().tgp_k_rmsnorm(_ptr(x), ldx, _ptr(g), _ptr(h), M, d, eps, _ptr(stream))
+    if rc:
+        raise TgpError(rc, "tgp_k_rmsnorm")
 
 
 def k_gemm(A, W, Cout, M, n, K, ldc, col0, accumulate, stream=None):
-    _k(lib().tgp_k_gemm(_ptr(A), _ptr(W), _ptr(Cout), M, n, K, ldc, col0, int(accumulate), _ptr(stream)), "tgp_k_gemm")
+    rc = _fast.gemm(A, W, Cout, M, n, K, ldc, col0, accumulate, stream)
+    if rc is None:
+        rc = lib().tgp_k_gemm(_ptr(A), _ptr(W), _ptr(Cout), M, n, K, ldc, col0, int(accumulate), _ptr(stream))
+    if rc:
+        raise TgpError(rc, "tgp_k_gemm")
 
 
 def k_gemm_group(A, Ws, Couts, M, ns, K, ldcs, accumulate=False, stream=None):
     """Products of the same activations A [M, K] with several weight blocks Ws[s] [ns[s], K] into Couts[s] (row stride ldcs[s])."""
-    c = len(Ws)
-    _k(lib().tgp_k_gemm_group(_ptr(A), c, _pointers(Ws, c), _pointers(Couts, c),
-                              (_U32 * c)(*ns), (_U32 * c)(*ldcs), M, K, int(accumulate), _ptr(stream)), "tgp_k_gemm_group")
+    rc = _fast.gemm_group(A, Ws, Couts, M, ns, K, ldcs, accumulate, stream)
+    if rc is None:
+        c = len(Ws)
+        rc = lib().tgp_k_gemm_group(_ptr(A), c, _pointers(Ws, c), _pointers(Couts, c), (_U32 * c)(*ns), (_U32 * c)(*ldcs), M, K, int(accumulate), _ptr(stream))
+    if rc:
+        raise TgpError(rc, "tgp_k_gemm_group")
 
 
 def k_gemm_group_key(M, n, K):
@@ -557,13 +596,21 @@ def k_rope_tables(Dh, max_len, base, cos, sin):
 
 
 def k_rope_kv(q32, k32, v32, qb, k_tiles, v_tiles, cos, sin, cfg, B, q_len, pos0, stream=None):
-    ka, va, n = _tile_arrays(k_tiles, v_tiles)
-    _k(lib().tgp_k_rope_kv(_ptr(q32), _ptr(k32), _ptr(v32), _ptr(qb), ka, va, n, _ptr(cos), _ptr(sin), C.byref(cfg), B, q_len, pos0, _ptr(stream)), "tgp_k_rope_kv")
+    rc = _fast.rope_kv(q32, k32, v32, qb, k_tiles, v_tiles, cos, sin, cfg, B, q_len, pos0, stream)
+    if rc is None:
+        ka, va, n = _tile_arrays(k_tiles, v_tiles)
+        rc = lib().tgp_k_rope_kv(_ptr(q32), _ptr(k32), _ptr(v32), _ptr(qb), ka, va, n, _ptr(cos), _ptr(sin), C.byref(cfg), B, q_len, pos0, _ptr(stream))
+    if rc:
+        raise TgpError(rc, "tgp_k_rope_kv")
 
 
 def k_attn(qb, k_tiles, v_tiles, ob, cfg, B, q_len, pos0, scratch=None, stream=None):
-    ka, va, n = _tile_arrays(k_tiles, v_tiles)
-    _k(lib().tgp_k_attn(_ptr(qb), ka, va, n, _ptr(ob), C.byref(cfg), B, q_len, pos0, _ptr(scratch), _ptr(stream)), "tgp_k_attn")
+    rc = _fast.attn(qb, k_tiles, v_tiles, ob, cfg, B, q_len, pos0, scratch, stream)
+    if rc is None:
+        ka, va, n = _tile_arrays(k_tiles, v_tiles)
+        rc = lib().tgp_k_attn(_ptr(qb), ka, va, n, _ptr(ob), C.byref(cfg), B, q_len, pos0, _ptr(scratch), _ptr(stream))
+    if rc:
+        raise TgpError(rc, "tgp_k_attn")
 
 
 STATIC_SCRATCH_BYTES = 4 << 20
@@ -583,8 +630,16 @@ def k_attn_scratch_bytes(cfg):
 
 
 def k_swiglu(g, u, ab, n, stream=None):
-    _k(lib().tgp_k_swiglu(_ptr(g), _ptr(u), _ptr(ab), n, _ptr(stream)), "tgp_k_swiglu")
+    rc = _fast.swiglu(g, u, ab, n, stream)
+    if rc is None:
+        rc = lib().tgp_k_swiglu(_ptr(g), _ptr(u), _ptr(ab), n, _ptr(stream))
+    if rc:
+        raise TgpError(rc, "tgp_k_swiglu")
 
 
 def k_argmax(logits, out, B, V, stream=None):
-    _k(lib().tgp_k_argmax(_ptr(logits), _ptr(out), B, V, _ptr(stream)), "tgp_k_argmax")
+    rc = _fast.argmax(logits, out, B, V, stream)
+    if rc is None:
+        rc = lib().tgp_k_argmax(_ptr(logits), _ptr(out), B, V, _ptr(stream))
+    if rc:
+        raise TgpError(rc, "tgp_k_argmax")

@@ -534,3 +534,47 @@ def test_null_tiles_are_refused_where_the_call_uses_them():
         with pytest.raises(tb.TgpError) as e:
             tb.k_attn_decode_static(16, k, v, 16, mc, 1, p)
         assert e.value.code == tb.E_INVAL
+
+
+def test_calls_without_ctypes_take_and_refuse_what_the_general_path_does(monkeypatch):
+    """The extension's functions leave what they do not know to the general path, having done nothing, and return the library's code for the rest: the same
+    outcome with and without them, for arguments of every kind (no rows, or refused: nothing is launched)."""
+    import torch
+    t, a = torch.zeros(64), np.zeros(64, dtype=np.float32)
+    mc = tb.ModelCfg()
+    mc.B, mc.Hq, mc.Hkv, mc.Dh, mc.TK, mc.max_len = 1, 2, 1, 64, 16, 48
+
+    class Holder:
+        cuda_stream = 0
+
+    def outcome(f):
+        try:
+            return f()
+        except tb.TgpError as e:
+            return "TgpError", e.code, str(e)
+        except Exception as e:
+            return type(e), str(e)
+
+    calls = []
+    for p in (None, 16, True, t, torch.nn.Parameter(t), t[3:], a, "x", 1.5, Holder(), [1]):
+        calls += [lambda p=p: tb.k_embed(p, 16, p, 0, 8, 8), lambda p=p: tb.k_rmsnorm(p, 8, p, 16, 0, 8, 1e-5, 0), lambda p=p: tb.k_gemm(p, 16, p, 0, 8, 8, 8, 0, False),
+                  lambda p=p: tb.k_gemm(16, p, 16, 1, 8, 12, 8, 0, 0), lambda p=p: tb.k_swiglu(p, p, 16, 0), lambda p=p: tb.k_argmax(p, 16, 0, 8), lambda p=p: tb.k_rmsnorm(16, 8, 16, 16, 0, 8, 1e-5, p),
+                  lambda p=p: tb.k_gemm_group(p, [16, p], [16, 16], 0, [8, 8], 64, [8, 8]), lambda p=p: tb.k_attn(16, [p], [16], 16, mc, 0, 1, 0, p)]
+    for n in (0, np.uint32(0), 0.0, True, None, "0", -1 << 32, 1 << 32):
+        calls += [lambda n=n: tb.k_embed(16, 16, 16, n, 8, 8) if n is not True else None, lambda n=n: tb.k_rmsnorm(16, 8, 16, 16, n, 8, 1e-5) if n is not True else None, lambda n=n: tb.k_gemm(16, 16, 16, 0, 8, 8, 8, 0, n),
+                  lambda n=n: tb.k_gemm_group(16, [16], [16], 0, [n], 64, [8]), lambda n=n: tb.k_rope_kv(16, 16, 16, 16, [16], [16], 16, 16, mc, 0, 1, n), lambda n=n: tb.k_rmsnorm(16, 8, 16, 16, 0, 8, n)]
+    for k, v in (([], []), ([16], (32,)), ((16, 32), [16]), ([16], [16, 32]), (range(2), [16, 32]), ([16] * 300, [16] * 300), (t.tolist()[:1], [16]), (16, 16)):
+        calls += [lambda k=k, v=v: tb.k_attn(16, k, v, 16, mc, 0, 1, 0), lambda k=k, v=v: tb.k_rope_kv(16, 16, 16, 16, k, v, 16, 16, mc, 0, 1, 0),
+                  lambda k=k, v=v: tb.k_gemm_group(16, k, v, 0, [8] * 2, 64, [8] * 2), lambda k=k, v=v: tb.k_gemm_group(16, [16, 16], [16, 16], 0, k, 64, v)]
+    for c in (None, 16, tb.Machine(), a):
+        calls += [lambda c=c: tb.k_attn(16, [16], [16], 16, c, 0, 1, 0), lambda c=c: tb.k_rope_kv(16, 16, 16, 16, [16], [16], 16, 16, c, 0, 1, 0)]
+    calls.append(lambda: tb.k_gemm(A=16, W=16, Cout=16, M=0, n=8, K=8, ldc=8, col0=0, accumulate=False, stream=None))
+    calls.append(lambda: tb.k_gemm(16, 16))
+    tb.lib()
+    assert tb._fast.__name__.endswith("_fastcall")
+    assert tb._fast.gemm(t, 16, 16, 0, 8, 8, 8, 0, False, None) == 0 and tb._fast.gemm(a, 16, 16, 0, 8, 8, 8, 0, False, None) is None
+    fast = [outcome(f) for f in calls]
+    monkeypatch.setattr(tb, "_fast", tb._General())
+    monkeypatch.setattr(tb._General, "__getattr__", lambda self, name: lambda *args: None)
+    assert fast == [outcome(f) for f in calls]
+    assert sum(o is None for o in fast) > 40 and sum(isinstance(o, tuple) for o in fast) > 40
