@@ -665,6 +665,7 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
     // every kernel of the step is launched from here on the compute stream: consecutive products over the same activations
     // may read them before their predecessor has finished
     struct ChainScope { bool was; ChainScope() : was(tgpk_chain_ok) { tgpk_chain_ok = true; } ~ChainScope() { tgpk_chain_ok = was; } } chain_scope;
+    struct EdgeScope { ~EdgeScope() { tgpk_whole_edge = false; } } edge_scope;
     // however the step ends, tgp_expert_counts() waits for the router kernels it has launched
     struct CountScope {
         TgpEngine *e; cudaStream_t cs; size_t before;
@@ -769,6 +770,9 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
                 cudaEvent_t ev;
                 if ((rc = get_event(ctx, e->copied_ev, j, &ev))) return rc;
                 CU(ctx, cudaStreamWaitEvent(cs, ev, 0));
+                // in a graph an edge from a load kernel and a programmatic one into the same node make the graph six times as long to instantiate (16 steps: 10.7 against
+                // 2.8 ms), and the kernel has the load to wait for anyway
+                tgpk_whole_edge = e->capturing && e->small_loads;
             }
         const uint32_t ti = i - st.op0;
         if (e->op_timing) {
@@ -910,6 +914,7 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
         default:
             return tgp_fail(ctx, TGP_E_MISMATCH, "op kind the bound model cannot run");
         }
+        tgpk_whole_edge = false;
         if (rc) return tgp_fail(ctx, rc, "kernel launch failed");
         if (e->tap) {
             auto tap_copy = [&](uint64_t tag, uint64_t sub, const void *src, uint64_t bytes) -> int {
@@ -1180,6 +1185,7 @@ extern "C" int tgp_run_capture_end(tgp_ctx *ctx) {
     }
     e->graph = g;
     CU(ctx, cudaGraphInstantiate(&e->graph_exec, e->graph, 0));
+    if (e->small_loads) CU(ctx, cudaGraphUpload(e->graph_exec, e->cap_cs));      // (or the first launch would take a third longer than the next)
     return TGP_OK;
 }
 

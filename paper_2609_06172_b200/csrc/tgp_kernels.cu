@@ -61,6 +61,8 @@ static int device_sms() {
 }
 
 static int g_small_pdl = 1;      // small kernels are launched as programmatic dependents of their predecessor (0: plain launches)
+thread_local bool tgpk_whole_edge = false;     // this thread's next launches wait for their predecessors as a whole, however the switches stand
+static int small_overlap() { return g_small_pdl && !tgpk_whole_edge ? 1 : 0; }
 
 template <typename... KArgs, typename... Args>
 static void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
@@ -68,7 +70,7 @@ static void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = small_overlap();
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
@@ -1435,7 +1437,7 @@ int tgpk_router(const void *h, const void *Wr, const float *bias, int32_t *idx, 
     cfg.gridDim = dim3(M <= 2 ? M : M <= 4 ? 4 : 8); cfg.blockDim = dim3(ROUTE_WARPS * 32); cfg.stream = st;        // one cluster
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = small_overlap();
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = cfg.gridDim.x; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
@@ -1498,7 +1500,7 @@ static int g_gemm_group = 1;     // products over the same activations: one laun
 bool tgpk_gemm_grouping() { return g_gemm_group != 0; }
 static int g_gemv_balance = 1;   // grouped skinny launches: rows per group chosen so that every persistent CTA gets the same number of groups
 static int g_gemv_pdl = 1;       // consecutive weight-streaming launches may overlap (programmatic dependent launch)
-bool tgpk_launch_overlap() { return g_gemv_pdl != 0; }
+bool tgpk_launch_overlap() { return g_gemv_pdl != 0 && !tgpk_whole_edge; }
 
 // Launches a kernel that streams weights through registers.  Its loads under way take up L1, 64 KB of them and more per SM, and a kernel without a
 // preference of its own runs on the split of L1 and shared memory that the SM has: next to nothing is left of L1 behind an attention or tcgen05
@@ -1533,7 +1535,7 @@ static void launch_gemv(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, 
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     launch_weights<tgp_wstream_kernel<MT, R, U>>(cfg, A, W, C, Mrows, n, K, ldc, col0, acc);
@@ -1894,7 +1896,7 @@ static void launch_skinny(const bf16 *A, GemvParts p, const SkinnyPick &k, uint3
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     uint32_t total = 0;
@@ -1938,7 +1940,7 @@ static void launch_gemv_splitk(const bf16 *A, const bf16 *W, float *C, uint32_t 
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     launch_weights<tgp_wstream_splitk_kernel<MT, RB, U>>(cfg, A, W, C, Mrows, n, K, ldc, col0, acc);
@@ -2002,7 +2004,7 @@ static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows,
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     launch_weights<tgp_wstream_group_kernel<MT, 8, FUSED>>(cfg, A, p, Mrows, n_total, K, acc, src);
@@ -2335,7 +2337,7 @@ int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *c
     cfg.gridDim = dim3(std::min((groups + RG - 1) / RG, full)); cfg.blockDim = dim3(nw * 32); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = g_gemv_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
 #define TGP_EXPERT_ROWS(NB_) do { \
@@ -2355,7 +2357,7 @@ static void launch_experts(const ExpertParts &p, uint32_t T, cudaStream_t st) {
     cfg.gridDim = dim3(16 / warps * (uint32_t)device_sms()); cfg.blockDim = dim3(32 * warps); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = small_overlap();
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (warps == 8) { if (T == 8) launch_weights<tgp_expert_mma_kernel<1, 8, GLU>>(cfg, p); else launch_weights<tgp_expert_mma_kernel<2, 8, GLU>>(cfg, p); }
@@ -2567,7 +2569,7 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
             cfg.gridDim = dim3(parts, c->Hkv, B); cfg.blockDim = dim3(DEC_WARPS * 32); cfg.dynamicSmemBytes = smem; cfg.stream = st;
             cudaLaunchAttribute attr[2];
             attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;
+            attr[0].val.programmaticStreamSerializationAllowed = small_overlap();
             attr[1].id = cudaLaunchAttributeClusterDimension;
             attr[1].val.clusterDim.x = parts; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
             cfg.attrs = attr;
@@ -2643,7 +2645,7 @@ int tgpk_argmax(const float *logits, int32_t *out, int32_t *out2, uint32_t B, ui
     cfg.gridDim = dim3(B * parts); cfg.blockDim = dim3(256); cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = g_small_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = small_overlap();
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = parts; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;

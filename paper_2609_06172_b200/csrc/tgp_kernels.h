@@ -31,6 +31,7 @@ int tgpk_gemm_tc_list(const void *A, uint32_t count, const void *const *W, float
 // a kernel other than the automatic choice is selected (tgp_k_gemm_tc_variant)
 bool tgpk_gemm_tc_forced();
 // programmatic dependent launches are switched on (tgp_k_gemv_overlap)
+extern thread_local bool tgpk_whole_edge;      // (and this thread has not set them aside for its next launches)
 bool tgpk_launch_overlap();
 // true if a product of M activation rows takes the tensor-core GEMM, whose epilogue can apply SwiGLU (M > 128, tensor cores selected)
 bool tgpk_swiglu_fusable(uint32_t M);
