@@ -699,6 +699,7 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
         int32_t g_expert = -1;
         bool g_gather = false, g_scatter = false;
         uint32_t gbase = i;                                  // first product of the span (after a fused norm / SwiGLU op: i + 1)
+        bool with_attn = false;                              // op i is the rotation and append of a decode step, op i + 1 its attention
         int fuse = 0;                                        // 1: op i is an RMSNorm computed by its consumers; 2: a SwiGLU computed by its consumers
         // products from op `base` on that may share a launch: same layer, activations, accumulation, K and group key
         auto form_group = [&](uint32_t base, uint32_t *key_out) -> uint32_t {
@@ -738,6 +739,11 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
                 g_gather |= r.kind == TGP_K_WG && r.row0 == 0;
                 g_scatter |= r.kind == TGP_K_WD && r.row0 + r.rows == c.d;
             }
+        } else if (ring && o.kind == TGP_OP_ROPE_KV && !e->tap && q_len == 1 && i + 1 < st.op0 + st.nops && ctx->ops[i + 1].kind == TGP_OP_ATTN && ctx->ops[i + 1].layer == o.layer &&
+                   !ctx->plan.op_is_wait_target[i] && (ctx->plan.op_last_place[i] < 0 || (size_t)ctx->plan.op_last_place[i] < e->next_cmd) &&
+                   (ctx->plan.op_last_place[i + 1] < 0 || (size_t)ctx->plan.op_last_place[i + 1] < e->next_cmd)) {
+            span = 2;                                    // the decode attention rotates and appends for itself (bit for bit), where its kernel can
+            with_attn = true;
         } else if (ring && g_fuse_small && !e->tap && !c.E && q_len == 1 && M <= 2 && (o.kind == TGP_OP_RMSNORM || o.kind == TGP_OP_SWIGLU) &&
                    i + 1 < st.op0 + st.nops && (ctx->plan.op_last_place[i] < 0 || (size_t)ctx->plan.op_last_place[i] < e->next_cmd)) {
             // Launch-bound decode steps of small models (one or two sequences, rows of at most 1024 elements): the products
@@ -879,21 +885,25 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
             TgpTilePtrs tp;
             memset(&tp, 0, sizeof(tp));
             uint32_t nt = 0;
-            for (uint32_t k = 0; k < o.nacc; ++k) {
-                const TgpRole *rp = role_of(ctx, o, k);
+            const TgpOp &ot = with_attn ? ctx->ops[i + 1] : o;           // whose tiles: attention's are all up to the new position's
+            for (uint32_t k = 0; k < ot.nacc; ++k) {
+                const TgpRole *rp = role_of(ctx, ot, k);
                 if (!rp || (rp->kind != TGP_K_KTILE && rp->kind != TGP_K_VTILE)) return tgp_fail(ctx, TGP_E_MISMATCH, "attention op on a tensor that is not a bound KV tile");
                 const TgpRole &r = *rp;
                 if (r.block >= TGP_MAX_TILES) return tgp_fail(ctx, TGP_E_TOO_LARGE, "KV tile index");
-                (r.kind == TGP_K_KTILE ? tp.k : tp.v)[r.block] = where(ctx, o, k);
+                (r.kind == TGP_K_KTILE ? tp.k : tp.v)[r.block] = where(ctx, ot, k);
                 nt = std::max(nt, r.block + 1);
             }
             {   // every tile the kernel will address must have been listed by the op (an append touches the tiles of the new
                 // positions, attention every tile below the cached length)
-                const uint32_t t_lo = o.kind == TGP_OP_ROPE_KV ? pos0 / c.TK : 0, t_hi = (pos0 + q_len - 1) / c.TK;
+                const uint32_t t_lo = ot.kind == TGP_OP_ROPE_KV ? pos0 / c.TK : 0, t_hi = (pos0 + q_len - 1) / c.TK;
                 for (uint32_t j = t_lo; j <= t_hi; ++j)
                     if (j >= TGP_MAX_TILES || !tp.k[j] || !tp.v[j]) return tgp_fail(ctx, TGP_E_MISMATCH, "the trace does not list a KV tile this step addresses");
             }
-            if (o.kind == TGP_OP_ROPE_KV) rc = tgpk_rope_kv(e->q32, e->k32, e->v32, e->qb, tp, e->cos_t, e->sin_t, &c, B, q_len, pos0, cs);
+            if (with_attn) {
+                const TgpRopeIn in{e->q32, e->k32, e->v32, e->cos_t, e->sin_t};
+                rc = tgpk_attn(e->qb, tp, (c.max_len + c.TK - 1) / c.TK, e->ob, &c, B, q_len, pos0, e->scratch, cs, &in);
+            } else if (o.kind == TGP_OP_ROPE_KV) rc = tgpk_rope_kv(e->q32, e->k32, e->v32, e->qb, tp, e->cos_t, e->sin_t, &c, B, q_len, pos0, cs);
             else rc = tgpk_attn(e->qb, tp, (c.max_len + c.TK - 1) / c.TK, e->ob, &c, B, q_len, pos0, e->scratch, cs);
             break;
         }

@@ -508,6 +508,10 @@ __global__ void __launch_bounds__(256) tgp_matmul_simt_kernel(const bf16 *A, con
 }
 
 // ---- RoPE + bf16 rounding + KV append -----------------------------------------------------------
+// A dimension and its partner half a head away, rotated, with explicit roundings: the decode attention that rotates for itself gives the same bits.
+__device__ __forceinline__ float rope_lo(float x0, float x1, float c, float s) { return __fmaf_rn(x0, c, -__fmul_rn(x1, s)); }
+__device__ __forceinline__ float rope_hi(float x0, float x1, float c, float s) { return __fmaf_rn(x1, c, __fmul_rn(x0, s)); }
+
 struct RopeArgs {
     const float *q32, *k32, *v32; bf16 *qb; const float *cos_t, *sin_t;
     uint32_t Hq, Hkv, Dh, TK, q_len, pos0;
@@ -526,15 +530,15 @@ __global__ void tgp_rope_kv_kernel(RopeArgs a) {
             const float *s = a.q32 + (size_t)m * qd + h * a.Dh;
             float x0 = s[i], x1 = s[i + half], c = cs[i], sv = sn[i];
             bf16 *o = a.qb + (size_t)m * qd + h * a.Dh;
-            o[i] = __float2bfloat16_rn(x0 * c - x1 * sv);
-            o[i + half] = __float2bfloat16_rn(x1 * c + x0 * sv);
+            o[i] = __float2bfloat16_rn(rope_lo(x0, x1, c, sv));
+            o[i + half] = __float2bfloat16_rn(rope_hi(x0, x1, c, sv));
         } else if (h < a.Hq + a.Hkv) {
             const uint32_t hk = h - a.Hq;
             const float *s = a.k32 + (size_t)m * kd + hk * a.Dh;
             float x0 = s[i], x1 = s[i + half], c = cs[i], sv = sn[i];
             bf16 *o = reinterpret_cast<bf16 *>(a.tiles.k[j]) + ((size_t)(b * a.Hkv + hk) * a.TK + slot) * a.Dh;
-            o[i] = __float2bfloat16_rn(x0 * c - x1 * sv);
-            o[i + half] = __float2bfloat16_rn(x1 * c + x0 * sv);
+            o[i] = __float2bfloat16_rn(rope_lo(x0, x1, c, sv));
+            o[i + half] = __float2bfloat16_rn(rope_hi(x0, x1, c, sv));
         } else {
             const uint32_t hk = h - a.Hq - a.Hkv;
             const float *s = a.v32 + (size_t)m * kd + hk * a.Dh;
@@ -565,8 +569,8 @@ __global__ void __launch_bounds__(256) tgp_rope_kv_vec_kernel(RopeArgs a) {
         if (rot) {
             const float4 c = *reinterpret_cast<const float4 *>(a.cos_t + (size_t)pos * HALF + i), sv = *reinterpret_cast<const float4 *>(a.sin_t + (size_t)pos * HALF + i);
             const float4 y0 = x0, y1 = x1;
-            x0 = make_float4(y0.x * c.x - y1.x * sv.x, y0.y * c.y - y1.y * sv.y, y0.z * c.z - y1.z * sv.z, y0.w * c.w - y1.w * sv.w);
-            x1 = make_float4(y1.x * c.x + y0.x * sv.x, y1.y * c.y + y0.y * sv.y, y1.z * c.z + y0.z * sv.z, y1.w * c.w + y0.w * sv.w);
+            x0 = make_float4(rope_lo(y0.x, y1.x, c.x, sv.x), rope_lo(y0.y, y1.y, c.y, sv.y), rope_lo(y0.z, y1.z, c.z, sv.z), rope_lo(y0.w, y1.w, c.w, sv.w));
+            x1 = make_float4(rope_hi(y0.x, y1.x, c.x, sv.x), rope_hi(y0.y, y1.y, c.y, sv.y), rope_hi(y0.z, y1.z, c.z, sv.z), rope_hi(y0.w, y1.w, c.w, sv.w));
         }
         bf16 *o = h < a.Hq ? a.qb + (size_t)m * qd + hk * DH
                            : reinterpret_cast<bf16 *>(rot ? a.tiles.k[j] : a.tiles.v[j]) + ((size_t)(b * a.Hkv + hk) * a.TK + slot) * DH;
@@ -583,6 +587,7 @@ struct AttnArgs {
     float scale;
     TgpTilePtrs tiles;
     uint32_t n_parts;                 // partials per head the merge kernel reads; 0: one per KV tile with valid keys
+    TgpRopeIn rope;                   // of the instances that rotate for themselves: the new position's projections and the tables
 };
 
 // One warp per query row, 32 keys per pass: lane = key for the scores, lane = output dims for P.V.
@@ -945,7 +950,10 @@ __device__ __forceinline__ float fast_ex2(float x) { float y; asm("ex2.approx.ft
 // shared memory leaves room for: told so, the compiler keeps its loads apart with 177 - 179 registers at DH = 128; left to itself it takes 141 to 165,
 // by what the instance holds besides, and is up to 20 % slower: 8 heads over one, 9000 keys of one sequence 19.1 -> 15.0 us with the norm before, in clusters 3 - 6 %.  All bits of P
 // take 151 registers at DH = 64, and the few CTAs they are for fit an SM in threes.)
-template <int DH, int G, bool SPLIT_P, bool CLUSTER>
+// ROPE: the kernel does what tgp_rope_kv_vec_kernel does, too, with its bits: every CTA rotates its queries in registers, and the warp whose chunk holds the new
+// position rotates its key, puts key and value into the stage behind the copies, and writes both to the tiles.  One launch and its hand-over less per layer
+// of a decode step (one sequence, 32 heads over 8 x 64, 300 keys: 6.1 us for both, 4.6 so).
+template <int DH, int G, bool SPLIT_P, bool CLUSTER, bool ROPE>
 __global__ void __launch_bounds__(DEC_WARPS * 32, DH == 128 ? 2 : SPLIT_P ? 3 : 4) tgp_attn_decode_mma_kernel(AttnArgs a, uint32_t chunks_per_cta) {
     pdl_enter();
     extern __shared__ __align__(128) uint8_t dec_sm[];
@@ -961,7 +969,39 @@ __global__ void __launch_bounds__(DEC_WARPS * 32, DH == 128 ? 2 : SPLIT_P ? 3 : 
 
     // Q fragments of this group: rows 0..G-1 real, the rest zero; held in registers for the whole kernel
     uint32_t qf[DH / 16][2];
-    {
+    constexpr uint32_t HALF = DH / 2;
+    auto bits2 = [](float lo, float hi) { const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi); return *reinterpret_cast<const uint32_t *>(&p); };
+    uint32_t new_k[2] = {0u, 0u}, new_v[2] = {0u, 0u};                // ROPE: dimensions 2 lane and half a head on of the new key and value
+    const uint32_t in_tiles = ROPE ? kvlen - 1 : kvlen;               // keys that the tiles hold
+    if constexpr (ROPE) {
+        const float *cs = a.rope.cos_t + (size_t)a.pos0 * HALF, *sn = a.rope.sin_t + (size_t)a.pos0 * HALF;
+        const float *q = a.rope.q32 + ((size_t)b * a.Hq + hk * G + (r < G ? r : 0)) * DH;
+#pragma unroll
+        for (int ks = 0; ks < DH / 32; ++ks)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const uint32_t i = ks * 16 + 2 * c + 8 * e;
+                const float2 x0 = *reinterpret_cast<const float2 *>(q + i), x1 = *reinterpret_cast<const float2 *>(q + HALF + i);
+                const float2 co = *reinterpret_cast<const float2 *>(cs + i), si = *reinterpret_cast<const float2 *>(sn + i);
+                qf[ks][e] = r < G ? bits2(rope_lo(x0.x, x1.x, co.x, si.x), rope_lo(x0.y, x1.y, co.y, si.y)) : 0u;
+                qf[ks + DH / 32][e] = r < G ? bits2(rope_hi(x0.x, x1.x, co.x, si.x), rope_hi(x0.y, x1.y, co.y, si.y)) : 0u;
+            }
+        if (q_hi == nchunks && (nchunks - 1 - q_lo) % DEC_WARPS == warp && 2 * lane < HALF) {      // this warp has the chunk of the new position
+            const size_t row = ((size_t)b * a.Hkv + hk) * DH;
+            const uint32_t i = 2 * lane, tile = a.pos0 / a.TK;
+            const float2 x0 = *reinterpret_cast<const float2 *>(a.rope.k32 + row + i), x1 = *reinterpret_cast<const float2 *>(a.rope.k32 + row + HALF + i);
+            const float2 v0 = *reinterpret_cast<const float2 *>(a.rope.v32 + row + i), v1 = *reinterpret_cast<const float2 *>(a.rope.v32 + row + HALF + i);
+            const float2 co = *reinterpret_cast<const float2 *>(cs + i), si = *reinterpret_cast<const float2 *>(sn + i);
+            new_k[0] = bits2(rope_lo(x0.x, x1.x, co.x, si.x), rope_lo(x0.y, x1.y, co.y, si.y));
+            new_k[1] = bits2(rope_hi(x0.x, x1.x, co.x, si.x), rope_hi(x0.y, x1.y, co.y, si.y));
+            new_v[0] = bits2(v0.x, v0.y);
+            new_v[1] = bits2(v1.x, v1.y);
+            const size_t at = (((size_t)b * a.Hkv + hk) * a.TK + (a.pos0 - tile * a.TK)) * DH + i;
+            bf16 *kt = reinterpret_cast<bf16 *>(a.tiles.k[tile]) + at, *vt = reinterpret_cast<bf16 *>(a.tiles.v[tile]) + at;
+            *reinterpret_cast<uint32_t *>(kt) = new_k[0]; *reinterpret_cast<uint32_t *>(kt + HALF) = new_k[1];
+            *reinterpret_cast<uint32_t *>(vt) = new_v[0]; *reinterpret_cast<uint32_t *>(vt + HALF) = new_v[1];
+        }
+    } else {
         const bf16 *q = a.qb + ((size_t)b * a.Hq + hk * G) * DH + (size_t)r * DH;
 #pragma unroll
         for (int ks = 0; ks < DH / 16; ++ks) {
@@ -979,7 +1019,7 @@ __global__ void __launch_bounds__(DEC_WARPS * 32, DH == 128 ? 2 : SPLIT_P ? 3 : 
         for (uint32_t i = 0; i < DEC_KEYS * CPR / 32; ++i) {
             const uint32_t idx = i * 32 + lane, row = idx / CPR, j = idx % CPR;
             const uint32_t dst = row * ROW + ((j ^ (row & 7)) << 4);
-            const uint32_t nbytes = key0 + row < kvlen ? 16u : 0u;  // rows past the sequence are written as zeros, not read
+            const uint32_t nbytes = key0 + row < in_tiles ? 16u : 0u;  // rows past the sequence are written as zeros, not read
             cp_async16(base + dst, kg + (size_t)row * ROW + j * 16, nbytes);
             cp_async16(base + KV_BYTES + dst, vg + (size_t)row * ROW + j * 16, nbytes);
         }
@@ -1008,6 +1048,17 @@ __global__ void __launch_bounds__(DEC_WARPS * 32, DH == 128 ? 2 : SPLIT_P ? 3 : 
         __syncwarp();
         const uint32_t q = q_lo + warp + it * DEC_WARPS, key0 = q * DEC_KEYS;
         const uint32_t kb = mine_u + (it % DEC_STAGES) * STAGE, vb = kb + KV_BYTES;
+        if (ROPE && q + 1 == nchunks) {                               // the new position's row, over the zeros that the copy has put there
+            const uint32_t row = a.pos0 - key0;
+            if (2 * lane < HALF)
+#pragma unroll
+                for (uint32_t e = 0; e < 2; ++e) {
+                    const uint32_t i = 2 * lane + e * HALF, at = row * ROW + ((i / 8 ^ (row & 7)) << 4) + i % 8 * 2;
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(kb + at), "r"(new_k[e]) : "memory");
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(vb + at), "r"(new_v[e]) : "memory");
+                }
+            __syncwarp();
+        }
         // ---- S = Q K^T: two n-tiles of 8 keys ----
         float sacc[2][4];
 #pragma unroll
@@ -2516,11 +2567,32 @@ static int g_attn_decode_grouped = 1;   // decode: one pass over a KV tile serve
 static int g_attn_decode_impl = 0;      // decode: 0 and 2 the tensor-core kernel wherever its geometry allows, 1 the CUDA-core per-tile kernels only
 static int g_attn_impl = 0;      // q_len >= 16: 0 by problem size, 3 tcgen05 kernel, 2 mma.sync flash kernel, 1 warp-per-row CUDA-core kernel
 
+// Does the tensor-core decode kernel serve a step?  Whole 16-key chunks inside a tile, 16-byte aligned rows, 1, 2, 4 or 8 query heads per KV head.  It is ahead at any
+// length (us with the merge, against the per-tile kernels: 40 keys of 4 heads 1.8 / 4.3, which is one CTA per head and no merge; one sequence
+// of 32 over 8 heads x 64, 130 keys 4.2 / 5.8, 700 keys 4.9 / 6.6; 1500 keys of 8 heads over 1 x 128: 6.7 / 13.3)
+static bool decode_mma(const void *qb, const TgpTilePtrs &tiles, const tgp_model_cfg *c, uint32_t q_len, uint32_t pos0, const float *scratch) {
+    const uint32_t G = c->Hq / c->Hkv, nt = (pos0 + 1 + c->TK - 1) / c->TK;
+    if (q_len != 1 || !scratch || !g_attn_decode_grouped || (G != 1 && G != 2 && G != 4 && G != 8) || c->Hq % c->Hkv || g_attn_decode_impl == 1 || c->TK % DEC_KEYS) return false;
+    bool aligned = (reinterpret_cast<uintptr_t>(qb) & 3u) == 0;
+    for (uint32_t t = 0; t < nt && aligned; ++t) aligned = ((reinterpret_cast<uintptr_t>(tiles.k[t]) | reinterpret_cast<uintptr_t>(tiles.v[t])) & 15u) == 0;
+    return aligned;
+}
+
+// (rope: the projections of a decode step's new position, not yet rotated; qb is then written only where the two ops are launched apart)
 int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0,
-              float *scratch, cudaStream_t st) {
+              float *scratch, cudaStream_t st, const TgpRopeIn *rope) {
     if (!B || !q_len) return TGP_OK;
     if (c->Dh != 64 && c->Dh != 128) return TGP_E_INVAL;
-    AttnArgs a{(const bf16 *)qb, (bf16 *)ob, scratch, c->Hq, c->Hkv, c->Dh, c->TK, q_len, pos0, n_tiles, 1.0f / sqrtf((float)c->Dh), tiles};
+    AttnArgs a{(const bf16 *)qb, (bf16 *)ob, scratch, c->Hq, c->Hkv, c->Dh, c->TK, q_len, pos0, n_tiles, 1.0f / sqrtf((float)c->Dh), tiles, 0, {}};
+    bool rotates = false;
+    if (rope) {
+        const uintptr_t bits = reinterpret_cast<uintptr_t>(rope->q32) | reinterpret_cast<uintptr_t>(rope->k32) | reinterpret_cast<uintptr_t>(rope->v32) |
+                               reinterpret_cast<uintptr_t>(rope->cos_t) | reinterpret_cast<uintptr_t>(rope->sin_t);
+        const uint32_t G = c->Hkv ? c->Hq / c->Hkv : 0;
+        rotates = decode_mma(qb, tiles, c, q_len, pos0, scratch) && (bits & 15u) == 0 && G * c->Hkv == c->Hq;
+        if (rotates) a.rope = *rope;
+        else if (int rc = tgpk_rope_kv(rope->q32, rope->k32, rope->v32, const_cast<void *>(qb), tiles, rope->cos_t, rope->sin_t, c, B, q_len, pos0, st)) return rc;
+    }
     if (q_len == 1 && scratch) {
         const uint32_t nt = (pos0 + 1 + c->TK - 1) / c->TK, G = c->Hq / c->Hkv;
         if (G > 32) return TGP_E_TOO_LARGE;
@@ -2529,13 +2601,8 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
         if (split < 1) split = 1;
         dim3 grid(nt, c->Hkv, B);
         const bool grouped = g_attn_decode_grouped && (G == 1 || G == 2 || G == 4 || G == 8) && c->Hq % c->Hkv == 0;
-        // tensor-core decode kernel: whole 16-key chunks inside a tile, 16-byte aligned rows.  It is ahead at any length (us with
-        // the merge, against the per-tile kernels: 40 keys of 4 heads 1.8 / 4.3, which is one CTA per head and no merge; one sequence
-        // of 32 over 8 heads x 64, 130 keys 4.2 / 5.8, 700 keys 4.9 / 6.6; 1500 keys of 8 heads over 1 x 128: 6.7 / 13.3)
         const uint32_t nchunks = (pos0 + 1 + DEC_KEYS - 1) / DEC_KEYS;
-        bool aligned16 = (reinterpret_cast<uintptr_t>(qb) & 3u) == 0;
-        for (uint32_t t = 0; t < nt && aligned16; ++t) aligned16 = ((reinterpret_cast<uintptr_t>(tiles.k[t]) | reinterpret_cast<uintptr_t>(tiles.v[t])) & 15u) == 0;
-        if (grouped && g_attn_decode_impl != 1 && c->TK % DEC_KEYS == 0 && aligned16) {
+        if (decode_mma(qb, tiles, c, q_len, pos0, scratch)) {
             static int sms = 0;
             if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
             const uint32_t units = B * c->Hkv, per_sm = c->Dh == 64 ? 4 : 2;             // CTAs that fit an SM (96 / 48 KB of shared memory each)
@@ -2574,10 +2641,11 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
             attr[1].val.clusterDim.x = parts; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = cluster ? 2 : 1;
-#define TGP_DECODE_MMA_P(DH_, G_, SP_, CL_) do { \
+#define TGP_DECODE_MMA_R(DH_, G_, SP_, CL_, RO_) do { \
                 static bool attr_set = false; \
-                if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_decode_mma_kernel<DH_, G_, SP_, CL_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TGP_E_CUDA; attr_set = true; } \
-                cudaLaunchKernelEx(&cfg, tgp_attn_decode_mma_kernel<DH_, G_, SP_, CL_>, a, per_cta); } while (0)
+                if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_decode_mma_kernel<DH_, G_, SP_, CL_, RO_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TGP_E_CUDA; attr_set = true; } \
+                cudaLaunchKernelEx(&cfg, tgp_attn_decode_mma_kernel<DH_, G_, SP_, CL_, RO_>, a, per_cta); } while (0)
+#define TGP_DECODE_MMA_P(DH_, G_, SP_, CL_) do { if (rotates) TGP_DECODE_MMA_R(DH_, G_, SP_, CL_, true); else TGP_DECODE_MMA_R(DH_, G_, SP_, CL_, false); } while (0)
 #define TGP_DECODE_MMA(DH_, G_) do { if (cluster) { if (split_p) TGP_DECODE_MMA_P(DH_, G_, true, true); else TGP_DECODE_MMA_P(DH_, G_, false, true); } \
                 else { if (split_p) TGP_DECODE_MMA_P(DH_, G_, true, false); else TGP_DECODE_MMA_P(DH_, G_, false, false); } } while (0)
 #define TGP_DECODE_MMA_G(DH_) do { if (G == 1) TGP_DECODE_MMA(DH_, 1); else if (G == 2) TGP_DECODE_MMA(DH_, 2); else if (G == 4) TGP_DECODE_MMA(DH_, 4); else TGP_DECODE_MMA(DH_, 8); } while (0)
@@ -2586,6 +2654,7 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
 #undef TGP_DECODE_MMA_G
 #undef TGP_DECODE_MMA
 #undef TGP_DECODE_MMA_P
+#undef TGP_DECODE_MMA_R
             LAUNCH_CHECK(merge ? 2 : 1);
             return TGP_OK;
         }

@@ -37,8 +37,10 @@ bool tgpk_launch_overlap();
 bool tgpk_swiglu_fusable(uint32_t M);
 int tgpk_rope_kv(const float *q32, const float *k32, const float *v32, void *qb, const TgpTilePtrs &tiles, const float *cos_t, const float *sin_t,
                  const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0, cudaStream_t st);
+// what a decode step's attention needs to rotate for itself: the fp32 projections of its new position and the tables
+struct TgpRopeIn { const float *q32, *k32, *v32, *cos_t, *sin_t; };
 int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0,
-              float *scratch, cudaStream_t st);
+              float *scratch, cudaStream_t st, const TgpRopeIn *rope = nullptr);
 // tcgen05 causal attention for q_len > 1 (tgp_attn_sm100.cu); Dh 64 or 128
 int tgpk_attn_prefill_tc5(const void *qb, const TgpTilePtrs &tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0, cudaStream_t st);
 // mma.sync flash-style causal attention for q_len > 1 (tgp_attn_prefill.cu); Dh 64 or 128

@@ -1277,3 +1277,36 @@ def test_edge_shapes_single_token_prompt_no_decode_and_maximum_tile_count():
         r.step(tb.PREFILL, np.zeros((many.B, many.S + 1), np.int32), many.S + 1)      # more tokens than the workspace holds
     assert ei.value.code == tb.E_INVAL
     s.close()
+
+
+# one part, clusters of up to eight and the merge kernel; 1, 2, 4 and 8 query heads per KV head; new positions that begin a chunk of 16 keys and a tile; tiles of 8 keys (apart anyway)
+@pytest.mark.parametrize("Dh,Hq,Hkv,TK,B,S", [(64, 4, 4, 16, 1, 15), (64, 8, 4, 64, 3, 62), (128, 4, 1, 32, 2, 95), (128, 8, 1, 128, 1, 1023), (64, 8, 8, 256, 2, 766),
+                                              (128, 2, 2, 64, 5, 1599), (64, 4, 4, 8, 2, 30)])
+def test_decode_attention_that_rotates_for_itself_gives_the_bits_of_the_two_kernels(Dh, Hq, Hkv, TK, B, S):
+    """With the activation tap a decode step rotates and appends in a kernel of its own, without it in the attention: logits of every step and the KV tiles that the
+    last one leaves (read by the attention of one more step with the tap) are the same, and there is one launch less per layer."""
+    cfg = replace(si.CONFIGS[1], L=2, d=Hq * Dh, Hq=Hq, Hkv=Hkv, Dh=Dh, F=512, V=500, B=B, S=S, T=4, TK=TK, budget_rule="half_w")
+    lay, pool, s, blobs, T = setup(cfg, budget=256 << 20)
+    r = Runner(s, cfg.B * cfg.S)
+    tap = torch.zeros(512 << 20, dtype=torch.uint8, device="cuda:0")
+    prompt = si.prompt_tokens(cfg)
+    forced = (np.arange(B * T, dtype=np.int32).reshape(B, T) * 61 + 3) % cfg.V
+    runs, launches = [], []
+    for apart in (True, False):
+        r.reset()
+        s.ctx.set_tap(None, 0)
+        r.step(tb.PREFILL, prompt, cfg.S)
+        logits = []
+        for t in range(T):
+            s.ctx.set_tap(*((tap, tap.numel()) if apart or t == T - 1 else (None, 0)))
+            st = r.step(tb.DECODE, np.ascontiguousarray(forced[:, t:t + 1]), 1, want_stats=True)
+            logits.append(r.logits.cpu().numpy().copy())
+            if t == 1:
+                launches.append(st.n_launches)
+        runs.append(logits)
+    s.ctx.set_tap(None, 0)
+    s.close()
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
+    # (products that share a launch without the tap make the difference larger)
+    assert launches[0] - launches[1] >= (cfg.L if TK % 16 == 0 else 0)
