@@ -71,7 +71,10 @@ __device__ __forceinline__ uint64_t fma2(uint64_t x, uint64_t y, uint64_t z) { u
 __device__ __forceinline__ uint64_t add2(uint64_t x, uint64_t y) { uint64_t d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y)); return d; }
 __device__ __forceinline__ float max3(float x, float y, float z) { float d; asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(x), "f"(y), "f"(z)); return d; }
 
-template <int DH>
+// SPLIT: two CTAs of a cluster share the queries, each with half of the key blocks, for grids that leave SMs without a second CTA or without one: the chain of
+// key blocks is half as long.  They exchange what they have of half of the dimensions through shared memory, with the sums and exponent references, and
+// each stores the other half.
+template <int DH, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUtensorMap tmO, const TArgs a) {
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int KB = DH / 64;                          // 64-wide blocks of the head dimension
@@ -92,15 +95,16 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
         if (tid == 0) atomicCAS(&g_attn_tc_error, 0, 5);
         return;
     }
-    const uint32_t qblk = gridDim.x - 1 - blockIdx.x, hq = blockIdx.y, b = blockIdx.z, hk = hq / (a.Hq / a.Hkv);      // longest (latest) query blocks are launched first
+    const uint32_t half = SPLIT ? cluster_ctarank() : 0, qblk = SPLIT ? (gridDim.x - 1 - blockIdx.x) / 2 : gridDim.x - 1 - blockIdx.x, hq = blockIdx.y, b = blockIdx.z, hk = hq / (a.Hq / a.Hkv);      // longest (latest) query blocks are launched first
     const uint32_t q0 = qblk * BQ, kvlen = a.pos0 + a.q_len;
     const uint32_t last_q = min(a.q_len, q0 + BQ) - 1;
-    const uint32_t nblk = (a.pos0 + last_q + 1 + BKV - 1) / BKV;
+    const uint32_t all_blk = (a.pos0 + last_q + 1 + BKV - 1) / BKV, j_lo = SPLIT && half ? (all_blk + 1) / 2 : 0;
+    const uint32_t nblk = SPLIT && !half ? (all_blk + 1) / 2 : all_blk - j_lo;      // key blocks of this CTA, from j_lo on (below they are counted from 0)
 
     // The TMA thread (warp 5, lane 0) initialises the barriers and requests Q and the first K and V blocks at once, before
     // the TMEM allocation and the CTA-wide barrier below.  Its state: blocks requested so far (block i uses stage i & 1)
     // and, for the next K and V block, the KV tile and the key offset inside it.
-    uint32_t nk = 0, nv = 0, k_tile = 0, k_off = 0, v_tile = 0, v_off = 0;
+    uint32_t nk = 0, nv = 0, k_tile = j_lo * BKV / a.TK, k_off = j_lo * BKV - k_tile * a.TK, v_tile = k_tile, v_off = k_off;
     const uint32_t head_row = (b * a.Hkv + hk) * a.TK;
     auto load_kv = [&](uint8_t *dst, int y, uint64_t *bar, uint32_t more_bytes) {
         mbar_expect_tx(bar, KV_BYTES + more_bytes);
@@ -209,8 +213,8 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
                 const uint32_t st = jb & 1;
                 if (!wait(bar_p + st, (jb >> 1) & 1, 4)) break;
                 if (!wait(bar_v + st, (jb >> 1) & 1, 3)) break;
-                if (jb * BKV + BKV > kvlen) {                                    // rows past the sequence: whatever the tile holds there
-                    const uint32_t valid = kvlen - jb * BKV;
+                if ((j_lo + jb) * BKV + BKV > kvlen) {                           // rows past the sequence: whatever the tile holds there
+                    const uint32_t valid = kvlen - (j_lo + jb) * BKV;
                     for (uint32_t i = lane; i < (BKV - valid) * KB * 8; i += 32) {
                         const uint32_t r = valid + i / (KB * 8), kb = (i / 8) % KB, c = i % 8;
                         *reinterpret_cast<uint4 *>(Vs + st * KV_BYTES + kb * (BKV * 128) + r * 128 + c * 16) = make_uint4(0, 0, 0, 0);
@@ -249,10 +253,10 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
             tmem_ld64(tmem_S + lane_addr, s);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             mbar_arrive(bar_sfree);
-            if (jb * BKV + BKV - 1 > a.pos0 + q0) {                          // this block crosses the diagonal of some row
+            if ((j_lo + jb) * BKV + BKV - 1 > a.pos0 + q0) {                 // this block crosses the diagonal of some row
 #pragma unroll
                 for (uint32_t i = 0; i < BKV; ++i)
-                    if (jb * BKV + i > qpos) s[i] = -INFINITY;
+                    if ((j_lo + jb) * BKV + i > qpos) s[i] = -INFINITY;
             }
             auto row_max = [&]() {                                           // of the scaled scores (scale > 0: max commutes with it)
                 float m0 = max3(s[0], s[1], s[2]), m1 = max3(s[3], s[4], s[5]);
@@ -280,11 +284,14 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
             // The exponent reference m is the row max of block 0 (which holds key 0 <= qpos: finite).  Later blocks use it
             // as it is and never look for their own max: only when a block's sum says that a score of one of the warp's
             // rows lies more than about 2^40 above m (or overflowed) does the warp take the slow path.
+            // (the second half of the key blocks may begin with blocks that a row sees nothing of: its reference is the max of the first that it does)
             if (jb == 0) m_ref = row_max();
-            float lblk = exps(m_ref);
+            else if (SPLIT && __any_sync(0xffffffffu, m_ref == -INFINITY)) { const float m = row_max(); if (m_ref == -INFINITY) m_ref = m; }
+            auto reference = [&]() { return SPLIT && m_ref == -INFINITY ? 0.f : m_ref; };
+            float lblk = exps(reference());
             if (jb > 0 && __any_sync(0xffffffffu, !(lblk <= 0x1p40f))) {
                 if (!(ok = wait(bar_o + ((jb - 1) & 1), ((jb - 1) >> 1) & 1, 2))) break;           // P V_{j-1}: nothing is accumulating into O
-                const float m_new = fmaxf(m_ref, row_max()), alpha = ex2(m_ref - m_new);
+                const float m_new = fmaxf(m_ref, row_max()), alpha = SPLIT && m_ref == -INFINITY ? 1.f : ex2(m_ref - m_new);      // (nothing seen so far: zeros)
                 m_ref = m_new;
                 lrow *= alpha;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -297,7 +304,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
                     for (uint32_t i = 0; i < 32; ++i) u[i] = __float_as_uint(v[i] * alpha);
                     tmem_st32(tmem_O + lane_addr + h * 32, u);
                 }
-                lblk = exps(m_ref);
+                lblk = exps(reference());
             }
             lrow += lblk;
             if (jb >= 2 && !(ok = wait(bar_o + (jb & 1), ((jb - 2) >> 1) & 1, 2))) break;      // P V_{j-2}: this P buffer is free
@@ -308,7 +315,52 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
         }
         // ---- the last P V; normalise and store this thread's row ----
         if (ok) ok = wait(bar_o + ((nblk - 1) & 1), ((nblk - 1) >> 1) & 1, 2);
-        if (ok) {
+        if constexpr (SPLIT) {
+            // this row's outputs in the other CTA's dimensions, its sum and its reference go where K and V were (every load has landed, every product is done)
+            float *mine = reinterpret_cast<float *>(Ks) + tid;
+            constexpr uint32_t OUT = DH / 2;                                 // dimensions that a CTA stores
+            if (ok) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                for (uint32_t h = 0; h < OUT / 32; ++h) {
+                    float v[32];
+                    tmem_ld32(tmem_O + lane_addr + (half ^ 1) * OUT + h * 32, v);
+#pragma unroll
+                    for (uint32_t i = 0; i < 32; ++i) mine[(h * 32 + i) * BQ] = v[i];
+                }
+                mine[OUT * BQ] = m_ref;
+                mine[(OUT + 1) * BQ] = lrow;
+            }
+            __syncwarp();
+            cluster_sync_all();
+            const uint32_t theirs = smem_u32(mine), other = half ^ 1;
+            const uint32_t bad = ld_remote_u32(smem_u32((const void *)failed), 0) | ld_remote_u32(smem_u32((const void *)failed), 1);
+            if (ok && !bad) {
+                const float m_o = ld_remote_f32(theirs + OUT * BQ * 4, other), l_o = ld_remote_f32(theirs + (OUT + 1) * BQ * 4, other);
+                // (a NaN stays one: fmaxf drops it from the maximum, the weights of its side are NaN)
+                const float M = fmaxf(m_ref, m_o), w_m = m_ref == -INFINITY ? 0.f : ex2(m_ref - M), w_o = m_o == -INFINITY ? 0.f : ex2(m_o - M);
+                const float inv = 1.0f / (w_m * lrow + w_o * l_o), f_m = w_m * inv, f_o = w_o * inv;
+                bf16 *dst = a.ob + ((size_t)(b * a.q_len + q0 + tid) * a.Hq + hq) * DH + half * OUT;
+#pragma unroll
+                for (uint32_t h = 0; h < OUT / 32; ++h) {
+                    float v[32], x[32];
+#pragma unroll
+                    for (uint32_t i = 0; i < 32; ++i) x[i] = ld_remote_f32(theirs + (h * 32 + i) * BQ * 4, other);
+                    tmem_ld32(tmem_O + lane_addr + half * OUT + h * 32, v);
+#pragma unroll
+                    for (uint32_t c = 0; c < 4; ++c) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (uint32_t i = 0; i < 4; ++i) {
+                            const uint32_t e = c * 8 + 2 * i;
+                            __nv_bfloat162 pk = __floats2bfloat162_rn(v[e] * f_m + x[e] * f_o, v[e + 1] * f_m + x[e + 1] * f_o);
+                            w[i] = *reinterpret_cast<uint32_t *>(&pk);
+                        }
+                        if (row_ok) *reinterpret_cast<uint4 *>(dst + h * 32 + c * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                }
+            }
+        } else if (ok) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const float inv = 1.0f / lrow;
             const bool full_tile = q0 + BQ <= a.q_len;                       // a TMA store would spill padding rows into the next sequence
@@ -344,8 +396,10 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
             }
         }
     }
+    if (SPLIT && warp >= 4) { __syncwarp(); cluster_sync_all(); }            // (the softmax warps' exchange)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if constexpr (SPLIT) cluster_sync_all();                                 // neither CTA leaves while the other may still read its outputs
     if (warp == 4) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(256u) : "memory");
@@ -358,24 +412,39 @@ template <int DH> constexpr int smem_bytes() { return (DH / 64) * (BQ + 4 * BKV)
 
 extern thread_local uint64_t tgpk_launches;
 
-template <int DH>
+template <int DH, bool SPLIT>
 static int launch(const CUtensorMap &mq, const CUtensorMap &mkv, const CUtensorMap &mo, const TArgs &a, uint32_t B, cudaStream_t st) {
     static bool attr_set = false;
     if (!attr_set) {
-        if (cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<DH>()) != cudaSuccess) return TGP_E_CUDA;
-        cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<DH>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        if (cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<DH, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<DH>()) != cudaSuccess) return TGP_E_CUDA;
+        cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<DH, SPLIT>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         attr_set = true;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((a.q_len + BQ - 1) / BQ, a.Hq, B); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = smem_bytes<DH>(); cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3((a.q_len + BQ - 1) / BQ * (SPLIT ? 2 : 1), a.Hq, B); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = smem_bytes<DH>(); cfg.stream = st;
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, tgp_attn_prefill_tc_kernel<DH>, mq, mkv, mo, a) != cudaSuccess) return TGP_E_CUDA;
+    cfg.numAttrs = SPLIT ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, tgp_attn_prefill_tc_kernel<DH, SPLIT>, mq, mkv, mo, a) != cudaSuccess) return TGP_E_CUDA;
     tgpk_launches += 1;
     return TGP_OK;
+}
+
+// Two CTAs per query block and head where both of all of them fit the GPU at a time and the longest chain of key blocks makes up for the exchange, which takes longer
+// with 128 dimensions and where most SMs have two CTAs anyway (us with the norm before, one against two: 8 heads x 64, 128 queries behind 1000 keys 17.6 / 13.1, behind
+// 200 9.4 / 8.5; 16 heads x 128, 509 queries 14.3 / 11.6, 384 10.7 / 10.5; 32 heads x 128, 384 queries 11.5 / 13.5; 128 CTAs: 13 - 16 blocks 1.02 - 1.14 times as fast, 8
+// blocks 0.92 - 1.08; 192 CTAs of 27 blocks 33.1 / 37.9).
+static bool split_keys(const TArgs &a, uint32_t B, uint32_t Dh) {
+    static int sms = 0;
+    if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
+    const uint64_t ctas = (uint64_t)((a.q_len + BQ - 1) / BQ) * a.Hq * B;
+    const uint32_t blocks = (a.pos0 + a.q_len + BKV - 1) / BKV;
+    if (a.pos0 + (a.q_len < BQ ? a.q_len : BQ) <= BKV) return false;         // a block for each of the two, also of the first queries
+    return 3 * ctas <= 2 * (uint64_t)sms ? blocks >= (Dh == 128 ? 8u : 6u) : ctas <= (uint64_t)sms && blocks >= 12;
 }
 
 int tgpk_attn_prefill_tc5(const void *qb, const TgpTilePtrs &tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0, cudaStream_t st) {
@@ -405,7 +474,8 @@ int tgpk_attn_prefill_tc5(const void *qb, const TgpTilePtrs &tiles, void *ob, co
         !tensor_map_bf16_2d(&mkv, (const void *)lo, (hi - lo) / row_bytes + tile_rows, c->Dh, row_bytes, BKV) ||
         !tensor_map_bf16_2d(&mo, ob, (uint64_t)B * q_len, (uint64_t)c->Hq * c->Dh, (uint64_t)c->Hq * c->Dh * 2, BQ))
         return TGP_E_CUDA;
-    return c->Dh == 64 ? launch<64>(mq, mkv, mo, a, B, st) : launch<128>(mq, mkv, mo, a, B, st);
+    if (split_keys(a, B, c->Dh)) return c->Dh == 64 ? launch<64, true>(mq, mkv, mo, a, B, st) : launch<128, true>(mq, mkv, mo, a, B, st);
+    return c->Dh == 64 ? launch<64, false>(mq, mkv, mo, a, B, st) : launch<128, false>(mq, mkv, mo, a, B, st);
 }
 
 int tgpk_attn_wait_test(unsigned long long limit_ns, int withhold_step) {

@@ -1270,3 +1270,41 @@ def test_products_in_small_tiles_of_pairs_have_the_bits_of_the_largest(M, n, K):
     assert tb.k_gemm_status() == 0 and torch.equal(out[0], out[1])
     want = A.double() @ W.double().T
     assert float((out[0].double() - want).abs().max()) < 2e-5 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("Dh,Hq,Hkv,B,S,pos0,TK", [(64, 4, 4, 1, 384, 0, 64), (128, 4, 1, 2, 500, 0, 128), (64, 8, 2, 1, 129, 300, 64), (128, 2, 2, 3, 201, 1500, 256), (64, 2, 1, 1, 1000, 37, 128)])
+def test_prefill_attention_whose_key_blocks_two_ctas_share(Dh, Hq, Hkv, B, S, pos0, TK):
+    """Grids that leave SMs idle: two CTAs of a cluster take half of the key blocks each.  Ragged last query blocks, rows whose keys lie in the first half only or begin inside
+    the second, scores that grow towards the last keys (a moved exponent reference in one half), against 64 bits; an infinity in a key's score, an infinity in V."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(S + pos0)
+    n, kv, G = (pos0 + S + TK - 1) // TK, pos0 + S, Hq // Hkv
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=kv, T=0, B=B, d=Hq * Dh)
+    mc = model_cfg(cfg)
+    q = torch.randn((B, S, Hq, Dh), device=DEV, generator=gen).bfloat16()
+    q[..., 0] = 1
+
+    def check(K, V):
+        kt, vt = ([t.permute(1, 2, 0, 3).contiguous() for t in T.split(TK)] for T in (K, V))
+        ob = torch.zeros((B, S, Hq, Dh), device=DEV, dtype=torch.bfloat16)
+        tb.k_attn(q, kt, vt, ob, mc, B, S, pos0, None)
+        torch.cuda.synchronize()
+        assert tb.k_attn_status() == 0
+        k64, v64 = (T[:kv].permute(1, 2, 0, 3).double().repeat_interleave(G, 1) for T in (K, V))
+        sc = q.permute(0, 2, 1, 3).double() @ k64.transpose(-1, -2) / Dh ** 0.5
+        mask = torch.arange(kv, device=DEV)[None, :] > pos0 + torch.arange(S, device=DEV)[:, None]
+        want = (torch.softmax(sc.masked_fill(mask, -float("inf")), -1) @ v64).permute(0, 2, 1, 3)
+        # half a bf16 step of the output and of each of the probabilities, whose roundings average out: 2^-9 of the largest V, as in the tests above
+        assert float((ob.double() - want).abs().max()) < 2.0 ** -7 * float(want.abs().max()) + 1e-6
+
+    K, V = (torch.zeros((n * TK, B, Hkv, Dh), device=DEV, dtype=torch.bfloat16) for _ in range(2))
+    K[:kv], V[:kv] = (torch.randn((kv, B, Hkv, Dh), device=DEV, generator=gen).bfloat16() for _ in range(2))
+    check(K, V)
+    rising = K.clone()                                       # scores up to 150 in units of log2 above the first ones, and falling ones
+    rising[:kv, :, :, 0] = (torch.arange(kv, device=DEV)[:, None, None] / kv * 100 * Dh ** 0.5).bfloat16()
+    check(rising, V)
+    check((-rising.float()).bfloat16(), V)
+    hidden = K.clone()                                       # keys of score -inf, the whole first block of the second half among them
+    blocks = (kv + 63) // 64
+    hidden[64 * ((blocks + 1) // 2):64 * ((blocks + 1) // 2) + 64, :, :, 0] = -float("inf")
+    check(hidden, V)
