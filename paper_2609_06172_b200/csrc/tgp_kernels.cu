@@ -952,7 +952,7 @@ __device__ __forceinline__ float fast_ex2(float x) { float y; asm("ex2.approx.ft
 // take 151 registers at DH = 64, and the few CTAs they are for fit an SM in threes.)
 // ROPE: the kernel does what tgp_rope_kv_vec_kernel does, too, with its bits: every CTA rotates its queries in registers, and the warp whose chunk holds the new
 // position rotates its key, puts key and value into the stage behind the copies, and writes both to the tiles.  One launch and its hand-over less per layer
-// of a decode step (one sequence, 32 heads over 8 x 64, 300 keys: 6.1 us for both, 4.6 so).
+// of a decode step (one sequence, 16 layers of 32 heads over 8 x 64, a run of 192 steps: 41.2 -> 40.5 ms).
 template <int DH, int G, bool SPLIT_P, bool CLUSTER, bool ROPE>
 __global__ void __launch_bounds__(DEC_WARPS * 32, DH == 128 ? 2 : SPLIT_P ? 3 : 4) tgp_attn_decode_mma_kernel(AttnArgs a, uint32_t chunks_per_cta) {
     pdl_enter();
