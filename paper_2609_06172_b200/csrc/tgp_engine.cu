@@ -599,6 +599,33 @@ static bool gemm_target(const TgpEngine *e, const tgp_model_cfg &c, const TgpRol
     }
 }
 
+// Blocks of each of the gate and up projections that begin at op `first` and run as one launch with the SwiGLU op behind them: the whole matrices in the
+// same pieces, all on the device since earlier ops, and no copy waits for one of them (waiting for a copy that is under way, or keeping a slot
+// for longer, would cost the link more than the launches), and F > 1024: SwiGLU of shorter rows is what tgp_k_decode_fuse() moves into the down
+// projection, and with that switched off every op of such a model is a launch of its own, which is what the switch promises to take away.  0: they run one by one.
+static uint32_t glu_blocks(const tgp_ctx *ctx, uint32_t first, uint32_t end, uint32_t M) {
+    const tgp_model_cfg &c = ctx->cfg;
+    uint32_t rows[TGP_GEMM_GROUP_MAX / 2], nb = 0;
+    if (c.F <= 1024) return 0;
+    auto block = [&](uint32_t i, uint32_t kind) -> const TgpRole * {
+        if (i >= end || ctx->ops[i].kind != TGP_OP_GEMM || ctx->ops[i].layer != ctx->ops[first].layer || !ctx->ops[i].nacc) return nullptr;
+        const TgpRole *r = role_of(ctx, ctx->ops[i], 0);
+        if (!r || r->kind != kind || r->expert >= 0 || ctx->plan.op_is_wait_target[i] || ctx->plan.op_last_place[i] >= 0) return nullptr;
+        return tgpk_glu_rows_ok(M, r->rows, c.d) && ctx->tensors[ctx->acc[ctx->ops[i].acc0].tensor].size == 2ull * r->rows * c.d ? r : nullptr;
+    };
+    for (uint32_t at = 0; at < c.F; at += rows[nb++]) {
+        const TgpRole *r = nb < TGP_GEMM_GROUP_MAX / 2 ? block(first + nb, TGP_K_WG) : nullptr;
+        if (!r || r->row0 != at) return 0;
+        rows[nb] = r->rows;
+    }
+    for (uint32_t j = 0, at = 0; j < nb; at += rows[j++]) {
+        const TgpRole *r = block(first + nb + j, TGP_K_WU);
+        if (!r || r->row0 != at || r->rows != rows[j]) return 0;
+    }
+    const uint32_t last = first + 2 * nb;
+    return nb && last < end && ctx->ops[last].kind == TGP_OP_SWIGLU && ctx->ops[last].layer == ctx->ops[first].layer && ctx->plan.op_last_place[last] < 0 ? nb : 0;
+}
+
 // The expert ops of a layer, [first, first + result), as one launch of tgpk_experts(): every expert is traced (so none can be routed to
 // that is not here), the blocks fit its tables and are on the device or on their way, and no copy waits for one of them.
 // 0: they run one by one.
@@ -724,8 +751,11 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
             if (key_out) *key_out = key0;
             return cnt;
         };
+        const uint32_t glu = ring && o.kind == TGP_OP_GEMM && !e->tap && !c.E && q_len == 1 && M <= 2 ? glu_blocks(ctx, i, st.op0 + st.nops, M) : 0;
         if (moe_span && i == moe_first) {
             span = moe_span;
+        } else if (glu) {
+            span = 2 * glu + 1;                          // gate, up and SwiGLU of a decode step of one or two sequences (bit for bit)
         } else if (ring && o.kind == TGP_OP_GEMM && !e->tap) {
             uint32_t cnt = form_group(i, nullptr);
             // A grouped launch keeps the ring slots of its first blocks until its last block has arrived and the launch has
@@ -811,6 +841,12 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
         }
         case TGP_OP_GEMM: {
             if (moe_span && i == moe_first) { rc = tgpk_experts(moe, cs); break; }
+            if (glu) {
+                const void *gW[TGP_GEMM_GROUP_MAX];
+                for (uint32_t j = 0; j < 2 * glu; ++j) { gW[j] = where(ctx, ctx->ops[i + j], 0); gn[j] = role_of(ctx, ctx->ops[i + j], 0)->rows; }
+                rc = tgpk_glu_rows(e->h, glu, gW, gW + glu, gn, e->ab, M, c.d, cs);
+                break;
+            }
             const TgpRole *rp = role_of(ctx, o, 0);
             if (!rp || !rp->rows) return tgp_fail(ctx, TGP_E_MISMATCH, "GEMM op on a tensor with no model role");
             const tgp_access &a = ctx->acc[o.acc0];

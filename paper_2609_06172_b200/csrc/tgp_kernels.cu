@@ -340,6 +340,68 @@ __global__ void __launch_bounds__(256) tgp_wstream_group_kernel(const bf16 *A, c
     }
 }
 
+// Gate, up and SwiGLU of one or two rows in one launch, for the decode steps of a planned run: a warp takes a row of gate and the same row of up (blocks of a
+// matrix are walked as one list), so that the two sums meet in its registers and only a = bf16(silu(gate) * up) is stored.  HBM bounds it as it bounds the
+// products; what goes is the launch of tgp_swiglu_kernel and the ramp between the matrices.  A row's sums are those of
+// tgp_wstream_kernel and the expression is that of tgp_swiglu_kernel: the same bits.
+// (Whole captured runs of 48 steps, before and after: 4 layers of 2048 x 512 4.77 -> 4.44 ms, 4096 x 1024 8.27 -> 7.67, 8192 x 2048 18.28 -> 18.14, 5632 x 2048
+// 15.73 -> 15.34; two rows, 8192 x 2048 20.40 -> 20.18, 2 layers of 14336 x 4096 33.95 -> 33.40, 8960 x 1536 14.30 -> 13.78.)
+struct GluParts { const bf16 *gate[TGP_GEMM_GROUP_MAX / 2], *up[TGP_GEMM_GROUP_MAX / 2]; uint32_t n[TGP_GEMM_GROUP_MAX / 2], count; };
+
+template <int MT, int U>
+__global__ void __launch_bounds__(256) tgp_wstream_glu_kernel(const bf16 *A, const GluParts p, bf16 *out, uint32_t Mrows, uint32_t F, uint32_t K) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarp = (gridDim.x * blockDim.x) >> 5;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    bool synced = false;
+    for (uint32_t row = gwarp; row < F; row += nwarp) {
+        const bf16 *w[2] = {p.gate[0], p.up[0]};
+        uint32_t r = row, start = p.n[0];
+#pragma unroll
+        for (int s = 1; s < (int)TGP_GEMM_GROUP_MAX / 2; ++s)
+            if (s < (int)p.count) {
+                if (row >= start) { w[0] = p.gate[s]; w[1] = p.up[s]; r = row - start; }
+                start += p.n[s];
+            }
+        w[0] += (size_t)r * K;
+        w[1] += (size_t)r * K;
+        float acc[2][MT];
+#pragma unroll
+        for (int m = 0; m < MT; ++m) acc[0][m] = acc[1][m] = 0.f;
+        for (uint32_t k0 = lane * 8; k0 < K; k0 += 256 * U) {
+            uint4 wv[U][2];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) wv[u][i] = (k0 + 256 * u < K) ? __ldcs(reinterpret_cast<const uint4 *>(w[i] + k0 + 256 * u)) : make_uint4(0, 0, 0, 0);
+            if (!synced) { asm volatile("griddepcontrol.wait;" ::: "memory"); synced = true; }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t k = k0 + 256 * u;
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    float xf[8];
+                    unpack8((k < K && m < (int)Mrows) ? ld_act(reinterpret_cast<const uint4 *>(A + (size_t)m * K + k)) : make_uint4(0, 0, 0, 0), xf);
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        float wf[8];
+                        unpack8(wv[u][i], wf);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) acc[i][m] = fmaf(wf[j], xf[j], acc[i][m]);
+                    }
+                }
+            }
+        }
+        if (!synced) { asm volatile("griddepcontrol.wait;" ::: "memory"); synced = true; }       // a lane without columns
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            const float g = warp_sum(acc[0][m]), u = warp_sum(acc[1][m]);
+            if ((int)lane == m && m < (int)Mrows) out[(size_t)m * F + row] = __float2bfloat16_rn(g / (1.0f + expf(-g)) * u);
+        }
+    }
+    if (!synced) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Same product for blocks with few rows (n below two waves of warps): one CTA of 8 warps owns RB rows and its warps
 // split K in interleaved chunks of 256 elements, so n / RB CTAs spread over the SMs almost evenly where n warps of whole
 // rows leave a quarter of them with half the work.  The 8 partial sums of a row meet in shared memory and are added in
@@ -2510,6 +2572,48 @@ int tgpk_gemm_group_fused(int mode, const float *x, uint32_t ldx, const void *ga
     const ASrc src{mode, x, ldx, (const bf16 *)gain, eps, g32, u32};
     if (M == 1) launch_gemv_group<1, true>(nullptr, p, M, total, K, accumulate, st, src);
     else launch_gemv_group<2, true>(nullptr, p, M, total, K, accumulate, st, src);
+    LAUNCH_CHECK(1);
+    return TGP_OK;
+}
+
+template <int MT, int U>
+static void launch_glu(const bf16 *A, const GluParts &p, bf16 *out, uint32_t Mrows, uint32_t F, uint32_t K, cudaStream_t st) {
+    static int blocks_per_sm = 0;
+    if (!blocks_per_sm && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, tgp_wstream_glu_kernel<MT, U>, 256, 0) != cudaSuccess || blocks_per_sm < 1)) blocks_per_sm = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::min((F + 7) / 8, (uint32_t)(device_sms() * blocks_per_sm)));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = tgpk_launch_overlap() ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    launch_weights<tgp_wstream_glu_kernel<MT, U>>(cfg, A, p, out, Mrows, F, K);
+    tgpk_last_gemm_kernel = "tgp_wstream_glu_kernel";
+}
+
+// Would each of a matrix's blocks, alone or in a list, have the sums of tgp_wstream_kernel?
+bool tgpk_glu_rows_ok(uint32_t M, uint32_t n, uint32_t K) {
+    return g_gemm_group && M && M <= 2 && n && K && K % 8 == 0 && (n >= GEMV_MANY_ROWS || !(g_gemv_splitk && K >= 8192));
+}
+
+// a = bf16(silu(A gate^T) * (A up^T)) for M <= 2 rows, gate and up in `count` blocks of n[s] rows each, every one of them with tgpk_glu_rows_ok().
+int tgpk_glu_rows(const void *A, uint32_t count, const void *const *gate, const void *const *up, const uint32_t *n, void *out, uint32_t M, uint32_t K, cudaStream_t st) {
+    if (!count || count > TGP_GEMM_GROUP_MAX / 2) return TGP_E_INVAL;
+    GluParts p;
+    memset(&p, 0, sizeof(p));
+    uint32_t F = 0;
+    for (uint32_t s = 0; s < count; ++s) {
+        if (!tgpk_glu_rows_ok(M, n[s], K)) return TGP_E_INVAL;
+        p.gate[s] = (const bf16 *)gate[s]; p.up[s] = (const bf16 *)up[s]; p.n[s] = n[s]; F += n[s];
+    }
+    p.count = count;
+    // One row from K = 4096 on: all sixteen loads of 2048 columns under way (a run of 48 steps, 2 layers of 14336 x 4096 30.69 ms against 30.81 with eight;
+    // 4 x 4096 x 1024 7.67 with eight, 7.92 with sixteen).
+    if (M == 1 && K >= 4096) launch_glu<1, 8>((const bf16 *)A, p, (bf16 *)out, M, F, K, st);
+    else if (M == 1) launch_glu<1, 4>((const bf16 *)A, p, (bf16 *)out, M, F, K, st);
+    else launch_glu<2, 4>((const bf16 *)A, p, (bf16 *)out, M, F, K, st);
     LAUNCH_CHECK(1);
     return TGP_OK;
 }

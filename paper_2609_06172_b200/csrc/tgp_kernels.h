@@ -67,6 +67,9 @@ bool tgpk_expert_rows(uint32_t M, uint32_t K);
 int tgpk_gemm_rows(const void *A, uint32_t count, const void *const *W, float *const *C, const uint32_t *n, const uint32_t *ldc, uint32_t me, uint32_t K, cudaStream_t st);
 // products over the same activations may share a launch (tgp_k_gemm_group_select)
 bool tgpk_gemm_grouping();
+// gate, up and SwiGLU of at most two rows in one launch, blocks of gate and of up with the same rows (bit-identical to the separate launches)
+bool tgpk_glu_rows_ok(uint32_t M, uint32_t n, uint32_t K);
+int tgpk_glu_rows(const void *A, uint32_t count, const void *const *gate, const void *const *up, const uint32_t *n, void *out, uint32_t M, uint32_t K, cudaStream_t st);
 int tgpk_gather_rows(const void *src, const int32_t *rows, void *dst, uint32_t m, uint32_t d, cudaStream_t st);
 int tgpk_scatter_add(float *x, const float *y, const int32_t *rows, const float *gates, uint32_t m, uint32_t d, cudaStream_t st);
 // the result also goes to out2 if that is not NULL

@@ -1310,3 +1310,35 @@ def test_decode_attention_that_rotates_for_itself_gives_the_bits_of_the_two_kern
         assert np.array_equal(a, b)
     # (products that share a launch without the tap make the difference larger)
     assert launches[0] - launches[1] >= (cfg.L if TK % 16 == 0 else 0)
+
+
+# one and two rows; rows that leave warps of the last CTA idle; a K that is no multiple of 256 and one of sixteen load steps; one to four blocks per matrix, the last shorter; five blocks, and F = 1024 (apart)
+@pytest.mark.parametrize("d,F,cap,B,together", [(256, 1032, None, 1, 1), (320, 1096, None, 1, 1), (192, 1504, None, 2, 1), (128, 2000, 128 << 10, 2, 4), (128, 2000, 128 << 10, 1, 4),
+                                                (128, 2304, 128 << 10, 1, 0), (4096, 1032, None, 1, 1), (2048, 5000, None, 2, 1), (128, 1024, None, 1, 0)])
+def test_decode_steps_whose_gate_up_and_swiglu_share_a_launch_give_the_bits_of_the_separate_ones(d, F, cap, B, together):
+    """With the activation tap gate, up and SwiGLU of a decode step are launches of their own, without it one: the logits of every step are the same."""
+    Dh = 128 if d == 4096 else 64
+    cfg = replace(si.CONFIGS[1], L=2, d=d, Hq=d // Dh, Hkv=d // Dh, Dh=Dh, F=F, V=1500, B=B, S=20, T=3, TK=16, budget_rule="half_w")
+    lay, pool, s, blobs, T = setup(cfg, budget=512 << 20, cap=cap)
+    r = Runner(s, cfg.B * cfg.S)
+    tap = torch.zeros(256 << 20, dtype=torch.uint8, device="cuda:0")
+    prompt = si.prompt_tokens(cfg)
+    forced = (np.arange(B * T, dtype=np.int32).reshape(B, T) * 61 + 3) % cfg.V
+    runs, launches = [], []
+    for apart in (True, False):
+        r.reset()
+        s.ctx.set_tap(None, 0)
+        r.step(tb.PREFILL, prompt, cfg.S)
+        logits = []
+        for t in range(T):
+            s.ctx.set_tap(*((tap, tap.numel()) if apart else (None, 0)))
+            st = r.step(tb.DECODE, np.ascontiguousarray(forced[:, t:t + 1]), 1, want_stats=True)
+            logits.append(r.logits.cpu().numpy().copy())
+        launches.append(st.n_launches)
+        runs.append(logits)
+    s.ctx.set_tap(None, 0)
+    s.close()
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
+    # per layer: gate and up blocks and SwiGLU, one launch instead of 2 * together + 1; the rotation, the attention's, goes in any case
+    assert launches[0] - launches[1] >= cfg.L * (2 * together + 1)
