@@ -4,6 +4,8 @@ import ctypes
 import os
 import re
 import struct
+import subprocess
+import sys
 from dataclasses import replace
 
 import numpy as np
@@ -578,3 +580,59 @@ def test_calls_without_ctypes_take_and_refuse_what_the_general_path_does(monkeyp
     monkeypatch.setattr(tb._General, "__getattr__", lambda self, name: lambda *args: None)
     assert fast == [outcome(f) for f in calls]
     assert sum(o is None for o in fast) > 40 and sum(isinstance(o, tuple) for o in fast) > 40
+
+
+def test_lists_that_change_while_their_addresses_are_read_are_left_to_the_general_path():
+    """An active function mode (torch.device() installs one) makes a tensor's data_ptr() run Python, which may do anything to the list at hand, give the call an
+    exception, or call the library again: nothing that is gone is read.  In a process of its own, whose end says so."""
+    code = """
+import torch
+from torch.overrides import TorchFunctionMode
+from paper_2609_06172_b200 import binding as tb
+tb.lib()
+assert tb._fast.__name__.endswith("_fastcall")
+mc = tb.ModelCfg()
+mc.B, mc.Hq, mc.Hkv, mc.Dh, mc.TK, mc.max_len = 1, 2, 1, 64, 16, 256
+
+class Mode(TorchFunctionMode):
+    def __init__(self, at, act):
+        super().__init__()
+        self.n, self.at, self.act = 0, at, act
+    def __torch_function__(self, f, types, args=(), kwargs=None):
+        self.n += 1
+        if self.n == self.at:
+            self.act()
+        return f(*args, **(kwargs or {}))
+
+def swap(x):
+    x[:] = [torch.zeros(8) for _ in range(4)] + [16] * 4
+
+def nested():
+    assert tb._fast.gemm_group(16, [torch.zeros(8)] * 2, [16] * 2, 0, [8] * 2, 64, [8] * 2, 0, None) == 0
+    for i in range(20):                                       # types that fill the table of known ones while one is being looked at
+        tb._fast.swiglu(type("T%d" % i, (torch.Tensor,), {})(), 16, 16, 0, None)
+
+for act in (list.clear, list.pop, swap, lambda x: x.extend(x), lambda x: nested()):
+    for at in range(1, 8):
+        for call in (lambda x: tb._fast.gemm_group(16, x, [16] * 8, 0, [8] * 8, 64, [8] * 8, 0, None), lambda x: tb._fast.gemm_group(16, [16] * 8, x, 0, [8] * 8, 64, [8] * 8, 0, None),
+                     lambda x: tb._fast.attn(16, x, [16] * 8, 16, mc, 0, 1, 0, None, None), lambda x: tb._fast.rope_kv(16, 16, 16, 16, [16] * 8, x, 16, 16, mc, 0, 1, 0, None)):
+            x = [torch.zeros(8) for _ in range(8)]
+            with Mode(at, lambda: act(x)):
+                rc = call(x)
+            assert rc in ((0,) if len(x) == 8 else (None,)), (act, at, rc)
+
+def interrupt():
+    raise KeyboardInterrupt
+for act, out in ((lambda: 1 / 0, ZeroDivisionError), (interrupt, KeyboardInterrupt)):
+    x = [torch.zeros(8) for _ in range(8)]
+    try:
+        with Mode(2, act):
+            rc = tb.k_gemm_group(16, x, [16] * 8, 0, [8] * 8, 64, [8] * 8)
+    except KeyboardInterrupt as e:
+        assert out is KeyboardInterrupt
+    else:
+        assert out is ZeroDivisionError and rc is None        # raised once: the general path has taken the call
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(tb.__file__)))
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=root)
+    assert r.returncode == 0, (r.returncode, r.stderr)
