@@ -261,7 +261,9 @@ int  tgp_tap_index(tgp_ctx *ctx, uint64_t *out, uint64_t *n_words);
 /* Per-op timestamps (Section IV-E "Runtime Monitor": lightweight timestamping).  While enabled, tgp_step()
  * brackets every op with CUDA events on the compute stream (after the op's copies have been waited for, so
  * the figure is kernel time, not stall time).  Steps of a mixture run expert by expert meanwhile (the same bits; untimed steps of 3
- * to 32 tokens may run all experts of a layer in joint launches).  tgp_op_times() waits for the last timed step and returns one
+ * to 32 tokens may run all experts of a layer in joint launches), and decode steps rotate and append, attend, multiply by gate and up, and apply SwiGLU
+ * in launches of their own (the same bits; untimed ones join the first two, and the last three).  Products over the same activations may still share a
+ * launch; its time is that of the first.  tgp_op_times() waits for the last timed step and returns one
  * duration in ms per op of that step, ops [*first_op, *first_op + *n_ops) of the trace; ms == NULL asks
  * for the count only. */
 int  tgp_set_op_timing(tgp_ctx *ctx, int enable);

@@ -751,7 +751,8 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
             if (key_out) *key_out = key0;
             return cnt;
         };
-        const uint32_t glu = ring && o.kind == TGP_OP_GEMM && !e->tap && !c.E && q_len == 1 && M <= 2 ? glu_blocks(ctx, i, st.op0 + st.nops, M) : 0;
+        // (with timestamps these two stay apart, as a mixture's experts do: the bracket of a joint launch would be one op's and the others' empty)
+        const uint32_t glu = ring && o.kind == TGP_OP_GEMM && !e->tap && !e->op_timing && !c.E && q_len == 1 && M <= 2 ? glu_blocks(ctx, i, st.op0 + st.nops, M) : 0;
         if (moe_span && i == moe_first) {
             span = moe_span;
         } else if (glu) {
@@ -769,7 +770,7 @@ extern "C" int tgp_step(tgp_ctx *ctx, uint32_t step_kind, const int32_t *tokens_
                 g_gather |= r.kind == TGP_K_WG && r.row0 == 0;
                 g_scatter |= r.kind == TGP_K_WD && r.row0 + r.rows == c.d;
             }
-        } else if (ring && o.kind == TGP_OP_ROPE_KV && !e->tap && q_len == 1 && i + 1 < st.op0 + st.nops && ctx->ops[i + 1].kind == TGP_OP_ATTN && ctx->ops[i + 1].layer == o.layer &&
+        } else if (ring && o.kind == TGP_OP_ROPE_KV && !e->tap && !e->op_timing && q_len == 1 && i + 1 < st.op0 + st.nops && ctx->ops[i + 1].kind == TGP_OP_ATTN && ctx->ops[i + 1].layer == o.layer &&
                    !ctx->plan.op_is_wait_target[i] && (ctx->plan.op_last_place[i] < 0 || (size_t)ctx->plan.op_last_place[i] < e->next_cmd) &&
                    (ctx->plan.op_last_place[i + 1] < 0 || (size_t)ctx->plan.op_last_place[i + 1] < e->next_cmd)) {
             span = 2;                                    // the decode attention rotates and appends for itself (bit for bit), where its kernel can

@@ -1284,39 +1284,42 @@ def test_edge_shapes_single_token_prompt_no_decode_and_maximum_tile_count():
                                               (128, 2, 2, 64, 5, 1599), (64, 4, 4, 8, 2, 30)])
 def test_decode_attention_that_rotates_for_itself_gives_the_bits_of_the_two_kernels(Dh, Hq, Hkv, TK, B, S):
     """With the activation tap a decode step rotates and appends in a kernel of its own, without it in the attention: logits of every step and the KV tiles that the
-    last one leaves (read by the attention of one more step with the tap) are the same, and there is one launch less per layer."""
+    last one leaves (read by the attention of one more step with the tap) are the same.  Timestamps keep the two apart and nothing else, and there is one launch
+    less per layer without them."""
     cfg = replace(si.CONFIGS[1], L=2, d=Hq * Dh, Hq=Hq, Hkv=Hkv, Dh=Dh, F=512, V=500, B=B, S=S, T=4, TK=TK, budget_rule="half_w")
     lay, pool, s, blobs, T = setup(cfg, budget=256 << 20)
     r = Runner(s, cfg.B * cfg.S)
     tap = torch.zeros(512 << 20, dtype=torch.uint8, device="cuda:0")
     prompt = si.prompt_tokens(cfg)
     forced = (np.arange(B * T, dtype=np.int32).reshape(B, T) * 61 + 3) % cfg.V
-    runs, launches = [], []
-    for apart in (True, False):
+    runs, launches = [], {}
+    for mode in ("tap", "timed", "joint"):
         r.reset()
         s.ctx.set_tap(None, 0)
         r.step(tb.PREFILL, prompt, cfg.S)
         logits = []
+        s.ctx.set_op_timing(mode == "timed")
         for t in range(T):
-            s.ctx.set_tap(*((tap, tap.numel()) if apart or t == T - 1 else (None, 0)))
+            s.ctx.set_tap(*((tap, tap.numel()) if mode == "tap" or t == T - 1 else (None, 0)))
             st = r.step(tb.DECODE, np.ascontiguousarray(forced[:, t:t + 1]), 1, want_stats=True)
             logits.append(r.logits.cpu().numpy().copy())
             if t == 1:
-                launches.append(st.n_launches)
+                launches[mode] = st.n_launches
+        s.ctx.set_op_timing(False)
         runs.append(logits)
     s.ctx.set_tap(None, 0)
     s.close()
-    for a, b in zip(*runs):
-        assert np.array_equal(a, b)
-    # (products that share a launch without the tap make the difference larger)
-    assert launches[0] - launches[1] >= (cfg.L if TK % 16 == 0 else 0)
+    for a, b, c in zip(*runs):
+        assert np.array_equal(a, b) and np.array_equal(a, c)
+    assert launches["timed"] - launches["joint"] == (cfg.L if TK % 16 == 0 else 0)
 
 
 # one and two rows; rows that leave warps of the last CTA idle; a K that is no multiple of 256 and one of sixteen load steps; one to four blocks per matrix, the last shorter; five blocks, and F = 1024 (apart)
 @pytest.mark.parametrize("d,F,cap,B,together", [(256, 1032, None, 1, 1), (320, 1096, None, 1, 1), (192, 1504, None, 2, 1), (128, 2000, 128 << 10, 2, 4), (128, 2000, 128 << 10, 1, 4),
                                                 (128, 2304, 128 << 10, 1, 0), (4096, 1032, None, 1, 1), (2048, 5000, None, 2, 1), (128, 1024, None, 1, 0)])
 def test_decode_steps_whose_gate_up_and_swiglu_share_a_launch_give_the_bits_of_the_separate_ones(d, F, cap, B, together):
-    """With the activation tap gate, up and SwiGLU of a decode step are launches of their own, without it one: the logits of every step are the same."""
+    """With the activation tap every block of gate and up and SwiGLU of a decode step is a launch of its own, with timestamps the blocks share one, else all
+    are one: the logits of every step are the same."""
     Dh = 128 if d == 4096 else 64
     cfg = replace(si.CONFIGS[1], L=2, d=d, Hq=d // Dh, Hkv=d // Dh, Dh=Dh, F=F, V=1500, B=B, S=20, T=3, TK=16, budget_rule="half_w")
     lay, pool, s, blobs, T = setup(cfg, budget=512 << 20, cap=cap)
@@ -1324,21 +1327,47 @@ def test_decode_steps_whose_gate_up_and_swiglu_share_a_launch_give_the_bits_of_t
     tap = torch.zeros(256 << 20, dtype=torch.uint8, device="cuda:0")
     prompt = si.prompt_tokens(cfg)
     forced = (np.arange(B * T, dtype=np.int32).reshape(B, T) * 61 + 3) % cfg.V
-    runs, launches = [], []
-    for apart in (True, False):
+    runs, launches = [], {}
+    for mode in ("tap", "timed", "joint"):
         r.reset()
         s.ctx.set_tap(None, 0)
         r.step(tb.PREFILL, prompt, cfg.S)
         logits = []
+        s.ctx.set_op_timing(mode == "timed")
         for t in range(T):
-            s.ctx.set_tap(*((tap, tap.numel()) if apart else (None, 0)))
+            s.ctx.set_tap(*((tap, tap.numel()) if mode == "tap" else (None, 0)))
             st = r.step(tb.DECODE, np.ascontiguousarray(forced[:, t:t + 1]), 1, want_stats=True)
             logits.append(r.logits.cpu().numpy().copy())
-        launches.append(st.n_launches)
+        s.ctx.set_op_timing(False)
+        launches[mode] = st.n_launches
         runs.append(logits)
     s.ctx.set_tap(None, 0)
     s.close()
-    for a, b in zip(*runs):
-        assert np.array_equal(a, b)
-    # per layer: gate and up blocks and SwiGLU, one launch instead of 2 * together + 1; the rotation, the attention's, goes in any case
-    assert launches[0] - launches[1] >= cfg.L * (2 * together + 1)
+    for a, b, c in zip(*runs):
+        assert np.array_equal(a, b) and np.array_equal(a, c)
+    # per layer the rotation, which is the attention's, and SwiGLU (gate and up share a launch either way)
+    assert launches["timed"] - launches["joint"] == cfg.L * (1 + (together > 0))
+    # ... of which the blocks of q, k and v are one, too; with the tap all are apart
+    assert launches["tap"] - launches["timed"] >= cfg.L * (2 * together - 1)
+
+
+def test_timestamps_of_a_decode_step_are_of_the_ops_they_are_given_for():
+    """Attention over a long context takes much longer than the rotation of one position, and the rotation longer than nothing: their times say so."""
+    cfg = replace(si.CONFIGS[1], L=2, d=512, Hq=8, Hkv=8, Dh=64, F=512, V=500, B=2, S=8000, T=4, TK=256, budget_rule="half_w")
+    lay, pool, s, blobs, T = setup(cfg, budget=512 << 20)
+    r = Runner(s, cfg.B * cfg.S)
+    r.step(tb.PREFILL, si.prompt_tokens(cfg), cfg.S)
+    kinds = [o[3] for o in s.ctx.trace_ops()]
+    r.step(tb.DECODE, None, 1)
+    s.ctx.set_op_timing(True)
+    best = np.inf
+    for t in range(3):
+        r.step(tb.DECODE, None, 1, want_stats=True)
+        first, ms = s.ctx.op_times()
+        best = np.minimum(best, ms)
+    s.ctx.set_op_timing(False)
+    s.close()
+    rope, attn = (best[[kinds[first + j] == k for j in range(len(best))]] for k in (trace.OP_ROPE_KV, trace.OP_ATTN))
+    assert len(rope) == len(attn) == cfg.L
+    # 16 MB of keys and values per layer take 5 us of L2's rate and 2.5 of HBM's at the least, and are a chain of 16 chunks
+    assert attn.min() > 1.5 * rope.max() and attn.min() > 0.005 and rope.min() > 0, (rope, attn)
