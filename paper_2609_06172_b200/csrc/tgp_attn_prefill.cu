@@ -9,6 +9,7 @@
 // overlap); with 1600 keys it would be 67 -> 80 us and gain nothing.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <cfloat>
 #include <cstdint>
 #include "tgp.h"
 #include "tgp_kernels.h"
@@ -91,7 +92,7 @@ __global__ void __launch_bounds__(128) tgp_attn_prefill_mma_kernel(PArgs a) {
     float o[DH / 8][4];
 #pragma unroll
     for (int t = 0; t < DH / 8; ++t) { o[t][0] = o[t][1] = o[t][2] = o[t][3] = 0.f; }
-    float mrow[2] = {-INFINITY, -INFINITY}, lrow[2] = {0.f, 0.f};
+    float mrow[2] = {-FLT_MAX, -FLT_MAX}, lrow[2] = {0.f, 0.f};        // finite: a first block of scores -inf weighs nothing
     uint32_t qf[DH / 16][4];
     const uint32_t row_in_warp = lane >> 2;                 // accumulator rows: row_in_warp and row_in_warp + 8
     uint32_t qpos[2];

@@ -19,7 +19,7 @@
 //                                        stage (refilled with V_{j+2}).
 // An MMA accumulating into the same TMEM tile costs 75-90 cycles whatever its N <= 128, so S (8 MMAs) and P V (4) are
 // issued by different warps and overlap with each other and with the other CTA of the SM.
-// Softmax: the exponent reference m of a row is its max over block 0.  Later blocks use it as it is - P = exp2(S - m)
+// Softmax: the exponent reference m of a row is its max over block 0 (the lowest finite value where no score is above -inf).  Later blocks use it as it is - P = exp2(S - m)
 // may then exceed 1, which fp32 sums and bf16 P hold without loss of precision - and never compute a row max; only
 // when a block's sum of exponentials exceeds 2^40 (or overflowed) does the warp wait for the P V in flight, move m to
 // the new max and multiply its 32 rows of O in TMEM and its sums by 2^(m_old - m_new).  Scale-and-subtract and the sums
@@ -34,6 +34,7 @@
 // waits (bounded) for the loads it still has in flight, TMEM is freed and nothing is stored.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <cfloat>
 #include <cstdint>
 #include "tgp.h"
 #include "tgp_kernels.h"
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
         const bool row_ok = q0 + tid < a.q_len;
         const uint32_t qpos = a.pos0 + min(q0 + tid, a.q_len - 1);          // padding rows take the last query's mask
         const uint32_t lane_addr = (warp * 32u) << 16;                       // this warp's quarter of the TMEM lanes
-        float m_ref = -INFINITY, lrow = 0.f;                                 // exponent reference and running sum of this row
+        float m_ref = -FLT_MAX, lrow = 0.f;                                  // exponent reference and running sum of this row
         auto wait = [&](uint64_t *bar, uint32_t parity, int code) {
             bool ok = mbar_wait(bar, parity, failed);
             if (!ok) give_up(code);
@@ -281,17 +282,15 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
                 unpack2(add2(acc0, acc1), l0, l1);
                 return l0 + l1;
             };
-            // The exponent reference m is the row max of block 0 (which holds key 0 <= qpos: finite).  Later blocks use it
-            // as it is and never look for their own max: only when a block's sum says that a score of one of the warp's
-            // rows lies more than about 2^40 above m (or overflowed) does the warp take the slow path.
-            // (the second half of the key blocks may begin with blocks that a row sees nothing of: its reference is the max of the first that it does)
-            if (jb == 0) m_ref = row_max();
-            else if (SPLIT && __any_sync(0xffffffffu, m_ref == -INFINITY)) { const float m = row_max(); if (m_ref == -INFINITY) m_ref = m; }
-            auto reference = [&]() { return SPLIT && m_ref == -INFINITY ? 0.f : m_ref; };
-            float lblk = exps(reference());
+            // The exponent reference m is the row max of block 0.  Later blocks use it as it is and never look for their own max: only when a
+            // block's sum says that a score of one of the warp's rows lies more than about 2^40 above m (or overflowed) does the warp take
+            // the slow path.  A row that sees nothing of block 0 (keys of score -inf, or the second half of the key blocks) has the lowest
+            // finite reference: its sums are 0, and the first finite score takes the slow path.
+            if (jb == 0) m_ref = fmaxf(row_max(), -FLT_MAX);
+            float lblk = exps(m_ref);
             if (jb > 0 && __any_sync(0xffffffffu, !(lblk <= 0x1p40f))) {
                 if (!(ok = wait(bar_o + ((jb - 1) & 1), ((jb - 1) >> 1) & 1, 2))) break;           // P V_{j-1}: nothing is accumulating into O
-                const float m_new = fmaxf(m_ref, row_max()), alpha = SPLIT && m_ref == -INFINITY ? 1.f : ex2(m_ref - m_new);      // (nothing seen so far: zeros)
+                const float m_new = fmaxf(m_ref, row_max()), alpha = ex2(m_ref - m_new);
                 m_ref = m_new;
                 lrow *= alpha;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -304,7 +303,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
                     for (uint32_t i = 0; i < 32; ++i) u[i] = __float_as_uint(v[i] * alpha);
                     tmem_st32(tmem_O + lane_addr + h * 32, u);
                 }
-                lblk = exps(reference());
+                lblk = exps(m_ref);
             }
             lrow += lblk;
             if (jb >= 2 && !(ok = wait(bar_o + (jb & 1), ((jb - 2) >> 1) & 1, 2))) break;      // P V_{j-2}: this P buffer is free
@@ -338,7 +337,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
             if (ok && !bad) {
                 const float m_o = ld_remote_f32(theirs + OUT * BQ * 4, other), l_o = ld_remote_f32(theirs + (OUT + 1) * BQ * 4, other);
                 // (a NaN stays one: fmaxf drops it from the maximum, the weights of its side are NaN)
-                const float M = fmaxf(m_ref, m_o), w_m = m_ref == -INFINITY ? 0.f : ex2(m_ref - M), w_o = m_o == -INFINITY ? 0.f : ex2(m_o - M);
+                const float M = fmaxf(m_ref, m_o), w_m = ex2(m_ref - M), w_o = ex2(m_o - M);
                 const float inv = 1.0f / (w_m * lrow + w_o * l_o), f_m = w_m * inv, f_o = w_o * inv;
                 bf16 *dst = a.ob + ((size_t)(b * a.q_len + q0 + tid) * a.Hq + hq) * DH + half * OUT;
 #pragma unroll

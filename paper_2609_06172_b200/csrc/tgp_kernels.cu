@@ -669,7 +669,7 @@ __global__ void __launch_bounds__(128) tgp_attn_rows_kernel(AttnArgs a) {
     float o[DPL];
 #pragma unroll
     for (int i = 0; i < DPL; ++i) o[i] = 0.f;
-    float mx = -INFINITY, l = 0.f;
+    float mx = -FLT_MAX, l = 0.f;                           // finite: first keys of score -inf weigh nothing
     for (uint32_t j0 = 0; j0 < nkeys; j0 += 32) {
         const uint32_t j = j0 + lane;
         float s = -INFINITY;
@@ -732,7 +732,7 @@ __global__ void tgp_attn_decode_partial_kernel(AttnArgs a, uint32_t SPLIT) {
     float o[DPL];
 #pragma unroll
     for (int i = 0; i < DPL; ++i) o[i] = 0.f;
-    float mx = -INFINITY, l = 0.f;
+    float mx = -FLT_MAX, l = 0.f;                           // finite: first keys of score -inf weigh nothing
     const bf16 *kt = reinterpret_cast<const bf16 *>(a.tiles.k[tile]) + (size_t)(b * a.Hkv + hk) * a.TK * DH;
     const bf16 *vt = reinterpret_cast<const bf16 *>(a.tiles.v[tile]) + (size_t)(b * a.Hkv + hk) * a.TK * DH;
     for (uint32_t j0 = sp * 32; j0 < nk; j0 += SPLIT * 32) {
@@ -779,7 +779,7 @@ __global__ void tgp_attn_decode_partial_kernel(AttnArgs a, uint32_t SPLIT) {
 #pragma unroll
         for (int i = 0; i < DPL; ++i) acc[i] = 0.f;
         for (uint32_t k = 0; k < SPLIT; ++k) {
-            const float w = expf(p0[k * (DH + 2)] - m);     // a warp that saw no key has max -inf and weight 0
+            const float w = expf(p0[k * (DH + 2)] - m);     // a warp that saw no key has the lowest finite max and sums of 0
             lsum += w * p0[k * (DH + 2) + 1];
 #pragma unroll
             for (int i = 0; i < DPL; ++i) acc[i] += w * p0[k * (DH + 2) + 2 + lane + 32 * i];
@@ -818,7 +818,7 @@ __global__ void __launch_bounds__(256, 2) tgp_attn_decode_group_kernel(AttnArgs 
     float o[G][DPL], mx[G], l[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-        mx[g] = -INFINITY; l[g] = 0.f;
+        mx[g] = -FLT_MAX; l[g] = 0.f;                      // finite: first keys of score -inf weigh nothing
 #pragma unroll
         for (int i = 0; i < DPL; ++i) o[g][i] = 0.f;
     }
@@ -924,7 +924,7 @@ __global__ void __launch_bounds__(256, 2) tgp_attn_decode_group_kernel(AttnArgs 
 #pragma unroll
         for (int i = 0; i < DPL; ++i) accm[i] = 0.f;
         for (uint32_t k = 0; k < SPLIT; ++k) {
-            const float w = expf(p0[k * (DH + 2)] - m);     // a warp that saw no key has max -inf and weight 0
+            const float w = expf(p0[k * (DH + 2)] - m);     // a warp that saw no key has the lowest finite max and sums of 0
             lsum += w * p0[k * (DH + 2) + 1];
 #pragma unroll
             for (int i = 0; i < DPL; ++i) accm[i] += w * p0[k * (DH + 2) + 2 + lane * DPL + i];

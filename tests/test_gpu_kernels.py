@@ -1308,3 +1308,41 @@ def test_prefill_attention_whose_key_blocks_two_ctas_share(Dh, Hq, Hkv, B, S, po
     blocks = (kv + 63) // 64
     hidden[64 * ((blocks + 1) // 2):64 * ((blocks + 1) // 2) + 64, :, :, 0] = -float("inf")
     check(hidden, V)
+
+
+# a grid whose key blocks two CTAs share and one that leaves no SM idle, both head sizes; mma.sync by length and by choice; the CUDA-core kernels of few queries, of three
+# query heads per KV head, of tiles that are no multiple of 16 keys
+@pytest.mark.parametrize("Dh,Hq,Hkv,B,S,pos0,TK,impl", [(64, 4, 2, 1, 384, 0, 64, 0), (64, 32, 8, 4, 384, 0, 64, 0), (128, 4, 1, 1, 500, 0, 128, 0), (128, 32, 8, 3, 500, 0, 128, 0),
+                                                        (64, 4, 2, 1, 129, 300, 64, 0), (64, 4, 2, 2, 100, 200, 64, 0), (128, 4, 2, 1, 200, 100, 64, 2), (64, 2, 2, 1, 50, 100, 64, 1),
+                                                        (64, 4, 2, 2, 5, 120, 64, 0), (64, 3, 1, 2, 1, 170, 64, 0), (128, 4, 2, 1, 1, 170, 24, 0)])
+def test_attention_whose_first_keys_score_minus_infinity(Dh, Hq, Hkv, B, S, pos0, TK, impl):
+    """The first keys of every row, or all that a row sees, score -inf: they weigh nothing, and a row of nothing else is NaN, whichever kernel the grid, the number of
+    queries or the tiles choose.  As 64 bits have it."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(S + pos0 + Dh)
+    n, kv, G = (pos0 + S + TK - 1) // TK, pos0 + S, Hq // Hkv
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=kv, T=0, B=B, d=Hq * Dh)
+    mc = model_cfg(cfg)
+    q = torch.randn((B, S, Hq, Dh), device=DEV, generator=gen).bfloat16()
+    q[..., 0] = 1
+    K, V = (torch.zeros((n * TK, B, Hkv, Dh), device=DEV, dtype=torch.bfloat16) for _ in range(2))
+    K[:kv], V[:kv] = (torch.randn((kv, B, Hkv, Dh), device=DEV, generator=gen).bfloat16() for _ in range(2))
+    scratch = torch.zeros(tb.k_attn_scratch_bytes(mc) // 4, device=DEV) if S == 1 else None
+    mask = torch.arange(kv, device=DEV)[None, :] > pos0 + torch.arange(S, device=DEV)[:, None]
+    for lo, hi in ((0, 16), (0, 33), (0, 64), (0, 128), (64, 160), (0, kv)):
+        hidden = K.clone()
+        hidden[lo:min(hi, kv), :, :, 0] = -float("inf")
+        kt, vt = ([t.permute(1, 2, 0, 3).contiguous() for t in T.split(TK)] for T in (hidden, V))
+        ob = torch.zeros((B, S, Hq, Dh), device=DEV, dtype=torch.bfloat16)
+        tb.k_attn_select(impl)
+        tb.k_attn(q, kt, vt, ob, mc, B, S, pos0, scratch)
+        tb.k_attn_select(0)
+        torch.cuda.synchronize()
+        assert tb.k_attn_status() == 0
+        k64, v64 = (T[:kv].permute(1, 2, 0, 3).double().repeat_interleave(G, 1) for T in (hidden, V))
+        sc = q.permute(0, 2, 1, 3).double() @ k64.transpose(-1, -2) / Dh ** 0.5
+        want = (torch.softmax(sc.masked_fill(mask, -float("inf")), -1) @ v64).permute(0, 2, 1, 3)
+        got, fin = ob.double(), want.isfinite()
+        assert torch.equal(got.isfinite(), fin), (lo, hi)
+        # half a bf16 step of the output and of each of the probabilities, whose roundings average out: 2^-9 of the largest V, as in the tests above
+        assert not fin.any() or float((got - want)[fin].abs().max()) < 2.0 ** -7 * float(want[fin].abs().max()) + 1e-6
