@@ -295,9 +295,10 @@ static int get_event(tgp_ctx *ctx, std::vector<cudaEvent_t> &v, size_t i, cudaEv
 }
 
 // A load of a captured run whose loads are all small, by a kernel that reads the mapped pool, 16 bytes per thread and all of them under way at once.  The copy
-// engine takes 14 us for 512 KB (40 of the link's 55 GB/s: it starts anew for every copy), this 12 (a 12 MB model at half its size, 16 steps: 2735 -> 2439 us;
-// two steps 916 -> 797).  Not for plans with larger loads, whose start is a small part of them (blocks of 1 MB: 8230 us, 8680 so; small and large ones
-// mixed: 1253, 1279), and not outside a graph, where the launch costs the host as much as it saves.
+// engine takes 14 us for 512 KB (40 of the link's 55 GB/s: it starts anew for every copy), this 12, and the smaller the load the more that counts (a 12 MB model at
+// half its size, 16 steps, in blocks of 64 KB 9070 -> 4550 us, 128 KB 5430 -> 3230, 256 KB 3810 -> 2890, 512 KB 2757 -> 2460; four times the size, 512 KB 9060 ->
+// 8170).  Neighbours that share a load are held to the same size.  Not for plans with larger loads, whose start is a small part of them (blocks of 1 MB: 8230 us,
+// 8680 so; small and large ones mixed: 1253, 1279), and not outside a graph, where the launch costs the host as much as it saves.
 constexpr uint64_t GRAPH_LOAD_MAX = 512u << 10;
 __global__ void __launch_bounds__(512) tgp_graph_load_kernel(const char *src, char *dst, uint64_t bytes) {
     const uint64_t at = ((uint64_t)blockIdx.x * 512 + threadIdx.x) * 16;
@@ -343,17 +344,19 @@ static int pump(tgp_ctx *ctx, int32_t limit, cudaStream_t copy, uint32_t *n_cmds
             // a copy of a few hundred KiB is mostly latency, while merging megabytes would only delay the first tensor.
             size_t last = e->next_cmd;
             uint64_t span_bytes = c.bytes;
+            const char *mapped = pool.dev_alias ? pool.dev_alias + c.pool_off : nullptr;
+            const bool by_kernel = c.kind == CMD_H2D && e->capturing && e->small_loads && mapped && (((uintptr_t)mapped | (uintptr_t)dev) & 15u) == 0;
+            const uint64_t span_max = by_kernel ? GRAPH_LOAD_MAX : 1u << 20;
             if (c.kind == CMD_H2D && g_merge_copies)
                 while (last + 1 < pl.cmds.size()) {
                     const TgpCmd &d = pl.cmds[last + 1], &p = pl.cmds[last];
                     if (d.kind != CMD_H2D || d.wait_op > waited || d.wait_op > limit || ctx->tensors[d.tensor].pool != ctx->tensors[c.tensor].pool) break;
                     if (d.pool_off < p.pool_off + p.bytes || d.pool_off - p.pool_off != d.arena_off - p.arena_off || d.pool_off - (p.pool_off + p.bytes) >= 512) break;
-                    if (d.pool_off + d.bytes - c.pool_off > (1u << 20)) break;
+                    if (d.pool_off + d.bytes - c.pool_off > span_max) break;
                     span_bytes = d.pool_off + d.bytes - c.pool_off;
                     ++last;
                 }
-            const char *mapped = pool.dev_alias ? pool.dev_alias + c.pool_off : nullptr;
-            if (c.kind == CMD_H2D && e->capturing && e->small_loads && mapped && (((uintptr_t)mapped | (uintptr_t)dev) & 15u) == 0) {
+            if (by_kernel) {
                 tgp_graph_load_kernel<<<(uint32_t)((span_bytes + 8191) / 8192), 512, 0, mine>>>(mapped, dev, span_bytes);
                 CU(ctx, cudaGetLastError());
             } else if (c.kind == CMD_H2D) {

@@ -1,5 +1,6 @@
 """End-to-end parity on the GPU: the planned, oversubscribed forward pass through tgp_step() against the
 oracle (teacher-forced tokens), at the tolerance the benchmark spec states: max abs 3e-2, mean relative 1e-2."""
+import json
 from dataclasses import replace
 
 import numpy as np
@@ -1241,6 +1242,36 @@ def test_whole_run_cuda_graph_with_cluster_launched_and_tma_kernels():
     s.close()
 
 
+def graph_loads(r, tmp_path):
+    """Sizes in KB (rounded up to 8) of the loads by a kernel of one replay, and the number of host-to-device copies."""
+    r.replay()
+    r.sync()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        r.replay()
+        r.sync()
+    path = tmp_path / "trace.json"
+    prof.export_chrome_trace(str(path))
+    events = json.loads(path.read_text())["traceEvents"]
+    return ([8 * e["args"]["grid"][0] for e in events if e.get("cat") == "kernel" and "tgp_graph_load_kernel" in e["name"]],
+            sum(e.get("cat") == "gpu_memcpy" and "HtoD" in e["name"] for e in events))
+
+
+# blocks of 128 KB, of which neighbours are one load; of 512 KB, each a load; a plan with one block of 1 MB, whose loads are the copy engine's
+@pytest.mark.parametrize("kw,cap,by_kernel", [(dict(), 128 << 10, True), (dict(), 512 << 10, True), (dict(d=512, F=2048, Hq=8, Hkv=8), 1 << 20, False)])
+def test_captured_runs_whose_loads_are_small_load_by_a_kernel(kw, cap, by_kernel, tmp_path):
+    cfg = replace(si.CONFIGS[1], **kw)
+    lay, pool, s, blobs, T = setup(cfg, cap=cap)
+    r = Runner(s, cfg.B * cfg.S)
+    prompt = torch.from_numpy(si.prompt_tokens(cfg)).pin_memory()
+    plain, _ = r.generate(prompt.numpy(), T)
+    r.capture_run(prompt, T)
+    loads, copies = graph_loads(r, tmp_path)
+    assert np.array_equal(r.logits.cpu().numpy(), plain[-1])
+    s.close()
+    # (the prompt is a copy in any case)
+    assert (len(loads) > 100 and copies == 1 and 128 < max(loads) <= 512) if by_kernel else (not loads and copies > 100), (len(loads), copies, loads and max(loads))
+
+
 def test_edge_shapes_single_token_prompt_no_decode_and_maximum_tile_count():
     """Degenerate sizes: a prompt of one token with no decode step, and a context that needs all 64 KV tiles a kernel
     can address (TK = 1), both against the oracle; requests beyond the workspace or max_len are refused."""
@@ -1353,8 +1384,8 @@ def test_decode_steps_whose_gate_up_and_swiglu_share_a_launch_give_the_bits_of_t
 
 def test_timestamps_of_a_decode_step_are_of_the_ops_they_are_given_for():
     """Attention over a long context takes much longer than the rotation of one position, and the rotation longer than nothing: their times say so."""
-    cfg = replace(si.CONFIGS[1], L=2, d=512, Hq=8, Hkv=8, Dh=64, F=512, V=500, B=2, S=8000, T=4, TK=256, budget_rule="half_w")
-    lay, pool, s, blobs, T = setup(cfg, budget=512 << 20)
+    cfg = replace(si.CONFIGS[1], L=2, d=512, Hq=8, Hkv=8, Dh=64, F=512, V=500, B=6, S=8000, T=4, TK=256, budget_rule="half_w")
+    lay, pool, s, blobs, T = setup(cfg, budget=1 << 30)
     r = Runner(s, cfg.B * cfg.S)
     r.step(tb.PREFILL, si.prompt_tokens(cfg), cfg.S)
     kinds = [o[3] for o in s.ctx.trace_ops()]
@@ -1369,5 +1400,5 @@ def test_timestamps_of_a_decode_step_are_of_the_ops_they_are_given_for():
     s.close()
     rope, attn = (best[[kinds[first + j] == k for j in range(len(best))]] for k in (trace.OP_ROPE_KV, trace.OP_ATTN))
     assert len(rope) == len(attn) == cfg.L
-    # 16 MB of keys and values per layer take 5 us of L2's rate and 2.5 of HBM's at the least, and are a chain of 16 chunks
-    assert attn.min() > 1.5 * rope.max() and attn.min() > 0.005 and rope.min() > 0, (rope, attn)
+    # 98 MB of keys and values per layer take 15 us at HBM's rate at the least, the rotation is a launch (2 sequences: 6.0 - 7.5 us, attention 14.8 - 15.7)
+    assert attn.min() > rope.max() and attn.min() > 0.015 and rope.min() > 0, (rope, attn)
