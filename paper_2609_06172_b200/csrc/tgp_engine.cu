@@ -80,7 +80,7 @@ struct TgpEngine {
     std::vector<cudaEvent_t> ta, tb_;
     uint32_t timed_op0 = 0, timed_nops = 0;
     // whole-run CUDA graph (dense models): capture state and the instantiated graph
-    bool capturing = false, small_loads = false;         // small_loads: no load of the plan is larger than GRAPH_LOAD_MAX
+    bool capturing = false, small_loads = false;         // small_loads: no load of the plan is larger than GRAPH_LOAD_MAX, or from a managed pool
     cudaStream_t cap_cs = nullptr, cap_cp = nullptr;
     cudaEvent_t fork_ev = nullptr, join_cp = nullptr, join_wb = nullptr;
     cudaGraph_t graph = nullptr;
@@ -1196,7 +1196,8 @@ extern "C" int tgp_run_capture_begin(tgp_ctx *ctx, void *compute_stream, void *c
     e->n_copy = 1;                                       // in a graph the joins of several copy branches cost more than they hide (measured: the tiny
                                                          // configuration at 512 KiB blocks replays at 0.56 / 0.52 / 0.51 of its roofline with 1 / 2 / 3 copy streams)
     e->small_loads = true;
-    for (const TgpCmd &c : ctx->plan.cmds) e->small_loads &= c.kind != CMD_H2D || c.bytes <= GRAPH_LOAD_MAX;
+    for (const TgpCmd &c : ctx->plan.cmds)               // (a kernel that reads a managed pool would fault its pages in, one by one, and move them)
+        e->small_loads &= c.kind != CMD_H2D || (c.bytes <= GRAPH_LOAD_MAX && ctx->pools[ctx->tensors[c.tensor].pool].flags != TGP_POOL_MANAGED);
     CU(ctx, cudaStreamBeginCapture(e->cap_cs, cudaStreamCaptureModeRelaxed));
     // fork: the copy and write-back streams join the capture
     cudaError_t er = cudaEventRecord(e->fork_ev, e->cap_cs);

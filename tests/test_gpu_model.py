@@ -1272,6 +1272,30 @@ def test_captured_runs_whose_loads_are_small_load_by_a_kernel(kw, cap, by_kernel
     assert (len(loads) > 100 and copies == 1 and 128 < max(loads) <= 512) if by_kernel else (not loads and copies > 100), (len(loads), copies, loads and max(loads))
 
 
+def test_captured_runs_over_a_managed_pool_load_by_the_copy_engine(tmp_path):
+    """A kernel that reads managed memory faults its pages in and moves them; no kernel of the explicit engine does that for a load."""
+    from paper_2609_06172_b200 import uvm_baseline
+    cfg = si.CONFIGS[1]
+    lay, pool, s, blobs, T = setup(cfg, cap=128 << 10)
+    prompt = torch.from_numpy(si.prompt_tokens(cfg)).pin_memory()
+    plain, _ = Runner(s, cfg.B * cfg.S).generate(prompt.numpy(), T)
+    s.close()
+    mp = uvm_baseline.ManagedPool(lay.pool_bytes)
+    try:
+        si.fill_pool(lay, mp.numpy())
+        sm = Session(lay, MACHINE, pool_base=mp.ptr, pool_flags=tb.POOL_MANAGED)
+        sm.plan(T=T)
+        r = Runner(sm, cfg.B * cfg.S)
+        stepped, _ = r.generate(prompt.numpy(), T)
+        r.capture_run(prompt, T)
+        loads, copies = graph_loads(r, tmp_path)
+        assert not loads
+        assert np.array_equal(r.logits.cpu().numpy(), plain[-1]) and np.array_equal(stepped[-1], plain[-1])
+        sm.close()
+    finally:
+        mp.free()
+
+
 def test_edge_shapes_single_token_prompt_no_decode_and_maximum_tile_count():
     """Degenerate sizes: a prompt of one token with no decode step, and a context that needs all 64 KV tiles a kernel
     can address (TK = 1), both against the oracle; requests beyond the workspace or max_len are refused."""
