@@ -228,8 +228,7 @@ extern thread_local uint64_t tgpk_launches;
 template <int DH, bool SPLIT_P>
 static int launch(const PArgs &a, uint32_t B, cudaStream_t st) {
     constexpr int SM = (BM + 4 * BN) * DH * 2;
-    static bool attr_set = false;
-    if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_prefill_mma_kernel<DH, SPLIT_P>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM) != cudaSuccess) return TGP_E_CUDA; attr_set = true; }
+    if (!tgpk_allow_smem<tgp_attn_prefill_mma_kernel<DH, SPLIT_P>>(SM)) return TGP_E_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((a.q_len + BM - 1) / BM, a.Hq, B); cfg.blockDim = dim3(128); cfg.dynamicSmemBytes = SM; cfg.stream = st;
     cudaLaunchAttribute attr[1];

@@ -413,12 +413,7 @@ extern thread_local uint64_t tgpk_launches;
 
 template <int DH, bool SPLIT>
 static int launch(const CUtensorMap &mq, const CUtensorMap &mkv, const CUtensorMap &mo, const TArgs &a, uint32_t B, cudaStream_t st) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        if (cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<DH, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<DH>()) != cudaSuccess) return TGP_E_CUDA;
-        cudaFuncSetAttribute(tgp_attn_prefill_tc_kernel<DH, SPLIT>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        attr_set = true;
-    }
+    if (!tgpk_allow_smem<tgp_attn_prefill_tc_kernel<DH, SPLIT>>(smem_bytes<DH>(), true)) return TGP_E_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((a.q_len + BQ - 1) / BQ * (SPLIT ? 2 : 1), a.Hq, B); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = smem_bytes<DH>(); cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -438,8 +433,7 @@ static int launch(const CUtensorMap &mq, const CUtensorMap &mkv, const CUtensorM
 // 200 9.4 / 8.5; 16 heads x 128, 509 queries 14.3 / 11.6, 384 10.7 / 10.5; 32 heads x 128, 384 queries 11.5 / 13.5; 128 CTAs: 13 - 16 blocks 1.02 - 1.14 times as fast, 8
 // blocks 0.92 - 1.08; 192 CTAs of 27 blocks 33.1 / 37.9).
 static bool split_keys(const TArgs &a, uint32_t B, uint32_t Dh) {
-    static int sms = 0;
-    if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
+    const int sms = tgpk_sms();
     const uint64_t ctas = (uint64_t)((a.q_len + BQ - 1) / BQ) * a.Hq * B;
     const uint32_t blocks = (a.pos0 + a.q_len + BKV - 1) / BKV;
     if (a.pos0 + (a.q_len < BQ ? a.q_len : BQ) <= BKV) return false;         // a block for each of the two, also of the first queries

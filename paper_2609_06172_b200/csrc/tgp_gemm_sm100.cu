@@ -812,11 +812,7 @@ extern thread_local uint64_t tgpk_launches;
 
 template <int BN, int ST, int KH, bool SWAP = false>
 static bool launch_tile(const CUtensorMap &ma, const CUtensorMap &mb, float *C, uint32_t M, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int accumulate, cudaStream_t st, const Epi ep = Epi{nullptr, nullptr}) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        if (cudaFuncSetAttribute(tgp_matmul_tc_kernel<BN, ST, KH, SWAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<BN, ST, KH>::TOTAL) != cudaSuccess) return false;
-        attr_set = true;
-    }
+    if (!tgpk_allow_smem<tgp_matmul_tc_kernel<BN, ST, KH, SWAP>>(Smem<BN, ST, KH>::TOTAL)) return false;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(((M + BM - 1) / BM) * ((n + BN - 1) / BN)); cfg.blockDim = dim3(192); cfg.dynamicSmemBytes = Smem<BN, ST, KH>::TOTAL; cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -831,11 +827,7 @@ static int g_tc_variant = 0;     // 0 by size (see the top of this file), 1 forc
 
 bool tgpk_gemm_tc_forced() { return g_tc_variant != 0; }
 
-static uint32_t tc_sms() {
-    static int sms = 0;
-    if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
-    return (uint32_t)sms;
-}
+static uint32_t tc_sms() { return (uint32_t)tgpk_sms(); }
 
 // Does the paired kernel share the tiles of a block between two pairs?  Blocks of more than 128 activation rows and K >= 8192, more tiles than the one-tile-per-CTA
 // kernel holds in one wave of slices and at most a cluster's tile each in one wave.  The sums are those of half of K in four accumulators each, as near 64 bits as
@@ -887,11 +879,7 @@ constexpr uint32_t Q_RING = 227u * 1024u - 2048u;
 
 template <bool SHARED>
 static int launch_pair(ListArgs &p, cudaStream_t st) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        if (cudaFuncSetAttribute(tgp_matmul_tc_pair_kernel<SHARED>, cudaFuncAttributeMaxDynamicSharedMemorySize, Q_RING + 2048) != cudaSuccess) return TGP_E_CUDA;
-        attr_set = true;
-    }
+    if (!tgpk_allow_smem<tgp_matmul_tc_pair_kernel<SHARED>>(Q_RING + 2048)) return TGP_E_CUDA;
     const uint32_t stage = KH * (BM * BK * 2 + p.N / 2 * BK * 2);
     p.stages = std::min(8u, Q_RING / stage);
     const uint32_t tiles = p.tiles_m * p.tiles_n;
@@ -911,11 +899,7 @@ static int launch_pair(ListArgs &p, cudaStream_t st) {
 }
 
 static int launch_stream(ListArgs &p, cudaStream_t st) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        if (cudaFuncSetAttribute(tgp_wstream_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, S_RING_LONE + 2048) != cudaSuccess) return TGP_E_CUDA;
-        attr_set = true;
-    }
+    if (!tgpk_allow_smem<tgp_wstream_tc_kernel>(S_RING_LONE + 2048)) return TGP_E_CUDA;
     const uint32_t stage = BM * BK * 2 + p.N * BK * 2, ctas = p.tiles_m * p.tiles_n * p.slices;
     p.stages = std::min(S_STAGES, (ctas <= tc_sms() ? S_RING_LONE : S_RING) / stage);
     cudaLaunchConfig_t cfg = {};
@@ -1023,11 +1007,7 @@ int tgpk_gemm_tc(const void *A, const void *W, float *C, uint32_t M, uint32_t n,
     if (persistent) {
         const uint32_t tiles_p = ((M + BM - 1) / BM) * ((n + P_BN - 1) / P_BN);
         constexpr int SMEM = P_STAGES * (BM * BK * 2 + P_BN * BK * 2) + 128 + 1024;
-        static bool attr_p = false;
-        if (!attr_p) {
-            if (cudaFuncSetAttribute(tgp_matmul_tc_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess) return TGP_E_CUDA;
-            attr_p = true;
-        }
+        if (!tgpk_allow_smem<tgp_matmul_tc_persistent_kernel>(SMEM)) return TGP_E_CUDA;
         tgp_matmul_tc_persistent_kernel<<<tiles_p < sms ? tiles_p : sms, 192, SMEM, st>>>(ma, mb, C, M, n, K, ldc, col0, accumulate, ep);
     } else {
         // fewer tiles than SMs: one CTA per SM, so the ring may take all of shared memory (a 3-stage ring leaves a lone

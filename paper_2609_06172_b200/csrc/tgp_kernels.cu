@@ -54,11 +54,18 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-static int device_sms() {
-    static int sms = 0;
-    if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
+int tgpk_sms() {
+    static std::atomic<int> known[TGP_DEVICES];
+    const int dev = tgpk_device();
+    int sms = dev < 0 ? 0 : known[dev].load(std::memory_order_relaxed);
+    if (!sms) {
+        int d = 0;
+        if (cudaGetDevice(&d) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d) != cudaSuccess || sms < 1) return 148;
+        if (dev >= 0) known[dev].store(sms, std::memory_order_relaxed);
+    }
     return sms;
 }
+static int device_sms() { return tgpk_sms(); }
 
 static int g_small_pdl = 1;      // small kernels are launched as programmatic dependents of their predecessor (0: plain launches)
 thread_local bool tgpk_whole_edge = false;     // this thread's next launches wait for their predecessors as a whole, however the switches stand
@@ -2038,15 +2045,11 @@ static void launch_skinny_pick(const bf16 *A, const GemvParts &p, const SkinnyPi
 
 template <int MT, int RB, int U>
 static void launch_gemv_splitk(const bf16 *A, const bf16 *W, float *C, uint32_t Mrows, uint32_t n, uint32_t K, uint32_t ldc, uint32_t col0, int acc, cudaStream_t st) {
-    static int blocks_per_sm = 0, sms = 0;
+    static int blocks_per_sm = 0;
     if (!blocks_per_sm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, tgp_wstream_splitk_kernel<MT, RB, U>, 256, 0) != cudaSuccess || blocks_per_sm < 1) blocks_per_sm = 1;
-        if (sms < 1) sms = 148;
     }
-    uint32_t need = (n + RB - 1) / RB, full = (uint32_t)(sms * blocks_per_sm);
+    uint32_t need = (n + RB - 1) / RB, full = (uint32_t)(device_sms() * blocks_per_sm);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(need < full ? need : full);
     cfg.blockDim = dim3(256);
@@ -2102,15 +2105,11 @@ static void launch_gemv_rows(const bf16 *A, const bf16 *W, float *C, uint32_t Mr
 
 template <int MT, bool FUSED>
 static void launch_gemv_group(const bf16 *A, const GemvParts &p, uint32_t Mrows, uint32_t n_total, uint32_t K, int acc, cudaStream_t st, const ASrc &src = ASrc{}) {
-    static int blocks_per_sm = 0, sms = 0;
+    static int blocks_per_sm = 0;
     if (!blocks_per_sm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, tgp_wstream_group_kernel<MT, 8, FUSED>, 256, 0) != cudaSuccess || blocks_per_sm < 1) blocks_per_sm = 1;
-        if (sms < 1) sms = 148;
     }
-    uint32_t need = (n_total + 7) / 8, full = (uint32_t)(sms * blocks_per_sm);
+    uint32_t need = (n_total + 7) / 8, full = (uint32_t)(device_sms() * blocks_per_sm);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(need < full ? need : full);
     cfg.blockDim = dim3(256);
@@ -2399,8 +2398,7 @@ static void launch_expert_rows(cudaLaunchConfig_t &cfg, const bf16 *A, const Gem
         constexpr int U = decltype(steps)::value;
         constexpr size_t smem = (size_t)NW * RG * NB * 4 * 32 * 4;
         if constexpr (smem > 48 * 1024) {
-            static bool attr_set = false;
-            if (!attr_set) { cudaFuncSetAttribute(tgp_wstream_mma_group_kernel<NB, U, NW, RG, EXP_U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); attr_set = true; }
+            tgpk_allow_smem<tgp_wstream_mma_group_kernel<NB, U, NW, RG, EXP_U>>(smem);
             cfg.dynamicSmemBytes = smem;
         }
         launch_weights<tgp_wstream_mma_group_kernel<NB, U, NW, RG, EXP_U>>(cfg, A, p, me, groups, K, 0, rpc, 0);
@@ -2707,8 +2705,7 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
         const bool grouped = g_attn_decode_grouped && (G == 1 || G == 2 || G == 4 || G == 8) && c->Hq % c->Hkv == 0;
         const uint32_t nchunks = (pos0 + 1 + DEC_KEYS - 1) / DEC_KEYS;
         if (decode_mma(qb, tiles, c, q_len, pos0, scratch)) {
-            static int sms = 0;
-            if (!sms) { int dev = 0; cudaGetDevice(&dev); if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148; }
+            const int sms = device_sms();
             const uint32_t units = B * c->Hkv, per_sm = c->Dh == 64 ? 4 : 2;             // CTAs that fit an SM (96 / 48 KB of shared memory each)
             uint32_t parts = (uint32_t)sms * per_sm / units;                              // CTAs per (sequence, KV head): one wave at most
             const uint32_t slots = (uint32_t)sms * per_sm;
@@ -2746,8 +2743,7 @@ int tgpk_attn(const void *qb, const TgpTilePtrs &tiles, uint32_t n_tiles, void *
             cfg.attrs = attr;
             cfg.numAttrs = cluster ? 2 : 1;
 #define TGP_DECODE_MMA_R(DH_, G_, SP_, CL_, RO_) do { \
-                static bool attr_set = false; \
-                if (!attr_set) { if (cudaFuncSetAttribute(tgp_attn_decode_mma_kernel<DH_, G_, SP_, CL_, RO_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TGP_E_CUDA; attr_set = true; } \
+                if (!tgpk_allow_smem<tgp_attn_decode_mma_kernel<DH_, G_, SP_, CL_, RO_>>(smem)) return TGP_E_CUDA; \
                 cudaLaunchKernelEx(&cfg, tgp_attn_decode_mma_kernel<DH_, G_, SP_, CL_, RO_>, a, per_cta); } while (0)
 #define TGP_DECODE_MMA_P(DH_, G_, SP_, CL_) do { if (rotates) TGP_DECODE_MMA_R(DH_, G_, SP_, CL_, true); else TGP_DECODE_MMA_R(DH_, G_, SP_, CL_, false); } while (0)
 #define TGP_DECODE_MMA(DH_, G_) do { if (cluster) { if (split_p) TGP_DECODE_MMA_P(DH_, G_, true, true); else TGP_DECODE_MMA_P(DH_, G_, false, true); } \

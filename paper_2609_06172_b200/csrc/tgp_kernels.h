@@ -1,10 +1,29 @@
 // Internal launch interface between the step engine and the kernels.
 #pragma once
 #include <cuda_runtime.h>
+#include <atomic>
 #include <cstdint>
 #include "tgp.h"
 
 #define TGP_MAX_TILES 64      // KV tiles per layer a kernel can address (pointer table passed by value)
+
+// Function attributes and the number of SMs are a device's own, and a process may use several: what is kept of them is kept by device.
+#define TGP_DEVICES 64        // of these; further ones ask every time
+inline int tgpk_device() { int dev = 0; return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < TGP_DEVICES ? dev : -1; }
+int tgpk_sms();               // SMs of the current device
+
+// Dynamic shared memory above 48 KB for a kernel on the current device; `shared_first` also asks for the split of L1 and shared memory that leaves it all to the latter (a hint).
+template <auto KERNEL>
+inline bool tgpk_allow_smem(size_t bytes, bool shared_first = false) {
+    static std::atomic<uint64_t> allowed{0};                  // a bit per device
+    const int dev = tgpk_device();
+    const uint64_t bit = dev < 0 ? 0 : 1ull << dev;
+    if (bit & allowed.load(std::memory_order_relaxed)) return true;
+    if (cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
+    if (shared_first && cudaFuncSetAttribute(KERNEL, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess) cudaGetLastError();
+    allowed.fetch_or(bit, std::memory_order_relaxed);
+    return true;
+}
 
 struct TgpTilePtrs { void *k[TGP_MAX_TILES]; void *v[TGP_MAX_TILES]; };
 

@@ -62,3 +62,18 @@ def test_a_launch_hint_is_given_on_every_device_and_fails_no_product():
     body = re.search(r"static void launch_weights\(.*?\n\}\n", text, re.S).group(0)
     assert not re.search(r"static\s+(const\s+)?(cudaError_t|bool|auto)\b", body) and "cudaGetDevice" in body
     assert re.search(r"cudaFuncSetAttribute\([^;]*!= cudaSuccess\) cudaGetLastError\(\);", body)
+
+
+def test_what_is_a_devices_own_is_kept_by_device():
+    """A process may use several devices: an attribute that a flag of the process says is set, or a number of SMs asked for once, would be the first one's."""
+    sources = {f: re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, f)).read()) for f in sorted(os.listdir(CSRC)) if f.endswith((".cu", ".cuh", ".h", ".cpp"))}
+    for f, text in sources.items():
+        assert not re.search(r"static\s+(bool|int|uint32_t)\s+(\w+\s*=\s*0\s*,\s*)?(attr_\w+|sms)\b", text), f
+    held = {f: len(re.findall(r"cudaFuncSetAttribute\(", text)) for f, text in sources.items()}
+    # tgpk_allow_smem() and launch_weights(), a bit per device each
+    assert {f: n for f, n in held.items() if n} == {"tgp_kernels.h": 2, "tgp_kernels.cu": 1}
+    assert sum(len(re.findall(r"cudaDevAttrMultiProcessorCount", text)) for text in sources.values()) == 1
+    for f, name in (("tgp_kernels.h", "tgpk_allow_smem"), ("tgp_kernels.cu", "tgpk_sms")):
+        body = re.search(r"\b%s\([^;{]*\) \{\n.*?\n\}\n" % name, sources[f], re.S).group(0)
+        assert "tgpk_device()" in body, name
+    assert "cudaGetDevice" in re.search(r"inline int tgpk_device\(\).*", sources["tgp_kernels.h"]).group(0)
