@@ -636,3 +636,20 @@ for act, out in ((lambda: 1 / 0, ZeroDivisionError), (interrupt, KeyboardInterru
     root = os.path.dirname(os.path.dirname(os.path.abspath(tb.__file__)))
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=root)
     assert r.returncode == 0, (r.returncode, r.stderr)
+
+
+@pytest.mark.parametrize("cc", ["false", "/nonexistent/cc"])
+def test_a_machine_that_cannot_build_the_extension_still_builds_the_library(cc, monkeypatch, tmp_path):
+    """ctypes serves every call, so a missing C compiler is a warning; an extension of an earlier build does not stay beside a newer library."""
+    old = tmp_path / "_fastcall.so"
+    old.write_bytes(b"")
+    os.utime(old, (0, 0))
+    monkeypatch.setattr(tbuild, "FASTCALL", str(old))
+    monkeypatch.setenv("CC", cc)
+    assert tbuild.needs_build()
+    with pytest.warns(RuntimeWarning, match="ctypes"):
+        assert tbuild.build() == tbuild.LIB
+    assert not old.exists() and os.path.exists(tbuild.LIB)
+    monkeypatch.setenv("CC", "gcc")
+    tbuild.build()
+    assert old.stat().st_size and not tbuild.needs_build()
