@@ -1230,8 +1230,9 @@ def test_products_of_few_tiles_alone_have_the_bits_of_the_pairs(M, n, K, alone):
         assert float((one[:, :n].double() - exact).abs().max()) < 2e-5 * float(exact.abs().max())
 
 
-@pytest.mark.parametrize("M,n,K", [(129, 4097, 8192), (150, 4096, 8200), (257, 2100, 8192), (509, 2048, 8200), (512, 2048, 14336), (1100, 1000, 8328), (256, 4700, 8192)])
-def test_products_of_a_long_k_whose_tiles_two_pairs_share(M, n, K):
+# (the last: one tile more than clusters fit 148 SMs, so that slices of single CTAs serve it)
+@pytest.mark.parametrize("M,n,K", [(129, 4097, 8192), (150, 4096, 8200), (257, 2100, 8192), (509, 2048, 8200), (512, 2048, 14336), (1100, 1000, 8328), (256, 4600, 8192), (256, 4700, 8192)])
+def test_products_of_a_long_k_whose_tiles_two_pairs_share(M, n, K, tmp_path):
     """More than 128 activation rows, K >= 8192 and few tiles: a block alone and in a list of 2 and of 8 (more clusters than fit the GPU at a time) has
     the same bits, no other column changes, and it is as near the fp64 product as fp32 sums are."""
     gen = torch.Generator(device=DEV)
@@ -1239,6 +1240,12 @@ def test_products_of_a_long_k_whose_tiles_two_pairs_share(M, n, K):
     A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
     W = (torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16()
     want = A.double() @ W.double().T
+    scratch = torch.empty((M, n), device=DEV)
+    (name, args), = kernels_of(lambda: tb.k_gemm(A, W, scratch, M, n, K, n, 0, False), tmp_path)
+    if n == 4700:
+        assert "tgp_wstream_tc_kernel" in name, name
+    else:
+        assert "tgp_matmul_tc_pair_kernel" in name and ("true" in name or "(bool)1" in name) and args["grid"][0] % 4 == 0, (name, args["grid"])
     for acc in (False, True):
         c0 = torch.randn((M, n + 4), device=DEV, generator=gen)
         one = c0.clone()
@@ -1273,9 +1280,10 @@ def test_products_in_small_tiles_of_pairs_have_the_bits_of_the_largest(M, n, K):
 
 
 @pytest.mark.parametrize("Dh,Hq,Hkv,B,S,pos0,TK", [(64, 4, 4, 1, 384, 0, 64), (128, 4, 1, 2, 500, 0, 128), (64, 8, 2, 1, 129, 300, 64), (128, 2, 2, 3, 201, 1500, 256), (64, 2, 1, 1, 1000, 37, 128)])
-def test_prefill_attention_whose_key_blocks_two_ctas_share(Dh, Hq, Hkv, B, S, pos0, TK):
+def test_prefill_attention_whose_key_blocks_two_ctas_share(Dh, Hq, Hkv, B, S, pos0, TK, tmp_path):
     """Grids that leave SMs idle: two CTAs of a cluster take half of the key blocks each.  Ragged last query blocks, rows whose keys lie in the first half only or begin inside
-    the second, scores that grow towards the last keys (a moved exponent reference in one half), against 64 bits; an infinity in a key's score, an infinity in V."""
+    the second, scores that grow towards the last keys (a moved exponent reference in one half), against 64 bits; keys of score -inf; an infinity in V, which reaches the rows that see
+    its key, whichever half has it, and no row of a query block that ends before the key's block."""
     gen = torch.Generator(device=DEV)
     gen.manual_seed(S + pos0)
     n, kv, G = (pos0 + S + TK - 1) // TK, pos0 + S, Hq // Hkv
@@ -1284,18 +1292,26 @@ def test_prefill_attention_whose_key_blocks_two_ctas_share(Dh, Hq, Hkv, B, S, po
     q = torch.randn((B, S, Hq, Dh), device=DEV, generator=gen).bfloat16()
     q[..., 0] = 1
 
-    def check(K, V):
+    def run(K, V):
         kt, vt = ([t.permute(1, 2, 0, 3).contiguous() for t in T.split(TK)] for T in (K, V))
         ob = torch.zeros((B, S, Hq, Dh), device=DEV, dtype=torch.bfloat16)
-        tb.k_attn(q, kt, vt, ob, mc, B, S, pos0, None)
-        torch.cuda.synchronize()
+        (name, args), = kernels_of(lambda: tb.k_attn(q, kt, vt, ob, mc, B, S, pos0, None), tmp_path)
+        assert "tgp_attn_prefill_tc_kernel" in name and args["grid"] == [2 * ((S + 127) // 128), Hq, B], (name, args["grid"])
         assert tb.k_attn_status() == 0
+        return ob.double()
+
+    def exact(K, V):
         k64, v64 = (T[:kv].permute(1, 2, 0, 3).double().repeat_interleave(G, 1) for T in (K, V))
         sc = q.permute(0, 2, 1, 3).double() @ k64.transpose(-1, -2) / Dh ** 0.5
         mask = torch.arange(kv, device=DEV)[None, :] > pos0 + torch.arange(S, device=DEV)[:, None]
-        want = (torch.softmax(sc.masked_fill(mask, -float("inf")), -1) @ v64).permute(0, 2, 1, 3)
+        return (torch.softmax(sc.masked_fill(mask, -float("inf")), -1) @ v64).permute(0, 2, 1, 3)
+
+    def close(got, want):
         # half a bf16 step of the output and of each of the probabilities, whose roundings average out: 2^-9 of the largest V, as in the tests above
-        assert float((ob.double() - want).abs().max()) < 2.0 ** -7 * float(want.abs().max()) + 1e-6
+        assert float((got - want).abs().max()) < 2.0 ** -7 * float(want.abs().max()) + 1e-6
+
+    def check(K, V):
+        close(run(K, V), exact(K, V))
 
     K, V = (torch.zeros((n * TK, B, Hkv, Dh), device=DEV, dtype=torch.bfloat16) for _ in range(2))
     K[:kv], V[:kv] = (torch.randn((kv, B, Hkv, Dh), device=DEV, generator=gen).bfloat16() for _ in range(2))
@@ -1308,6 +1324,16 @@ def test_prefill_attention_whose_key_blocks_two_ctas_share(Dh, Hq, Hkv, B, S, po
     blocks = (kv + 63) // 64
     hidden[64 * ((blocks + 1) // 2):64 * ((blocks + 1) // 2) + 64, :, :, 0] = -float("inf")
     check(hidden, V)
+    finite, at = exact(K, V), pos0 + torch.arange(S, device=DEV)
+    last = pos0 + torch.clamp((torch.arange(S, device=DEV) // 128 + 1) * 128, max=S) - 1            # position of the last row of a row's query block
+    for key in (3, 64 * ((blocks + 1) // 2) - 1, 64 * ((blocks + 1) // 2), kv - 1):                 # the last query block's halves end and begin at the middle two
+        Vi = V.clone()
+        Vi[key, ..., 5], Vi[key, ..., 6] = float("inf"), -float("inf")
+        got, sees, clear = run(K, Vi), at >= key, last // 64 < key // 64
+        assert (got[:, sees][..., 5] == float("inf")).all() and (got[:, sees][..., 6] == -float("inf")).all()
+        close(got[:, clear], finite[:, clear]) if clear.any() else None
+        others = [i for i in range(Dh) if i not in (5, 6)]
+        close(got[..., others], finite[..., others])
 
 
 # a grid whose key blocks two CTAs share and one that leaves no SM idle, both head sizes; mma.sync by length and by choice; the CUDA-core kernels of few queries, of three
@@ -1346,3 +1372,65 @@ def test_attention_whose_first_keys_score_minus_infinity(Dh, Hq, Hkv, B, S, pos0
         assert torch.equal(got.isfinite(), fin), (lo, hi)
         # half a bf16 step of the output and of each of the probabilities, whose roundings average out: 2^-9 of the largest V, as in the tests above
         assert not fin.any() or float((got - want)[fin].abs().max()) < 2.0 ** -7 * float(want[fin].abs().max()) + 1e-6
+
+
+def test_products_whose_tiles_two_pairs_share_give_up_on_a_wait_that_runs_out_and_recover():
+    """The four CTAs of the first cluster never load their second stage: the waits for their tile run out in both pairs, none of the four stores anything, every other
+    tile is right, and the next launch is correct."""
+    M, n, K = 509, 2048, 8192
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(5)
+    A = torch.randn((M, K), device=DEV, generator=gen).bfloat16()
+    W = (torch.randn((n, K), device=DEV, generator=gen) * 0.02).bfloat16()
+    want = A.double() @ W.double().T
+    SENT = 12345.0
+    tb.k_status_clear()
+    try:
+        tb.k_wait_test(2_000_000, 1)
+        C = torch.full((M, n), SENT, device=DEV)
+        tb.k_gemm(A, W, C, M, n, K, n, 0, 0)
+        torch.cuda.synchronize()
+        assert tb.k_gemm_status() >> 8 in (2, 3)              # the MMA threads' waits for the stage, the epilogues' for the accumulators
+        untouched = C == SENT
+        rows = int(untouched[:, 0].sum())                     # (the tile's activation rows)
+        assert 32 <= rows <= 128 and rows % 32 == 0 and untouched[:rows, :256].all() and int(untouched.sum()) == 256 * rows
+        assert float((C.double() - want)[~untouched].abs().max()) < 2e-5 * float(want.abs().max())
+    finally:
+        tb.k_wait_test(0, -1)
+        tb.k_status_clear()
+    tb.k_gemm(A, W, C, M, n, K, n, 0, 0)
+    torch.cuda.synchronize()
+    assert tb.k_gemm_status() == 0 and float((C.double() - want).abs().max()) < 2e-5 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("Dh", [64, 128])
+def test_attention_whose_key_blocks_two_ctas_share_gives_up_on_a_wait_that_runs_out_and_recovers(Dh):
+    """The grid's first CTA - the first half of the key blocks of the last 128 queries of head 0 - never loads its second V block: its waits run out, neither it nor the CTA
+    that has the other half stores anything, all other rows are right, and the next launch is correct."""
+    S, Hq, Hkv, TK = 512, 4, 2, 64
+    cfg = replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hkv, TK=TK, S=S, T=0, B=1, d=Hq * Dh)
+    mc = model_cfg(cfg)
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(Dh)
+    q, K, V = (torch.randn((S, h, Dh), device=DEV, generator=gen).bfloat16() for h in (Hq, Hkv, Hkv))
+    kt, vt = ([t.permute(1, 0, 2).contiguous()[None] for t in T.split(TK)] for T in (K, V))
+    k64, v64 = (T.permute(1, 0, 2).double().repeat_interleave(Hq // Hkv, 0) for T in (K, V))
+    sc = (q.permute(1, 0, 2).double() @ k64.transpose(-1, -2) / Dh ** 0.5).masked_fill(torch.ones((S, S), device=DEV, dtype=torch.bool).triu(1), -float("inf"))
+    want = (torch.softmax(sc, -1) @ v64).permute(1, 0, 2)
+    tol = 2.0 ** -7 * float(want.abs().max()) + 1e-6          # as in the tests above
+    tb.k_status_clear()
+    try:
+        tb.k_wait_test(2_000_000, 1)
+        ob = torch.full((S, Hq, Dh), 768.0, dtype=torch.bfloat16, device=DEV)
+        tb.k_attn(q, kt, vt, ob, mc, 1, S, 0, None)
+        torch.cuda.synchronize()
+        assert tb.k_attn_status() in (1, 2, 3)
+        untouched = ob == 768.0
+        assert untouched[S - 128:, 0].all() and int(untouched.sum()) == 128 * Dh
+        assert float((ob.double() - want)[~untouched].abs().max()) < tol
+    finally:
+        tb.k_wait_test(0, -1)
+        tb.k_status_clear()
+    tb.k_attn(q, kt, vt, ob, mc, 1, S, 0, None)
+    torch.cuda.synchronize()
+    assert tb.k_attn_status() == 0 and float((ob.double() - want).abs().max()) < tol
