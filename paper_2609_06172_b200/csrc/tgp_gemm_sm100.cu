@@ -832,11 +832,16 @@ static uint32_t tc_sms() { return (uint32_t)tgpk_sms(); }
 // Does the paired kernel share the tiles of a block between two pairs?  Blocks of more than 128 activation rows and K >= 8192, more tiles than the one-tile-per-CTA
 // kernel holds in one wave of slices and at most a cluster's tile each in one wave.  The sums are those of half of K in four accumulators each, as near 64 bits as
 // that kernel's four slices with two (M=509, n=2048, K=8192: 29.2 us in slices, 23.9 shared; M=150, n=4096, K=14336: 44.8, 41.8; but n=2048, K=8192
-// 16.8, 18.3).  With a shorter K sharing gains 5 % at best over smaller tiles.  The choice depends on M, n and K of the block and on the
-// number of SMs (the bits may differ between devices of different sizes), not on a list.
+// 16.8, 18.3).  With a shorter K sharing gains 5 % at best over smaller tiles.  The choice depends on M, n, K and the number of SMs (the bits may differ between
+// devices of different sizes), not on a list.
+//   One wave: a cluster of four lies in one GPC, of which two to four SMs stay over, so that 148 SMs hold 33 clusters and not 37, fewer where GPCs are cut
+// differently; counted on are seven eighths, 32 (K=8192, M=236 in slices and shared: 32 tiles 29.0 / 25.5 us, 34 tiles 29.4 / 40.5; M=364, 27 tiles in rows
+// of 128, which is one wave, 23, in rows of 96, which would be one of 37, 32).
+static uint32_t shared_at_once() { return tc_sms() * 7 / 32; }
+
 static bool shared_tiles(uint32_t M, uint32_t n, uint32_t K) {
-    const uint64_t rows = (M + BM - 1) / BM, sms = tc_sms();
-    return M > BM && K >= 8192 && rows * ((n + BM - 1) / BM) * 4 > sms && rows * ((n + 2 * BM - 1) / (2 * BM)) * 4 <= sms;
+    const uint64_t rows = (M + BM - 1) / BM;
+    return M > BM && K >= 8192 && rows * ((n + BM - 1) / BM) * 4 > tc_sms() && rows * ((n + 2 * BM - 1) / (2 * BM)) <= shared_at_once();
 }
 
 // K slices of a block in the one-tile-per-CTA kernel, 0: the paired kernel serves it.  No list counts here either.  Measured (us; M=61):
@@ -944,7 +949,7 @@ int tgpk_gemm_tc_list(const void *A, uint32_t count, const void *const *W, float
         p.N = ((M + t - 1) / t + 15) / 16 * 16;
     } else {
         p.slices = g_tc_variant != 3 && shared_tiles(M, n[0], K) ? 2 : 1;
-        p.N = p.slices == 2 ? pair_rows(M, p.tiles_n, K / 2, tc_sms() / 4, 128) : pair_rows(M, p.tiles_n, K, tc_sms() / 2, 256);
+        p.N = p.slices == 2 ? pair_rows(M, p.tiles_n, K / 2, shared_at_once(), 128) : pair_rows(M, p.tiles_n, K, tc_sms() / 2, 256);
     }
     p.tiles_m = (M + p.N - 1) / p.N;
     if (!make_map(&p.x, A, M, K, stream ? p.N : p.N / 2)) return TGP_E_CUDA;
