@@ -858,12 +858,13 @@ static uint32_t cta_slices(uint32_t M, uint32_t n, uint32_t K) {
 
 // Estimated cycles of the paired kernel for `wt` tiles of 256 weight rows at M activation rows in tiles of N, with room for `at_once` tiles.  A 64-wide block of K
 // of a pair takes 2 N cycles of the tensor pipe (172 at least) and (16384 + 64 N) bytes per SM, which arrive at 80 a clock (what a full ring
-// asks for in the 1.4 us a load takes); the first stage arrives after 3000 cycles, and a tile's epilogue writes 512 N bytes per SM at 32 a clock (a few
-// of them are under way when it ends: 1600 cycles), under the MMAs of the next tile.
+// asks for in the 1.4 us a load takes); the first stage arrives after 3000 cycles, and a tile's epilogue, under the MMAs of the next one, takes 1600 cycles and
+// writes 512 N bytes per SM at 32 a clock (16 for residual adds, which shifts all choices alike).  The 1600 count for every tile, not only behind the last: 66 forms
+// of M=212 - 2000, K=64 - 2048 take 1.001 of the time of their best tiles so, 1.05 otherwise, by K=64 most (M=288, n=14464 in tiles of 144 rows 9.8 us, of 32 14.1).
 static uint64_t pair_cost(uint32_t M, uint32_t wt, uint32_t K, uint32_t N, uint32_t at_once) {
     const uint64_t tiles = (uint64_t)((M + N - 1) / N) * wt, rounds = (tiles + at_once - 1) / at_once;
-    const uint64_t mma = (uint64_t)((K + BK - 1) / BK) * std::max<uint64_t>(std::max(2 * N, 172u), (16384 + 64 * N) / 80), epi = 16 * N;
-    return 3000 + mma + (rounds - 1) * std::max(mma, epi) + epi + 1600;
+    const uint64_t mma = (uint64_t)((K + BK - 1) / BK) * std::max<uint64_t>(std::max(2 * N, 172u), (16384 + 64 * N) / 80), epi = 16 * N + 1600;
+    return 3000 + mma + (rounds - 1) * std::max(mma, epi) + epi;
 }
 
 // Activation rows per tile: what the estimate above says is fastest (us with the norm before; estimates rank the choices as the clock does: M=509, n=2048, K=2048
