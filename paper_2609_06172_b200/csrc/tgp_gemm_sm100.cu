@@ -861,9 +861,11 @@ static uint32_t cta_slices(uint32_t M, uint32_t n, uint32_t K) {
 // asks for in the 1.4 us a load takes); the first stage arrives after 3000 cycles, and a tile's epilogue, under the MMAs of the next one, takes 1600 cycles and
 // writes 512 N bytes per SM at 32 a clock (16 for residual adds, which shifts all choices alike).  The 1600 count for every tile, not only behind the last: 66 forms
 // of M=212 - 2000, K=64 - 2048 take 1.001 of the time of their best tiles so, 1.05 otherwise, by K=64 most (M=288, n=14464 in tiles of 144 rows 9.8 us, of 32 14.1).
+// Where K is no multiple of 64 the 128 bytes that a box takes of a row lie in two lines, and arrive at 70 a clock (M=501, n=11469+352+1013, K=5832 in tiles
+// of 256 rows 95 us, of 128, which 80 a clock would make the faster ones, 103; over 80 such forms 1.002 of the best, 1.007 otherwise).
 static uint64_t pair_cost(uint32_t M, uint32_t wt, uint32_t K, uint32_t N, uint32_t at_once) {
     const uint64_t tiles = (uint64_t)((M + N - 1) / N) * wt, rounds = (tiles + at_once - 1) / at_once;
-    const uint64_t mma = (uint64_t)((K + BK - 1) / BK) * std::max<uint64_t>(std::max(2 * N, 172u), (16384 + 64 * N) / 80), epi = 16 * N + 1600;
+    const uint64_t mma = (uint64_t)((K + BK - 1) / BK) * std::max<uint64_t>(std::max(2 * N, 172u), (16384 + 64 * N) / (K % BK ? 70 : 80)), epi = 16 * N + 1600;
     return 3000 + mma + (rounds - 1) * std::max(mma, epi) + epi;
 }
 

@@ -83,11 +83,12 @@ def test_what_is_a_devices_own_is_kept_by_device():
 # (activation rows, weight tiles, K): activation rows per tile that were within 3 % of the fastest, on 148 SMs (us; K = 64 and M = 288: 144 rows 9.8, 96 10.2, 64 11.1, 32 14.1)
 FASTEST = {(288, 57, 64): {144}, (288, 57, 256): {144}, (212, 59, 128): {224, 256}, (417, 40, 128): {144}, (1264, 42, 256): {256}, (1758, 30, 256): {256}, (509, 56, 512): {256},
            (300, 118, 64): {160}, (300, 118, 1024): {112, 160}, (603, 8, 64): {80, 96}, (603, 8, 2048): {80, 96}, (1024, 16, 128): {256}, (1024, 16, 2048): {256}, (2000, 8, 512): {224},
-           (400, 12, 64): {80}, (400, 12, 2048): {80}}
+           (400, 12, 64): {80}, (400, 12, 2048): {80},
+           (501, 51, 4584): {256}, (501, 51, 5832): {256}, (2493, 33, 4584): {240}, (2493, 33, 7000): {240}, (539, 59, 232): {192}}
 
 
 def test_tiles_of_the_paired_products_are_the_fastest_measured(tmp_path):
-    """The estimate that chooses the tiles, compiled by itself: it knows the cost of a tile's end, which is most of a short K."""
+    """The estimate that chooses the tiles, compiled by itself: it knows the cost of a tile's end, which is most of a short K, and of rows that begin inside a line."""
     text = open(os.path.join(CSRC, "tgp_gemm_sm100.cu")).read()
     body = "".join(re.search(r"static \w+ %s\(uint32_t M, uint32_t wt.*?\n\}\n" % f, text, re.S).group(0) for f in ("pair_cost", "pair_rows"))
     calls = "".join('printf("%%u\\n", pair_rows(%du, %du, %du, 74, 256));' % case for case in FASTEST)
