@@ -192,9 +192,18 @@ __global__ void __launch_bounds__(192) tgp_matmul_tc_kernel(const __grid_constan
                             *reinterpret_cast<float4 *>(dst + j) = o;
                         }
                     } else {
+                        // (a lane's row is a line of its own, and what L1 the ring leaves does not keep them from one element to the next: the old sums are all
+                        // requested before the first is stored)
+                        if (accumulate) {
+                            float old[32];
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) old[j] = col + j < n ? dst[j] : 0.f;
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) v[j] = old[j] + v[j];
+                        }
 #pragma unroll
                         for (int j = 0; j < 32; ++j)
-                            if (col + j < n) dst[j] = accumulate ? dst[j] + v[j] : v[j];
+                            if (col + j < n) dst[j] = v[j];
                     }
                 }
             }
