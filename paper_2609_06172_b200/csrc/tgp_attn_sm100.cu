@@ -429,15 +429,16 @@ static int launch(const CUtensorMap &mq, const CUtensorMap &mkv, const CUtensorM
 }
 
 // Two CTAs per query block and head where both of all of them fit the GPU at a time and the longest chain of key blocks makes up for the exchange, which takes longer
-// with 128 dimensions and where most SMs have two CTAs anyway (us with the norm before, one against two: 8 heads x 64, 128 queries behind 1000 keys 17.6 / 13.1, behind
-// 200 9.4 / 8.5; 16 heads x 128, 509 queries 14.3 / 11.6, 384 10.7 / 10.5; 32 heads x 128, 384 queries 11.5 / 13.5; 128 CTAs: 13 - 16 blocks 1.02 - 1.14 times as fast, 8
-// blocks 0.92 - 1.08; 192 CTAs of 27 blocks 33.1 / 37.9).
+// with 128 dimensions, and for what two CTAs of an SM take from each other.  The lines are where two are no slower by themselves, behind the rotation and in a whole
+// layer of k_* calls (us, one against two CTAs, behind the rotation; heads x dimensions, query blocks x sequences: key blocks): 8 x 128, 3 x 1: 8 11.6 / 10.4; 16 x 128, 4 x 1:
+// 10 16.1 / 12.6 (in a layer 35.3 / 35.6, with 8 34.0 / 34.5); 16 x 64, 3 x 2: 8 11.2 / 12.1, 12 14.1 / 13.7; 8 x 128, 4 x 4: 12 16.5 / 17.3, 14 18.1 / 18.2,
+// 17 20.2 / 19.3; 16 x 128, 4 x 2: 14 21.0 / 17.8.  192 CTAs of 27 blocks 33.1 / 37.9.
 static bool split_keys(const TArgs &a, uint32_t B, uint32_t Dh) {
     const int sms = tgpk_sms();
     const uint64_t ctas = (uint64_t)((a.q_len + BQ - 1) / BQ) * a.Hq * B;
     const uint32_t blocks = (a.pos0 + a.q_len + BKV - 1) / BKV;
     if (a.pos0 + (a.q_len < BQ ? a.q_len : BQ) <= BKV) return false;         // a block for each of the two, also of the first queries
-    return 3 * ctas <= 2 * (uint64_t)sms ? blocks >= (Dh == 128 ? 8u : 6u) : ctas <= (uint64_t)sms && blocks >= 12;
+    return ctas <= (uint64_t)sms && blocks >= (3 * ctas <= (uint64_t)sms ? 6u : 2 * ctas <= (uint64_t)sms ? 8u : 12u) + (Dh == 128 ? 2u : 0u);
 }
 
 int tgpk_attn_prefill_tc5(const void *qb, const TgpTilePtrs &tiles, void *ob, const tgp_model_cfg *c, uint32_t B, uint32_t q_len, uint32_t pos0, cudaStream_t st) {

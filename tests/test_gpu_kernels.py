@@ -1436,3 +1436,20 @@ def test_attention_whose_key_blocks_two_ctas_share_gives_up_on_a_wait_that_runs_
     tb.k_attn(q, kt, vt, ob, mc, 1, S, 0, None)
     torch.cuda.synchronize()
     assert tb.k_attn_status() == 0 and float((ob.double() - want).abs().max()) < tol
+
+
+# on either side of the lines: a third, a half and all of 148 SMs have a CTA
+@pytest.mark.parametrize("Dh,Hq,B,S,blocks,two", [(64, 12, 1, 500, 5, False), (64, 12, 1, 384, 6, True), (128, 16, 1, 300, 7, False), (128, 16, 1, 300, 8, True), (64, 16, 1, 500, 7, False),
+                                                  (64, 18, 1, 500, 8, True), (128, 16, 1, 500, 9, False), (128, 18, 1, 500, 10, True), (64, 19, 1, 500, 11, False), (64, 16, 3, 380, 12, True),
+                                                  (128, 19, 1, 500, 13, False), (128, 37, 1, 500, 14, True), (64, 38, 1, 500, 20, False)])
+def test_key_blocks_are_shared_where_that_is_faster(Dh, Hq, B, S, blocks, two, tmp_path):
+    kv, TK = 64 * blocks - 10, 128
+    n, pos0 = (kv + TK - 1) // TK, 64 * blocks - 10 - S
+    if pos0 < 0:
+        pos0, S = 0, kv
+    mc = model_cfg(replace(KCFG, Dh=Dh, Hq=Hq, Hkv=Hq, TK=TK, S=kv, T=0, B=B, d=Hq * Dh))
+    q = torch.randn((B, S, Hq, Dh), device=DEV).bfloat16()
+    kt, vt = ([torch.randn((B, Hq, TK, Dh), device=DEV).bfloat16() for _ in range(n)] for _ in range(2))
+    ob = torch.empty_like(q)
+    (name, args), = kernels_of(lambda: tb.k_attn(q, kt, vt, ob, mc, B, S, pos0, None), tmp_path)
+    assert "tgp_attn_prefill_tc_kernel" in name and args["grid"] == [(2 if two else 1) * ((S + 127) // 128), Hq, B], (name, args["grid"])
