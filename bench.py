@@ -31,8 +31,8 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 import seeded_inputs as si  # noqa: E402
 
-# roofline constants frozen for the planner (integers): sustained bf16 peak and HBM copy bandwidth measured on
-# this machine's B200, pinned host-link bandwidth at 256 MiB measured by this build (profiles/host_link.md)
+# roofline constants frozen for the planner (integers): measured sustained bf16 peak and HBM copy bandwidth of a B200,
+# and its pinned host-link bandwidth with copies of 256 MiB
 MACHINE = dict(peak_flops=1362800000000000, hbm_Bps=6541100000000, h2d_Bps=55570000000, d2h_Bps=56900000000)
 OP_NAMES = ["embed", "rmsnorm", "gemm", "rope_kv", "attn", "swiglu", "router", "argmax"]
 

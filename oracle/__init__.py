@@ -14,5 +14,5 @@ Parity status of each part:
                 is pinned by hand-computed toy rooflines, the schedule by the invariants
                 in validate.py, closed forms and a brute-force pin-set search.  The
                 policy *constants* (hold window, zero-copy ratio, ring minimum, alignment,
-                tie-breaks) are choices of this build: parity unpinned for those.
+                tie-breaks) are choices made here: parity unpinned for those.
 """

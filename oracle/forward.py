@@ -4,7 +4,7 @@ TEST INFRASTRUCTURE - see oracle/__init__.py.
 
 What is computed (the workload the paper runs under oversubscription, Section V-A:
 LLM inference; operator families named in Section III-C: GEMM/GEMV, elementwise /
-normalisation, attention).  Precision contract of this build (the paper states none):
+normalisation, attention).  Precision contract of this implementation (the paper states none):
 bf16 (round-to-nearest-even) at weights, the KV cache and every GEMM input activation;
 everything else (residual stream, accumulators, norm statistics, softmax, router,
 logits) is fp32 on the GPU.  The oracle accumulates in ``dtype`` (float64 by default)

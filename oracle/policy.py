@@ -11,7 +11,7 @@ The paper describes the policy in prose only.  What it fixes, and where:
   (Section IV-B, IV-E "Prefetch Engine");
 * link-bound kernels trigger proactive prefetch; tensors reused across consecutive kernels
   are held resident during their reuse window (Section IV-D look-ahead affinity, IV-E).
-Everything numeric below is this build's reading: the exact inequality, ties, the hold
+Everything numeric below is the reading taken here: the exact inequality, ties, the hold
 window W_AFF, the zero-copy ratio ZC_DEN, the ring minimum, the 512-byte alignment.
 
 Steps, in order (notation: P = peak flop/s, Bh = HBM bytes/s, Bl = host-link bytes/s):

@@ -3,8 +3,9 @@
 // One CTA of eight warps owns 128 consecutive queries of one (sequence, query head); the longest query blocks are
 // launched first.  Roles:
 //   warps 0-3  softmax: thread t is query row t and TMEM lane t;
-//   warp 4     lane 0 issues S_j = Q K_j^T;          warp 6  lane 0 issues O += P_j V_j;
-//   warp 5     lane 0 issues every TMA load;         warp 7  idle (completes the second warpgroup for setmaxnreg).
+//   warp 4     one thread issues S_j = Q K_j^T;      warp 6  one thread issues O += P_j V_j;
+//   warp 5     one thread issues every TMA load;     warp 7  idle (completes the second warpgroup for setmaxnreg).
+// The issuing threads are elected (elect.sync), by every election of a warp the same one: the TMA thread's state is its own registers.
 // Shared memory holds Q and two stages each of K and V blocks of 64 keys as 64-wide blocks of [rows x 128 B] with the
 // 128-byte swizzle (what a TMA box of 64 elements writes); K is then a K-major operand (head dimension contiguous) and
 // V, in the very same layout, an MN-major operand (its contiguous dimension is the output dimension of P V).  One tensor
@@ -17,21 +18,22 @@
 //                                        stage to the TMA warp, which refills it with K_{j+2};
 //   P_j written, V_j landed           -> P V warp issues O += P_j V_j; its completion releases the P buffer and the V
 //                                        stage (refilled with V_{j+2}).
-// An MMA accumulating into the same TMEM tile costs 75-90 cycles whatever its N <= 128, so S (8 MMAs) and P V (4) are
-// issued by different warps and overlap with each other and with the other CTA of the SM.
+// S (8 MMAs of 40 to 64 cycles) and P V (4) are issued by different warps and overlap with each other and with the other CTA of the SM.
 // Softmax: the exponent reference m of a row is its max over block 0 (the lowest finite value where no score is above -inf).  Later blocks use it as it is - P = exp2(S - m)
 // may then exceed 1, which fp32 sums and bf16 P hold without loss of precision - and never compute a row max; only
 // when a block's sum of exponentials exceeds 2^40 (or overflowed) does the warp wait for the P V in flight, move m to
 // the new max and multiply its 32 rows of O in TMEM and its sums by 2^(m_old - m_new).  Scale-and-subtract and the sums
 // use packed fp32 pairs.  At the end every thread reads its row of O once, divides by its sum, and the tile leaves
 // through the (now free) Q buffer by TMA store (partial tiles: plain stores).
+// Grids that leave SMs idle (split_keys()): the two CTAs of a cluster take half of the key blocks of one query block each, bring what they have of the
+// other's dimensions, their sums and references to each other through shared memory, and store half of the dimensions each, by plain stores.
 // Two CTAs fit on an SM (96 KB of shared memory, 256 TMEM columns, 128 registers per thread each, of which setmaxnreg
 // moves the single-thread warps' share to the softmax warps).  KV tiles must hold a multiple of 64 keys; other
 // geometries go to the mma.sync kernel.  Rows of the last V block past the sequence are zeroed in shared memory
 // (0 * stale NaN would poison O); stale K rows only produce masked scores.
 // P is rounded to bf16 for the second product (the one rounding of this path the CPU oracle does not mirror).
 // Every mbarrier wait is bounded; a wait that runs out sets an error word, every role leaves its loop, the TMA warp
-// waits (bounded) for the loads it still has in flight, TMEM is freed and nothing is stored.
+// waits (bounded) for the loads it still has in flight, TMEM is freed and nothing is stored, by neither CTA of a cluster.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cfloat>
@@ -102,7 +104,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
     const uint32_t all_blk = (a.pos0 + last_q + 1 + BKV - 1) / BKV, j_lo = SPLIT && half ? (all_blk + 1) / 2 : 0;
     const uint32_t nblk = SPLIT && !half ? (all_blk + 1) / 2 : all_blk - j_lo;      // key blocks of this CTA, from j_lo on (below they are counted from 0)
 
-    // The TMA thread (warp 5, lane 0) initialises the barriers and requests Q and the first K and V blocks at once, before
+    // The TMA thread (of warp 5) initialises the barriers and requests Q and the first K and V blocks at once, before
     // the TMEM allocation and the CTA-wide barrier below.  Its state: blocks requested so far (block i uses stage i & 1)
     // and, for the next K and V block, the KV tile and the key offset inside it.
     uint32_t nk = 0, nv = 0, k_tile = j_lo * BKV / a.TK, k_off = j_lo * BKV - k_tile * a.TK, v_tile = k_tile, v_off = k_off;
@@ -155,7 +157,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
     if (warp >= 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 64;" ::: "memory");
         if (warp == 5) {
-            // ======================= TMA warp: lane 0 requests the remaining K and V blocks =======================
+            // ======================= TMA warp: the same thread requests the remaining K and V blocks =======================
             if (elect_one()) {
                 // test hook: the first CTA of the grid never loads this V block, so the wait for it runs out
                 const uint32_t withhold = (blockIdx.x | blockIdx.y | blockIdx.z) == 0 ? (uint32_t)g_withhold_step : 0xffffffffu;
@@ -178,7 +180,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
                 }
             }
         } else if (warp == 4) {
-            // ======================= S warp: lane 0 issues S_j = Q K_j^T =======================
+            // ======================= S warp: one thread issues S_j = Q K_j^T =======================
             constexpr uint32_t idesc_s = umma_idesc(BKV);
             auto wait = [&](uint64_t *bar, uint32_t parity, int code) {
                 bool ok = mbar_wait(bar, parity, failed);
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(THREADS, 2) tgp_attn_prefill_tc_kernel(const _
                 __syncwarp();
             }
         } else if (warp == 6) {
-            // ======================= P V warp: lane 0 issues O += P_j V_j =======================
+            // ======================= P V warp: one thread issues O += P_j V_j =======================
             constexpr uint32_t idesc_o = umma_idesc(DH) | (1u << 16);           // bit 16: B operand is MN-major
             auto wait = [&](uint64_t *bar, uint32_t parity, int code) {
                 bool ok = mbar_wait(bar, parity, failed);

@@ -2,14 +2,14 @@
 // bf16 operands, fp32 accumulation in tensor memory.  tgpk_gemm_tc() and tgpk_gemm_tc_list() choose between
 //   tgp_wstream_tc_kernel         one tile of 128 weight rows x up to 128 activation rows per CTA, K in 1, 2 or 4 slices: up to 128
 //                                 activation rows, and more of them on few tiles with a long K;
-//   tgp_matmul_tc_pair_kernel     tiles of 256 weight rows x up to 256 activation rows on the two SMs of a CTA pair: the rest;
+//   tgp_matmul_tc_pair_kernel     tiles of 256 weight rows x up to 256 activation rows on the two SMs of a CTA pair, or shared by two pairs: the rest;
 //   tgp_matmul_tc_kernel          one narrow tile per CTA (below): more than 128 activation rows on few tiles, launched alone.
 // tgp_matmul_tc_persistent_kernel and the other forms of tgp_matmul_tc_kernel run by request only (tgp_k_gemm_tc_variant): they
 // cross-check the others.
 //
 // tgp_matmul_tc_kernel:
-// One CTA computes a 128 x BN tile.  Warp 0 (one lane) feeds a shared-memory ring of ST stages with TMA
-// (128-byte swizzle, 64 bf16 of K per stage); warp 1 (one lane) issues tcgen05.mma (M=128, N=BN, K=16,
+// One CTA computes a 128 x BN tile.  Warp 0 (one elected thread) feeds a shared-memory ring of ST stages with TMA
+// (128-byte swizzle, 64 bf16 of K per stage); warp 1 (one elected thread) issues tcgen05.mma (M=128, N=BN, K=16,
 // four per stage) into a TMEM accumulator and releases stages with tcgen05.commit; warps 2-5 wait for the
 // last commit, read the accumulator with tcgen05.ld (each warp its own 32-lane quarter) and store fp32 rows.
 // Out-of-range rows / columns / K are zero-filled by TMA and masked in the epilogue, so any M, n and
@@ -868,7 +868,7 @@ static uint32_t cta_slices(uint32_t M, uint32_t n, uint32_t K) {
 // Estimated cycles of the paired kernel for `wt` tiles of 256 weight rows at M activation rows in tiles of N, with room for `at_once` tiles.  A 64-wide block of K
 // of a pair takes 2 N cycles of the tensor pipe (172 at least) and (16384 + 64 N) bytes per SM, which arrive at 80 a clock (what a full ring
 // asks for in the 1.4 us a load takes); the first stage arrives after 3000 cycles, and a tile's epilogue, under the MMAs of the next one, takes 1600 cycles and
-// writes 512 N bytes per SM at 32 a clock (16 for residual adds, which shifts all choices alike).  The 1600 count for every tile, not only behind the last: 66 forms
+// writes 512 N bytes per SM at 32 a clock (residual adds leave at 16, which is not counted).  The 1600 count for every tile, not only behind the last: 66 forms
 // of M=212 - 2000, K=64 - 2048 take 1.001 of the time of their best tiles so, 1.05 otherwise, by K=64 most (M=288, n=14464 in tiles of 144 rows 9.8 us, of 32 14.1).
 // Where K is no multiple of 64 the 128 bytes that a box takes of a row lie in two lines, and arrive at 70 a clock (M=501, n=11469+352+1013, K=5832 in tiles
 // of 256 rows 95 us, of 128, which 80 a clock would make the faster ones, 103; over 80 such forms 1.002 of the best, 1.007 otherwise).
