@@ -80,7 +80,7 @@ struct TgpEngine {
     std::vector<cudaEvent_t> ta, tb_;
     uint32_t timed_op0 = 0, timed_nops = 0;
     // whole-run CUDA graph (dense models): capture state and the instantiated graph
-    bool capturing = false, small_loads = false;         // small_loads: no load of the plan is larger than GRAPH_LOAD_MAX, or from a managed pool
+    bool capturing = false, small_loads = false;         // small_loads: every load of the plan can be a kernel's (tgp_graph_load_kernel)
     cudaStream_t cap_cs = nullptr, cap_cp = nullptr;
     cudaEvent_t fork_ev = nullptr, join_cp = nullptr, join_wb = nullptr;
     cudaGraph_t graph = nullptr;
@@ -300,10 +300,10 @@ static int get_event(tgp_ctx *ctx, std::vector<cudaEvent_t> &v, size_t i, cudaEv
 // 8170).  Neighbours that share a load are held to the same size.  Not for plans with larger loads, whose start is a small part of them (blocks of 1 MB: 8230 us,
 // 8680 so; small and large ones mixed: 1253, 1279), and not outside a graph, where the launch costs the host as much as it saves.
 constexpr uint64_t GRAPH_LOAD_MAX = 512u << 10;
+// (Sub-ranges of a pool and arena slots begin on 512 bytes; tgp_run_capture_begin() looks at their sizes.)
 __global__ void __launch_bounds__(512) tgp_graph_load_kernel(const char *src, char *dst, uint64_t bytes) {
     const uint64_t at = ((uint64_t)blockIdx.x * 512 + threadIdx.x) * 16;
-    if (at + 16 <= bytes) *reinterpret_cast<uint4 *>(dst + at) = __ldcs(reinterpret_cast<const uint4 *>(src + at));
-    else for (uint64_t i = at; i < bytes; ++i) dst[i] = src[i];
+    if (at < bytes) *reinterpret_cast<uint4 *>(dst + at) = __ldcs(reinterpret_cast<const uint4 *>(src + at));
 }
 
 // Enqueue, in plan order, every command whose wait_op has been enqueued (wait_op <= limit).
@@ -344,8 +344,7 @@ static int pump(tgp_ctx *ctx, int32_t limit, cudaStream_t copy, uint32_t *n_cmds
             // a copy of a few hundred KiB is mostly latency, while merging megabytes would only delay the first tensor.
             size_t last = e->next_cmd;
             uint64_t span_bytes = c.bytes;
-            const char *mapped = pool.dev_alias ? pool.dev_alias + c.pool_off : nullptr;
-            const bool by_kernel = c.kind == CMD_H2D && e->capturing && e->small_loads && mapped && (((uintptr_t)mapped | (uintptr_t)dev) & 15u) == 0;
+            const bool by_kernel = c.kind == CMD_H2D && e->capturing && e->small_loads;
             const uint64_t span_max = by_kernel ? GRAPH_LOAD_MAX : 1u << 20;
             if (c.kind == CMD_H2D && g_merge_copies)
                 while (last + 1 < pl.cmds.size()) {
@@ -357,7 +356,7 @@ static int pump(tgp_ctx *ctx, int32_t limit, cudaStream_t copy, uint32_t *n_cmds
                     ++last;
                 }
             if (by_kernel) {
-                tgp_graph_load_kernel<<<(uint32_t)((span_bytes + 8191) / 8192), 512, 0, mine>>>(mapped, dev, span_bytes);
+                tgp_graph_load_kernel<<<(uint32_t)((span_bytes + 8191) / 8192), 512, 0, mine>>>(pool.dev_alias + c.pool_off, dev, span_bytes);
                 CU(ctx, cudaGetLastError());
             } else if (c.kind == CMD_H2D) {
                 CU(ctx, cudaMemcpyAsync(dev, host, span_bytes, cudaMemcpyHostToDevice, mine));
@@ -1196,8 +1195,10 @@ extern "C" int tgp_run_capture_begin(tgp_ctx *ctx, void *compute_stream, void *c
     e->n_copy = 1;                                       // in a graph the joins of several copy branches cost more than they hide (measured: the tiny
                                                          // configuration at 512 KiB blocks replays at 0.56 / 0.52 / 0.51 of its roofline with 1 / 2 / 3 copy streams)
     e->small_loads = true;
-    for (const TgpCmd &c : ctx->plan.cmds)               // (a kernel that reads a managed pool would fault its pages in, one by one, and move them)
-        e->small_loads &= c.kind != CMD_H2D || (c.bytes <= GRAPH_LOAD_MAX && ctx->pools[ctx->tensors[c.tensor].pool].flags != TGP_POOL_MANAGED);
+    for (const TgpCmd &c : ctx->plan.cmds) {             // (a kernel that reads a managed pool would fault its pages in, one by one, and move them)
+        const TgpPool &pool = ctx->pools[ctx->tensors[c.tensor].pool];
+        e->small_loads &= c.kind != CMD_H2D || (c.bytes <= GRAPH_LOAD_MAX && c.bytes % 16 == 0 && pool.flags != TGP_POOL_MANAGED && pool.dev_alias);
+    }
     CU(ctx, cudaStreamBeginCapture(e->cap_cs, cudaStreamCaptureModeRelaxed));
     // fork: the copy and write-back streams join the capture
     cudaError_t er = cudaEventRecord(e->fork_ev, e->cap_cs);
